@@ -17,6 +17,8 @@
 // that a node can take 2^20 contributions of the largest size without
 // overflow; the fixed point then resolves 2^-42 of that size, far below fp32
 // rounding of the contributions themselves.
+#include <algorithm>
+
 #include "launch.h"
 #include "profile.h"
 
@@ -34,57 +36,47 @@ int blocks_for(int64_t n)
 
 // Cell and offset of the position x + u along an axis of n points, clamped
 // into [0, n - 1]; returns whether the position was inside (a non-finite u
-// counts as outside, at 0). The integer part of u is split off first, so x +
-// u is not rounded in fp32.
-__device__ __forceinline__ bool field_axis(int x, float u, int n, int &cell, float &f)
+// counts as outside: NaN and -inf at 0, +inf at n - 1). No branches: u is
+// clamped to [lo, hi] = [-x, n - 1 - x] (exact floats, axes are shorter than
+// 2^22), and one round-toward-minus-infinity add of 1.5 * 2^23 leaves floor(u)
+// in the low mantissa bits; the integer part is split off first, so x + u is
+// not rounded in fp32.
+__device__ __forceinline__ bool field_axis(int x, float u, float lo, float hi, int n,
+                                                int &cell, float &f)
 {
-    const float fl = floorf(u);
-    if (!(fabsf(fl) < 1.0e9f)) {  // non-finite or far outside
-        const bool hi = u > 0.0f;   // NaN -> low face
-        cell = hi ? n - 2 : 0;
-        f = hi ? 1.0f : 0.0f;
-        return false;
-    }
-    const int iy = x + (int)fl;
-    const float fr = u - fl;
-    if (iy < 0) {
-        cell = 0;
-        f = 0.0f;
-        return false;
-    }
-    if (iy > n - 1 || (iy == n - 1 && fr > 0.0f)) {
-        cell = n - 2;
-        f = 1.0f;
-        return false;
-    }
+    constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23, bit pattern 0x4B400000
+    const float uc = fminf(fmaxf(u, lo), hi);
+    const float t = __fadd_rd(uc, kMagic);
+    const int iy = x + (__float_as_int(t) - 0x4B400000);
+    const float fr = uc - (t - kMagic);
     cell = min(iy, n - 2);
-    f = fr + (float)(iy - cell);
-    return true;
+    f = iy > cell ? fr + 1.0f : fr;  // the last face: all weight on the last point
+    return u >= lo && u <= hi;
 }
 
-struct FieldSample {
-    int cell[3];
-    float f[3];
-    bool in[3];
-};
-
-// (the field read is u * sc; sc is a power of two, so the product is exact)
+// Interpolant of one component (times sc) in the cell at p, every linear step
+// as fma(1 - f, a, f b). In 3D the two z faces are packed pairs.
 template <int D>
-__device__ __forceinline__ FieldSample field_sample(const Grid &g, int x, int y, int z,
-                                                    const float *__restrict__ u, int64_t v,
-                                                    float sc = 1.0f)
+__device__ __forceinline__ float interp_field(const float *__restrict__ p, int sy, int sz,
+                                              float fx, float fy, float fz, float sc)
 {
-    FieldSample s;
-    s.in[0] = field_axis(x, __ldg(u + v) * sc, g.X, s.cell[0], s.f[0]);
-    s.in[1] = field_axis(y, __ldg(u + g.nv + v) * sc, g.Y, s.cell[1], s.f[1]);
-    if (D == 3) {
-        s.in[2] = field_axis(z, __ldg(u + 2 * (int64_t)g.nv + v) * sc, g.Z, s.cell[2], s.f[2]);
+    const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
+    if constexpr (D == 2) {
+        const float c0 = fmaf(gx, __ldg(p) * sc, fx * (__ldg(p + 1) * sc));
+        const float c1 = fmaf(gx, __ldg(p + sy) * sc, fx * (__ldg(p + sy + 1) * sc));
+        return fmaf(gy, c0, fy * c1);
     } else {
-        s.cell[2] = 0;
-        s.f[2] = 0.0f;
-        s.in[2] = false;
+        const float *q = p + sz;
+        const float2 a = make_float2(__ldg(p) * sc, __ldg(q) * sc);
+        const float2 b = make_float2(__ldg(p + 1) * sc, __ldg(q + 1) * sc);
+        const float2 c = make_float2(__ldg(p + sy) * sc, __ldg(q + sy) * sc);
+        const float2 d = make_float2(__ldg(p + sy + 1) * sc, __ldg(q + sy + 1) * sc);
+        const float2 gx2 = make_float2(gx, gx), fx2 = make_float2(fx, fx);
+        const float2 c0 = __ffma2_rn(gx2, a, __fmul2_rn(fx2, b));
+        const float2 c1 = __ffma2_rn(gx2, c, __fmul2_rn(fx2, d));
+        const float2 r = __ffma2_rn(make_float2(gy, gy), c0, __fmul2_rn(make_float2(fy, fy), c1));
+        return fmaf(gz, r.x, fz * r.y);
     }
-    return s;
 }
 
 __global__ void __launch_bounds__(kDiffeoThreads)
@@ -95,52 +87,80 @@ __global__ void __launch_bounds__(kDiffeoThreads)
         out[e] = in[e] * s;
 }
 
-// One squaring: out = u + u~(x + u), the field read as u * sc (sc = 2^-K on
-// the first squaring, which then reads v itself and also writes u_0 = v sc
-// to u0 when given; otherwise 1). Scaling by a power of two is exact, so
-// this equals scaling v in a pass of its own first.
-template <int D, bool SCALED>
-__global__ void __launch_bounds__(kDiffeoThreads, 8)
-    k_compose(Grid g, const float *__restrict__ u, float *__restrict__ out, float scale,
-              float *__restrict__ u0)
+// One squaring of a 2D field: out = u + u~(x + u), the field read as u * sc
+// (sc = 2^-K on the first squaring, which then reads v itself and also writes
+// u_0 = v sc to u0 when given; otherwise 1). Scaling by a power of two is
+// exact, so this equals scaling v in a pass of its own first.
+template <bool SCALED>
+__global__ void __launch_bounds__(kDiffeoThreads)
+    k_compose2(Grid g, const float *__restrict__ u, float *__restrict__ out, float scale,
+               float *__restrict__ u0)
 {
     const float sc = SCALED ? scale : 1.0f;  // a compile-time 1 on every squaring but the first
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < g.nv;
-         v += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(v % g.X), y = (int)((v / g.X) % g.Y), z = (int)(v / ((int64_t)g.X * g.Y));
-        const FieldSample s = field_sample<D>(g, x, y, z, u, v, sc);
-        const int64_t base = ((int64_t)s.cell[2] * g.Y + s.cell[1]) * g.X + s.cell[0];
-        const int64_t sx = 1, sy = g.X, sz = (int64_t)g.X * g.Y;
-#pragma unroll
-        for (int i = 0; i < D; ++i) {
-            const float *p = u + (int64_t)i * g.nv + base;
-            float r;
-            if (D == 3) {
-                const float c00 = (1.0f - s.f[0]) * (__ldg(p) * sc) + s.f[0] * (__ldg(p + sx) * sc);
-                const float c10 =
-                    (1.0f - s.f[0]) * (__ldg(p + sy) * sc) + s.f[0] * (__ldg(p + sy + sx) * sc);
-                const float c01 =
-                    (1.0f - s.f[0]) * (__ldg(p + sz) * sc) + s.f[0] * (__ldg(p + sz + sx) * sc);
-                const float c11 = (1.0f - s.f[0]) * (__ldg(p + sz + sy) * sc) +
-                                  s.f[0] * (__ldg(p + sz + sy + sx) * sc);
-                const float c0 = (1.0f - s.f[1]) * c00 + s.f[1] * c10;
-                const float c1 = (1.0f - s.f[1]) * c01 + s.f[1] * c11;
-                r = (1.0f - s.f[2]) * c0 + s.f[2] * c1;
-            } else {
-                const float c0 = (1.0f - s.f[0]) * (__ldg(p) * sc) + s.f[0] * (__ldg(p + sx) * sc);
-                const float c1 =
-                    (1.0f - s.f[0]) * (__ldg(p + sy) * sc) + s.f[0] * (__ldg(p + sy + sx) * sc);
-                r = (1.0f - s.f[1]) * c0 + s.f[1] * c1;
-            }
-            if constexpr (SCALED) {
-                const float own = __ldg(u + (int64_t)i * g.nv + v) * sc;
-                if (u0)
-                    u0[(int64_t)i * g.nv + v] = own;
-                out[(int64_t)i * g.nv + v] = own + r;
-            } else {
-                out[(int64_t)i * g.nv + v] = __ldg(u + (int64_t)i * g.nv + v) + r;
-            }
+    const int v = blockIdx.x * kDiffeoThreads + threadIdx.x;
+    if (v >= g.nv)
+        return;
+    const int y = v / g.X, x = v - y * g.X;
+    const float a0 = __ldg(u + v) * sc, a1 = __ldg(u + g.nv + v) * sc;
+    int cx, cy;
+    float fx, fy;
+    field_axis(x, a0, -(float)x, (float)(g.X - 1 - x), g.X, cx, fx);
+    field_axis(y, a1, -(float)y, (float)(g.Y - 1 - y), g.Y, cy, fy);
+    const float *p = u + cy * g.X + cx;
+    const float r0 = interp_field<2>(p, g.X, 0, fx, fy, 0.0f, sc);
+    const float r1 = interp_field<2>(p + g.nv, g.X, 0, fx, fy, 0.0f, sc);
+    if (SCALED && u0) {
+        u0[v] = a0;
+        u0[g.nv + v] = a1;
+    }
+    out[v] = a0 + r0;
+    out[g.nv + v] = a1 + r1;
+}
+
+// The same squaring of a 3D field: a warp takes 32 consecutive x of a row and
+// marches through zc slices, so that the index arithmetic is done once per
+// column and the cells come without branches. Bound by the L1's wavefronts (24
+// gathers a voxel) and their latency: 134 us a squaring at 256 x 256 x 160
+// (217 us the scaled one) with 64-bit divisions and branches per voxel, 81 us
+// (98 us) so; two passes over memory take 37 us. Four blocks per SM (64
+// registers) against six: 525 and 544 us for the six squarings; 16 slices
+// instead of 8 took 544, 32 took 830.
+template <bool SCALED>
+__global__ void __launch_bounds__(kDiffeoThreads, 4)
+    k_compose3(Grid g, const float *__restrict__ u, float *__restrict__ out, float scale,
+               float *__restrict__ u0, int ntx, int nty, int zc)
+{
+    const float sc = SCALED ? scale : 1.0f;
+    const int tile = blockIdx.x, tx = tile % ntx, ty = (tile / ntx) % nty, tz = tile / (ntx * nty);
+    const int x = tx * 32 + (threadIdx.x & 31), y = ty * (kDiffeoThreads / 32) + (threadIdx.x >> 5);
+    if (x >= g.X || y >= g.Y)
+        return;
+    const int sy = g.X, sz = g.X * g.Y;
+    const float xlo = -(float)x, xhi = (float)(g.X - 1 - x);
+    const float ylo = -(float)y, yhi = (float)(g.Y - 1 - y);
+    const int z1 = min((tz + 1) * zc, g.Z);
+    const float *u1 = u + g.nv, *u2 = u1 + g.nv;
+    float *o1 = out + g.nv, *o2 = o1 + g.nv;
+    int v = (tz * zc * g.Y + y) * g.X + x;
+    for (int z = tz * zc; z < z1; ++z, v += sz) {
+        const float a0 = __ldg(u + v) * sc, a1 = __ldg(u1 + v) * sc, a2 = __ldg(u2 + v) * sc;
+        int cx, cy, cz;
+        float fx, fy, fz;
+        field_axis(x, a0, xlo, xhi, g.X, cx, fx);
+        field_axis(y, a1, ylo, yhi, g.Y, cy, fy);
+        field_axis(z, a2, -(float)z, (float)(g.Z - 1 - z), g.Z, cz, fz);
+        const int base = (cz * g.Y + cy) * g.X + cx;  // nv < 2^31
+        const float r0 = interp_field<3>(u + base, sy, sz, fx, fy, fz, sc);
+        const float r1 = interp_field<3>(u1 + base, sy, sz, fx, fy, fz, sc);
+        const float r2 = interp_field<3>(u2 + base, sy, sz, fx, fy, fz, sc);
+        if (SCALED && u0) {
+            u0[v] = a0;
+            u0[g.nv + v] = a1;
+            u0[2 * (int64_t)g.nv + v] = a2;
         }
+        out[v] = a0 + r0;
+        o1[v] = a1 + r1;
+        o2[v] = a2 + r2;
     }
 }
 
@@ -172,103 +192,111 @@ __device__ __forceinline__ float fixed_scale(unsigned int maxbits)
     return ldexpf(1.0f, s);
 }
 
-// Local terms of one squaring's adjoint into h, the scatter into acc.
-// Consecutive lanes take consecutive voxels (all lanes run the same number of
-// iterations, so the warp shuffles see every lane). The scatter to the +x
-// corners of a sample is usually the scatter to the -x corners of the next
-// lane's sample (a smooth displacement keeps neighbours in neighbouring
-// cells): that lane adds it to its own contribution, as 64-bit integers, and
-// one atomic serves both. Integer addition is exact, so the result does not
-// change.
+// round(p) of |p| <= 2^42 as a 64-bit integer, ties to even like
+// __float2ll_rn, by fp32 adds. The 64-bit conversion instructions issue at the
+// rate of this part's FP64 pipe, 16 cycles per warp, and 24 of them per voxel
+// bounded the scatter. p = hi 2^21 + lo with hi = round(p / 2^21), |hi| <= 2^21,
+// and lo = p - hi 2^21, |lo| <= 2^20, exact (a multiple of p's last place);
+// adding 1.5 * 2^23 leaves an integer in the low mantissa bits. hi 2^21 is
+// even, so round(p) = hi 2^21 + round(lo) to even.
+__device__ __forceinline__ long long fixed_of(float p)
+{
+    constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23
+    constexpr int kBits = 0x4B400000;
+    const float t = __fmaf_rn(p, 0x1p-21f, kMagic);
+    const float lo = __fmaf_rn(__fsub_rn(t, kMagic), -0x1p21f, p);
+    const int ih = __float_as_int(t) - kBits;
+    const int il = __float_as_int(__fadd_rn(lo, kMagic)) - kBits;
+    return (long long)ih * 2097152ll + il;
+}
+
+// (float)q rounded to nearest even, like __ll2float_rn, with 32-bit
+// conversions only: the top 32 significant bits of |q| with the bits below
+// them or-ed into the last (more than the 24 that are kept, so one rounding).
+__device__ __forceinline__ float float_of(long long q)
+{
+    const unsigned long long m = q < 0 ? 0ull - (unsigned long long)q : (unsigned long long)q;
+    const unsigned hi = (unsigned)(m >> 32), lo = (unsigned)m;
+    float f;
+    if (hi == 0) {
+        f = __uint2float_rn(lo);
+    } else {
+        const int k = __clz(hi);
+        const unsigned top = __funnelshift_l(lo, hi, k), rest = lo << k;
+        // top has its leading bit set; times 2^(32 - k), exact
+        f = __uint2float_rn(top | (rest != 0u)) * __int_as_float((127 + 32 - k) << 23);
+    }
+    return q < 0 ? -f : f;
+}
+
+// The scatter of one sample whose gradient component does not fit the fixed
+// point, one component (its plane's accumulators from the sample's cell).
 template <int D>
+__device__ __noinline__ void scatter_far(unsigned long long *acc, int sy, int sz,
+                                         float fx, float fy, float fz, float gv, float S)
+{
+    for (int c = 0; c < (1 << D); ++c) {
+        const int cx = c & 1, cy = (c >> 1) & 1, cz = c >> 2;
+        const float wyz = (cy ? fy : 1.0f - fy) * (D == 3 ? (cz ? fz : 1.0f - fz) : 1.0f);
+        const float w = (cx ? fx : 1.0f - fx) * wyz;
+        atomicAdd(acc + cz * sz + cy * sy + cx,
+                  (unsigned long long)__float2ll_rn(w * gv * S));
+    }
+}
+
+// Local terms of one squaring's adjoint of a 2D field into h, the scatter into
+// acc.
 __global__ void __launch_bounds__(kDiffeoThreads)
-    k_compose_adjoint(Grid g, const float *__restrict__ u, const float *__restrict__ gin,
-                      float *__restrict__ h, unsigned long long *__restrict__ acc,
-                      const unsigned int *__restrict__ maxbits)
+    k_compose_adjoint2(Grid g, const float *__restrict__ u, const float *__restrict__ gin,
+                       float *__restrict__ h, unsigned long long *__restrict__ acc,
+                       const unsigned int *__restrict__ maxbits)
 {
     const float S = fixed_scale(*maxbits);
-    const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t v0 = blockIdx.x * (int64_t)blockDim.x; v0 < g.nv; v0 += stride) {
-        const int64_t v = v0 + threadIdx.x;
-        const bool valid = v < g.nv;
-        const int64_t vv = valid ? v : 0;
-        const int x = (int)(vv % g.X), y = (int)((vv / g.X) % g.Y),
-                  z = (int)(vv / ((int64_t)g.X * g.Y));
-        const FieldSample s = field_sample<D>(g, x, y, z, u, vv);
-        const int base = (s.cell[2] * g.Y + s.cell[1]) * g.X + s.cell[0];  // nv < 2^31
-        const int sy = g.X, sz = g.X * g.Y;
-        float gv[D], loc[D];
+    const int v = blockIdx.x * kDiffeoThreads + threadIdx.x;
+    if (v >= g.nv)
+        return;
+    const int y = v / g.X, x = v - y * g.X, sy = g.X;
+    int cx, cy;
+    float fx, fy;
+    const bool inx = field_axis(x, __ldg(u + v), -(float)x, (float)(g.X - 1 - x), g.X, cx, fx);
+    const bool iny =
+        field_axis(y, __ldg(u + g.nv + v), -(float)y, (float)(g.Y - 1 - y), g.Y, cy, fy);
+    const int base = cy * g.X + cx;
+    const float gx = 1.0f - fx, gy = 1.0f - fy;
+    const float gv[2] = {__ldg(gin + v), __ldg(gin + g.nv + v)};
+    float loc[2] = {gv[0], gv[1]};
+    // derivative of the interpolant of each component at the sample
 #pragma unroll
-        for (int i = 0; i < D; ++i) {
-            gv[i] = valid ? __ldg(gin + (int64_t)i * g.nv + vv) : 0.0f;
-            loc[i] = gv[i];
+    for (int i = 0; i < 2; ++i) {
+        const float *p = u + (int64_t)i * g.nv + base;
+        const float a00 = __ldg(p), a01 = __ldg(p + 1), a10 = __ldg(p + sy),
+                    a11 = __ldg(p + sy + 1);
+        const float d0 = fmaf(gy, a01 - a00, fy * (a11 - a10));
+        const float d1 = fmaf(gx, a10 - a00, fx * (a11 - a01));
+        if (inx)
+            loc[0] = fmaf(d0, gv[i], loc[0]);
+        if (iny)
+            loc[1] = fmaf(d1, gv[i], loc[1]);
+    }
+    h[v] = loc[0];
+    h[g.nv + v] = loc[1];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        unsigned long long *ap = acc + (int64_t)i * g.nv + base;
+        const float gs = gv[i] * S;
+        if (!(fabsf(gs) <= 0x1p42f)) {  // an infinity or a NaN
+            scatter_far<2>(ap, sy, 0, fx, fy, 0.0f, gv[i], S);
+            continue;
         }
-        // derivative of the interpolant of each component at the sample
-#pragma unroll
-        for (int i = 0; i < D; ++i) {
-            const float *p = u + (int64_t)i * g.nv + base;
-            float d0, d1, d2 = 0.0f;
-            if (D == 3) {
-                const float a000 = __ldg(p), a001 = __ldg(p + 1), a010 = __ldg(p + sy),
-                            a011 = __ldg(p + sy + 1), a100 = __ldg(p + sz),
-                            a101 = __ldg(p + sz + 1), a110 = __ldg(p + sz + sy),
-                            a111 = __ldg(p + sz + sy + 1);
-                const float fx = s.f[0], fy = s.f[1], fz = s.f[2];
-                d0 = (1.0f - fz) * ((1.0f - fy) * (a001 - a000) + fy * (a011 - a010)) +
-                     fz * ((1.0f - fy) * (a101 - a100) + fy * (a111 - a110));
-                d1 = (1.0f - fz) * ((1.0f - fx) * (a010 - a000) + fx * (a011 - a001)) +
-                     fz * ((1.0f - fx) * (a110 - a100) + fx * (a111 - a101));
-                d2 = (1.0f - fy) * ((1.0f - fx) * (a100 - a000) + fx * (a101 - a001)) +
-                     fy * ((1.0f - fx) * (a110 - a010) + fx * (a111 - a011));
-            } else {
-                const float a00 = __ldg(p), a01 = __ldg(p + 1), a10 = __ldg(p + sy),
-                            a11 = __ldg(p + sy + 1);
-                d0 = (1.0f - s.f[1]) * (a01 - a00) + s.f[1] * (a11 - a10);
-                d1 = (1.0f - s.f[0]) * (a10 - a00) + s.f[0] * (a11 - a01);
-            }
-            if (s.in[0])
-                loc[0] = fmaf(d0, gv[i], loc[0]);
-            if (s.in[1])
-                loc[1] = fmaf(d1, gv[i], loc[1]);
-            if (D == 3 && s.in[2])
-                loc[D - 1] = fmaf(d2, gv[i], loc[D - 1]);
-        }
-        if (valid) {
-#pragma unroll
-            for (int i = 0; i < D; ++i)
-                h[(int64_t)i * g.nv + vv] = loc[i];
-        }
-        // transposed interpolation: the sample's weights onto the corners,
-        // the -x and +x corner of each (y, z) corner pair together
-#pragma unroll
-        for (int cz = 0; cz < (D == 3 ? 2 : 1); ++cz)
-#pragma unroll
-            for (int cy = 0; cy < 2; ++cy) {
-                const float wyz = (cy ? s.f[1] : 1.0f - s.f[1]) *
-                                  (D == 3 ? (cz ? s.f[2] : 1.0f - s.f[2]) : 1.0f);
-                const float w0 = (1.0f - s.f[0]) * wyz, w1 = s.f[0] * wyz;
-                const int n0 = valid ? base + cz * sz + cy * sy : -2, n1 = valid ? n0 + 1 : -4;
-                // the previous lane's +x node is this lane's -x node: take its value;
-                // the next lane's -x node is this lane's +x node: give this value
-                const int prev_n1 = __shfl_up_sync(FULL, n1, 1);
-                const int next_n0 = __shfl_down_sync(FULL, n0, 1);
-                const bool take = lane > 0 && prev_n1 == n0;
-                const bool give = lane < 31 && next_n0 == n1;
-#pragma unroll
-                for (int i = 0; i < D; ++i) {
-                    long long q0 = valid ? __float2ll_rn(w0 * gv[i] * S) : 0ll;
-                    const long long q1 = valid ? __float2ll_rn(w1 * gv[i] * S) : 0ll;
-                    const long long qp = __shfl_up_sync(FULL, q1, 1);
-                    if (take)
-                        q0 += qp;
-                    if (q0 != 0)
-                        atomicAdd(acc + (int64_t)i * g.nv + n0, (unsigned long long)q0);
-                    if (!give && q1 != 0)
-                        atomicAdd(acc + (int64_t)i * g.nv + n1, (unsigned long long)q1);
-                }
-            }
+        auto add = [&](unsigned long long *a, float w) {
+            const long long q = fixed_of(w * gs);
+            if (q != 0)
+                atomicAdd(a, (unsigned long long)q);
+        };
+        add(ap, gx * gy);
+        add(ap + 1, fx * gy);
+        add(ap + sy, gx * fy);
+        add(ap + sy + 1, fx * fy);
     }
 }
 
@@ -276,7 +304,17 @@ __global__ void __launch_bounds__(kDiffeoThreads)
 // largest |h| (the next step's input) into *maxnext, as k_absmax does, so that
 // step needs no pass of its own for it.
 // With dest (the last step), (h + acc / 2^s) * dsc goes to dest instead, for
-// every entry (the exponential's final 2^-K).
+// every entry (the exponential's final 2^-K). Memory bound (24 bytes a value:
+// acc and h read and written): four consecutive values a thread, so that 48
+// bytes are in flight per thread and loads are 16 bytes.
+// (256 x 256 x 160: 220 us with one value a thread and the 64-bit conversion,
+// 107 us so, the rate of a copy.)
+__device__ __forceinline__ float finish_one(float hv, unsigned long long a, float inv)
+{
+    const long long q = (long long)a;
+    return q != 0 ? hv + float_of(q) * inv : hv;
+}
+
 __global__ void __launch_bounds__(kDiffeoThreads)
     k_compose_finish(float *__restrict__ h, unsigned long long *__restrict__ acc, int64_t n,
                      const unsigned int *__restrict__ maxbits, unsigned int *__restrict__ maxnext,
@@ -284,30 +322,43 @@ __global__ void __launch_bounds__(kDiffeoThreads)
 {
     const float inv = 1.0f / fixed_scale(*maxbits);  // a power of two: exact
     float m = 0.0f;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const long long q = (long long)acc[e];
-        float hv;
-        if (dest) {
-            hv = h[e];
-            if (q != 0) {
-                hv = hv + __ll2float_rn(q) * inv;
-                acc[e] = 0ull;
-            }
-            dest[e] = hv * dsc;
-            continue;
-        }
-        if (q != 0) {
-            hv = h[e] + __ll2float_rn(q) * inv;
-            h[e] = hv;
-            acc[e] = 0ull;
-        } else if (maxnext) {
-            hv = h[e];
-        } else {
-            continue;
-        }
-        const float a = fabsf(hv);
+    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    auto put = [&](float v) {
+        const float a = fabsf(v);
         m = a > m ? a : m;  // a NaN never wins
+    };
+    for (int64_t e = tid; e < n / 4; e += stride) {
+        ulonglong2 *ap = reinterpret_cast<ulonglong2 *>(acc) + 2 * e;
+        float4 *hp = reinterpret_cast<float4 *>(h) + e;
+        const ulonglong2 a0 = ap[0], a1 = ap[1];
+        float4 v = *hp;
+        v.x = finish_one(v.x, a0.x, inv);
+        v.y = finish_one(v.y, a0.y, inv);
+        v.z = finish_one(v.z, a1.x, inv);
+        v.w = finish_one(v.w, a1.y, inv);
+        ap[0] = make_ulonglong2(0ull, 0ull);
+        ap[1] = make_ulonglong2(0ull, 0ull);
+        if (dest) {
+            reinterpret_cast<float4 *>(dest)[e] =
+                make_float4(v.x * dsc, v.y * dsc, v.z * dsc, v.w * dsc);
+        } else {
+            *hp = v;
+            put(v.x);
+            put(v.y);
+            put(v.z);
+            put(v.w);
+        }
+    }
+    for (int64_t e = n / 4 * 4 + tid; e < n; e += stride) {
+        const float v = finish_one(h[e], acc[e], inv);
+        acc[e] = 0ull;
+        if (dest) {
+            dest[e] = v * dsc;
+        } else {
+            h[e] = v;
+            put(v);
+        }
     }
     if (!maxnext)
         return;
@@ -324,6 +375,170 @@ __global__ void __launch_bounds__(kDiffeoThreads)
             m = fmaxf(m, wm[w]);
         atomicMax(maxnext, __float_as_uint(m));
     }
+}
+
+// fixed_of in its two halves, value hi 2^21 + lo. Sums of a few stay far inside
+// 32 bits each.
+struct Fix {
+    int hi, lo;
+};
+
+// fixed_of of the pair (w.x g, w.y g) with packed operations.
+__device__ __forceinline__ void fixed_pair(float2 w, float gs, Fix &a, Fix &b)
+{
+    constexpr float kMagic = 12582912.0f;
+    constexpr int kBits = 0x4B400000;
+    const float2 m = make_float2(kMagic, kMagic);
+    const float2 p = __fmul2_rn(w, make_float2(gs, gs));
+    const float2 t = __ffma2_rn(p, make_float2(0x1p-21f, 0x1p-21f), m);
+    const float2 d = __fadd2_rn(t, make_float2(-kMagic, -kMagic));
+    const float2 l = __fadd2_rn(__ffma2_rn(d, make_float2(-0x1p21f, -0x1p21f), p), m);
+    a = {__float_as_int(t.x) - kBits, __float_as_int(l.x) - kBits};
+    b = {__float_as_int(t.y) - kBits, __float_as_int(l.y) - kBits};
+}
+
+__device__ __forceinline__ void add_fix(unsigned long long *a, Fix q)
+{
+    atomicAdd(a, (unsigned long long)((long long)q.hi * 2097152ll + q.lo));
+}
+
+// The adjoint of one squaring of a 3D field in tiles like k_compose3's: local
+// terms into h, the scatter into acc. Bound by the accumulator's atomics in L2
+// (a microbenchmark: 20 G warp instructions of 32 consecutive 64-bit
+// reductions per second). The contributions to the far z corners of a sample
+// stay in registers as exact integers and join the next slice's sample when
+// its cell is the next one, which halves them where the displacement is
+// smooth; exchanging x corners between lanes as well (as a version before did)
+// takes more instructions than it saves atomics. 256 x 256 x 160: 428 us a step
+// with 64-bit conversions and x corners merged by shuffles, 358 us with
+// fixed_of, 335 us so; 467 us with one atomic per corner. Sums are of exact
+// integers, so the result is the same whatever merges.
+__global__ void __launch_bounds__(kDiffeoThreads, 3)
+    k_compose_adjoint3(Grid g, const float *__restrict__ u, const float *__restrict__ gin,
+                       float *__restrict__ h, unsigned long long *__restrict__ acc,
+                       const unsigned int *__restrict__ maxbits, int ntx, int nty, int zc)
+{
+    const float S = fixed_scale(*maxbits);
+    const int tile = blockIdx.x, tx = tile % ntx, ty = (tile / ntx) % nty, tz = tile / (ntx * nty);
+    const int x = tx * 32 + (threadIdx.x & 31), y = ty * (kDiffeoThreads / 32) + (threadIdx.x >> 5);
+    if (x >= g.X || y >= g.Y)
+        return;
+    const int sy = g.X, sz = g.X * g.Y;
+    const float xlo = -(float)x, xhi = (float)(g.X - 1 - x);
+    const float ylo = -(float)y, yhi = (float)(g.Y - 1 - y);
+    const int z1 = min((tz + 1) * zc, g.Z);
+    const float *u1 = u + g.nv, *u2 = u1 + g.nv;
+    const float *g1 = gin + g.nv, *g2 = g1 + g.nv;
+    float *h1 = h + g.nv, *h2 = h1 + g.nv;
+    int v = (tz * zc * g.Y + y) * g.X + x;
+    // contributions to the corners (y, x) at the far z of the last sample's cell
+    Fix carry[3][4] = {};
+    int cb = -1;  // their first node
+#pragma unroll 1
+    for (int z = tz * zc; z < z1; ++z, v += sz) {
+        const float a0 = __ldg(u + v), a1 = __ldg(u1 + v), a2 = __ldg(u2 + v);
+        const float gv[3] = {__ldg(gin + v), __ldg(g1 + v), __ldg(g2 + v)};
+        int cx, cy, cz;
+        float fx, fy, fz;
+        const bool inx = field_axis(x, a0, xlo, xhi, g.X, cx, fx);
+        const bool iny = field_axis(y, a1, ylo, yhi, g.Y, cy, fy);
+        const bool inz = field_axis(z, a2, -(float)z, (float)(g.Z - 1 - z), g.Z, cz, fz);
+        const int base = (cz * g.Y + cy) * g.X + cx;
+        const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
+        float loc[3] = {gv[0], gv[1], gv[2]};
+        const float2 m1 = make_float2(-1.0f, -1.0f), fx2 = make_float2(fx, fx),
+                     fy2 = make_float2(fy, fy);
+        // derivative of the interpolant of each component at the sample, the
+        // corners of the two z faces as packed pairs
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const float *p = (i == 0 ? u : i == 1 ? u1 : u2) + base;
+            const float *q = p + sz;
+            const float2 c00 = make_float2(__ldg(p), __ldg(q));
+            const float2 c01 = make_float2(__ldg(p + 1), __ldg(q + 1));
+            const float2 c10 = make_float2(__ldg(p + sy), __ldg(q + sy));
+            const float2 c11 = make_float2(__ldg(p + sy + 1), __ldg(q + sy + 1));
+            const float2 d0 = __ffma2_rn(c00, m1, c01), d1 = __ffma2_rn(c10, m1, c11);
+            const float2 dx = __ffma2_rn(fy2, __ffma2_rn(d0, m1, d1), d0);
+            const float2 l0 = __ffma2_rn(fx2, d0, c00), l1 = __ffma2_rn(fx2, d1, c10);
+            const float2 dy = __ffma2_rn(l0, m1, l1), b = __ffma2_rn(fy2, dy, l0);
+            if (inx)
+                loc[0] = fmaf(fmaf(fz, dx.y - dx.x, dx.x), gv[i], loc[0]);
+            if (iny)
+                loc[1] = fmaf(fmaf(fz, dy.y - dy.x, dy.x), gv[i], loc[1]);
+            if (inz)
+                loc[2] = fmaf(b.y - b.x, gv[i], loc[2]);
+        }
+        h[v] = loc[0];
+        h1[v] = loc[1];
+        h2[v] = loc[2];
+        const float2 wy0 = make_float2(gx * gy, fx * gy), wy1 = make_float2(gx * fy, fx * fy);
+        const float2 gz2 = make_float2(gz, gz), fz2 = make_float2(fz, fz);
+        const float2 w00 = __fmul2_rn(wy0, gz2), w10 = __fmul2_rn(wy1, gz2);
+        const float2 w01 = __fmul2_rn(wy0, fz2), w11 = __fmul2_rn(wy1, fz2);
+        const bool on = cb == base;
+        if (!on && cb >= 0) {
+            unsigned long long *ap = acc + cb;
+#pragma unroll
+            for (int i = 0; i < 3; ++i, ap += g.nv) {
+                add_fix(ap, carry[i][0]);
+                add_fix(ap + 1, carry[i][1]);
+                add_fix(ap + sy, carry[i][2]);
+                add_fix(ap + sy + 1, carry[i][3]);
+            }
+        }
+        unsigned long long *ap = acc + base;
+#pragma unroll
+        for (int i = 0; i < 3; ++i, ap += g.nv) {
+            float gs = gv[i] * S;
+            if (!(fabsf(gs) <= 0x1p42f)) {  // an infinity or a NaN
+                scatter_far<3>(ap, sy, sz, fx, fy, fz, gv[i], S);
+                gs = 0.0f;
+            }
+            Fix q[4];
+            fixed_pair(w00, gs, q[0], q[1]);
+            fixed_pair(w10, gs, q[2], q[3]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                q[k].hi += on ? carry[i][k].hi : 0;
+                q[k].lo += on ? carry[i][k].lo : 0;
+            }
+            fixed_pair(w01, gs, carry[i][0], carry[i][1]);
+            fixed_pair(w11, gs, carry[i][2], carry[i][3]);
+            add_fix(ap, q[0]);
+            add_fix(ap + 1, q[1]);
+            add_fix(ap + sy, q[2]);
+            add_fix(ap + sy + 1, q[3]);
+        }
+        cb = base + sz;
+    }
+    unsigned long long *ap = acc + cb;
+#pragma unroll
+    for (int i = 0; i < 3; ++i, ap += g.nv) {
+        add_fix(ap, carry[i][0]);
+        add_fix(ap + 1, carry[i][1]);
+        add_fix(ap + sy, carry[i][2]);
+        add_fix(ap + sy + 1, carry[i][3]);
+    }
+}
+
+// Tiles of the marching kernels: 32 x 8 columns a block and zc slices, 8 of
+// them or fewer while that leaves less than eight blocks per SM.
+struct Tiles {
+    int ntx, nty, zc, blocks;
+};
+
+Tiles tiles_of(const Grid &g)
+{
+    Tiles t;
+    t.ntx = (g.X + 31) / 32;
+    t.nty = (g.Y + kDiffeoThreads / 32 - 1) / (kDiffeoThreads / 32);
+    t.zc = 8;
+    while (t.zc > 1 &&
+           (int64_t)t.ntx * t.nty * ((g.Z + t.zc - 1) / t.zc) < 8 * (int64_t)device_sms())
+        t.zc /= 2;
+    t.blocks = t.ntx * t.nty * ((g.Z + t.zc - 1) / t.zc);
+    return t;
 }
 
 template <int D>
@@ -365,12 +580,24 @@ cudaError_t exp_run(const Grid &g, int K, const float *v, float *u, float *traj,
             nxt = traj + (int64_t)(k + 1) * n;
         else
             nxt = ((K - 1 - k) % 2 == 0) ? u : tmp;
-        if (k == 0 && scale0 != 1.0f)
-            k_compose<D, true><<<blocks_for(g.nv), kDiffeoThreads, 0, s>>>(g, cur, nxt, scale0,
-                                                                          traj);
-        else
-            k_compose<D, false><<<blocks_for(g.nv), kDiffeoThreads, 0, s>>>(g, cur, nxt, 1.0f,
-                                                                           nullptr);
+        const bool scaled = k == 0 && scale0 != 1.0f;
+        float *u0 = scaled ? traj : nullptr;
+        if constexpr (D == 3) {
+            const Tiles t = tiles_of(g);
+            if (scaled)
+                k_compose3<true><<<t.blocks, kDiffeoThreads, 0, s>>>(g, cur, nxt, scale0, u0,
+                                                                     t.ntx, t.nty, t.zc);
+            else
+                k_compose3<false><<<t.blocks, kDiffeoThreads, 0, s>>>(g, cur, nxt, 1.0f, u0,
+                                                                      t.ntx, t.nty, t.zc);
+        } else {
+            if (scaled)
+                k_compose2<true><<<blocks_for(g.nv), kDiffeoThreads, 0, s>>>(g, cur, nxt, scale0,
+                                                                             u0);
+            else
+                k_compose2<false><<<blocks_for(g.nv), kDiffeoThreads, 0, s>>>(g, cur, nxt, 1.0f,
+                                                                              u0);
+        }
         e = cudaGetLastError();
         cur = nxt;
     }
@@ -393,7 +620,7 @@ cudaError_t exp_adjoint_run(const Grid &g, int K, const float *traj, const float
     // mx[0], mx[1]: the largest |g| of a step's input; the first from a pass of
     // its own, the others from the previous step's finish
     if (e == cudaSuccess && K > 0) {
-        e = cudaMemsetAsync(mx, 0, 2 * sizeof(unsigned int), s);
+        e = cudaMemsetAsync(mx, 0, sizeof(unsigned int), s);
         if (e == cudaSuccess) {
             k_absmax<<<blocks_for(n) < 4 * device_sms() ? blocks_for(n) : 4 * device_sms(),
                        kDiffeoThreads, 0, s>>>(gin, n, mx);
@@ -402,12 +629,20 @@ cudaError_t exp_adjoint_run(const Grid &g, int K, const float *traj, const float
     }
     for (int k = K - 1, j = 0; k >= 0 && e == cudaSuccess; --k, j ^= 1) {
         const float *u = traj + (int64_t)k * n;
-        unsigned int *mcur = mx + j, *mnext = k > 0 ? mx + (j ^ 1) : nullptr;
-        k_compose_adjoint<D><<<blocks_for(g.nv), kDiffeoThreads, 0, s>>>(g, u, gin, out, acc, mcur);
+        const unsigned int *mcur = mx + j;
+        unsigned int *mnext = k > 0 ? mx + (j ^ 1) : nullptr;
+        if constexpr (D == 3) {
+            const Tiles t = tiles_of(g);
+            k_compose_adjoint3<<<t.blocks, kDiffeoThreads, 0, s>>>(g, u, gin, out, acc, mcur,
+                                                                   t.ntx, t.nty, t.zc);
+        } else {
+            k_compose_adjoint2<<<blocks_for(g.nv), kDiffeoThreads, 0, s>>>(g, u, gin, out, acc,
+                                                                           mcur);
+        }
         if (mnext && (e = cudaMemsetAsync(mnext, 0, sizeof(unsigned int), s)) != cudaSuccess)
             break;
         // the last step writes (its result) * 2^-K to gv directly
-        const int fb = blocks_for(n) < 4 * device_sms() ? blocks_for(n) : 4 * device_sms();
+        const int fb = std::min(blocks_for((n + 3) / 4), 16 * device_sms());
         k_compose_finish<<<fb, kDiffeoThreads, 0, s>>>(out, acc, n, mcur, mnext,
                                                        k == 0 ? gv : nullptr, ldexpf(1.0f, -K));
         e = cudaGetLastError();
