@@ -405,21 +405,24 @@ static al_status objective_unfused(const al_problem *pr, const Grid &g, const La
         return AL_ERR_CUDA;
     if (launch_warp(g, moving, u, W, m, s) != cudaSuccess)
         return AL_ERR_CUDA;
-    if (launch_similarity(g, pr->sim.kind, pr->sim.lcc_window, pr->sim.eps, fixed, W, m, vals,
-                          grad_ctrl ? gW : nullptr, scratch, s) != cudaSuccess)
+    int gw = GW_NONE, count = 0;
+    if (launch_similarity_scalars(g, pr->sim.kind, pr->sim.lcc_window, pr->sim.eps, fixed, W, m,
+                                  true, vals, grad_ctrl ? gW : nullptr, scratch, &gw, s) != cudaSuccess)
         return AL_ERR_CUDA;
-    if (launch_regulariser(g, u, pr->lambda, vals + 2, grad_ctrl ? gu : nullptr, scratch, s) !=
-        cudaSuccess)
+    // R's partials stay where nothing is read any more until the last launch:
+    // dS/dW's buffer, or W's when dS/dW (LCC, unscaled) is in use (nv floats hold
+    // the at most ceil(nv / 256) doubles)
+    double *part = (double *)(gw == GW_SCALED ? W : gW);
+    const AdjointArgs a = {moving, fixed, W, gW, m, (const double *)scratch};
+    if (launch_regulariser_adjoint(g, u, pr->lambda, grad_ctrl ? gw : GW_NONE, a,
+                                   grad_ctrl ? gu : nullptr, part, &count, nullptr,
+                                   s) != cudaSuccess)
         return AL_ERR_CUDA;
-    if (grad_ctrl) {
-        if (launch_warp_adjoint(g, moving, u, m, gW, gu, 1, s) != cudaSuccess)
-            return AL_ERR_CUDA;
-        if (launch_displacement_adjoint(g, L, gu, grad_ctrl, scratch, s) != cudaSuccess)
-            return AL_ERR_CUDA;
-    }
-    return launched(launch_combine(vals, vals + 2, pr->lambda, value_dev, s));
+    if (grad_ctrl && launch_displacement_adjoint(g, L, gu, grad_ctrl, scratch, s) != cudaSuccess)
+        return AL_ERR_CUDA;
+    return launched(
+        launch_combine(vals, part, count, 1.0 / (double)g.nv, pr->lambda, value_dev, s));
 }
-
 al_status al_objective_grad_unfused(const al_problem *pr, const float *fixed, const float *moving,
                                     const float *ctrl, double *value_dev, float *grad_ctrl,
                                     void *workspace, size_t workspace_bytes, al_stream stream)
@@ -663,7 +666,8 @@ al_status al_exp_field_adjoint(const al_grid *gr, int32_t steps, const float *tr
         !aligned16(grad_velocity) || !aligned16(workspace))
         return AL_ERR_ALIGN;
     return launched(
-        launch_exp_adjoint(g, steps, trajectory, grad_disp, grad_velocity, workspace, S(stream)));
+        launch_exp_adjoint(g, steps, trajectory, grad_disp, grad_velocity, workspace, nullptr,
+                           S(stream)));
 }
 
 size_t al_exp_field_adjoint_workspace_bytes(const al_grid *gr)
@@ -754,21 +758,31 @@ al_status al_objective_grad_diffeo(const al_problem *pr, int32_t steps, const fl
     double *vals = (double *)(w + lay.vals);
     void *scratch = w + lay.scratch;
     const cudaStream_t s = S(stream);
+    int gw = GW_NONE, count = 0;
     if (launch_displacement(g, L, ctrl, v, s) != cudaSuccess ||
         launch_exp(g, steps, v, u, traj, nullptr, s) != cudaSuccess ||
         launch_warp(g, moving, u, W, m, s) != cudaSuccess ||
-        launch_similarity(g, pr->sim.kind, pr->sim.lcc_window, pr->sim.eps, fixed, W, m, vals,
-                          grad_ctrl ? gW : nullptr, scratch, s) != cudaSuccess ||
-        launch_regulariser(g, u, pr->lambda, vals + 2, grad_ctrl ? gu : nullptr, scratch, s) !=
-            cudaSuccess)
+        launch_similarity_scalars(g, pr->sim.kind, pr->sim.lcc_window, pr->sim.eps, fixed, W, m,
+                                  true, vals, grad_ctrl ? gW : nullptr, scratch, &gw, s) != cudaSuccess)
         return AL_ERR_CUDA;
-    if (grad_ctrl) {
-        if (launch_warp_adjoint(g, moving, u, m, gW, gu, 1, s) != cudaSuccess ||
-            launch_exp_adjoint(g, steps, traj, gu, gv, scratch, s) != cudaSuccess ||
-            launch_displacement_adjoint(g, L, gv, grad_ctrl, scratch, s) != cudaSuccess)
-            return AL_ERR_CUDA;
-    }
-    return launched(launch_combine(vals, vals + 2, pr->lambda, value_dev, s));
+    // R's partials: as in objective_unfused
+    double *part = (double *)(gw == GW_SCALED ? W : gW);
+    const AdjointArgs a = {moving, fixed, W, gW, m, (const double *)scratch};
+    // the similarity's scalars are in use until the gradient is formed, so the
+    // exponential's largest |gradient| goes to the last value slot first
+    unsigned int *mx = (unsigned int *)(vals + 3);
+    if (grad_ctrl && cudaMemsetAsync(mx, 0, sizeof(unsigned int), s) != cudaSuccess)
+        return AL_ERR_CUDA;
+    if (launch_regulariser_adjoint(g, u, pr->lambda, grad_ctrl ? gw : GW_NONE, a,
+                                   grad_ctrl ? gu : nullptr, part, &count,
+                                   grad_ctrl ? mx : nullptr, s) != cudaSuccess)
+        return AL_ERR_CUDA;
+    if (grad_ctrl &&
+        (launch_exp_adjoint(g, steps, traj, gu, gv, scratch, mx, s) != cudaSuccess ||
+         launch_displacement_adjoint(g, L, gv, grad_ctrl, scratch, s) != cudaSuccess))
+        return AL_ERR_CUDA;
+    return launched(
+        launch_combine(vals, part, count, 1.0 / (double)g.nv, pr->lambda, value_dev, s));
 }
 
 al_status al_lcc_set_wait(int32_t drop_slice)

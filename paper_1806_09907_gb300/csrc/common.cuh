@@ -389,6 +389,71 @@ __device__ __forceinline__ void block_reduce_fd(float (&v)[K], double (&out)[K],
     }
 }
 
+// An fp32 sum kept as its value and the sum of its rounding errors (each add's
+// error is exact, Knuth's two-sum), about 2^-45 of the terms' size: what an
+// FP64 sum of fp32 terms is wanted for, on the full-rate fp32 pipe (an FP64 add
+// or conversion takes 16 cycles per warp on this part).
+struct Sum2 {
+    float s = 0.0f, e = 0.0f;
+    __device__ __forceinline__ void add(float v)
+    {
+        const float t = __fadd_rn(s, v);
+        const float b = __fsub_rn(t, s);
+        e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b)));
+        s = t;
+    }
+    __device__ __forceinline__ void add(const Sum2 &o)
+    {
+        e = __fadd_rn(e, o.e);
+        add(o.s);
+    }
+    // a sum that left fp32's range has a NaN for its error
+    __device__ __forceinline__ double value() const
+    {
+        return isfinite(s) ? (double)s + (double)e : (double)s;
+    }
+};
+
+// Deterministic block sum of K Sum2 per thread (fixed trees): pairs within each
+// warp, then warp 0 adds the warps' sums in FP64, which has the range for any
+// number of them. Valid in thread 0. `scratch` holds at least
+// K * (blockDim.x / 32) doubles.
+template <int K>
+__device__ __forceinline__ void block_reduce_s2(Sum2 (&v)[K], double (&out)[K], double *scratch)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nwarp = (blockDim.x + 31) >> 5;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            Sum2 o;
+            o.s = __shfl_down_sync(0xffffffffu, v[k].s, off);
+            o.e = __shfl_down_sync(0xffffffffu, v[k].e, off);
+            v[k].add(o);
+        }
+    }
+    __syncthreads();  // scratch may still be in use by a previous call
+    if (lane == 0)
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            scratch[k * nwarp + warp] = v[k].value();
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+        out[k] = 0.0;
+    if (warp == 0) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            double t = lane < nwarp ? scratch[k * nwarp + lane] : 0.0;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1)
+                t += __shfl_down_sync(0xffffffffu, t, off);
+            out[k] = t;
+        }
+    }
+}
+
 // Adam's bias-correction factor 1 / (1 - beta^t) at step t >= 1 (Kingma and
 // Ba), as float. beta^t is formed in FP64 by binary exponentiation (at most
 // 2 log2 t products) instead of a library pow: FP64 issues slowly on this

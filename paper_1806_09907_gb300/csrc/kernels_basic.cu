@@ -1,5 +1,7 @@
 // Step kernels of the unfused path: A1 B-spline expansion, A6 its adjoint,
 // A2 warp, A5 warp adjoint, A4 diffusion regulariser (voxel form).
+#include <algorithm>
+
 #include "launch.h"
 
 namespace airgb {
@@ -8,53 +10,68 @@ namespace {
 
 constexpr int kDispTX = 128;  // x extent of a displacement tile (threads)
 constexpr int kDispTY = 8;    // rows per tile
-constexpr int kDispMaxJX = kDispTX + 5;  // control columns a tile can touch (delta >= 1)
-constexpr int kDispMaxJY = kDispTY + 5;
+
+// Control columns / rows a tile of n voxels can touch.
+__host__ __device__ constexpr int disp_span(int n, int delta) { return (n - 1) / delta + 5; }
 
 // A1: u_i(x) = sum_j c_{i,j} prod_k w. One CTA = one z slice, 8 rows, 128
 // columns. Separable: z-contraction of the touched control block into smem,
-// then y-contraction per row, then 4 x-taps per voxel.
+// then y-contraction per row, then 4 x-taps per voxel. The two buffers are
+// sized by the spacing (4.4 KB at 6, not the 33 KB that spacing 1 needs), so
+// that 16 CTAs are resident per SM instead of 6: it is the latency of the three
+// short phases that bounds the kernel (256 x 256 x 160, spacing 6: 63.6 us with
+// the fixed buffers and divided indices, 49.3 us so; writing u takes 18.5 us).
 template <int D>
-__global__ void __launch_bounds__(kDispTX) k_displacement(Grid g, Lattice L,
-                                                          const float *__restrict__ c,
-                                                          float *__restrict__ u)
+__global__ void __launch_bounds__(kDispTX)
+    k_displacement(Grid g, const __grid_constant__ Lattice L, const float *__restrict__ c,
+                   float *__restrict__ u)
 {
-    __shared__ float tz[D][kDispMaxJY][kDispMaxJX];
-    __shared__ float ty[D][kDispTY][kDispMaxJX];
+    extern __shared__ float disp_smem[];
     const int x0 = blockIdx.x * kDispTX, y0 = blockIdx.y * kDispTY, z = blockIdx.z;
     const int delta = L.delta;
     const int jx0 = x0 / delta, jy0 = y0 / delta;
     const int xl = min(x0 + kDispTX, g.X) - 1, yl = min(y0 + kDispTY, g.Y) - 1;
     const int njx = xl / delta + 4 - jx0, njy = yl / delta + 4 - jy0;
+    float *tz = disp_smem;                                    // [D][njy][njx]
+    float *ty = tz + D * disp_span(kDispTY, delta) * njx;     // [D][kDispTY][njx]
     const int qz = z / delta, pz = z - qz * delta;
+    // a warp per row of control columns, so that no index is divided
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // z contraction
-    for (int e = threadIdx.x; e < D * njy * njx; e += blockDim.x) {
-        const int i = e / (njy * njx), r = e - i * njy * njx;
-        const int jyl = r / njx, jxl = r - jyl * njx;
-        const int jy = jy0 + jyl, jx = jx0 + jxl;
-        float acc = 0.0f;
-        if (D == 3) {
+    for (int row = warp; row < D * njy; row += kDispTX / 32) {
+        const int i = D == 3 ? (row >= njy) + (row >= 2 * njy) : (row >= njy);
+        const int jyl = row - i * njy;
+        const float *src = D == 3
+                               ? c + (((int64_t)i * L.nz + qz) * L.ny + jy0 + jyl) * L.nx + jx0
+                               : c + ((int64_t)i * L.ny + jy0 + jyl) * L.nx + jx0;
+        const int64_t pl = (int64_t)L.ny * L.nx;
+        for (int j = lane; j < njx; j += 32) {
+            float acc = 0.0f;
+            if (D == 3) {
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
-                acc = fmaf(L.w[pz][a],
-                           __ldg(c + (((int64_t)i * L.nz + qz + a) * L.ny + jy) * L.nx + jx), acc);
-        } else {
-            acc = __ldg(c + ((int64_t)i * L.ny + jy) * L.nx + jx);
+                for (int a = 0; a < 4; ++a)
+                    acc = fmaf(L.w[pz][a], __ldg(src + a * pl + j), acc);
+            } else {
+                acc = __ldg(src + j);
+            }
+            tz[row * njx + j] = acc;
         }
-        tz[i][jyl][jxl] = acc;
     }
     __syncthreads();
     // y contraction
-    for (int e = threadIdx.x; e < D * kDispTY * njx; e += blockDim.x) {
-        const int i = e / (kDispTY * njx), r = e - i * kDispTY * njx;
-        const int yr = r / njx, jxl = r - yr * njx;
+#pragma unroll 2
+    for (int row = warp; row < D * kDispTY; row += kDispTX / 32) {
+        const int i = row / kDispTY, yr = row % kDispTY;
         const int y = min(y0 + yr, g.Y - 1);
         const int qy = y / delta, py = y - qy * delta;
-        float acc = 0.0f;
-#pragma unroll
-        for (int b = 0; b < 4; ++b)
-            acc = fmaf(L.w[py][b], tz[i][qy - jy0 + b][jxl], acc);
-        ty[i][yr][jxl] = acc;
+        const float b0 = L.w[py][0], b1 = L.w[py][1], b2 = L.w[py][2], b3 = L.w[py][3];
+        const float *t = tz + (i * njy + qy - jy0) * njx;
+        for (int j = lane; j < njx; j += 32) {
+            float acc = fmaf(b0, t[j], 0.0f);
+            acc = fmaf(b1, t[njx + j], acc);
+            acc = fmaf(b2, t[2 * njx + j], acc);
+            ty[row * njx + j] = fmaf(b3, t[3 * njx + j], acc);
+        }
     }
     __syncthreads();
     const int x = x0 + threadIdx.x;
@@ -63,91 +80,277 @@ __global__ void __launch_bounds__(kDispTX) k_displacement(Grid g, Lattice L,
     const int qx = x / delta, px = x - qx * delta;
     const float w0 = L.w[px][0], w1 = L.w[px][1], w2 = L.w[px][2], w3 = L.w[px][3];
     const int jxl = qx - jx0;
-    for (int yr = 0; yr < kDispTY && y0 + yr < g.Y; ++yr) {
+#pragma unroll
+    for (int yr = 0; yr < kDispTY; ++yr) {
+        if (y0 + yr >= g.Y)
+            break;
         const int64_t v = ((int64_t)z * g.Y + y0 + yr) * g.X + x;
 #pragma unroll
         for (int i = 0; i < D; ++i) {
-            float acc = w0 * ty[i][yr][jxl];
-            acc = fmaf(w1, ty[i][yr][jxl + 1], acc);
-            acc = fmaf(w2, ty[i][yr][jxl + 2], acc);
-            acc = fmaf(w3, ty[i][yr][jxl + 3], acc);
+            const float *t = ty + (i * kDispTY + yr) * njx + jxl;
+            float acc = w0 * t[0];
+            acc = fmaf(w1, t[1], acc);
+            acc = fmaf(w2, t[2], acc);
+            acc = fmaf(w3, t[3], acc);
             u[(int64_t)i * g.nv + v] = acc;
         }
     }
 }
 
-// A6, one axis of the separable transpose: out[.., j, ..] = sum over the
-// 4*delta inputs t of axis `axis` in j's support of w(t, j) * in[.., t, ..].
-// Each output is a gather in fixed order (ascending t). Shapes are given
-// as (outer, len_in, inner) -> (outer, len_out, inner).
-__global__ void k_bspline_transpose_axis(const float *__restrict__ in, float *__restrict__ out,
-                                         int64_t outer, int len_in, int len_out, int64_t inner,
-                                         Lattice L)
+// A6 along x and y for one z slice of one component and a band of bj control
+// rows: out[o][jy][jx] = sum_y w(y, jy) sum_x w(x, jx) in[o][y][x]. A warp
+// walks the rows of the band's support: a row comes in coalesced loads (the
+// next one's are in flight meanwhile), is contracted along x in two steps (each
+// cell's four weighted sums of its delta voxels, then per control point the
+// sum over the up to four cells it supports) and kept; then the kept rows are
+// contracted along y. A row's buffers belong to its warp, so only the y step
+// waits for the block, and lanes stride along x, so no index is divided. Fixed
+// order, no atomics. 256 x 256 x 160, spacing 6: 168 us for x and 31 us for y
+// with one thread per output reading 4 delta values delta apart, 70 us so;
+// reading the field takes 18.5 us.
+constexpr int kTransThreads = 256;
+constexpr int kTransWarps = kTransThreads / 32;
+constexpr int kTransWidth = 320;  // voxels of a staged row at most
+
+struct TransPlan {
+    int jt, bj;         // control columns and rows of a block
+    int nxt, nbands;    // blocks per slice along x and y
+    size_t smem;
+};
+
+// A block's columns: up to kTransWidth voxels of support (a whole row of most
+// volumes; the buffers stay within 48 KB); its rows: 16, so that 3/16 of the
+// rows are read twice, or 8 or 4 when that leaves fewer than four blocks per SM
+// of a 152-SM GB300.
+TransPlan trans_plan(const Grid &g, const Lattice &L)
 {
-    const int64_t total = outer * len_out * inner;
+    TransPlan t;
+    t.jt = std::min(L.nx, std::max(4, std::min(kTransWidth / L.delta - 3, 96)));
+    t.nxt = (L.nx + t.jt - 1) / t.jt;
+    for (t.bj = 16; t.bj > 4; t.bj /= 2)
+        if ((int64_t)g.ndim * g.Z * t.nxt * ((L.ny + t.bj - 1) / t.bj) >= 4 * 152)
+            break;
+    t.nbands = (L.ny + t.bj - 1) / t.bj;
+    const int cells = t.jt + 3;
+    t.smem = 4 * (kMaxDelta * 4 + (size_t)kTransWarps * cells * (L.delta + 4) +
+                  (size_t)(t.bj + 3) * L.delta * t.jt);
+    return t;
+}
+
+__global__ void __launch_bounds__(kTransThreads)
+    k_transpose_xy(const float *__restrict__ in, float *__restrict__ out, int X, int Y, int jt,
+                   int bj, int nxt, int nbands, const __grid_constant__ Lattice L)
+{
+    extern __shared__ __align__(16) float trans_sm[];
+    const int delta = L.delta, cells = jt + 3, width = cells * delta;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float4 *w4 = reinterpret_cast<float4 *>(trans_sm);   // [delta] weights of a phase
+    float *raw = trans_sm + kMaxDelta * 4 + warp * width;                       // [width]
+    float *sums = trans_sm + kMaxDelta * 4 + kTransWarps * width + warp * cells * 4;  // [4][cells]
+    float *t1 = trans_sm + kMaxDelta * 4 + kTransWarps * (width + cells * 4);   // [rows][jt]
+    if (threadIdx.x < delta)
+        w4[threadIdx.x] = make_float4(L.w[threadIdx.x][0], L.w[threadIdx.x][1],
+                                      L.w[threadIdx.x][2], L.w[threadIdx.x][3]);
+    const int tile = blockIdx.x, tx = tile % nxt, band = (tile / nxt) % nbands;
+    const int64_t o = tile / (nxt * nbands);
+    const int jx0 = tx * jt, jy0 = band * bj;
+    const int nj = min(jt, L.nx - jx0), nb = min(bj, L.ny - jy0);
+    // voxel (column) 0 of the tile, row 0 of the band
+    const int x0 = (jx0 - 3) * delta, y0 = (jy0 - 3) * delta;
+    const int rows = (nb + 3) * delta;
+    const float *src = in + o * Y * X + x0;
+    constexpr int PER = kTransWidth / 32;
+    float next[PER];
+    auto fetch = [&](int r) {
+        const int y = y0 + r;
+        const bool ok = r < rows && y >= 0 && y < Y;
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            const int i = lane + 32 * k;
+            next[k] = ok && i < width && x0 + i >= 0 && x0 + i < X
+                          ? __ldg(src + (int64_t)y * X + i) : 0.0f;
+        }
+    };
+    fetch(warp);
+    __syncthreads();
+    for (int r = warp; r < rows; r += kTransWarps) {
+#pragma unroll
+        for (int k = 0; k < PER; ++k)
+            if (lane + 32 * k < width)
+                raw[lane + 32 * k] = next[k];
+        __syncwarp();
+        fetch(r + kTransWarps);
+        for (int e = lane; e < cells; e += 32) {
+            const float *v = raw + e * delta;
+            float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, s3 = 0.0f;
+#pragma unroll 4
+            for (int k = 0; k < delta; ++k) {
+                const float a = v[k];
+                const float4 w = w4[k];
+                s0 = fmaf(w.x, a, s0);
+                s1 = fmaf(w.y, a, s1);
+                s2 = fmaf(w.z, a, s2);
+                s3 = fmaf(w.w, a, s3);
+            }
+            sums[e] = s0;
+            sums[cells + e] = s1;
+            sums[2 * cells + e] = s2;
+            sums[3 * cells + e] = s3;
+        }
+        __syncwarp();
+        // control point j is fed by the cells j - 3 .. j (weights 3 .. 0)
+        for (int j = lane; j < nj; j += 32) {
+            const float *d = sums + j;
+            t1[r * jt + j] =
+                ((d[3 * cells] + d[2 * cells + 1]) + d[cells + 2]) + d[3];
+        }
+    }
+    __syncthreads();
+    for (int jb = warp; jb < nb; jb += kTransWarps)
+        for (int j = lane; j < nj; j += 32) {
+            const float *v = t1 + jb * delta * jt + j;
+            float s3 = 0.0f, s2 = 0.0f, s1 = 0.0f, s0 = 0.0f;
+#pragma unroll 4
+            for (int k = 0; k < delta; ++k, v += jt) {
+                const float4 w = w4[k];
+                s3 = fmaf(w.w, v[0], s3);
+                s2 = fmaf(w.z, v[delta * jt], s2);
+                s1 = fmaf(w.y, v[2 * delta * jt], s1);
+                s0 = fmaf(w.x, v[3 * delta * jt], s0);
+            }
+            out[(o * L.ny + jy0 + jb) * L.nx + jx0 + j] = ((s3 + s2) + s1) + s0;
+        }
+}
+
+// A6 along z: in[o][Z][inner] -> out[o][nz][inner], one thread per output,
+// ascending z.
+__global__ void __launch_bounds__(kTransThreads)
+    k_transpose_z(const float *__restrict__ in, float *__restrict__ out, int outer, int Z, int nz,
+                  int inner, const __grid_constant__ Lattice L)
+{
+    const int64_t total = (int64_t)outer * nz * inner;
     const int delta = L.delta;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
          e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t o = e / ((int64_t)len_out * inner);
-        const int64_t r = e - o * len_out * inner;
-        const int j = (int)(r / inner);
-        const int64_t k = r - (int64_t)j * inner;
-        const int t0 = max(0, (j - 3) * delta), t1 = min(len_in, (j + 1) * delta);
-        const float *src = in + (o * len_in) * inner + k;
+        const int o = (int)(e / ((int64_t)nz * inner));
+        const int64_t r = e - (int64_t)o * nz * inner;
+        const int j = (int)(r / inner), k = (int)(r - (int64_t)j * inner);
+        const float *src = in + (int64_t)o * Z * inner + k;
         float acc = 0.0f;
-        for (int t = t0; t < t1; ++t) {
-            const int q = t / delta, p = t - q * delta;
-            acc = fmaf(L.w[p][j - q], __ldg(src + (int64_t)t * inner), acc);
+#pragma unroll
+        for (int a = 3; a >= 0; --a) {
+            const int t0 = (j - a) * delta;
+            if (t0 < 0)
+                continue;
+            const int n = min(delta, Z - t0);
+            const float *p = src + (int64_t)t0 * inner;
+#pragma unroll 4
+            for (int q = 0; q < n; ++q)
+                acc = fmaf(L.w[q][a], __ldg(p + (int64_t)q * inner), acc);
         }
         out[e] = acc;
     }
 }
 
-// A2: backward warp with mask.
-template <int D>
-__global__ void k_warp(Grid g, const float *__restrict__ M, const float *__restrict__ u,
-                       float *__restrict__ W, uint8_t *__restrict__ mask)
+// ---- marching tiles ---------------------------------------------------------
+// The point-wise kernels take 32 x 8 columns a block (a warp per row) and march
+// through zc slices, so that a column's index arithmetic is done once and its
+// z neighbours stay in registers. Tiles beyond the grid's blocks follow in
+// order (tile += gridDim).
+constexpr int kTileX = 32, kTileY = 8;
+
+struct March {
+    int ntx, nty, ntiles, zc;
+};
+
+// Slices of a column: 16, fewer while that leaves less than eight blocks per SM.
+March march_plan(const Grid &g)
 {
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < g.nv;
-         v += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(v % g.X);
-        const int64_t r = v / g.X;
-        const int y = (int)(r % g.Y), z = (int)(r / g.Y);
-        AxisSample sx, sy, sz;
-        bool in = axis_sample(x, __ldg(u + v), g.X, sx);
-        in &= axis_sample(y, __ldg(u + g.nv + v), g.Y, sy);
-        if (D == 3)
-            in &= axis_sample(z, __ldg(u + 2 * (int64_t)g.nv + v), g.Z, sz);
-        float w = 0.0f;
-        if (in)
-            w = (D == 3) ? trilinear(M, g.X, g.Y, g.Z, sx, sy, sz).v : bilinear(M, g.X, g.Y, sx, sy).v;
-        W[v] = w;
+    March m;
+    m.ntx = (g.X + kTileX - 1) / kTileX;
+    m.nty = (g.Y + kTileY - 1) / kTileY;
+    m.zc = 16;
+    while (m.zc > 1 &&
+           (int64_t)m.ntx * m.nty * ((g.Z + m.zc - 1) / m.zc) < 8 * (int64_t)device_sms())
+        m.zc /= 2;
+    m.ntiles = m.ntx * m.nty * ((g.Z + m.zc - 1) / m.zc);
+    return m;
+}
+
+struct Column {
+    int x, y, z0, z1;
+    bool on;
+};
+
+__device__ __forceinline__ Column march_column(const Grid &g, const March &m, int tile)
+{
+    Column c;
+    c.x = tile % m.ntx * kTileX + (threadIdx.x & 31);
+    c.y = tile / m.ntx % m.nty * kTileY + (threadIdx.x >> 5);
+    c.z0 = tile / (m.ntx * m.nty) * m.zc;
+    c.z1 = min(c.z0 + m.zc, g.Z);
+    c.on = c.x < g.X && c.y < g.Y;
+    return c;
+}
+
+// Sample at voxel (x, y, z) displaced by (ux, uy, uz): inside, and the
+// interpolant there (whatever the cell holds when outside). All axes are
+// shorter than 2^22 (axis_cell).
+template <int D>
+__device__ __forceinline__ bool sample_at(const Grid &g, const float *__restrict__ M, int x, int y,
+                                          int z, float ux, float uy, float uz, Interp &ip)
+{
+    AxisSample sx, sy, sz;
+    bool in = axis_cell(x, ux, -(float)x, (float)(g.X - 1 - x), g.X, sx.cell, sx.f);
+    in &= axis_cell(y, uy, -(float)y, (float)(g.Y - 1 - y), g.Y, sy.cell, sy.f);
+    if (D == 3)
+        in &= axis_cell(z, uz, -(float)z, (float)(g.Z - 1 - z), g.Z, sz.cell, sz.f);
+    ip = D == 3 ? trilinear(M, g.X, g.Y, g.Z, sx, sy, sz) : bilinear(M, g.X, g.Y, sx, sy);
+    return in;
+}
+
+// A2: backward warp with mask. Bound by instructions and gathers, not memory
+// (256 x 256 x 160: 74 us with 64-bit index divisions and branches per voxel,
+// 53 us so; its bytes take 32 us).
+template <int D>
+__global__ void __launch_bounds__(kTileX *kTileY)
+    k_warp(Grid g, March mp, const float *__restrict__ M, const float *__restrict__ u,
+           float *__restrict__ W, uint8_t *__restrict__ mask)
+{
+    const Column c = march_column(g, mp, blockIdx.x);
+    if (!c.on)
+        return;
+    const int sz = g.X * g.Y;
+    int v = (c.z0 * g.Y + c.y) * g.X + c.x;
+#pragma unroll 2
+    for (int z = c.z0; z < c.z1; ++z, v += sz) {
+        Interp ip;
+        const bool in = sample_at<D>(g, M, c.x, c.y, z, __ldg(u + v), __ldg(u + g.nv + v),
+                                     D == 3 ? __ldg(u + 2 * (int64_t)g.nv + v) : 0.0f, ip);
+        W[v] = in ? ip.v : 0.0f;
         mask[v] = in ? 1 : 0;
     }
 }
 
 // A5: grad_disp[k] = mask * grad_warped * dM~/dy_k (+ grad_disp if accumulate).
 template <int D>
-__global__ void k_warp_adjoint(Grid g, const float *__restrict__ M, const float *__restrict__ u,
-                               const uint8_t *__restrict__ mask, const float *__restrict__ gw,
-                               float *__restrict__ gu, int accumulate)
+__global__ void __launch_bounds__(kTileX *kTileY)
+    k_warp_adjoint(Grid g, March mp, const float *__restrict__ M, const float *__restrict__ u,
+                   const uint8_t *__restrict__ mask, const float *__restrict__ gw,
+                   float *__restrict__ gu, int accumulate)
 {
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < g.nv;
-         v += (int64_t)gridDim.x * blockDim.x) {
+    const Column c = march_column(g, mp, blockIdx.x);
+    if (!c.on)
+        return;
+    const int sz = g.X * g.Y;
+    int v = (c.z0 * g.Y + c.y) * g.X + c.x;
+    for (int z = c.z0; z < c.z1; ++z, v += sz) {
         float gx = 0.0f, gy = 0.0f, gz = 0.0f;
         const float gwv = __ldg(gw + v);
         if (__ldg(mask + v) && gwv != 0.0f) {
-            const int x = (int)(v % g.X);
-            const int64_t r = v / g.X;
-            const int y = (int)(r % g.Y), z = (int)(r / g.Y);
-            AxisSample sx, sy, sz;
-            bool in = axis_sample(x, __ldg(u + v), g.X, sx);
-            in &= axis_sample(y, __ldg(u + g.nv + v), g.Y, sy);
-            if (D == 3)
-                in &= axis_sample(z, __ldg(u + 2 * (int64_t)g.nv + v), g.Z, sz);
-            if (in) {
-                const Interp ip =
-                    (D == 3) ? trilinear(M, g.X, g.Y, g.Z, sx, sy, sz) : bilinear(M, g.X, g.Y, sx, sy);
+            Interp ip;
+            if (sample_at<D>(g, M, c.x, c.y, z, __ldg(u + v), __ldg(u + g.nv + v),
+                             D == 3 ? __ldg(u + 2 * (int64_t)g.nv + v) : 0.0f, ip)) {
                 gx = gwv * ip.gx;
                 gy = gwv * ip.gy;
                 gz = gwv * ip.gz;
@@ -168,46 +371,135 @@ __global__ void k_warp_adjoint(Grid g, const float *__restrict__ M, const float 
 }
 
 // A4: R = (1/|X|) sum_i sum_k sum_{x_k < N_k-1} (u_i(x+e_k) - u_i(x))^2 and
-// grad = weight * dR/du. One thread per voxel; per-block FP64 partial sums.
-template <int D>
-__global__ void __launch_bounds__(256) k_regulariser(Grid g, const float *__restrict__ u,
-                                                     float gscale, float *__restrict__ gu,
-                                                     double *__restrict__ partials)
+// grad = gscale * its derivative (+ the adjoint of the warp with
+// GW != GW_NONE: mask * dS/dW * dM~/dy, dS/dW formed from the similarity's
+// scalars without a pass of its own). A column's z neighbours are carried in
+// registers and its x and y neighbours come from L1; one FP64 partial per
+// block. 256 x 256 x 160: 139 us (one voxel a thread, an FP64 block reduction
+// per 256 voxels) + 135 us (warp adjoint, reading and writing the gradient
+// again) + 19 us (the scaling of dS/dW), 156 us so; its bytes take 51 us.
+// maxbits (nullable): the largest |grad| as the bits of a float (a NaN never
+// wins), for al_exp_field_adjoint's fixed point.
+template <int D, int GW>
+__global__ void __launch_bounds__(kTileX *kTileY)
+    k_regulariser(Grid g, March mp, const float *__restrict__ u, float gscale,
+                  float *__restrict__ gu, double *__restrict__ partials, AdjointArgs a,
+                  unsigned int *__restrict__ maxbits)
 {
-    __shared__ double red[8];
-    double acc[1] = {0.0};
-    const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (v < g.nv) {
-        const int x = (int)(v % g.X);
-        const int64_t r = v / g.X;
-        const int y = (int)(r % g.Y), z = (int)(r / g.Y);
-        const int64_t st[3] = {1, g.X, (int64_t)g.X * g.Y};
-        const int pos[3] = {x, y, z};
-        const int n[3] = {g.X, g.Y, g.Z};
-        float sum = 0.0f;
+    __shared__ double red[kTileX * kTileY / 32];
+    __shared__ float wm[kTileX * kTileY / 32];
+    Sum2 total[1];
+    float big = 0.0f;
+    float k0 = 0.0f, k1 = 0.0f, k2 = 0.0f, k3 = 0.0f;
+    if (GW == GW_MSE || GW == GW_SCALED)
+        k0 = (float)a.scal[0];
+    if (GW == GW_NCC)
+        k0 = (float)a.scal[0], k1 = (float)a.scal[1], k2 = (float)a.scal[3], k3 = (float)a.scal[4];
+    const int sy = g.X, sz = g.X * g.Y;
+    const int64_t nv = g.nv;
+    for (int tile = blockIdx.x; tile < mp.ntiles; tile += gridDim.x) {
+        const Column c = march_column(g, mp, tile);
+        if (!c.on)
+            continue;
+        int v = (c.z0 * g.Y + c.y) * g.X + c.x;
+        float below[D], cur[D];
 #pragma unroll
         for (int i = 0; i < D; ++i) {
-            const float *ui = u + (int64_t)i * g.nv;
-            const float c = __ldg(ui + v);
-            float lap = 0.0f;  // sum_k (u(x) - u(x-e_k)) - (u(x+e_k) - u(x))
-#pragma unroll
-            for (int k = 0; k < D; ++k) {
-                if (pos[k] + 1 < n[k]) {
-                    const float d = __ldg(ui + v + st[k]) - c;
-                    sum = fmaf(d, d, sum);
-                    lap -= d;
-                }
-                if (pos[k] > 0)
-                    lap += c - __ldg(ui + v - st[k]);
-            }
-            if (gu)
-                gu[(int64_t)i * g.nv + v] = gscale * lap;
+            cur[i] = __ldg(u + i * nv + v);
+            below[i] = D == 3 && c.z0 > 0 ? __ldg(u + i * nv + v - sz) : 0.0f;
         }
-        acc[0] = sum;
+        // neighbours beyond the grid are read at the voxel itself and dropped
+        const bool xu = c.x + 1 < g.X, xd = c.x > 0, yu = c.y + 1 < g.Y, yd = c.y > 0;
+        const int oxu = xu ? 1 : 0, oxd = xd ? -1 : 0, oyu = yu ? sy : 0, oyd = yd ? -sy : 0;
+#pragma unroll 1
+        for (int z = c.z0; z < c.z1; ++z, v += sz) {
+            const bool zu = D == 3 && z + 1 < g.Z, zd = D == 3 && z > 0;
+            float sum = 0.0f, lap[D], next[D], wxu[D], wxd[D], wyu[D], wyd[D];
+#pragma unroll
+            for (int i = 0; i < D; ++i) {
+                const float *ui = u + i * nv + v;
+                next[i] = D == 3 ? __ldg(ui + (zu ? sz : 0)) : 0.0f;
+                wxu[i] = __ldg(ui + oxu);
+                wxd[i] = __ldg(ui + oxd);
+                wyu[i] = __ldg(ui + oyu);
+                wyd[i] = __ldg(ui + oyd);
+            }
+#pragma unroll
+            for (int i = 0; i < D; ++i) {
+                const float m = cur[i];
+                float l = 0.0f;  // sum_k (u(x) - u(x-e_k)) - (u(x+e_k) - u(x))
+                auto up = [&](bool ok, float w) {
+                    const float d = ok ? w - m : 0.0f;
+                    sum = fmaf(d, d, sum);
+                    l -= d;
+                };
+                up(xu, wxu[i]);
+                l += xd ? m - wxd[i] : 0.0f;
+                up(yu, wyu[i]);
+                l += yd ? m - wyd[i] : 0.0f;
+                if (D == 3) {
+                    up(zu, next[i]);
+                    l += zd ? m - below[i] : 0.0f;
+                }
+                lap[i] = l;
+            }
+            total[0].add(sum);
+            if (gu) {
+                float gx = 0.0f, gy = 0.0f, gz = 0.0f;
+                if (GW != GW_NONE) {
+                    const bool on = __ldg(a.mask + v) != 0;
+                    float gwv = 0.0f;
+                    if (on) {
+                        if (GW == GW_MSE)
+                            gwv = k0 * (__ldg(a.W + v) - __ldg(a.F + v));
+                        else if (GW == GW_NCC)
+                            gwv = fmaf(k2, __ldg(a.F + v) - k0, k3 * (__ldg(a.W + v) - k1));
+                        else
+                            gwv = __fmul_rn(__ldg(a.gw + v), k0);
+                    }
+                    if (on && gwv != 0.0f) {
+                        Interp ip;
+                        if (sample_at<D>(g, a.M, c.x, c.y, z, cur[0], cur[1],
+                                         D == 3 ? cur[D - 1] : 0.0f, ip)) {
+                            gx = __fmul_rn(gwv, ip.gx);
+                            gy = __fmul_rn(gwv, ip.gy);
+                            gz = __fmul_rn(gwv, ip.gz);
+                        }
+                    }
+                }
+                const float add[3] = {gx, gy, gz};
+#pragma unroll
+                for (int i = 0; i < D; ++i) {
+                    const float r = __fadd_rn(__fmul_rn(gscale, lap[i]), add[i]);
+                    gu[i * nv + v] = r;
+                    const float ar = fabsf(r);
+                    big = ar > big ? ar : big;
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < D; ++i) {
+                below[i] = cur[i];
+                cur[i] = next[i];
+            }
+        }
     }
-    block_reduce_d<1>(acc, red);
+    double R[1];
+    block_reduce_s2<1>(total, R, red);
     if (threadIdx.x == 0)
-        partials[blockIdx.x] = acc[0];
+        partials[blockIdx.x] = R[0];
+    if (!maxbits)
+        return;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+        big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, off));
+    if ((threadIdx.x & 31) == 0)
+        wm[threadIdx.x >> 5] = big;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kTileX * kTileY / 32; ++w)
+            big = fmaxf(big, wm[w]);
+        atomicMax(maxbits, __float_as_uint(big));
+    }
 }
 
 // Fixed-order sum of `count` partials (one block), scaled, into out[0].
@@ -223,11 +515,19 @@ __global__ void k_sum_partials(const double *__restrict__ partials, int count, d
         out[0] = acc[0] * scale;
 }
 
-__global__ void k_combine(const double *__restrict__ sim, const double *__restrict__ reg,
-                          double lambda, double *__restrict__ out)
+// {J, S, R, n_mask} of the unfused pieces; R as reg[0], or (count > 0) as the
+// fixed-order sum of `count` partials times scale.
+__global__ void __launch_bounds__(256)
+    k_combine(const double *__restrict__ sim, const double *__restrict__ reg, int count,
+              double scale, double lambda, double *__restrict__ out)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        const double S = sim[0], n = sim[1], R = reg[0];
+    __shared__ double red[8];
+    double acc[1] = {0.0};
+    for (int i = threadIdx.x; i < count; i += blockDim.x)
+        acc[0] += reg[i];
+    block_reduce_d<1>(acc, red);
+    if (threadIdx.x == 0) {
+        const double S = sim[0], n = sim[1], R = count > 0 ? acc[0] * scale : reg[0];
         out[0] = S + lambda * R;
         out[1] = S;
         out[2] = R;
@@ -248,10 +548,12 @@ cudaError_t launch_displacement(const Grid &g, const Lattice &L, const float *ct
                                 cudaStream_t s)
 {
     dim3 grid((g.X + kDispTX - 1) / kDispTX, (g.Y + kDispTY - 1) / kDispTY, g.Z);
+    const size_t smem = (size_t)g.ndim * std::min(disp_span(kDispTX, L.delta), L.nx) *
+                        (disp_span(kDispTY, L.delta) + kDispTY) * 4;
     if (g.ndim == 3)
-        k_displacement<3><<<grid, kDispTX, 0, s>>>(g, L, ctrl, disp);
+        k_displacement<3><<<grid, kDispTX, smem, s>>>(g, L, ctrl, disp);
     else
-        k_displacement<2><<<grid, kDispTX, 0, s>>>(g, L, ctrl, disp);
+        k_displacement<2><<<grid, kDispTX, smem, s>>>(g, L, ctrl, disp);
     return cudaGetLastError();
 }
 
@@ -267,24 +569,18 @@ cudaError_t launch_displacement_adjoint(const Grid &g, const Lattice &L, const f
                                         float *grad_ctrl, void *ws, cudaStream_t s)
 {
     const int D = g.ndim;
-    float *t1 = (float *)ws;
-    size_t t1n = (size_t)D * g.Z * g.Y * L.nx;
+    // x and y: (D*Z, Y, X) -> (D*Z, ny, nx); in 2D this is the result, in 3D the
+    // second part of the workspace
+    const size_t t1n = (size_t)D * g.Z * g.Y * L.nx;
     float *t2 = (float *)((char *)ws + ((t1n * 4 + 255) / 256) * 256);
-    const int th = 256;
-    // x: (D*Z*Y, X, 1) -> (D*Z*Y, nx, 1)
-    int64_t n1 = (int64_t)D * g.Z * g.Y * L.nx;
-    k_bspline_transpose_axis<<<elementwise_grid(n1, th), th, 0, s>>>(
-        grad_disp, t1, (int64_t)D * g.Z * g.Y, g.X, L.nx, 1, L);
-    // y: (D*Z, Y, nx) -> (D*Z, ny, nx); in 2D this is the result
-    float *ydst = (D == 3) ? t2 : grad_ctrl;
-    int64_t n2 = (int64_t)D * g.Z * L.ny * L.nx;
-    k_bspline_transpose_axis<<<elementwise_grid(n2, th), th, 0, s>>>(
-        t1, ydst, (int64_t)D * g.Z, g.Y, L.ny, L.nx, L);
+    const TransPlan t = trans_plan(g, L);
+    k_transpose_xy<<<D * g.Z * t.nxt * t.nbands, kTransThreads, t.smem, s>>>(
+        grad_disp, D == 3 ? t2 : grad_ctrl, g.X, g.Y, t.jt, t.bj, t.nxt, t.nbands, L);
     if (D == 3) {
         // z: (D, Z, ny*nx) -> (D, nz, ny*nx)
-        int64_t n3 = (int64_t)D * L.nz * L.ny * L.nx;
-        k_bspline_transpose_axis<<<elementwise_grid(n3, th), th, 0, s>>>(
-            t2, grad_ctrl, D, g.Z, L.nz, (int64_t)L.ny * L.nx, L);
+        const int64_t n3 = (int64_t)D * L.nc;
+        k_transpose_z<<<elementwise_grid(n3, kTransThreads), kTransThreads, 0, s>>>(
+            t2, grad_ctrl, D, g.Z, L.nz, L.ny * L.nx, L);
     }
     return cudaGetLastError();
 }
@@ -292,11 +588,11 @@ cudaError_t launch_displacement_adjoint(const Grid &g, const Lattice &L, const f
 cudaError_t launch_warp(const Grid &g, const float *moving, const float *disp, float *warped,
                         uint8_t *mask, cudaStream_t s)
 {
-    const int th = 256;
+    const March m = march_plan(g);
     if (g.ndim == 3)
-        k_warp<3><<<elementwise_grid(g.nv, th), th, 0, s>>>(g, moving, disp, warped, mask);
+        k_warp<3><<<m.ntiles, kTileX * kTileY, 0, s>>>(g, m, moving, disp, warped, mask);
     else
-        k_warp<2><<<elementwise_grid(g.nv, th), th, 0, s>>>(g, moving, disp, warped, mask);
+        k_warp<2><<<m.ntiles, kTileX * kTileY, 0, s>>>(g, m, moving, disp, warped, mask);
     return cudaGetLastError();
 }
 
@@ -304,15 +600,13 @@ cudaError_t launch_warp_adjoint(const Grid &g, const float *moving, const float 
                                 const uint8_t *mask, const float *grad_warped, float *grad_disp,
                                 int accumulate, cudaStream_t s)
 {
-    const int th = 256;
+    const March m = march_plan(g);
     if (g.ndim == 3)
-        k_warp_adjoint<3><<<elementwise_grid(g.nv, th), th, 0, s>>>(g, moving, disp, mask,
-                                                                     grad_warped, grad_disp,
-                                                                     accumulate);
+        k_warp_adjoint<3><<<m.ntiles, kTileX * kTileY, 0, s>>>(g, m, moving, disp, mask,
+                                                               grad_warped, grad_disp, accumulate);
     else
-        k_warp_adjoint<2><<<elementwise_grid(g.nv, th), th, 0, s>>>(g, moving, disp, mask,
-                                                                     grad_warped, grad_disp,
-                                                                     accumulate);
+        k_warp_adjoint<2><<<m.ntiles, kTileX * kTileY, 0, s>>>(g, m, moving, disp, mask,
+                                                               grad_warped, grad_disp, accumulate);
     return cudaGetLastError();
 }
 
@@ -322,25 +616,58 @@ size_t regulariser_ws(const Grid &g)
     return blocks * sizeof(double);
 }
 
-cudaError_t launch_regulariser(const Grid &g, const float *disp, double weight, double *value_dev,
-                               float *grad_disp, void *ws, cudaStream_t s)
+// Blocks of k_regulariser: at most what its partials' workspace holds.
+int regulariser_blocks(const Grid &g, const March &m)
 {
-    const int th = 256;
-    const int blocks = (int)((g.nv + th - 1) / th);
-    double *partials = (double *)ws;
+    const int64_t slots = ((int64_t)g.nv + 255) / 256;
+    return (int)std::min<int64_t>(std::min<int64_t>(m.ntiles, slots), 8192);
+}
+
+template <int D>
+static void run_regulariser(const Grid &g, const March &m, int blocks, int gw, const float *u,
+                            float gscale, float *gu, double *part, const AdjointArgs &a,
+                            unsigned int *maxbits, cudaStream_t s)
+{
+    constexpr int T = kTileX * kTileY;
+    switch (gw) {
+    case GW_MSE: k_regulariser<D, GW_MSE><<<blocks, T, 0, s>>>(g, m, u, gscale, gu, part, a, maxbits); break;
+    case GW_NCC: k_regulariser<D, GW_NCC><<<blocks, T, 0, s>>>(g, m, u, gscale, gu, part, a, maxbits); break;
+    case GW_SCALED: k_regulariser<D, GW_SCALED><<<blocks, T, 0, s>>>(g, m, u, gscale, gu, part, a, maxbits); break;
+    default: k_regulariser<D, GW_NONE><<<blocks, T, 0, s>>>(g, m, u, gscale, gu, part, a, maxbits); break;
+    }
+}
+
+cudaError_t launch_regulariser_adjoint(const Grid &g, const float *disp, double weight, int gw,
+                                       const AdjointArgs &a, float *grad_disp, double *partials,
+                                       int *count, unsigned int *maxbits, cudaStream_t s)
+{
+    const March m = march_plan(g);
+    *count = regulariser_blocks(g, m);
     const float gscale = (float)(2.0 * weight / (double)g.nv);
     if (g.ndim == 3)
-        k_regulariser<3><<<blocks, th, 0, s>>>(g, disp, gscale, grad_disp, partials);
+        run_regulariser<3>(g, m, *count, gw, disp, gscale, grad_disp, partials, a, maxbits, s);
     else
-        k_regulariser<2><<<blocks, th, 0, s>>>(g, disp, gscale, grad_disp, partials);
-    k_sum_partials<<<1, 1024, 0, s>>>(partials, blocks, 1.0 / (double)g.nv, value_dev);
+        run_regulariser<2>(g, m, *count, gw, disp, gscale, grad_disp, partials, a, maxbits, s);
     return cudaGetLastError();
 }
 
-cudaError_t launch_combine(const double *sim_value, const double *reg_value, double lambda,
-                           double *out, cudaStream_t s)
+cudaError_t launch_regulariser(const Grid &g, const float *disp, double weight, double *value_dev,
+                               float *grad_disp, void *ws, cudaStream_t s)
 {
-    k_combine<<<1, 32, 0, s>>>(sim_value, reg_value, lambda, out);
+    double *partials = (double *)ws;
+    int count = 0;
+    const cudaError_t e = launch_regulariser_adjoint(g, disp, weight, GW_NONE, AdjointArgs{},
+                                                     grad_disp, partials, &count, nullptr, s);
+    if (e != cudaSuccess)
+        return e;
+    k_sum_partials<<<1, 256, 0, s>>>(partials, count, 1.0 / (double)g.nv, value_dev);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_combine(const double *sim_value, const double *reg, int count, double scale,
+                           double lambda, double *out, cudaStream_t s)
+{
+    k_combine<<<1, 256, 0, s>>>(sim_value, reg, count, scale, lambda, out);
     return cudaGetLastError();
 }
 

@@ -606,7 +606,7 @@ cudaError_t exp_run(const Grid &g, int K, const float *v, float *u, float *traj,
 
 template <int D>
 cudaError_t exp_adjoint_run(const Grid &g, int K, const float *traj, const float *gu, float *gv,
-                            char *ws, cudaStream_t s)
+                            char *ws, const unsigned int *gmax, cudaStream_t s)
 {
     const int64_t n = (int64_t)D * g.nv;
     unsigned long long *acc = (unsigned long long *)ws;
@@ -617,9 +617,9 @@ cudaError_t exp_adjoint_run(const Grid &g, int K, const float *traj, const float
     cudaError_t e = cudaMemsetAsync(acc, 0, (size_t)n * 8, s);
     const float *gin = gu;
     float *out = b0;
-    // mx[0], mx[1]: the largest |g| of a step's input; the first from a pass of
-    // its own, the others from the previous step's finish
-    if (e == cudaSuccess && K > 0) {
+    // mx[0], mx[1]: the largest |g| of a step's input; the first from the caller
+    // or from a pass of its own, the others from the previous step's finish
+    if (e == cudaSuccess && K > 0 && !gmax) {
         e = cudaMemsetAsync(mx, 0, sizeof(unsigned int), s);
         if (e == cudaSuccess) {
             k_absmax<<<blocks_for(n) < 4 * device_sms() ? blocks_for(n) : 4 * device_sms(),
@@ -629,7 +629,7 @@ cudaError_t exp_adjoint_run(const Grid &g, int K, const float *traj, const float
     }
     for (int k = K - 1, j = 0; k >= 0 && e == cudaSuccess; --k, j ^= 1) {
         const float *u = traj + (int64_t)k * n;
-        const unsigned int *mcur = mx + j;
+        const unsigned int *mcur = k == K - 1 && gmax ? gmax : mx + j;
         unsigned int *mnext = k > 0 ? mx + (j ^ 1) : nullptr;
         if constexpr (D == 3) {
             const Tiles t = tiles_of(g);
@@ -672,10 +672,10 @@ cudaError_t launch_exp(const Grid &g, int K, const float *v, float *u, float *tr
 }
 
 cudaError_t launch_exp_adjoint(const Grid &g, int K, const float *traj, const float *gu, float *gv,
-                               void *ws, cudaStream_t s)
+                               void *ws, const unsigned int *gmax, cudaStream_t s)
 {
-    return g.ndim == 3 ? exp_adjoint_run<3>(g, K, traj, gu, gv, (char *)ws, s)
-                       : exp_adjoint_run<2>(g, K, traj, gu, gv, (char *)ws, s);
+    return g.ndim == 3 ? exp_adjoint_run<3>(g, K, traj, gu, gv, (char *)ws, gmax, s)
+                       : exp_adjoint_run<2>(g, K, traj, gu, gv, (char *)ws, gmax, s);
 }
 
 }  // namespace airgb

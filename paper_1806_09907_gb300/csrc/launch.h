@@ -30,11 +30,36 @@ size_t regulariser_ws(const Grid &g);
 cudaError_t launch_regulariser(const Grid &g, const float *disp, double weight, double *value_dev,
                                float *grad_disp, void *ws, cudaStream_t s);
 
+// The regulariser's gradient and the adjoint of the warp in one pass:
+// grad_disp = weight dR/du + mask dS/dW dM~/dy, with dS/dW formed on the fly
+// from the similarity's scalars (MSE: scal[0] (W - F); NCC: scal[3] (F - scal[0])
+// + scal[4] (W - scal[1]); scaled: gw scal[0]). Per-block partials of R |X| go
+// to `partials` (*count of them, at most ceil(nv / 256)); maxbits (nullable):
+// the largest |grad_disp| as float bits, atomicMax-ed.
+enum { GW_NONE = 0, GW_MSE = 1, GW_NCC = 2, GW_SCALED = 3 };
+struct AdjointArgs {
+    const float *M, *F, *W, *gw;
+    const uint8_t *mask;
+    const double *scal;
+};
+cudaError_t launch_regulariser_adjoint(const Grid &g, const float *disp, double weight, int gw,
+                                       const AdjointArgs &a, float *grad_disp, double *partials,
+                                       int *count, unsigned int *maxbits, cudaStream_t s);
+
 // ---- A3: similarity (unfused) ------------------------------------------------
 size_t similarity_ws(const Grid &g, int kind, int window);
 cudaError_t launch_similarity(const Grid &g, int kind, int window, double eps, const float *fixed,
                               const float *warped, const uint8_t *mask, double *value_dev,
                               float *grad_warped, void *ws, cudaStream_t s);
+
+// The value, and the scalars at the head of ws (256 bytes) that dS/dW follows
+// from, without writing dS/dW: LCC leaves it unscaled in grad_unscaled (null:
+// value only), see AdjointArgs. w_masked: as in launch_lcc. Returns the GW_
+// kind in *gw.
+cudaError_t launch_similarity_scalars(const Grid &g, int kind, int window, double eps,
+                                      const float *fixed, const float *warped,
+                                      const uint8_t *mask, bool w_masked, double *value_dev,
+                                      float *grad_unscaled, void *ws, int *gw, cudaStream_t s);
 
 // Streaming multiprocessors of the current device (queried once per device;
 // 152, a GB300's count, if the query fails). Sizes grids and z chunks only:
@@ -84,8 +109,9 @@ cudaError_t launch_fused(const Grid &g, const Lattice &L, int kind, int window, 
                          double *value_dev, float *grad_ctrl, void *ws, cudaStream_t s);
 
 // J = S + lambda * R from the unfused pieces: out[0..3] = {J, S, R, n_mask}.
-cudaError_t launch_combine(const double *sim_value /*S, n_mask*/, const double *reg_value /*R*/,
-                           double lambda, double *out, cudaStream_t s);
+// R = reg[0], or the sum of `count` partials times scale when count > 0.
+cudaError_t launch_combine(const double *sim_value /*S, n_mask*/, const double *reg, int count,
+                           double scale, double lambda, double *out, cudaStream_t s);
 
 // ---- optimisation loop: Adam, pyramid level, coefficient refinement ---------
 struct AdamArgs {
@@ -169,8 +195,10 @@ cudaError_t launch_batch(int delta, int tile, int blocks, const BatchProblem *pr
 cudaError_t launch_exp(const Grid &g, int K, const float *v, float *u, float *traj, float *tmp,
                        cudaStream_t s);
 size_t exp_adjoint_ws(const Grid &g);
+// gmax (nullable): device word with the largest |gu| as float bits; otherwise
+// a pass of its own finds it.
 cudaError_t launch_exp_adjoint(const Grid &g, int K, const float *traj, const float *gu, float *gv,
-                               void *ws, cudaStream_t s);
+                               void *ws, const unsigned int *gmax, cudaStream_t s);
 
 // ---- learned initialisation: convolution layers and the network's glue ------
 // A 3x3x3 convolution layer, zero padding 1: batch nb of D x H x W voxels
