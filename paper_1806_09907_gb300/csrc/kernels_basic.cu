@@ -11,66 +11,63 @@ namespace {
 constexpr int kDispTX = 128;  // x extent of a displacement tile (threads)
 constexpr int kDispTY = 8;    // rows per tile
 
-// Control columns / rows a tile of n voxels can touch.
-__host__ __device__ constexpr int disp_span(int n, int delta) { return (n - 1) / delta + 5; }
+// Control columns a tile of n voxels can touch.
+constexpr int disp_span(int n, int delta) { return (n - 1) / delta + 5; }
 
 // A1: u_i(x) = sum_j c_{i,j} prod_k w. One CTA = one z slice, 8 rows, 128
-// columns. Separable: z-contraction of the touched control block into smem,
-// then y-contraction per row, then 4 x-taps per voxel. The two buffers are
-// sized by the spacing (4.4 KB at 6, not the 33 KB that spacing 1 needs), so
-// that 16 CTAs are resident per SM instead of 6: it is the latency of the three
-// short phases that bounds the kernel (256 x 256 x 160, spacing 6: 63.6 us with
-// the fixed buffers and divided indices, 49.3 us so; writing u takes 18.5 us).
+// columns. Separable: a thread per touched control column contracts along z
+// and y together, keeping the four z-contracted points that the row needs in
+// registers and forming the next one every delta rows, into a row buffer in
+// shared memory; then 4 x-taps per voxel. Bound by instructions: 63.6 us at
+// 256 x 256 x 160, spacing 6, with a z and a y phase over elements whose
+// indices were divided out and buffers sized for spacing 1 (6 CTAs per SM),
+// 44.8 us so; writing u takes 18.5 us. (96 registers; held to 64, 46.6 us, to 40,
+// 61.9 us.)
 template <int D>
 __global__ void __launch_bounds__(kDispTX)
     k_displacement(Grid g, const __grid_constant__ Lattice L, const float *__restrict__ c,
                    float *__restrict__ u)
 {
-    extern __shared__ float disp_smem[];
+    extern __shared__ float disp_smem[];  // [D][kDispTY][njx]
     const int x0 = blockIdx.x * kDispTX, y0 = blockIdx.y * kDispTY, z = blockIdx.z;
     const int delta = L.delta;
     const int jx0 = x0 / delta, jy0 = y0 / delta;
-    const int xl = min(x0 + kDispTX, g.X) - 1, yl = min(y0 + kDispTY, g.Y) - 1;
-    const int njx = xl / delta + 4 - jx0, njy = yl / delta + 4 - jy0;
-    float *tz = disp_smem;                                    // [D][njy][njx]
-    float *ty = tz + D * disp_span(kDispTY, delta) * njx;     // [D][kDispTY][njx]
-    const int qz = z / delta, pz = z - qz * delta;
-    // a warp per row of control columns, so that no index is divided
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // z contraction
-    for (int row = warp; row < D * njy; row += kDispTX / 32) {
-        const int i = D == 3 ? (row >= njy) + (row >= 2 * njy) : (row >= njy);
-        const int jyl = row - i * njy;
-        const float *src = D == 3
-                               ? c + (((int64_t)i * L.nz + qz) * L.ny + jy0 + jyl) * L.nx + jx0
-                               : c + ((int64_t)i * L.ny + jy0 + jyl) * L.nx + jx0;
-        const int64_t pl = (int64_t)L.ny * L.nx;
-        for (int j = lane; j < njx; j += 32) {
-            float acc = 0.0f;
-            if (D == 3) {
+    const int xl = min(x0 + kDispTX, g.X) - 1;
+    const int njx = xl / delta + 4 - jx0;
+    const int rows = min(kDispTY, g.Y - y0);
+    const int qz = z / delta, pz = z - qz * delta, py0 = y0 - jy0 * delta;
+    const float z0 = L.w[pz][0], z1 = L.w[pz][1], z2 = L.w[pz][2], z3 = L.w[pz][3];
+    const int nxy = L.nx * L.ny;
+    for (int col = threadIdx.x; col < D * njx; col += kDispTX) {
+        const int i = D == 3 ? (col >= njx) + (col >= 2 * njx) : (col >= njx);
+        const float *src = c + (int64_t)i * L.nc + (D == 3 ? qz * nxy : 0) + jy0 * L.nx + jx0 +
+                           (col - i * njx);
+        auto point = [&](int jy) {
+            const float *p = src + jy * L.nx;
+            if (D == 2)
+                return __ldg(p);
+            float acc = fmaf(z0, __ldg(p), 0.0f);
+            acc = fmaf(z1, __ldg(p + nxy), acc);
+            acc = fmaf(z2, __ldg(p + 2 * nxy), acc);
+            return fmaf(z3, __ldg(p + 3 * nxy), acc);
+        };
+        float t0 = point(0), t1 = point(1), t2 = point(2), t3 = point(3);
+        float *d = disp_smem + i * kDispTY * njx + (col - i * njx);
+        int p = py0, jy = 3;
 #pragma unroll
-                for (int a = 0; a < 4; ++a)
-                    acc = fmaf(L.w[pz][a], __ldg(src + a * pl + j), acc);
-            } else {
-                acc = __ldg(src + j);
+        for (int yr = 0; yr < kDispTY; ++yr) {
+            if (yr >= rows)
+                break;
+            if (p == delta) {  // the same row for every column: uniform
+                p = 0;
+                t0 = t1, t1 = t2, t2 = t3;
+                t3 = point(++jy);
             }
-            tz[row * njx + j] = acc;
-        }
-    }
-    __syncthreads();
-    // y contraction
-#pragma unroll 2
-    for (int row = warp; row < D * kDispTY; row += kDispTX / 32) {
-        const int i = row / kDispTY, yr = row % kDispTY;
-        const int y = min(y0 + yr, g.Y - 1);
-        const int qy = y / delta, py = y - qy * delta;
-        const float b0 = L.w[py][0], b1 = L.w[py][1], b2 = L.w[py][2], b3 = L.w[py][3];
-        const float *t = tz + (i * njy + qy - jy0) * njx;
-        for (int j = lane; j < njx; j += 32) {
-            float acc = fmaf(b0, t[j], 0.0f);
-            acc = fmaf(b1, t[njx + j], acc);
-            acc = fmaf(b2, t[2 * njx + j], acc);
-            ty[row * njx + j] = fmaf(b3, t[3 * njx + j], acc);
+            float acc = fmaf(L.w[p][0], t0, 0.0f);
+            acc = fmaf(L.w[p][1], t1, acc);
+            acc = fmaf(L.w[p][2], t2, acc);
+            d[yr * njx] = fmaf(L.w[p][3], t3, acc);
+            ++p;
         }
     }
     __syncthreads();
@@ -79,21 +76,22 @@ __global__ void __launch_bounds__(kDispTX)
         return;
     const int qx = x / delta, px = x - qx * delta;
     const float w0 = L.w[px][0], w1 = L.w[px][1], w2 = L.w[px][2], w3 = L.w[px][3];
-    const int jxl = qx - jx0;
+    const float *t = disp_smem + (qx - jx0);
+    float *o = u + ((int64_t)z * g.Y + y0) * g.X + x;
 #pragma unroll
     for (int yr = 0; yr < kDispTY; ++yr) {
-        if (y0 + yr >= g.Y)
+        if (yr >= rows)
             break;
-        const int64_t v = ((int64_t)z * g.Y + y0 + yr) * g.X + x;
 #pragma unroll
         for (int i = 0; i < D; ++i) {
-            const float *t = ty + (i * kDispTY + yr) * njx + jxl;
-            float acc = w0 * t[0];
-            acc = fmaf(w1, t[1], acc);
-            acc = fmaf(w2, t[2], acc);
-            acc = fmaf(w3, t[3], acc);
-            u[(int64_t)i * g.nv + v] = acc;
+            const float *r = t + (i * kDispTY + yr) * njx;
+            float acc = w0 * r[0];
+            acc = fmaf(w1, r[1], acc);
+            acc = fmaf(w2, r[2], acc);
+            acc = fmaf(w3, r[3], acc);
+            o[(int64_t)i * g.nv] = acc;
         }
+        o += g.X;
     }
 }
 
@@ -263,13 +261,13 @@ struct March {
     int ntx, nty, ntiles, zc;
 };
 
-// Slices of a column: 16, fewer while that leaves less than eight blocks per SM.
+// Slices of a column: 8, fewer while that leaves less than eight blocks per SM.
 March march_plan(const Grid &g)
 {
     March m;
     m.ntx = (g.X + kTileX - 1) / kTileX;
     m.nty = (g.Y + kTileY - 1) / kTileY;
-    m.zc = 16;
+    m.zc = 8;
     while (m.zc > 1 &&
            (int64_t)m.ntx * m.nty * ((g.Z + m.zc - 1) / m.zc) < 8 * (int64_t)device_sms())
         m.zc /= 2;
@@ -381,7 +379,7 @@ __global__ void __launch_bounds__(kTileX *kTileY)
 // maxbits (nullable): the largest |grad| as the bits of a float (a NaN never
 // wins), for al_exp_field_adjoint's fixed point.
 template <int D, int GW>
-__global__ void __launch_bounds__(kTileX *kTileY)
+__global__ void __launch_bounds__(kTileX *kTileY, 5)
     k_regulariser(Grid g, March mp, const float *__restrict__ u, float gscale,
                   float *__restrict__ gu, double *__restrict__ partials, AdjointArgs a,
                   unsigned int *__restrict__ maxbits)
@@ -417,12 +415,12 @@ __global__ void __launch_bounds__(kTileX *kTileY)
             float sum = 0.0f, lap[D], next[D], wxu[D], wxd[D], wyu[D], wyd[D];
 #pragma unroll
             for (int i = 0; i < D; ++i) {
-                const float *ui = u + i * nv + v;
-                next[i] = D == 3 ? __ldg(ui + (zu ? sz : 0)) : 0.0f;
-                wxu[i] = __ldg(ui + oxu);
-                wxd[i] = __ldg(ui + oxd);
-                wyu[i] = __ldg(ui + oyu);
-                wyd[i] = __ldg(ui + oyd);
+                const float *ui = u + i * nv;
+                next[i] = D == 3 ? __ldg(ui + (unsigned)(zu ? v + sz : v)) : 0.0f;
+                wxu[i] = __ldg(ui + (unsigned)(v + oxu));
+                wxd[i] = __ldg(ui + (unsigned)(v + oxd));
+                wyu[i] = __ldg(ui + (unsigned)(v + oyu));
+                wyd[i] = __ldg(ui + (unsigned)(v + oyd));
             }
 #pragma unroll
             for (int i = 0; i < D; ++i) {
@@ -548,8 +546,8 @@ cudaError_t launch_displacement(const Grid &g, const Lattice &L, const float *ct
                                 cudaStream_t s)
 {
     dim3 grid((g.X + kDispTX - 1) / kDispTX, (g.Y + kDispTY - 1) / kDispTY, g.Z);
-    const size_t smem = (size_t)g.ndim * std::min(disp_span(kDispTX, L.delta), L.nx) *
-                        (disp_span(kDispTY, L.delta) + kDispTY) * 4;
+    const size_t smem =
+        (size_t)g.ndim * std::min(disp_span(kDispTX, L.delta), L.nx) * kDispTY * 4;
     if (g.ndim == 3)
         k_displacement<3><<<grid, kDispTX, smem, s>>>(g, L, ctrl, disp);
     else
