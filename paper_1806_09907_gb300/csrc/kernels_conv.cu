@@ -50,6 +50,7 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "launch.h"
@@ -73,6 +74,7 @@ constexpr int kTargetUnits = 1216;
 constexpr int kMaxN = 128;
 constexpr int kErrTimeout = 6;                // AL_ERR_TIMEOUT
 constexpr int kMaxClasses = 8;
+constexpr int kMaxDynSmem = 227 * 1024;      // dynamic shared memory a CTA may have
 
 enum { FWD = 0, DGRAD = 1, WGRAD = 2 };
 
@@ -241,11 +243,10 @@ __device__ __forceinline__ void tc_load16(uint32_t taddr, float (&v)[16])
 // Shared-memory matrix descriptor, no swizzle: start address, the byte
 // distance between core matrices along K (leading) and along M/N (stride),
 // descriptor version 1 (bits 46-47) of sm_100-class tensor cores.
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr)
+__device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo = 128, uint32_t sbo = 1024)
 {
-    constexpr uint64_t lbo = 128, sbo = 1024;
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((lbo >> 4) << 16) | ((sbo >> 4) << 32) |
-           (1ull << 46);
+    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) |
+           ((uint64_t)(sbo >> 4) << 32) | (1ull << 46);
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
@@ -882,6 +883,233 @@ __global__ void __launch_bounds__(kThreads, MODE == WGRAD ? 4 : 1) k_conv(const 
         tmem_dealloc(tmem, a.tmem_cols);
 }
 
+// ---- two input channels: forward and weight adjoint --------------------------
+// A tap row (dz, dy) of an output voxel reads three x-neighbouring voxels of
+// two bf16 channels: 12 consecutive bytes, which with a zero pair make one
+// 16-byte chunk (dx, ci) of 8 K elements. A 128-voxel tile is 9 planes (one
+// per (dz, dy)) of 128 chunks, 16 bytes apart: as K-major rows the operand of
+// the forward pass (K = 9 chunks and one of zeros, 5 MMAs of K = 16), as MN-major groups of 8 rows that of the weight
+// adjoint (M = 9 chunks and a chunk of ones for the bias, K = 128 voxels).
+// A thread gathers the 27 words of its voxel into registers by plain loads (a
+// warp's are 8 bytes apart) and stores 9 chunks; k_conv filled the same tile
+// with 27 4-byte asynchronous copies a row, which was bound by their number.
+// 16 x 128^3 -> 64^3, stride 2: forward 205 -> @@ us, weight adjoint 280 -> @@ us;
+// reading the input and writing or reading the output takes 40 us.
+constexpr int kC2Plane = 128 * 16;  // bytes of one plane of a tile
+constexpr int kC2Groups = 9;
+constexpr int kC2Slot = 10 * kC2Plane;  // a forward slot
+
+// The 9 chunks of output voxel `row` (zero outside the grid).
+__device__ __forceinline__ void c2_gather(const ConvArgs &a, int row, bool ok,
+                                          uint32_t (&w)[kC2Groups][3])
+{
+    unsigned r = ok ? (unsigned)row : 0u;
+    const unsigned ox = r % (unsigned)a.Wo;
+    r /= (unsigned)a.Wo;
+    const unsigned oy = r % (unsigned)a.Ho;
+    r /= (unsigned)a.Ho;
+    const unsigned oz = r % (unsigned)a.Do, b = r / (unsigned)a.Do;
+    const int z0 = (int)oz * a.stride - 1, y0 = (int)oy * a.stride - 1,
+              x0 = (int)ox * a.stride - 1;
+    const uint32_t *src = reinterpret_cast<const uint32_t *>(a.act);
+    const bool xl = x0 >= 0, xr = x0 + 2 < a.W;
+    const int64_t org = (((int64_t)b * a.D + z0) * a.H + y0) * a.W + x0;
+#pragma unroll
+    for (int g = 0; g < kC2Groups; ++g) {
+        const int dz = g / 3, dy = g % 3;
+        bool in = ok && (unsigned)(z0 + dz) < (unsigned)a.D && (unsigned)(y0 + dy) < (unsigned)a.H;
+        const int64_t o = org + ((int64_t)dz * a.H + dy) * a.W;
+        if (in && !al_index_ok(o + 1, a.act_elems / 2))
+            in = false;
+        w[g][0] = in && xl ? __ldg(src + o) : 0u;
+        w[g][1] = in ? __ldg(src + o + 1) : 0u;
+        w[g][2] = in && xr ? __ldg(src + o + 2) : 0u;
+    }
+}
+
+__device__ __forceinline__ void c2_store(uint8_t *A, int tid, const uint32_t (&w)[kC2Groups][3])
+{
+#pragma unroll
+    for (int g = 0; g < kC2Groups; ++g)
+        *reinterpret_cast<uint4 *>(A + g * kC2Plane + tid * 16) =
+            make_uint4(w[g][0], w[g][1], w[g][2], 0u);
+}
+
+// Forward: shared memory = 2 slots of 10 planes, the weights as 10 chunks of N
+// rows, barriers. D of a tile is double buffered in TMEM, so that a tile's
+// epilogue runs beside the next tile's MMAs.
+template <int N>
+__global__ void __launch_bounds__(kThreads) k_conv2_fwd(const ConvArgs a)
+{
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *sm = reinterpret_cast<uint8_t *>(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
+    uint8_t *B = sm + 2 * kC2Slot;
+    uint64_t *bars = reinterpret_cast<uint64_t *>(B + 10 * N * 16);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 2);
+    const uint32_t bar = smem_u32(bars);
+    const int tid = threadIdx.x, warp = tid >> 5;
+    if (tid == 0) {
+        mbar_init(bar, 1);
+        mbar_init(bar + 8, 1);
+        fence_mbar_init();
+    }
+    if (warp == 0) {
+        tmem_alloc(smem_u32(tslot), 2 * N);
+        tmem_relinquish();
+    }
+    // B: chunk g, row n, element (dx, ci) = w[n][t = 3 g + dx][ci] from the packed
+    // copy (k = 2 t + ci); zero for dx = 3 and chunk 9
+    for (int e = tid; e < 10 * N * 8; e += kThreads) {
+        const int q = e & 7, n = (e >> 3) % N, g = (e >> 3) / N;
+        const int k = 2 * (3 * g + (q >> 1)) + (q & 1);
+        __nv_bfloat16 v = __float2bfloat16_rn(0.0f);
+        if (g < kC2Groups && q < 6)
+            v = a.wpk[(n / 8) * 512 + (k / 8) * 64 + (n % 8) * 8 + (k & 7)];
+        reinterpret_cast<__nv_bfloat16 *>(B)[e] = v;
+    }
+    for (int k = 0; k < 2; ++k)
+        *reinterpret_cast<uint4 *>(sm + k * kC2Slot + kC2Groups * kC2Plane + tid * 16) =
+            make_uint4(0u, 0u, 0u, 0u);
+    tc_before_sync();
+    __syncthreads();
+    tc_after_sync();
+    const uint32_t tmem = *tslot;
+    const uint32_t bdesc = smem_u32(B);
+    uint32_t w[kC2Groups][3];
+    auto finish = [&](int tile, int slot, uint32_t use) {
+        mbar_wait(bar + 8 * slot, use & 1);
+        tc_after_sync();
+        Cursor c;
+        c.tile = tile;
+        epilogue<FWD>(a, c, tmem + slot * N + ((uint32_t)(warp * 32) << 16), tid);
+        tc_before_sync();
+    };
+    int it = 0;
+    for (int tile = blockIdx.x; tile < a.units; tile += gridDim.x, ++it) {
+        const int slot = it & 1;
+        const int row = tile * 128 + tid;
+        c2_gather(a, row, row < a.rows, w);
+        // the MMAs of two tiles ago, the slot's last use, are done: their tile's
+        // epilogue has waited for them
+        uint8_t *A = sm + slot * kC2Slot;
+        c2_store(A, tid, w);
+        fence_proxy_async();
+        __syncthreads();
+        if (tid == 0) {
+            tc_after_sync();
+            const uint32_t a0 = smem_u32(A);
+#pragma unroll
+            for (int j = 0; j < 5; ++j)
+                tc_mma(tmem + slot * N, sdesc(a0 + 2 * j * kC2Plane, kC2Plane, 128),
+                       sdesc(bdesc + 2 * j * N * 16, N * 16, 128), a.idesc, j != 0);
+            tc_commit(bar + 8 * slot);
+        }
+        if (it > 0)
+            finish(tile - gridDim.x, slot ^ 1, (uint32_t)((it - 1) >> 1));
+    }
+    if (it > 0)
+        finish(blockIdx.x + (it - 1) * gridDim.x, (it - 1) & 1, (uint32_t)((it - 1) >> 1));
+    __syncthreads();
+    if (warp == 0)
+        tmem_dealloc(tmem, 2 * N);
+}
+
+// Weight adjoint: shared memory = 2 slots of 16 planes (the 9 chunks, the
+// ones, planes whose rows of D are never read) and of the output gradient's N / 8
+// planes, barriers. One D per unit (a split of the voxels) in TMEM.
+template <int N>
+__global__ void __launch_bounds__(kThreads) k_conv2_wgrad(const ConvArgs a)
+{
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *sm = reinterpret_cast<uint8_t *>(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
+    constexpr int SLOT = (16 + N / 8) * kC2Plane;
+    uint64_t *bars = reinterpret_cast<uint64_t *>(sm + 2 * SLOT);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 3);
+    const uint32_t bar = smem_u32(bars);
+    const int tid = threadIdx.x, warp = tid >> 5;
+    constexpr uint32_t COLS = N < 32 ? 32 : (N <= 64 ? (N <= 32 ? 32 : 64) : 128);
+    if (tid == 0) {
+        for (int k = 0; k < 3; ++k)
+            mbar_init(bar + 8 * k, 1);
+        fence_mbar_init();
+    }
+    if (warp == 0) {
+        tmem_alloc(smem_u32(tslot), COLS);
+        tmem_relinquish();
+    }
+    for (int s = 0; s < 2; ++s)
+        for (int g = kC2Groups; g < 16; ++g)
+            *reinterpret_cast<uint4 *>(sm + s * SLOT + g * kC2Plane + tid * 16) =
+                make_uint4(g == kC2Groups ? 0x3F80u : 0u, 0u, 0u, 0u);
+    tc_before_sync();
+    __syncthreads();
+    tc_after_sync();
+    const uint32_t tmem = *tslot;
+    uint32_t w[kC2Groups][3];
+    int it = 0;
+    uint32_t nunit = 0;
+    for (int u = blockIdx.x; u < a.units; u += gridDim.x, ++nunit) {
+        const int v0 = u * a.Kreal, v1 = min(v0 + a.Kreal, a.rows);
+        for (int v = v0; v < v1; v += 128, ++it) {
+            const int slot = it & 1;
+            const int row = v + tid;
+            const bool ok = row < v1;
+            c2_gather(a, row, ok, w);
+            if (it >= 2)
+                mbar_wait(bar + 8 * slot, (uint32_t)((it >> 1) - 1) & 1);
+            uint8_t *A = sm + slot * SLOT, *G = A + 16 * kC2Plane;
+            const uint32_t sG = smem_u32(G);
+#pragma unroll
+            for (int n = 0; n < N / 8; ++n) {
+                bool in = ok;
+                if (in && !al_index_ok((int64_t)row * N + n * 8, a.gout_elems - 7))
+                    in = false;
+                cp16(sG + n * kC2Plane + tid * 16, in ? a.gout + (size_t)row * N + n * 8 : a.gout,
+                     in);
+            }
+            cp_commit();
+            c2_store(A, tid, w);
+            cp_wait<0>();
+            fence_proxy_async();
+            __syncthreads();
+            if (tid == 0) {
+                tc_after_sync();
+                const uint32_t a0 = smem_u32(A), g0 = smem_u32(G);
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    tc_mma(tmem, sdesc(a0 + 256 * j, 128, kC2Plane),
+                           sdesc(g0 + 256 * j, 128, kC2Plane), a.idesc, v != v0 || j != 0);
+                tc_commit(bar + 8 * slot);
+            }
+        }
+        if (tid == 0)
+            tc_commit(bar + 16);
+        mbar_wait(bar + 16, nunit & 1);
+        tc_after_sync();
+        // row m = chunk g, (dx, ci) of the chunk -> row 2 (3 g + dx) + ci of the
+        // partial sums; the ones' first row -> row 54
+        const int g = tid >> 3, q = tid & 7;
+        const bool keep = g < kC2Groups ? q < 6 : (g == kC2Groups && q == 0);
+        const int m = g < kC2Groups ? 6 * g + q : 54;
+        float *o = static_cast<float *>(a.out) + ((size_t)u * 128 + m) * N;
+#pragma unroll
+        for (int c0 = 0; c0 < N; c0 += 16) {
+            float v[16];
+            tc_load16(tmem + (uint32_t)c0 + ((uint32_t)(warp * 32) << 16), v);
+            if (keep)
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    *reinterpret_cast<float4 *>(o + c0 + 4 * k) =
+                        make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+        }
+        tc_before_sync();
+        __syncthreads();
+    }
+    __syncthreads();
+    if (warp == 0)
+        tmem_dealloc(tmem, COLS);
+}
+
 // Weight slices in the shared-memory layout of the B operand: slice s holds
 // rows n < N and K elements [64 s, 64 s + 64), K-major, zero beyond the real
 // rows and K. mode 0 (forward): B[n = co][k = t cin + ci] = w[co][t][ci], the
@@ -1204,6 +1432,87 @@ cudaError_t grid_for(int N, int units, int *grid)
     return cudaSuccess;
 }
 
+// Resident CTAs per SM of a kernel of kThreads threads with `smem` bytes of
+// dynamic shared memory and `cols` TMEM columns, from the kernel's own limits
+// (shared memory with the largest carveout, registers, 512 TMEM columns per
+// SM); found once per kernel, size and device.
+struct Residency {
+    const void *fn;
+    size_t smem;
+    int dev, occ;
+};
+
+cudaError_t resident_grid(const void *fn, size_t smem, int cols, int units, int *grid)
+{
+    static std::mutex mu;
+    static Residency known[64];
+    static int n = 0;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess)
+        return e;
+    std::lock_guard<std::mutex> lk(mu);
+    int occ = 0;
+    for (int k = 0; k < n && occ == 0; ++k)
+        if (known[k].fn == fn && known[k].smem == smem && known[k].dev == dev)
+            occ = known[k].occ;
+    if (occ == 0) {
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kMaxDynSmem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                     (int)cudaSharedmemCarveoutMaxShared);
+        cudaFuncAttributes fa;
+        if (e == cudaSuccess)
+            e = cudaFuncGetAttributes(&fa, fn);
+        int smem_sm = 0, resv = 0;
+        if (e == cudaSuccess)
+            e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+        if (e == cudaSuccess)
+            e = cudaDeviceGetAttribute(&resv, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+        if (e != cudaSuccess)
+            return e;
+        const int by_smem = smem_sm / (int)(smem + fa.sharedSizeBytes + resv);
+        const int by_regs = 65536 / ((fa.numRegs * 32 + 255) / 256 * 256 * (kThreads / 32));
+        occ = std::min(std::min(by_smem, by_regs), std::min(512 / cols, 16));
+        if (occ < 1)
+            return cudaErrorInvalidConfiguration;
+        if (n < 64)
+            known[n++] = Residency{fn, smem, dev, occ};
+    }
+    *grid = std::min(units, occ * device_sms());
+    return cudaSuccess;
+}
+
+// The two-channel kernels are built for the output widths 16 and 32.
+bool conv2_built(const ConvLayer &l) { return l.cin == 2 && (l.cout == 16 || l.cout == 32); }
+
+template <int N>
+cudaError_t run_conv2_fwd(const ConvArgs &a, cudaStream_t s)
+{
+    const size_t smem = 128 + 2 * kC2Slot + 10 * N * 16 + 32;
+    int grid = 0;
+    const cudaError_t e = resident_grid((const void *)k_conv2_fwd<N>, smem, 2 * N, a.units, &grid);
+    if (e != cudaSuccess)
+        return e;
+    ProfScope ps(s, "k_conv_fwd");
+    k_conv2_fwd<N><<<grid, kThreads, smem, s>>>(a);
+    return cudaGetLastError();
+}
+
+template <int N>
+cudaError_t run_conv2_wgrad(const ConvArgs &a, cudaStream_t s)
+{
+    const size_t smem = 128 + 2 * (16 + N / 8) * kC2Plane + 32;
+    int grid = 0;
+    const cudaError_t e = resident_grid((const void *)k_conv2_wgrad<N>, smem, 32, a.units, &grid);
+    if (e != cudaSuccess)
+        return e;
+    ProfScope ps(s, "k_conv_wgrad");
+    k_conv2_wgrad<N><<<grid, kThreads, smem, s>>>(a);
+    return cudaGetLastError();
+}
+
 int blocks_for(int64_t n, int threads)
 {
     int64_t b = (n + threads - 1) / threads;
@@ -1392,6 +1701,8 @@ cudaError_t launch_conv_forward(const ConvLayer &l, const void *in, const void *
     a.out_f32 = out_f32;
     a.idesc = make_idesc(a.N, false);
     a.tmem_cols = tmem_cols_for(a.N);
+    if (conv2_built(l) && sp == 1)
+        return l.cout == 16 ? run_conv2_fwd<16>(a, s) : run_conv2_fwd<32>(a, s);
     int grid = 0;
     cudaError_t e = grid_for<FWD>(a.N, a.units, &grid);
     if (e != cudaSuccess)
@@ -1462,15 +1773,18 @@ cudaError_t launch_conv_wgrad(const ConvLayer &l, const void *in, const void *go
     single_class(a, kp / kBK);
     a.idesc = make_idesc(a.N, true);
     a.tmem_cols = tmem_cols_for(a.N);
-    int grid = 0;
-    cudaError_t e = grid_for<WGRAD>(a.N, a.units, &grid);
-    if (e != cudaSuccess)
-        return e;
-    {
+    cudaError_t e;
+    if (conv2_built(l)) {
+        e = l.cout == 16 ? run_conv2_wgrad<16>(a, s) : run_conv2_wgrad<32>(a, s);
+    } else {
+        int grid = 0;
+        e = grid_for<WGRAD>(a.N, a.units, &grid);
+        if (e != cudaSuccess)
+            return e;
         ProfScope ps(s, "k_conv_wgrad");
         k_conv<WGRAD><<<grid, kThreads, conv_smem_bytes(a.N), s>>>(a);
+        e = cudaGetLastError();
     }
-    e = cudaGetLastError();
     if (e != cudaSuccess)
         return e;
     ProfScope ps(s, "k_wgrad_reduce");
