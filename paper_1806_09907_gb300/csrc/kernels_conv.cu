@@ -71,7 +71,6 @@ constexpr int kATile = 128 * kBK * 2;         // bytes of one A slot (16 KB)
 // not the device's SM count: the split counts size workspaces, which must not
 // depend on the device the sizes are queried on.
 constexpr int kTargetUnits = 1216;
-constexpr int kMaxN = 128;
 constexpr int kErrTimeout = 6;                // AL_ERR_TIMEOUT
 constexpr int kMaxClasses = 8;
 constexpr int kMaxDynSmem = 227 * 1024;      // dynamic shared memory a CTA may have
@@ -93,6 +92,7 @@ struct ConvArgs {
     int units, mtiles;           // work units (tiles); WGRAD: M tiles (units = mtiles x splits)
     int rows;                    // FWD: output voxels; DGRAD: input voxels; WGRAD: output voxels
     int relu, out_f32, add_stride, add_off;
+    int wide;                    // out and mask lie on 32 bytes: a row's 16 columns are one access
     int64_t act_elems, gout_elems;  // elements of act and gout (checked builds)
     float *part;                 // FWD with split K: fp32 partials [class][rows][N]
     int classes;                 // DGRAD with stride 2: 8 parity classes; otherwise 1
@@ -154,6 +154,11 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes)
                  : "memory");
 }
 
+__device__ __forceinline__ void mbar_arrive(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes,
                                           uint32_t bar)
 {
@@ -213,6 +218,23 @@ __device__ __forceinline__ void tc_mma(uint32_t d, uint64_t adesc, uint64_t bdes
         : "memory");
 }
 
+// tc_mma by the lane that has `on`, every lane of the warp calling with the same
+// operands: they stay in uniform registers, which the instruction takes.
+__device__ __forceinline__ void tc_mma_if(bool on, uint32_t d, uint64_t adesc, uint64_t bdesc,
+                                          uint32_t idesc, uint32_t accumulate)
+{
+    if (on)
+        tc_mma(d, adesc, bdesc, idesc, accumulate);
+}
+
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t ok;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(ok));
+    return ok != 0;
+}
+
 // Arrive on `bar` once every tcgen05.mma issued so far by this thread is done.
 __device__ __forceinline__ void tc_commit(uint32_t bar)
 {
@@ -240,6 +262,33 @@ __device__ __forceinline__ void tc_load16(uint32_t taddr, float (&v)[16])
         v[i] = __uint_as_float(r[i]);
 }
 
+// The same without waiting: the values are good after tc_load_wait, which takes
+// them so that no use can be moved before it.
+__device__ __forceinline__ void tc_load16_async(uint32_t taddr, uint32_t (&r)[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
+        "%11, %12, %13, %14, %15}, [%16];\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+          "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+}
+
+__device__ __forceinline__ void tc_load_wait(uint32_t (&r)[16], uint32_t (&q)[16])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]),
+                   "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]),
+                   "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(q[0]), "+r"(q[1]),
+                   "+r"(q[2]), "+r"(q[3]), "+r"(q[4]), "+r"(q[5]), "+r"(q[6]), "+r"(q[7]),
+                   "+r"(q[8]), "+r"(q[9]), "+r"(q[10]), "+r"(q[11]), "+r"(q[12]), "+r"(q[13]),
+                   "+r"(q[14]), "+r"(q[15])
+                 :
+                 : "memory");
+}
+
 // Shared-memory matrix descriptor, no swizzle: start address, the byte
 // distance between core matrices along K (leading) and along M/N (stride),
 // descriptor version 1 (bits 46-47) of sm_100-class tensor cores.
@@ -247,6 +296,22 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo = 128, ui
 {
     return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) |
            ((uint64_t)(sbo >> 4) << 32) | (1ull << 46);
+}
+
+// 32 bytes of a 32-byte aligned address.
+__device__ __forceinline__ void store32(void *p, const uint32_t (&w)[8])
+{
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(w[0]),
+                 "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                 : "memory");
+}
+
+__device__ __forceinline__ void load32(const void *p, uint4 (&w)[2])
+{
+    asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(w[0].x), "=r"(w[0].y), "=r"(w[0].z), "=r"(w[0].w), "=r"(w[1].x),
+                   "=r"(w[1].y), "=r"(w[1].z), "=r"(w[1].w)
+                 : "l"(p));
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
@@ -268,6 +333,15 @@ __device__ __forceinline__ int mnmajor_off(int g, int k) { return g * 1024 + (k 
 __device__ __forceinline__ void cp16(uint32_t dst, const void *src, bool ok)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
+                 "r"(ok ? 16 : 0)
+                 : "memory");
+}
+
+// The same through L1: pieces of one 32-byte sector that go to different planes
+// fetch it once.
+__device__ __forceinline__ void cp16_l1(uint32_t dst, const void *src, bool ok)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
                  "r"(ok ? 16 : 0)
                  : "memory");
 }
@@ -367,9 +441,81 @@ __device__ __forceinline__ void build_tables(const ConvArgs &a, Tables &T, int t
 struct UnitState {
     int64_t rowoff;  // FWD/DGRAD: element offset of the row's tap origin (used only with a valid tap)
     uint32_t mask;   // FWD/DGRAD: valid taps (bit t, or bit ti for a parity class)
-    int m0;          // WGRAD: first M row of this thread's 8 groups
-    int kreal;       // WGRAD: 27 cin
+    int g0;          // WGRAD: first group of 8 M rows of the unit's M tile
+    int vend;        // WGRAD: end of the unit's voxels
+    int ox, oy, oz, b, vox;  // WGRAD: the thread's next voxel
 };
+
+// WGRAD: the pieces of a slice of 64 voxels are 16 bytes each, (group, voxel).
+// 2^sh consecutive lanes take consecutive groups of one voxel and tap (2^sh
+// divides a tap's groups, so they are contiguous bytes), the next lanes the next
+// voxels: a pass of the threads covers nvox voxels, and a thread's voxels are
+// nvox apart through the whole unit, so they are advanced by adding nvox in
+// mixed radix (Wo, Ho, Do) instead of being divided out.
+struct WLanes {
+    int sh, nvox, dx, dy, dz, db;
+};
+
+__device__ __forceinline__ WLanes wgrad_lanes(const ConvArgs &a)
+{
+    WLanes w;
+    const int nc = a.cin >> 3;
+    w.sh = a.cin == 2 ? 0 : (nc & 7) == 0 ? 3 : (nc & 3) == 0 ? 2 : (nc & 1) == 0 ? 1 : 0;
+    w.nvox = min(kThreads >> w.sh, kBK);
+    int r = w.nvox;
+    w.dx = r % a.Wo;
+    r /= a.Wo;
+    w.dy = r % a.Ho;
+    r /= a.Ho;
+    w.dz = r % a.Do;
+    w.db = r / a.Do;
+    return w;
+}
+
+__device__ __forceinline__ void wgrad_advance(const ConvArgs &a, const WLanes &w, UnitState &st)
+{
+    st.vox += w.nvox;
+    st.ox += w.dx;
+    st.oy += w.dy;
+    st.oz += w.dz;
+    st.b += w.db;
+    if (st.ox >= a.Wo) {
+        st.ox -= a.Wo;
+        ++st.oy;
+    }
+    if (st.oy >= a.Ho) {
+        st.oy -= a.Ho;
+        ++st.oz;
+    }
+    if (st.oz >= a.Do) {
+        st.oz -= a.Do;
+        ++st.b;
+    }
+}
+
+// The thread's voxel: element offset of its tap origin and the taps inside the
+// grid (none beyond the unit).
+__device__ __forceinline__ uint32_t wgrad_taps(const ConvArgs &a, const UnitState &st, int64_t &org)
+{
+    const int z = st.oz * a.stride - 1, y = st.oy * a.stride - 1, x = st.ox * a.stride - 1;
+    org = ((((int64_t)st.b * a.D + z) * a.H + y) * a.W + x) * a.cin;
+    // an axis's first tap is inside unless it reads -1, its last unless it reads
+    // n, its middle one always; taps t = 9 tz + 3 ty + tx
+    uint32_t m = (1u << 27) - 1u;
+    if (x < 0)
+        m &= ~0x1249249u;
+    if (x + 2 >= a.W)
+        m &= ~(0x1249249u << 2);
+    if (y < 0)
+        m &= ~0x1C0E07u;
+    if (y + 2 >= a.H)
+        m &= ~(0x1C0E07u << 6);
+    if (z < 0)
+        m &= ~0x1FFu;
+    if (z + 2 >= a.D)
+        m &= ~(0x1FFu << 18);
+    return st.vox < st.vend ? m : 0u;
+}
 
 template <int MODE>
 __device__ __forceinline__ void unit_begin(const ConvArgs &a, const Cursor &c, int tid,
@@ -460,17 +606,27 @@ __device__ __forceinline__ void unit_begin(const ConvArgs &a, const Cursor &c, i
             }
         }
     } else {
-        const int mt = c.u % a.mtiles;
-        st.m0 = mt * 128 + (tid >> 6) * 64;
-        st.kreal = 27 * a.cin;
+        const int split = c.u / a.mtiles;
+        st.g0 = (c.u - split * a.mtiles) * 16;
+        st.vend = min((split + 1) * a.Kreal, a.rows);
+        const WLanes w = wgrad_lanes(a);
+        st.vox = split * a.Kreal + ((tid >> w.sh) & (kBK - 1));
+        unsigned r = (unsigned)st.vox;  // beyond the rows only where nothing is read
+        st.ox = (int)(r % (unsigned)a.Wo);
+        r /= (unsigned)a.Wo;
+        st.oy = (int)(r % (unsigned)a.Ho);
+        r /= (unsigned)a.Ho;
+        st.oz = (int)(r % (unsigned)a.Do);
+        st.b = (int)(r / (unsigned)a.Do);
     }
 }
 
 // This thread's share of one work item (slot A, B).
 template <int MODE>
-__device__ __forceinline__ void fill_item(const ConvArgs &a, const Cursor &c, const UnitState &st,
+__device__ __forceinline__ void fill_item(const ConvArgs &a, const Cursor &c, UnitState &st,
                                           uint8_t *A, uint8_t *B, int tid, const int *tapoff,
-                                          const int (*ctoff)[8], int kslice0)
+                                          const int (*ctoff)[8], int kslice0, const WLanes &wl,
+                                          const int2 *gtab)
 {
     const uint32_t sA = (uint32_t)__cvta_generic_to_shared(A);
     if (MODE == FWD) {
@@ -521,93 +677,87 @@ __device__ __forceinline__ void fill_item(const ConvArgs &a, const Cursor &c, co
             cp16(sA + kmajor_off(tid, kc), ok ? a.act + st.rowoff + off + co : a.act, ok);
         }
     } else {
-        // A: rows m = (t, ci) of the M tile, K = 64 voxels. Thread tid owns
-        // voxel k = tid % 64 of the slice and half h = tid / 64 of the M
-        // groups; 8 consecutive lanes write 8 consecutive K rows of one core
-        // matrix (128 contiguous bytes).
-        const int vbeg = (c.u / a.mtiles) * a.Kreal;
-        const int vend = min(vbeg + a.Kreal, a.rows);
-        const int k = tid & (kBK - 1), h = tid >> 6;
-        const int vox = vbeg + c.kk * kBK + k;
-        const bool vok = vox < vend;
-        int r = vok ? vox : 0;
-        const int ox = r % a.Wo;
-        r /= a.Wo;
-        const int oy = r % a.Ho;
-        r /= a.Ho;
-        const int oz = r % a.Do;
-        const int bb = r / a.Do;
-        const int zz = oz * a.stride - 1, yy = oy * a.stride - 1, xx = ox * a.stride - 1;
-        uint32_t mz = 0, my = 0, mx = 0;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            mz |= (uint32_t)((unsigned)(zz + d) < (unsigned)a.D) << d;
-            my |= (uint32_t)((unsigned)(yy + d) < (unsigned)a.H) << d;
-            mx |= (uint32_t)((unsigned)(xx + d) < (unsigned)a.W) << d;
-        }
-        if (!vok)
-            mz = 0;
-        const int64_t org = ((((int64_t)bb * a.D + zz) * a.H + yy) * a.W + xx) * a.cin;
+        // A: rows m = (t, ci) of the M tile, K = 64 voxels
+        const int v0 = st.vox - ((tid >> wl.sh) & (kBK - 1));  // first voxel of the slice
         if (a.cin == 2) {
-            // word t of the 55 rows (tap t, 2 channels; t = 27 the bias row),
-            // 14 words per thread; words 28..31 and the groups past them stay
-            // zero (cleared once: a 2-channel layer has one M tile)
+            // Thread tid owns voxel tid % 64 of the slice and half h = tid / 64 of the
+            // words: word t of the 55 rows (tap t, 2 channels; t = 27 the bias row), 14
+            // words per thread; words 28..31 and the groups past them stay zero
+            // (cleared once: a 2-channel layer has one M tile)
+            const int k = tid & (kBK - 1), h = tid >> 6;
+            int64_t org;
+            const uint32_t taps = wgrad_taps(a, st, org);
             const uint32_t *src = reinterpret_cast<const uint32_t *>(a.act);
 #pragma unroll
             for (int j = 0; j < 14; ++j) {
                 const int t = h * 14 + j;
                 const int off = mnmajor_off(t >> 2, k) + (t & 3) * 4;
                 if (t == 27) {
-                    *reinterpret_cast<uint32_t *>(A + off) = vok ? 0x3F80u : 0u;
+                    *reinterpret_cast<uint32_t *>(A + off) = st.vox < st.vend ? 0x3F80u : 0u;
                 } else {
-                    bool ok = ((mz >> (t / 9)) & (my >> ((t / 3) % 3)) & (mx >> (t % 3))) & 1u;
+                    bool ok = (taps >> t) & 1u;
                     if (ok && !al_index_ok(org + tapoff[t], a.act_elems - 1))
                         ok = false;
                     cp4(sA + off, ok ? src + (org + tapoff[t]) / 2 : src, ok);
                 }
             }
+            wgrad_advance(a, wl, st);
         } else {
-            int m0 = st.m0;
-            int t = m0 / a.cin, ci = m0 - t * a.cin;
-#pragma unroll
-            for (int j = 0; j < 8; ++j, m0 += 8) {
-                const int g = h * 8 + j;
-                const int off = mnmajor_off(g, k);
-                if (m0 < st.kreal) {
-                    bool ok = ((mz >> (t / 9)) & (my >> ((t / 3) % 3)) & (mx >> (t % 3))) & 1u;
-                    if (ok && !al_index_ok(org + tapoff[t] + ci, a.act_elems - 7))
-                        ok = false;
-                    cp16(sA + off, ok ? a.act + org + tapoff[t] + ci : a.act, ok);
-                } else if (m0 == st.kreal) {
-                    *reinterpret_cast<uint4 *>(A + off) = make_uint4(vok ? 0x3F80u : 0u, 0, 0, 0);
-                } else if (a.mtiles > 1) {
-                    *reinterpret_cast<uint4 *>(A + off) = make_uint4(0, 0, 0, 0);
+            const int gbias = 27 * (a.cin >> 3);
+            const int cl = tid & ((1 << wl.sh) - 1);
+            // with one lane per voxel, the threads' second half takes the odd groups
+            const int half = wl.sh == 0 ? tid >> 6 : 0;
+            const int first = (half << wl.sh) + cl, gstep = wl.sh == 0 ? 2 : 1 << wl.sh;
+            for (int done = 0; done < kBK; done += wl.nvox) {
+                const int k = st.vox - v0;
+                int64_t org;
+                const uint32_t taps = wgrad_taps(a, st, org);
+                const uint32_t row = sA + mnmajor_off(0, k);
+#pragma unroll 4
+                for (int gl = first; gl < 16; gl += gstep) {
+                    const int g = st.g0 + gl;
+                    if (g < gbias) {
+                        const int2 e = gtab[g];
+                        bool ok = (taps >> e.y) & 1u;
+                        const int64_t at = org + e.x;
+                        if (ok && !al_index_ok(at, a.act_elems - 7))
+                            ok = false;
+                        cp16(row + gl * 1024, ok ? a.act + at : a.act, ok);
+                    } else if (g == gbias) {
+                        *reinterpret_cast<uint4 *>(A + mnmajor_off(gl, k)) =
+                            make_uint4(st.vox < st.vend ? 0x3F80u : 0u, 0, 0, 0);
+                    } else if (a.mtiles > 1) {
+                        *reinterpret_cast<uint4 *>(A + mnmajor_off(gl, k)) = make_uint4(0, 0, 0, 0);
+                    }
                 }
-                ci += 8;
-                if (ci >= a.cin) {
-                    ci -= a.cin;
-                    ++t;
-                }
+                wgrad_advance(a, wl, st);
             }
         }
-        // B: rows n = co (N / 8 groups) x 64 voxels
-        const int kbase = vbeg + c.kk * kBK;
+        // B: rows n = co (N / 8 groups) x 64 voxels, contiguous in memory
         const uint32_t sB = (uint32_t)__cvta_generic_to_shared(B);
-        const int ng = a.N >> 3;
-        for (int idx = tid; idx < ng * kBK; idx += kThreads) {
-            const int krow = idx & 7, cm = idx >> 3;
-            const int g = cm % ng, kg = cm / ng;
-            const int kk2 = kg * 8 + krow;
-            const int v = kbase + kk2;
-            bool ok = v < vend;
-            if (ok && !al_index_ok((int64_t)v * a.cout + g * 8, a.gout_elems - 7))
+        const int ng = a.N >> 3, dv = kThreads / ng, dg = kThreads - dv * ng;
+        int v = tid / ng, g = tid - v * ng;
+        const __nv_bfloat16 *src = a.gout + (size_t)v0 * a.cout + tid * 8;
+        for (int idx = tid; idx < ng * kBK; idx += kThreads, src += kThreads * 8) {
+            bool ok = v0 + v < st.vend;
+            if (ok && !al_index_ok((int64_t)v0 * a.cout + (int64_t)idx * 8, a.gout_elems - 7))
                 ok = false;
-            cp16(sB + mnmajor_off(g, kk2), ok ? a.gout + (size_t)v * a.cout + g * 8 : a.gout, ok);
+            cp16(sB + mnmajor_off(g, v), ok ? src : a.gout, ok);
+            v += dv;
+            g += dg;
+            if (g >= ng) {
+                g -= ng;
+                ++v;
+            }
         }
     }
 }
 
 // ---- epilogue: row tid of the finished tile from TMEM lane tid -------------
+template <int MODE>
+__device__ __forceinline__ void epilogue_row(const ConvArgs &a, size_t orow, bool valid,
+                                             uint32_t lane_addr, int cls = 0);
+
 template <int MODE>
 __device__ __forceinline__ void epilogue(const ConvArgs &a, const Cursor &c, uint32_t lane_addr,
                                          int tid)
@@ -640,74 +790,96 @@ __device__ __forceinline__ void epilogue(const ConvArgs &a, const Cursor &c, uin
         const int mt = c.u % a.mtiles, split = c.u / a.mtiles;
         orow = (size_t)split * a.mtiles * 128 + (size_t)mt * 128 + tid;
     }
+    epilogue_row<MODE>(a, orow, valid, lane_addr, c.cls);
+}
+
+// Columns c0 .. c0 + 15 of output row orow. cls: K partition of a split forward
+// pass. mask: the row's ReLU factors already loaded (nullable).
+template <int MODE>
+__device__ __forceinline__ void epilogue_chunk(const ConvArgs &a, size_t orow, float (&v)[16],
+                                               int c0, int cls, const uint4 *mask = nullptr)
+{
+    if (MODE == FWD && a.part) {
+        // split K: this K partition's partial sums, reduced by k_fwd_reduce
+        float4 *o = reinterpret_cast<float4 *>(a.part + ((size_t)cls * a.rows + orow) * a.N + c0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        return;
+    }
+    if (MODE == FWD) {
+        if (a.bias) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+                v[i] += __ldg(a.bias + c0 + i);
+        }
+        if (a.relu) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+                v[i] = fmaxf(v[i], 0.0f);
+        }
+    } else if (MODE == DGRAD) {
+        if (a.addend) {
+            const uint4 *p =
+                reinterpret_cast<const uint4 *>(a.addend + orow * a.add_stride + a.add_off + c0);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const uint4 w = __ldg(p + q);
+                const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    v[8 * q + 2 * h] += bf16_lo(ws[h]);
+                    v[8 * q + 2 * h + 1] += bf16_hi(ws[h]);
+                }
+            }
+        }
+        if (a.mask) {
+            const uint4 *p = reinterpret_cast<const uint4 *>(a.mask + orow * a.N + c0);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const uint4 w = mask ? mask[q] : __ldg(p + q);
+                const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    if (!(bf16_lo(ws[h]) > 0.0f))
+                        v[8 * q + 2 * h] = 0.0f;
+                    if (!(bf16_hi(ws[h]) > 0.0f))
+                        v[8 * q + 2 * h + 1] = 0.0f;
+                }
+            }
+        }
+    }
+    if (MODE == WGRAD || (MODE == FWD && a.out_f32)) {
+        float4 *o = reinterpret_cast<float4 *>(static_cast<float *>(a.out) + orow * a.N + c0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    } else {
+        uint32_t w[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            w[i] = pack_bf16(v[2 * i], v[2 * i + 1]);
+        uint4 *o = reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(a.out) + orow * a.N + c0);
+        if (a.wide) {
+            store32(o, w);
+        } else {
+            o[0] = make_uint4(w[0], w[1], w[2], w[3]);
+            o[1] = make_uint4(w[4], w[5], w[6], w[7]);
+        }
+    }
+}
+
+// Output row orow (when valid) from N columns of this thread's TMEM lane; every
+// lane of the warp calls.
+template <int MODE>
+__device__ __forceinline__ void epilogue_row(const ConvArgs &a, size_t orow, bool valid,
+                                             uint32_t lane_addr, int cls)
+{
     for (int c0 = 0; c0 < a.N; c0 += 16) {
         float v[16];
         tc_load16(lane_addr + (uint32_t)c0, v);
-        if (!valid)
-            continue;
-        if (MODE == FWD && a.part) {
-            // split K: this K partition's partial sums, reduced by k_fwd_reduce
-            float4 *o = reinterpret_cast<float4 *>(a.part + ((size_t)c.cls * a.rows + orow) * a.N + c0);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-            continue;
-        }
-        if (MODE == FWD) {
-            if (a.bias) {
-#pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    v[i] += __ldg(a.bias + c0 + i);
-            }
-            if (a.relu) {
-#pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    v[i] = fmaxf(v[i], 0.0f);
-            }
-        } else if (MODE == DGRAD) {
-            if (a.addend) {
-                const uint4 *p = reinterpret_cast<const uint4 *>(a.addend + orow * a.add_stride +
-                                                                 a.add_off + c0);
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const uint4 w = __ldg(p + q);
-                    const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                    for (int h = 0; h < 4; ++h) {
-                        v[8 * q + 2 * h] += bf16_lo(ws[h]);
-                        v[8 * q + 2 * h + 1] += bf16_hi(ws[h]);
-                    }
-                }
-            }
-            if (a.mask) {
-                const uint4 *p = reinterpret_cast<const uint4 *>(a.mask + orow * a.N + c0);
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const uint4 w = __ldg(p + q);
-                    const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                    for (int h = 0; h < 4; ++h) {
-                        if (!(bf16_lo(ws[h]) > 0.0f))
-                            v[8 * q + 2 * h] = 0.0f;
-                        if (!(bf16_hi(ws[h]) > 0.0f))
-                            v[8 * q + 2 * h + 1] = 0.0f;
-                    }
-                }
-            }
-        }
-        if (MODE == WGRAD || (MODE == FWD && a.out_f32)) {
-            float4 *o = reinterpret_cast<float4 *>(static_cast<float *>(a.out) + orow * a.N + c0);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-        } else {
-            uint4 *o = reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(a.out) + orow * a.N +
-                                                 c0);
-            o[0] = make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]),
-                              pack_bf16(v[6], v[7]));
-            o[1] = make_uint4(pack_bf16(v[8], v[9]), pack_bf16(v[10], v[11]),
-                              pack_bf16(v[12], v[13]), pack_bf16(v[14], v[15]));
-        }
+        if (valid)
+            epilogue_chunk<MODE>(a, orow, v, c0, cls);
     }
 }
 
@@ -762,6 +934,8 @@ __global__ void __launch_bounds__(kThreads, MODE == WGRAD ? 4 : 1) k_conv(const 
     int *s_nst = s_unit0 + kMaxClasses + 1;
     int *s_slice0 = s_nst + kMaxClasses;
     Tables &T = *reinterpret_cast<Tables *>(s_slice0 + kMaxClasses);
+    // WGRAD: per group of 8 M rows, element offset from a voxel's tap origin and tap
+    int2 *gtab = reinterpret_cast<int2 *>(((uintptr_t)(&T + 1) + 7) & ~(uintptr_t)7);
     const uint32_t bar_full = smem_u32(bars), bar_free = bar_full + 8 * kStages,
                    bar_done = bar_full + 16 * kStages;
     const int tid = threadIdx.x, warp = tid >> 5;
@@ -773,6 +947,14 @@ __global__ void __launch_bounds__(kThreads, MODE == WGRAD ? 4 : 1) k_conv(const 
         s_slice0[tid] = a.cls_slice0[tid < a.classes ? tid : 0];
     }
     build_tables(a, T, tid, MODE);
+    if (MODE == WGRAD && a.cin != 2) {
+        const int nc = a.cin >> 3;
+        for (int g = tid; g < 27 * nc; g += kThreads) {
+            const int t = g / nc;
+            gtab[g] = make_int2(((t / 9 * a.H + t / 3 % 3) * a.W + t % 3) * a.cin + (g - t * nc) * 8, t);
+        }
+    }
+    const WLanes wl = MODE == WGRAD ? wgrad_lanes(a) : WLanes{};
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(bar_full + 8 * s, 1);
@@ -820,7 +1002,7 @@ __global__ void __launch_bounds__(kThreads, MODE == WGRAD ? 4 : 1) k_conv(const 
                           (uint32_t)btile, bar_full + 8 * s);
             }
             fill_item<MODE>(a, prod, ust, sA + s * kATile, B, tid, T.tapoff, T.ctoff,
-                            MODE == FWD ? s_slice0[prod.cls] : 0);
+                            MODE == FWD ? s_slice0[prod.cls] : 0, wl, gtab);
             ++pit;
             if (++prod.kk >= prod.nst) {
                 prod.kk = 0;
@@ -885,21 +1067,29 @@ __global__ void __launch_bounds__(kThreads, MODE == WGRAD ? 4 : 1) k_conv(const 
 
 // ---- two input channels: forward and weight adjoint --------------------------
 // A tap row (dz, dy) of an output voxel reads three x-neighbouring voxels of
-// two bf16 channels: 12 consecutive bytes, which with a zero pair make one
+// two bf16 channels: 12 consecutive bytes, which with a fourth pair make one
 // 16-byte chunk (dx, ci) of 8 K elements. A 128-voxel tile is 9 planes (one
 // per (dz, dy)) of 128 chunks, 16 bytes apart: as K-major rows the operand of
-// the forward pass (K = 9 chunks and one of zeros, 5 MMAs of K = 16), as MN-major groups of 8 rows that of the weight
-// adjoint (M = 9 chunks and a chunk of ones for the bias, K = 128 voxels).
-// A thread gathers the 27 words of its voxel into registers by plain loads (a
-// warp's are 8 bytes apart) and stores 9 chunks; k_conv filled the same tile
+// the forward pass (K = 9 chunks and one of zeros, 5 MMAs of K = 16), as
+// MN-major groups of 8 rows that of the weight adjoint (M = 9 groups, K = 128
+// voxels; the first chunk's fourth pair holds the one that gives the bias).
+// A thread gathers the 27 words of its voxel into registers by plain loads
+// (with stride 2 and an even row, one 8-byte load per tap row and the third
+// word from the lane before) and stores 9 chunks; k_conv filled the same tile
 // with 27 4-byte asynchronous copies a row, which was bound by their number.
-// 16 x 128^3 -> 64^3, stride 2: forward 205 -> @@ us, weight adjoint 280 -> @@ us;
-// reading the input and writing or reading the output takes 40 us.
+// One tile in shared memory: the next tile's loads are in flight in registers
+// while its MMAs run, and the room left is better used by more CTAs per SM.
+// 16 x 128^3 -> 64^3, stride 2: forward 205 -> @@ us, weight adjoint 280 -> @@ us
+// (103 and 145 us with two slots and three loads per tap row); reading the
+// input and writing or reading the output takes 40 us.
 constexpr int kC2Plane = 128 * 16;  // bytes of one plane of a tile
 constexpr int kC2Groups = 9;
-constexpr int kC2Slot = 10 * kC2Plane;  // a forward slot
 
-// The 9 chunks of output voxel `row` (zero outside the grid).
+// The 9 chunks of output voxel `row` (zero outside the grid). PAIR: stride 2
+// and an even W, so that voxels 2 ox and 2 ox + 1 are one aligned 8-byte load
+// and voxel 2 ox - 1 is the second of the lane before, when that lane has the
+// voxel before. Every lane of the warp calls.
+template <bool PAIR>
 __device__ __forceinline__ void c2_gather(const ConvArgs &a, int row, bool ok,
                                           uint32_t (&w)[kC2Groups][3])
 {
@@ -909,10 +1099,11 @@ __device__ __forceinline__ void c2_gather(const ConvArgs &a, int row, bool ok,
     const unsigned oy = r % (unsigned)a.Ho;
     r /= (unsigned)a.Ho;
     const unsigned oz = r % (unsigned)a.Do, b = r / (unsigned)a.Do;
-    const int z0 = (int)oz * a.stride - 1, y0 = (int)oy * a.stride - 1,
-              x0 = (int)ox * a.stride - 1;
+    const int st = PAIR ? 2 : a.stride;
+    const int z0 = (int)oz * st - 1, y0 = (int)oy * st - 1, x0 = (int)ox * st - 1;
     const uint32_t *src = reinterpret_cast<const uint32_t *>(a.act);
     const bool xl = x0 >= 0, xr = x0 + 2 < a.W;
+    const bool alone = (threadIdx.x & 31) == 0 && xl;  // no lane before it
     const int64_t org = (((int64_t)b * a.D + z0) * a.H + y0) * a.W + x0;
 #pragma unroll
     for (int g = 0; g < kC2Groups; ++g) {
@@ -921,40 +1112,57 @@ __device__ __forceinline__ void c2_gather(const ConvArgs &a, int row, bool ok,
         const int64_t o = org + ((int64_t)dz * a.H + dy) * a.W;
         if (in && !al_index_ok(o + 1, a.act_elems / 2))
             in = false;
-        w[g][0] = in && xl ? __ldg(src + o) : 0u;
-        w[g][1] = in ? __ldg(src + o + 1) : 0u;
-        w[g][2] = in && xr ? __ldg(src + o + 2) : 0u;
+        if (PAIR) {
+            const uint2 p = in ? __ldg(reinterpret_cast<const uint2 *>(src + o + 1))
+                               : make_uint2(0u, 0u);
+            w[g][0] = in && alone ? __ldg(src + o) : 0u;
+            w[g][1] = p.x;
+            w[g][2] = p.y;
+        } else {
+            w[g][0] = in && xl ? __ldg(src + o) : 0u;
+            w[g][1] = in ? __ldg(src + o + 1) : 0u;
+            w[g][2] = in && xr ? __ldg(src + o + 2) : 0u;
+        }
     }
 }
 
-__device__ __forceinline__ void c2_store(uint8_t *A, int tid, const uint32_t (&w)[kC2Groups][3])
+// Stores the chunks (every lane calls); fourth: the fourth pair of chunk 0.
+template <bool PAIR>
+__device__ __forceinline__ void c2_store(const ConvArgs &a, uint8_t *A, int row, bool ok,
+                                         uint32_t fourth, const uint32_t (&w)[kC2Groups][3])
 {
+    const int tid = threadIdx.x;
+    const bool left = PAIR && (tid & 31) != 0 && ok && (unsigned)row % (unsigned)a.Wo != 0;
 #pragma unroll
-    for (int g = 0; g < kC2Groups; ++g)
+    for (int g = 0; g < kC2Groups; ++g) {
+        uint32_t w0 = w[g][0];
+        if (PAIR) {
+            const uint32_t up = __shfl_up_sync(0xffffffffu, w[g][2], 1);
+            w0 = left ? up : w0;
+        }
         *reinterpret_cast<uint4 *>(A + g * kC2Plane + tid * 16) =
-            make_uint4(w[g][0], w[g][1], w[g][2], 0u);
+            make_uint4(w0, w[g][1], w[g][2], g == 0 ? fourth : 0u);
+    }
 }
 
-// Forward: shared memory = 2 slots of 10 planes, the weights as 10 chunks of N
-// rows, barriers. D of a tile is double buffered in TMEM, so that a tile's
-// epilogue runs beside the next tile's MMAs.
-template <int N>
+// Forward: shared memory = the tile's 10 planes, the weights as 10 chunks of N
+// rows, barrier.
+template <int N, bool PAIR>
 __global__ void __launch_bounds__(kThreads) k_conv2_fwd(const ConvArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t *sm = reinterpret_cast<uint8_t *>(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
-    uint8_t *B = sm + 2 * kC2Slot;
+    uint8_t *A = reinterpret_cast<uint8_t *>(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
+    uint8_t *B = A + 10 * kC2Plane;
     uint64_t *bars = reinterpret_cast<uint64_t *>(B + 10 * N * 16);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 2);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 1);
     const uint32_t bar = smem_u32(bars);
     const int tid = threadIdx.x, warp = tid >> 5;
     if (tid == 0) {
         mbar_init(bar, 1);
-        mbar_init(bar + 8, 1);
         fence_mbar_init();
     }
     if (warp == 0) {
-        tmem_alloc(smem_u32(tslot), 2 * N);
+        tmem_alloc(smem_u32(tslot), 32);
         tmem_relinquish();
     }
     // B: chunk g, row n, element (dx, ci) = w[n][t = 3 g + dx][ci] from the packed
@@ -967,130 +1175,118 @@ __global__ void __launch_bounds__(kThreads) k_conv2_fwd(const ConvArgs a)
             v = a.wpk[(n / 8) * 512 + (k / 8) * 64 + (n % 8) * 8 + (k & 7)];
         reinterpret_cast<__nv_bfloat16 *>(B)[e] = v;
     }
-    for (int k = 0; k < 2; ++k)
-        *reinterpret_cast<uint4 *>(sm + k * kC2Slot + kC2Groups * kC2Plane + tid * 16) =
-            make_uint4(0u, 0u, 0u, 0u);
+    *reinterpret_cast<uint4 *>(A + kC2Groups * kC2Plane + tid * 16) = make_uint4(0u, 0u, 0u, 0u);
     tc_before_sync();
     __syncthreads();
     tc_after_sync();
     const uint32_t tmem = *tslot;
-    const uint32_t bdesc = smem_u32(B);
+    const uint32_t a0 = smem_u32(A), b0 = smem_u32(B);
     uint32_t w[kC2Groups][3];
-    auto finish = [&](int tile, int slot, uint32_t use) {
-        mbar_wait(bar + 8 * slot, use & 1);
+    auto finish = [&](int tile, int it) {
+        mbar_wait(bar, (uint32_t)it & 1);
         tc_after_sync();
-        Cursor c;
-        c.tile = tile;
-        epilogue<FWD>(a, c, tmem + slot * N + ((uint32_t)(warp * 32) << 16), tid);
+        const int row = tile * 128 + tid;
+        epilogue_row<FWD>(a, (size_t)row, row < a.rows, tmem + ((uint32_t)(warp * 32) << 16));
         tc_before_sync();
     };
     int it = 0;
     for (int tile = blockIdx.x; tile < a.units; tile += gridDim.x, ++it) {
-        const int slot = it & 1;
         const int row = tile * 128 + tid;
-        c2_gather(a, row, row < a.rows, w);
-        // the MMAs of two tiles ago, the slot's last use, are done: their tile's
-        // epilogue has waited for them
-        uint8_t *A = sm + slot * kC2Slot;
-        c2_store(A, tid, w);
+        const bool ok = row < a.rows;
+        c2_gather<PAIR>(a, row, ok, w);
+        if (it > 0)
+            finish(tile - gridDim.x, it - 1);
+        c2_store<PAIR>(a, A, row, ok, 0u, w);
         fence_proxy_async();
         __syncthreads();
         if (tid == 0) {
             tc_after_sync();
-            const uint32_t a0 = smem_u32(A);
 #pragma unroll
             for (int j = 0; j < 5; ++j)
-                tc_mma(tmem + slot * N, sdesc(a0 + 2 * j * kC2Plane, kC2Plane, 128),
-                       sdesc(bdesc + 2 * j * N * 16, N * 16, 128), a.idesc, j != 0);
-            tc_commit(bar + 8 * slot);
+                tc_mma(tmem, sdesc(a0 + 2 * j * kC2Plane, kC2Plane, 128),
+                       sdesc(b0 + 2 * j * N * 16, N * 16, 128), a.idesc, j != 0);
+            tc_commit(bar);
         }
-        if (it > 0)
-            finish(tile - gridDim.x, slot ^ 1, (uint32_t)((it - 1) >> 1));
     }
     if (it > 0)
-        finish(blockIdx.x + (it - 1) * gridDim.x, (it - 1) & 1, (uint32_t)((it - 1) >> 1));
+        finish(blockIdx.x + (it - 1) * gridDim.x, it - 1);
     __syncthreads();
     if (warp == 0)
-        tmem_dealloc(tmem, 2 * N);
+        tmem_dealloc(tmem, 32);
 }
 
-// Weight adjoint: shared memory = 2 slots of 16 planes (the 9 chunks, the
-// ones, planes whose rows of D are never read) and of the output gradient's N / 8
-// planes, barriers. One D per unit (a split of the voxels) in TMEM.
-template <int N>
+// Weight adjoint: shared memory = 16 planes (the 9 of the tile, the N / 8 of
+// the output gradient, and what M = 128 reads beyond them, rows of D that are
+// never used), barriers. One D per unit (a split of the voxels) in TMEM.
+template <int N, bool PAIR>
 __global__ void __launch_bounds__(kThreads) k_conv2_wgrad(const ConvArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t *sm = reinterpret_cast<uint8_t *>(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
-    constexpr int SLOT = (16 + N / 8) * kC2Plane;
-    uint64_t *bars = reinterpret_cast<uint64_t *>(sm + 2 * SLOT);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 3);
+    uint8_t *A = reinterpret_cast<uint8_t *>(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
+    uint8_t *G = A + kC2Groups * kC2Plane;
+    uint64_t *bars = reinterpret_cast<uint64_t *>(A + 16 * kC2Plane);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 2);
     const uint32_t bar = smem_u32(bars);
     const int tid = threadIdx.x, warp = tid >> 5;
-    constexpr uint32_t COLS = N < 32 ? 32 : (N <= 64 ? (N <= 32 ? 32 : 64) : 128);
+    static_assert(kC2Groups + N / 8 <= 16, "the output gradient's planes lie inside the 16");
     if (tid == 0) {
-        for (int k = 0; k < 3; ++k)
-            mbar_init(bar + 8 * k, 1);
+        mbar_init(bar, 1);
+        mbar_init(bar + 8, 1);
         fence_mbar_init();
     }
     if (warp == 0) {
-        tmem_alloc(smem_u32(tslot), COLS);
+        tmem_alloc(smem_u32(tslot), 32);
         tmem_relinquish();
     }
-    for (int s = 0; s < 2; ++s)
-        for (int g = kC2Groups; g < 16; ++g)
-            *reinterpret_cast<uint4 *>(sm + s * SLOT + g * kC2Plane + tid * 16) =
-                make_uint4(g == kC2Groups ? 0x3F80u : 0u, 0u, 0u, 0u);
     tc_before_sync();
     __syncthreads();
     tc_after_sync();
     const uint32_t tmem = *tslot;
+    const uint32_t a0 = smem_u32(A), g0 = smem_u32(G);
     uint32_t w[kC2Groups][3];
     int it = 0;
     uint32_t nunit = 0;
     for (int u = blockIdx.x; u < a.units; u += gridDim.x, ++nunit) {
         const int v0 = u * a.Kreal, v1 = min(v0 + a.Kreal, a.rows);
         for (int v = v0; v < v1; v += 128, ++it) {
-            const int slot = it & 1;
             const int row = v + tid;
             const bool ok = row < v1;
-            c2_gather(a, row, ok, w);
-            if (it >= 2)
-                mbar_wait(bar + 8 * slot, (uint32_t)((it >> 1) - 1) & 1);
-            uint8_t *A = sm + slot * SLOT, *G = A + 16 * kC2Plane;
-            const uint32_t sG = smem_u32(G);
+            c2_gather<PAIR>(a, row, ok, w);
+            uint4 gr[N / 8];
 #pragma unroll
             for (int n = 0; n < N / 8; ++n) {
                 bool in = ok;
                 if (in && !al_index_ok((int64_t)row * N + n * 8, a.gout_elems - 7))
                     in = false;
-                cp16(sG + n * kC2Plane + tid * 16, in ? a.gout + (size_t)row * N + n * 8 : a.gout,
-                     in);
+                gr[n] = in ? __ldg(reinterpret_cast<const uint4 *>(a.gout + (size_t)row * N) + n)
+                           : make_uint4(0u, 0u, 0u, 0u);
             }
-            cp_commit();
-            c2_store(A, tid, w);
-            cp_wait<0>();
+            if (it > 0)
+                mbar_wait(bar, (uint32_t)(it - 1) & 1);
+            c2_store<PAIR>(a, A, row, ok, ok ? 0x3F80u : 0u, w);
+#pragma unroll
+            for (int n = 0; n < N / 8; ++n)
+                *reinterpret_cast<uint4 *>(G + n * kC2Plane + tid * 16) = gr[n];
             fence_proxy_async();
             __syncthreads();
             if (tid == 0) {
                 tc_after_sync();
-                const uint32_t a0 = smem_u32(A), g0 = smem_u32(G);
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
                     tc_mma(tmem, sdesc(a0 + 256 * j, 128, kC2Plane),
                            sdesc(g0 + 256 * j, 128, kC2Plane), a.idesc, v != v0 || j != 0);
-                tc_commit(bar + 8 * slot);
+                tc_commit(bar);
             }
         }
         if (tid == 0)
-            tc_commit(bar + 16);
-        mbar_wait(bar + 16, nunit & 1);
+            tc_commit(bar + 8);
+        mbar_wait(bar + 8, nunit & 1);
         tc_after_sync();
-        // row m = chunk g, (dx, ci) of the chunk -> row 2 (3 g + dx) + ci of the
-        // partial sums; the ones' first row -> row 54
+        // row of chunk g, element (dx, ci) -> row 2 (3 g + dx) + ci of the partial
+        // sums; the one (chunk 0, fourth pair) -> row 54
         const int g = tid >> 3, q = tid & 7;
-        const bool keep = g < kC2Groups ? q < 6 : (g == kC2Groups && q == 0);
-        const int m = g < kC2Groups ? 6 * g + q : 54;
+        const bool keep = (g < kC2Groups && q < 6) || tid == 6;
+        const int m = tid == 6 ? 54 : 6 * g + q;
         float *o = static_cast<float *>(a.out) + ((size_t)u * 128 + m) * N;
 #pragma unroll
         for (int c0 = 0; c0 < N; c0 += 16) {
@@ -1107,7 +1303,550 @@ __global__ void __launch_bounds__(kThreads) k_conv2_wgrad(const ConvArgs a)
     }
     __syncthreads();
     if (warp == 0)
-        tmem_dealloc(tmem, COLS);
+        tmem_dealloc(tmem, 32);
+}
+
+__device__ __forceinline__ int class_ntaps(int cls);
+
+// ---- passes from a staged slab -------------------------------------------------
+// k_conv gathers every row of the im2col operand tap by tap, so each input
+// value passes through L2 and shared memory up to 27 times, and those copies
+// bound it. Here a CTA stages the input of a band of R output rows once, as
+// planes of 8 channels (16 bytes) per voxel, voxels P apart per row. With the
+// no-swizzle layout a K-major operand is 16-byte rows of consecutive addresses,
+// so the rows of 128 consecutive positions of the band, shifted by a tap, are
+// the same memory at another start address: every tap is a descriptor, and the
+// operand costs nothing beyond the staging (halo columns make a few of the 128
+// rows idle). Read as MN-major groups of 8 rows, the same planes are the operand
+// of the weight adjoint: the voxels are K, and 16 consecutive planes one MMA's
+// 128 rows at one shift.
+//
+// The kinds (q: output position; for the stride-2 input adjoint q indexes voxel
+// pairs, and the 8 parity classes of 2 q + c accumulate side by side in TMEM
+// from the same slab):
+//   FWD1   source q + d                    3 slices, rows and columns q - 1 .. q + 1
+//   FWD2   source 2 q + d, split by parity: odd sources 2 q - 1 and 2 q + 1 are
+//          neighbours in the odd block, 2 q is in the even block
+//   DGRAD1 source q - d                    as FWD1 with the taps mirrored
+//   DGRAD2 source q and q + 1              2 slices, rows q, q + 1, columns q, q + 1
+//   WGRAD2 the slab of FWD2 against the output gradient of the band's positions
+// Planes lie in the order (y, x parity block; z slice; 8 channels). The blocks'
+// order (odd y, even x), (odd, odd), (even, odd), (even, even) makes the planes
+// that a shift of WGRAD2 uses consecutive: all at (0, 0), blocks 1-2 one column
+// on, 0-1 one row on, 1 both.
+//
+// Warps: the first 8 (16 for the input adjoints, whose epilogues read and write
+// the most) take the epilogue, the warps of a TMEM quarter sharing its columns;
+// one issues the MMAs; the others stage the slabs (16-byte asynchronous copies
+// along rows) into a ring, two in flight. D is double buffered in TMEM, so
+// staging, MMAs and epilogues of successive bands overlap. What it took, measured
+// on 16 x 64^3 -> 32^3, 16 -> 32 channels, stride 2 (forward / input adjoint /
+// weight adjoint):
+//   k_conv                                                   124 / 332 / 178 us
+//   a slab, the roles in turn, two CTAs per SM               106 / 154 us
+//   roles in warps, MMAs issued by one thread from a table
+//   in shared memory (its descriptors reach the uniform
+//   registers one by one, over 100 cycles an MMA)            150 / 154 / 187 us
+//   descriptors computed by the whole warp in uniform
+//   registers, one elected lane issuing                       83 / 125 / 100 us
+//   copies through L1 (two 16-byte pieces of a sector go to
+//   two planes; past L1 they fetched it twice), 15 staging
+//   warps, 16 epilogue warps, ReLU factors one group ahead    61 /  88 /  70 us
+// The bytes take 25, 45 and 25 us; staging bounds the forward pass and the weight
+// adjoint, the epilogue's loads and stores the input adjoint. The tensor core
+// needs about 60 cycles per MMA here whatever N <= 64 (its A operand's 4 KB), so
+// DGRAD2 joins the classes that share a shift into one MMA over their columns: the
+// class order 0 1 5 4 6 7 3 2 makes most of them adjacent, 17 MMAs per 16 channels
+// instead of 27.
+enum { FWD1 = 0, FWD2 = 1, DGRAD1 = 2, DGRAD2 = 3, WGRAD2 = 4 };
+// Epilogue and staging warps of a kind.
+__host__ __device__ constexpr int slab_epi(int kind)
+{
+    return kind == DGRAD1 || kind == DGRAD2 ? 16 : 8;
+}
+__host__ __device__ constexpr int slab_prod(int kind)
+{
+    return kind == DGRAD1 || kind == DGRAD2 ? 7 : 15;
+}
+__host__ __device__ constexpr int slab_threads(int kind)
+{
+    return 32 * (slab_epi(kind) + 1 + slab_prod(kind));
+}
+
+struct SlabArgs {
+    const __nv_bfloat16 *src;  // staged tensor, C channels
+    int Sz, Sy, Sx;            // its grid
+    int Qz, Qy, Qx;            // positions
+    int P;                     // positions per staged row
+    int R, T;                  // output rows of a band, 128-position tiles of it
+    int RB;                    // staged rows of a block
+    int nzb;                   // z slices
+    int plane;                 // bytes of a plane (8 channels)
+    int stage;                 // bytes of a ring stage
+    int gplane;                // WGRAD2: bytes of an output gradient plane
+    int goff;                  // WGRAD2: their offset in a stage
+    int ksteps;                // WGRAD2: K steps of 16 positions of a band
+    int nst;                   // ring stages
+    int slack;                 // bytes behind the ring that a window may read
+    int nacc;                  // accumulator sets (2: double buffered)
+    int nk;                    // MMAs of a tile or K step
+    int accs;                  // TMEM columns of one accumulator set
+    int bands, items;
+    int upu;                   // WGRAD2: items of a unit
+    int wbytes;                // weights in shared memory
+    int64_t src_elems;
+};
+
+// DGRAD2: the column order of the classes, and a shift's runs of adjacent classes.
+struct ShiftRun {
+    int shift, pos, n, first;  // shift bits (z, y, x), first place in the class order, classes
+};
+constexpr int kRuns = 17;
+// Shifts in descending order, so that a class sums its taps in the packed order;
+// the class whose first tap a shift is starts its sum by an MMA of its own.
+struct Runs {
+    ShiftRun r[kRuns] = {{7, 5, 1, 1}, {6, 4, 1, 1}, {6, 5, 1, 0}, {5, 2, 1, 1}, {5, 5, 1, 0},
+                         {4, 3, 1, 1}, {4, 2, 1, 0}, {4, 4, 2, 0}, {3, 6, 1, 1}, {3, 5, 1, 0},
+                         {2, 7, 1, 1}, {2, 4, 3, 0}, {1, 1, 1, 1}, {1, 2, 1, 0}, {1, 5, 2, 0},
+                         {0, 0, 1, 1}, {0, 1, 7, 0}};
+};
+__constant__ Runs c_runs = {};
+__constant__ int c_cls_order[8] = {0, 1, 5, 4, 6, 7, 3, 2};
+
+__device__ __forceinline__ int class_ntaps(int cls);
+
+template <int C, int KIND>
+__global__ void __launch_bounds__(slab_threads(KIND), 1) k_conv_slab(const ConvArgs a, const SlabArgs s)
+{
+    constexpr int NC = C / 8, NK16 = C / 16;
+    constexpr int kSlabEpi = slab_epi(KIND), kSlabProd = slab_prod(KIND),
+                  kSlabThreads = slab_threads(KIND);
+    constexpr int PARTS = kSlabEpi / 4;  // warps of a TMEM quarter
+    constexpr bool S2 = KIND == FWD2 || KIND == WGRAD2;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *ring = reinterpret_cast<uint8_t *>(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
+    // behind the last stage: what a window or a shifted tile reads beyond it
+    uint8_t *wsm = ring + s.nst * s.stage + s.slack;
+    uint64_t *bars = reinterpret_cast<uint64_t *>(wsm + ((s.wbytes + 127) & ~127));
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 12);
+    // DGRAD2: class and first column in it of each 16 columns (c + 8 column)
+    uint16_t *chunks = reinterpret_cast<uint16_t *>(tslot + 1);
+    const uint32_t bar_full = smem_u32(bars), bar_empty = bar_full + 32, bar_acc = bar_full + 64,
+                   bar_free = bar_full + 80;
+    const uint32_t ring0 = smem_u32(ring), w0 = smem_u32(wsm);
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform to the compiler
+
+    if (tid == 0) {
+        for (int k = 0; k < s.nst; ++k) {
+            mbar_init(bar_full + 8 * k, 32 * kSlabProd);
+            mbar_init(bar_empty + 8 * k, 1);
+        }
+        for (int k = 0; k < 2; ++k) {
+            mbar_init(bar_acc + 8 * k, 1);
+            mbar_init(bar_free + 8 * k, 32 * kSlabEpi);
+        }
+        fence_mbar_init();
+    }
+    if (warp == 0) {
+        tmem_alloc(smem_u32(tslot), a.tmem_cols);
+        tmem_relinquish();
+    }
+    if (KIND == DGRAD2 && tid < s.accs / 16) {
+        const int pos = 16 * tid / a.N;
+        chunks[tid] = (uint16_t)(c_cls_order[pos] | (16 * tid - pos * a.N) << 3);
+    }
+    if (KIND == WGRAD2) {
+        // zero the ring once: positions that no copy writes (the parity blocks' spare
+        // row and column) are read as K elements
+        for (int i = tid; i < (int)(wsm - ring) / 16; i += kSlabThreads)
+            reinterpret_cast<uint4 *>(ring)[i] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+        // the plane of ones behind the slab's planes: its first row sums the
+        // output gradient (the bias)
+        const int np = 12 * NC;
+        for (int i = tid; i < s.nst * (s.plane / 16); i += kSlabThreads) {
+            const int st = i / (s.plane / 16), k = i - st * (s.plane / 16);
+            *reinterpret_cast<uint32_t *>(ring + st * s.stage + np * s.plane + k * 16) = 0x3F80u;
+        }
+    } else {
+        // weights: 16-byte pieces (row n, 8 of K) of the packed copy
+        const uint4 *src = reinterpret_cast<const uint4 *>(a.wpk);
+        if (KIND == DGRAD2) {
+            // step (run, c16): rows of its classes, core matrices 128 bytes apart
+            // along K, 256 along N
+            const int per = a.N * 2;  // pieces of one class of one step
+            for (int e = tid; e < 27 * NK16 * per; e += kSlabThreads) {
+                int j = e / per, r = e - j * per;  // j: (run, c16, class of the run)
+                int run = 0;
+                while (j >= c_runs.r[run].n * NK16)
+                    j -= c_runs.r[run++].n * NK16;
+                const int c16 = j / c_runs.r[run].n, m = j - c16 * c_runs.r[run].n;
+                const int cls = c_cls_order[c_runs.r[run].pos + m], sh = c_runs.r[run].shift;
+                const int kc = r & 1, n = r >> 1;
+                // the tap of class cls at this shift: on an odd axis the first tap
+                // reads q + 1, the second q
+                const int cz = cls >> 2, cy = (cls >> 1) & 1, cx = cls & 1;
+                const int ix = cx & ~sh & 1, iy = cy & ~(sh >> 1) & 1, iz = cz & ~(sh >> 2) & 1;
+                const int kk = ((iz * (1 + cy) + iy) * (1 + cx) + ix) * NK16 + c16;
+                const int from = (a.cls_slice0[cls] + kk / 4) * a.N * 8 + (n >> 3) * 64 +
+                                 ((kk & 3) * 2 + kc) * 8 + (n & 7);
+                uint8_t *d = wsm + (size_t)(e / per - m) * a.N * 32;
+                const int rn = m * a.N + n;
+                *reinterpret_cast<uint4 *>(d + (rn >> 3) * 256 + kc * 128 + (rn & 7) * 16) =
+                    __ldg(src + from);
+            }
+        } else {
+            for (int e = tid; e < s.wbytes / 16; e += kSlabThreads)
+                reinterpret_cast<uint4 *>(wsm)[e] = __ldg(src + e);
+        }
+    }
+    fence_proxy_async();  // weights, ones and zeros were written by plain stores
+    tc_before_sync();
+    __syncthreads();
+    tc_after_sync();
+    const uint32_t tmem = *tslot;
+    const uint32_t stage16 = (uint32_t)s.stage >> 4;
+
+    // a CTA's items: strided by the grid, or (WGRAD2) upu consecutive ones per unit
+    const int units = KIND == WGRAD2 ? a.units : s.items;
+    const int per = KIND == WGRAD2 ? s.upu : 1;
+    auto decode = [&](int item, int &b, int &qz, int &y0) {
+        const int r = item / s.bands;
+        y0 = (item - r * s.bands) * s.R;
+        b = r / s.Qz;
+        qz = r - b * s.Qz;
+    };
+    if (warp > kSlabEpi) {
+        // ---- staging: a warp per source row, lanes along its 16-byte pieces
+        const int pw = warp - kSlabEpi - 1;
+        const int ny = S2 ? 2 * s.R + 1 : s.RB, nx = S2 ? 2 * s.Qx + 1 : s.P;
+        const int o0 = KIND == DGRAD2 ? 0 : -1, mul = S2 ? 2 : 1;
+        // lane: channels 8 cl .. 8 cl + 7 of voxels xl, xl + XS, ... of a row (lanes
+        // beyond XS NC idle)
+        constexpr int XS = 32 / NC;
+        const int cl = lane % NC, xl = lane < XS * NC ? lane / NC : nx;
+        // the output gradient's pieces the same way
+        const int ng = a.N >> 3, gs = ng <= 32 ? 32 / ng : 1;
+        const int gl = lane % ng, gx = lane < gs * ng ? lane / ng : s.P;
+        uint32_t n = 0;
+        for (int u = blockIdx.x; u < units; u += gridDim.x)
+            for (int item = u * per; item < min((u + 1) * per, s.items); ++item, ++n) {
+                const int st = (int)(n % (uint32_t)s.nst);
+                const uint32_t use = n / (uint32_t)s.nst;
+                if (use > 0)
+                    mbar_wait(bar_empty + 8 * st, (use - 1) & 1);
+                int b, qz, y0;
+                decode(item, b, qz, y0);
+                const uint32_t base = ring0 + st * s.stage;
+                for (int row = pw; row < s.nzb * ny; row += kSlabProd) {
+                    const int zi = row / ny, yi = row - zi * ny;
+                    const int sz = mul * qz + o0 + zi, sy = mul * y0 + o0 + yi;
+                    const bool rowok = (unsigned)sz < (unsigned)s.Sz && (unsigned)sy < (unsigned)s.Sy;
+                    const int64_t at = ((((int64_t)b * s.Sz + sz) * s.Sy + sy) * s.Sx + o0) * C;
+                    // S2: odd sources (yi, xi even) and even ones go to their blocks
+                    const int blk_o = S2 ? ((yi & 1) ? 2 : 1) : 0, blk_e = (yi & 1) ? 3 : 0;
+                    const int r0 = (S2 ? yi >> 1 : yi) * s.P;
+                    const uint32_t d_o = base + (blk_o * s.nzb + zi) * NC * s.plane + r0 * 16;
+                    const uint32_t d_e = base + (blk_e * s.nzb + zi) * NC * s.plane + r0 * 16;
+                    // a lane keeps its 8 channels, and (32 / NC even) its x parity
+                    const __nv_bfloat16 *from = s.src + at + (xl * NC + cl) * 8;
+                    uint32_t to = (S2 ? ((xl & 1) ? d_e : d_o) + (xl >> 1) * 16 : d_o + xl * 16) +
+                                  cl * s.plane;
+                    if (!S2 || XS % 2 == 0) {
+#pragma unroll 4
+                        for (int xi = xl; xi < nx; xi += XS) {
+                            bool ok = rowok && (unsigned)(o0 + xi) < (unsigned)s.Sx;
+                            if (ok && !al_index_ok(from - s.src, s.src_elems - 7))
+                                ok = false;
+                            cp16_l1(to, ok ? from : s.src, ok);
+                            from += XS * C;
+                            to += S2 ? XS * 8 : XS * 16;
+                        }
+                    } else {
+                        for (int xi = xl; xi < nx; xi += XS) {
+                            bool ok = rowok && (unsigned)(o0 + xi) < (unsigned)s.Sx;
+                            if (ok && !al_index_ok(from - s.src, s.src_elems - 7))
+                                ok = false;
+                            to = ((xi & 1) ? d_e : d_o) + (xi >> 1) * 16 + cl * s.plane;
+                            cp16_l1(to, ok ? from : s.src, ok);
+                            from += XS * C;
+                        }
+                    }
+                }
+                if (KIND == WGRAD2) {
+                    // the output gradient at the band's positions, zero elsewhere
+                    for (int r = pw; r * s.P < s.ksteps * 16; r += kSlabProd) {
+                        const bool rowok = r < s.R && y0 + r < s.Qy;
+                        const int64_t at =
+                            ((((int64_t)b * s.Qz + qz) * s.Qy + y0 + r) * s.Qx) * a.N;
+                        const __nv_bfloat16 *from = a.gout + at + (gx * ng + gl) * 8;
+                        uint32_t to = base + s.goff + gl * s.gplane + (r * s.P + gx) * 16;
+                        const int nxg = min(s.P, s.ksteps * 16 - r * s.P);
+#pragma unroll 4
+                        for (int x = gx; x < nxg; x += gs) {
+                            bool ok = rowok && x < s.Qx;
+                            if (ok && !al_index_ok(from - a.gout, a.gout_elems - 7))
+                                ok = false;
+                            cp16_l1(to, ok ? from : a.gout, ok);
+                            from += gs * a.N;
+                            to += gs * 16;
+                        }
+                    }
+                }
+                if (KIND == DGRAD2 && a.mask) {
+                    // the ReLU factors of the item's voxels towards L2: the epilogue reads
+                    // them one item later
+                    const int line = 128 / (2 * a.N) > 0 ? 128 / (2 * a.N) : 1;  // voxels
+                    for (int row = pw; row < 4 * s.R; row += kSlabProd) {
+                        const int z = 2 * qz + row / (2 * s.R), y = 2 * y0 + row % (2 * s.R);
+                        if (z < a.D && y < a.H)
+                            for (int x = lane * line; x < a.W; x += 32 * line)
+                                asm volatile("prefetch.global.L2 [%0];" ::"l"(
+                                    a.mask + vox_index(b, z, y, x, a.D, a.H, a.W) * a.N));
+                    }
+                }
+                cp_commit();
+                if (n > 0) {
+                    cp_wait<1>();  // the item before has landed
+                    fence_proxy_async();
+                    mbar_arrive(bar_full + 8 * (int)((n - 1) % (uint32_t)s.nst));
+                }
+            }
+        if (n > 0) {
+            cp_wait<0>();
+            fence_proxy_async();
+            mbar_arrive(bar_full + 8 * (int)((n - 1) % (uint32_t)s.nst));
+        }
+    } else if (warp == kSlabEpi) {
+        // ---- MMAs: the whole warp computes the (uniform) operands, one lane issues
+        const bool one = elect_one();
+        const uint32_t pl = (uint32_t)s.plane >> 4, P = (uint32_t)s.P, N = (uint32_t)a.N;
+        const uint32_t id0 = a.idesc & ~(0x3Fu << 17);  // without N
+        // descriptor bits above the address
+        const uint64_t ka = sdesc(0, s.plane, 128), kb = sdesc(0),
+                       kbd = sdesc(0, 128, 256), ma = sdesc(0, 128, s.plane),
+                       mb = sdesc(0, 128, s.gplane);
+        const uint32_t w16 = w0 >> 4, r16 = ring0 >> 4;
+        uint32_t n = 0, nu = 0;
+        for (int u = blockIdx.x; u < units; u += gridDim.x, ++nu) {
+            const uint32_t acc = nu % (uint32_t)s.nacc, use = nu / (uint32_t)s.nacc;
+            if (use > 0)
+                mbar_wait(bar_free + 8 * acc, (use - 1) & 1);
+            const uint32_t d0 = tmem + acc * (a.tmem_cols / 2);
+            const int i0 = u * per, i1 = min((u + 1) * per, s.items);
+            for (int item = i0; item < i1; ++item, ++n) {
+                const int st = (int)(n % (uint32_t)s.nst);
+                mbar_wait(bar_full + 8 * st, (n / (uint32_t)s.nst) & 1);
+                tc_after_sync();
+                const uint32_t base = r16 + st * stage16;
+                if (KIND == WGRAD2) {
+                    // windows of 16 planes: all at shift (0, 0), blocks 1-2 one column
+                    // on, 0-1 one row on, 1 both
+                    constexpr int B = 3 * NC, n00 = (4 * B + 1 + 15) / 16, n2 = (2 * B + 15) / 16,
+                                  n11 = (B + 15) / 16;
+                    const uint32_t g0 = base + ((uint32_t)s.goff >> 4);
+#pragma unroll 1
+                    for (int j = 0; j < s.ksteps; ++j) {
+                        const uint32_t on = item != i0 || j != 0;
+                        const uint64_t b = mb + g0 + 16 * j;
+                        const uint32_t a0 = base + 16 * j;
+#pragma unroll
+                        for (int k = 0; k < n00 + 2 * n2 + n11; ++k) {
+                            const int sx = (k >= n00 && k < n00 + n2) || k >= n00 + 2 * n2;
+                            const int sy = k >= n00 + n2;
+                            const int p0 = k < n00               ? 16 * k
+                                           : k < n00 + n2        ? B + 16 * (k - n00)
+                                           : k < n00 + 2 * n2    ? 16 * (k - n00 - n2)
+                                                                 : B + 16 * (k - n00 - 2 * n2);
+                            tc_mma_if(one, d0 + k * N, ma + a0 + p0 * pl + sy * P + sx, b, a.idesc,
+                                      on);
+                        }
+                    }
+                } else {
+#pragma unroll 1
+                    for (int m = 0; m < s.T; ++m) {
+                        const uint32_t a0 = base + 128 * m, dm = d0 + m * s.accs;
+                        if (KIND == DGRAD2) {
+                            constexpr Runs runs{};
+                            uint32_t b = w16;
+#pragma unroll
+                            for (int k = 0; k < kRuns; ++k) {
+                                const ShiftRun r = runs.r[k];
+                                const uint32_t id = id0 | ((uint32_t)r.n * (N >> 3) << 17);
+                                const uint32_t sh = (r.shift >> 1 & 1) * P + (r.shift & 1);
+#pragma unroll
+                                for (int j = 0; j < NK16; ++j) {
+                                    tc_mma_if(one, dm + r.pos * N,
+                                              ka + a0 + ((r.shift >> 2) * NC + 2 * j) * pl + sh,
+                                              kbd + b, id, !r.first || j != 0);
+                                    b += r.n * N * 2;  // rows of 32 bytes
+                                }
+                            }
+                        } else {
+#pragma unroll
+                            for (int k = 0; k < 27 * NK16; ++k) {
+                                const int t = k / NK16, c16 = k % NK16;
+                                int tz = t / 9, ty = t / 3 % 3, tx = t % 3, blk = 0;
+                                if (KIND == DGRAD1)
+                                    tz = 2 - tz, ty = 2 - ty, tx = 2 - tx;
+                                if (KIND == FWD2) {
+                                    // block of the tap's parities and its place in it
+                                    const bool ey = ty == 1, ex = tx == 1;
+                                    blk = ey ? (ex ? 3 : 2) : (ex ? 0 : 1);
+                                    ty = ty == 2, tx = tx == 2;
+                                }
+                                tc_mma_if(one, dm,
+                                          ka + a0 + ((blk * 3 + tz) * NC + 2 * c16) * pl + ty * P + tx,
+                                          kb + w16 + (k / 4) * N * 8 + (k % 4) * 16, a.idesc, k != 0);
+                            }
+                        }
+                    }
+                }
+                if (one)
+                    tc_commit(bar_empty + 8 * st);
+            }
+            if (one)
+                tc_commit(bar_acc + 8 * acc);
+        }
+        __syncwarp();
+    } else {
+        // ---- epilogue
+        const int quarter = warp & 3, half = warp >> 2;
+        const uint32_t lanes = (uint32_t)(quarter * 32) << 16;
+        // this lane's position in the two tiles
+        const int l0 = quarter * 32 + lane, l1 = l0 + 128;
+        const int r0 = l0 / s.P, x0 = l0 - r0 * s.P, r1 = l1 / s.P, x1 = l1 - r1 * s.P;
+        const bool in0 = x0 < s.Qx && r0 < s.R, in1 = x1 < s.Qx && r1 < s.R;
+        uint32_t nu = 0;
+        for (int u = blockIdx.x; u < units; u += gridDim.x, ++nu) {
+            const uint32_t acc = nu % (uint32_t)s.nacc;
+            const uint32_t d0 = tmem + acc * (a.tmem_cols / 2) + lanes;
+            if (KIND == WGRAD2) {
+                mbar_wait(bar_acc + 8 * acc, (nu / (uint32_t)s.nacc) & 1);
+                tc_after_sync();
+                // row of window k: plane p0 + row / 8, element row % 8
+                constexpr int B = 3 * NC;
+                const int n00 = (4 * B + 1 + 15) / 16, n2 = (2 * B + 15) / 16;
+                for (int k = 0; k < s.nk; ++k) {
+                    int sy = 0, sx = 0, p0 = 16 * k, b0 = 0, b1 = 4;
+                    if (k >= n00 + 2 * n2)
+                        sy = sx = 1, p0 = B + 16 * (k - n00 - 2 * n2), b0 = 1, b1 = 2;
+                    else if (k >= n00 + n2)
+                        sy = 1, p0 = 16 * (k - n00 - n2), b1 = 2;
+                    else if (k >= n00)
+                        sx = 1, p0 = B + 16 * (k - n00), b0 = 1, b1 = 3;
+                    const int row = quarter * 32 + lane, p = p0 + (row >> 3);
+                    const int blk = p / B, r = p - blk * B, zi = r / NC, c = r - zi * NC;
+                    // blocks: (odd, even), (odd, odd), (even, odd), (even, even)
+                    const int ty = blk >= 2 ? 1 : (sy ? 2 : 0);
+                    const int tx = blk == 0 || blk == 3 ? 1 : (sx ? 2 : 0);
+                    const bool ones = k < n00 && p == 4 * B && (row & 7) == 0;
+                    const bool on = (blk >= b0 && blk < b1) || ones;
+                    const int m = ones ? 27 * C : ((zi * 3 + ty) * 3 + tx) * C + c * 8 + (row & 7);
+                    for (int c0 = 16 * half; c0 < a.N; c0 += 16 * PARTS) {
+                        float v[16];
+                        tc_load16(d0 + k * a.N + c0, v);
+                        if (on)
+                            epilogue_chunk<WGRAD>(a, (size_t)u * a.mtiles * 128 + m, v, c0, 0);
+                    }
+                }
+            } else {
+                int b, qz, y0;
+                decode(u, b, qz, y0);
+                // G chunks of 16 columns at a time (this warp's are PARTS apart); the ReLU
+                // factors of the next G are loaded before the sums of these are read
+                constexpr bool BWD = KIND == DGRAD1 || KIND == DGRAD2;
+                constexpr int G = 1;
+                const int per_tile = (s.accs - 16 * half + 16 * PARTS - 1) / (16 * PARTS);  // chunks
+                struct Group {
+                    size_t row[G];
+                    int nn[G];
+                    bool on[G];
+                    uint4 mask[G][2];
+                };
+                // group i: tile, first chunk
+                auto load = [&](int m, int j, Group &q) {
+                    const int x = m ? x1 : x0, y = y0 + (m ? r1 : r0);
+                    const bool in = (m ? in1 : in0) && y < s.Qy;
+#pragma unroll
+                    for (int k = 0; k < G; ++k) {
+                        const int c0 = 16 * (half + PARTS * (j + k));
+                        bool on = in && c0 < s.accs;
+                        size_t row = 0;
+                        int nn = c0;
+                        if (KIND == DGRAD2) {
+                            const int pc = on ? chunks[c0 >> 4] : 0, cls = pc & 7;
+                            nn = pc >> 3;
+                            const int z = 2 * qz + (cls >> 2), yy = 2 * y + ((cls >> 1) & 1),
+                                      xx = 2 * x + (cls & 1);
+                            on = on && z < a.D && yy < a.H && xx < a.W;
+                            if (on)
+                                row = vox_index(b, z, yy, xx, a.D, a.H, a.W);
+                        } else if (on) {
+                            row = (((size_t)b * s.Qz + qz) * s.Qy + y) * s.Qx + x;
+                        }
+                        q.nn[k] = nn;
+                        q.row[k] = row;
+                        q.on[k] = on;
+                        if (BWD && a.mask && on) {
+                            const uint4 *p =
+                                reinterpret_cast<const uint4 *>(a.mask + row * a.N + nn);
+                            if (a.wide) {
+                                load32(p, q.mask[k]);
+                            } else {
+                                q.mask[k][0] = __ldg(p);
+                                q.mask[k][1] = __ldg(p + 1);
+                            }
+                        }
+                    }
+                };
+                Group cur, nxt;
+                if (per_tile > 0)
+                    load(0, 0, cur);
+                // every warp waits for the sums, also one that has no columns: the set
+                // is free again when all of them have come by
+                mbar_wait(bar_acc + 8 * acc, (nu / (uint32_t)s.nacc) & 1);
+                tc_after_sync();
+                int m = per_tile > 0 ? 0 : s.T, j = 0;
+#pragma unroll 1
+                while (m < s.T) {
+                    int m2 = m, j2 = j + G;
+                    if (j2 >= per_tile) {
+                        ++m2;
+                        j2 = 0;
+                    }
+                    if (m2 < s.T)
+                        load(m2, j2, nxt);
+                    uint32_t v[2][16];
+#pragma unroll
+                    for (int k = 0; k < G; ++k) {  // past the sums: any columns of the set
+                        const int c0 = 16 * (half + PARTS * (j + k));
+                        tc_load16_async(d0 + m * s.accs + (c0 < s.accs ? c0 : 0), v[k]);
+                    }
+                    tc_load_wait(v[0], v[G - 1]);
+#pragma unroll
+                    for (int k = 0; k < G; ++k)
+                        if (cur.on[k]) {
+                            float f[16];
+#pragma unroll
+                            for (int e = 0; e < 16; ++e)
+                                f[e] = __uint_as_float(v[k][e]);
+                            epilogue_chunk<BWD ? DGRAD : FWD>(a, cur.row[k], f, cur.nn[k], 0,
+                                                              cur.mask[k]);
+                        }
+                    cur = nxt;
+                    m = m2;
+                    j = j2;
+                }
+            }
+            tc_before_sync();
+            mbar_arrive(bar_free + 8 * acc);
+        }
+    }
+    __syncthreads();
+    if (warp == 0)
+        tmem_dealloc(tmem, a.tmem_cols);
 }
 
 // Weight slices in the shared-memory layout of the B operand: slice s holds
@@ -1342,12 +2081,12 @@ uint32_t tmem_cols_for(int N)
 }
 
 // Dynamic shared memory: 1024-byte alignment slack, the ring's A and B
-// slots, 2 kStages + 1 mbarriers, the TMEM address, the class tables and
-// the tap offset tables.
-size_t conv_smem_bytes(int N)
+// slots, 2 kStages + 1 mbarriers, the TMEM address, the class tables, the tap
+// offset tables and (WGRAD) the group table.
+size_t conv_smem_bytes(int N, int groups)
 {
     return 1024 + kStages * (size_t)kATile + kStages * (size_t)N * 128 + 8 * (2 * kStages + 1) +
-           4 + 4 * (3 * kMaxClasses + 1) + sizeof(Tables);
+           4 + 4 * (3 * kMaxClasses + 1) + sizeof(Tables) + 8 + groups * sizeof(int2);
 }
 
 // Parity classes of the stride-2 dgrad (host side): units, K slices and
@@ -1372,67 +2111,7 @@ int dgrad_classes(const ConvLayer &l, int *unit0, int *nst, int *slice0, int *to
     return u;
 }
 
-struct DevInfo {
-    int sms = 0;
-    int occ[3][kMaxN / 16 + 1] = {};
-};
-std::mutex g_info_mu;
-DevInfo g_info[64];
-
-template <int MODE>
-cudaError_t grid_for(int N, int units, int *grid)
-{
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess)
-        return e;
-    if (dev < 0 || dev >= 64)
-        return cudaErrorInvalidDevice;
-    std::lock_guard<std::mutex> lk(g_info_mu);
-    DevInfo &d = g_info[dev];
-    if (d.sms == 0) {
-        e = cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess)
-            return e;
-    }
-    int &occ = d.occ[MODE][N / 16];
-    if (occ == 0) {
-        // resident CTAs per SM from the kernel's own limits: shared memory
-        // (with the largest carveout), registers, and TMEM columns (512 per SM)
-        e = cudaFuncSetAttribute(k_conv<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)conv_smem_bytes(kMaxN));
-        if (e != cudaSuccess)
-            return e;
-        e = cudaFuncSetAttribute(k_conv<MODE>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 (int)cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess)
-            return e;
-        cudaFuncAttributes fa;
-        e = cudaFuncGetAttributes(&fa, k_conv<MODE>);
-        if (e != cudaSuccess)
-            return e;
-        int smem_sm = 0, resv = 0;
-        e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-        if (e != cudaSuccess)
-            return e;
-        e = cudaDeviceGetAttribute(&resv, cudaDevAttrReservedSharedMemoryPerBlock, dev);
-        if (e != cudaSuccess)
-            return e;
-        const int by_smem = smem_sm / (int)(conv_smem_bytes(N) + fa.sharedSizeBytes + resv);
-        const int regs_warp = (fa.numRegs * 32 + 255) / 256 * 256;
-        const int by_regs = 65536 / (regs_warp * (kThreads / 32));
-        const int by_tmem = 512 / (int)tmem_cols_for(N);
-        occ = by_smem < by_regs ? by_smem : by_regs;
-        occ = occ < by_tmem ? occ : by_tmem;
-        occ = occ < 16 ? occ : 16;
-        if (occ < 1)
-            return cudaErrorInvalidConfiguration;
-    }
-    *grid = units < d.sms * occ ? units : d.sms * occ;
-    return cudaSuccess;
-}
-
-// Resident CTAs per SM of a kernel of kThreads threads with `smem` bytes of
+// Resident CTAs per SM of a kernel of `threads` threads with `smem` bytes of
 // dynamic shared memory and `cols` TMEM columns, from the kernel's own limits
 // (shared memory with the largest carveout, registers, 512 TMEM columns per
 // SM); found once per kernel, size and device.
@@ -1442,7 +2121,7 @@ struct Residency {
     int dev, occ;
 };
 
-cudaError_t resident_grid(const void *fn, size_t smem, int cols, int units, int *grid)
+cudaError_t resident_grid(const void *fn, size_t smem, int cols, int threads, int units, int *grid)
 {
     static std::mutex mu;
     static Residency known[64];
@@ -1473,7 +2152,7 @@ cudaError_t resident_grid(const void *fn, size_t smem, int cols, int units, int 
         if (e != cudaSuccess)
             return e;
         const int by_smem = smem_sm / (int)(smem + fa.sharedSizeBytes + resv);
-        const int by_regs = 65536 / ((fa.numRegs * 32 + 255) / 256 * 256 * (kThreads / 32));
+        const int by_regs = 65536 / ((fa.numRegs * 32 + 255) / 256 * 256 * (threads / 32));
         occ = std::min(std::min(by_smem, by_regs), std::min(512 / cols, 16));
         if (occ < 1)
             return cudaErrorInvalidConfiguration;
@@ -1484,33 +2163,180 @@ cudaError_t resident_grid(const void *fn, size_t smem, int cols, int units, int 
     return cudaSuccess;
 }
 
+// Resident grid of k_conv<MODE>; *smem receives its dynamic shared memory.
+template <int MODE>
+cudaError_t conv_grid(const ConvArgs &a, int *grid, size_t *smem)
+{
+    *smem = conv_smem_bytes(a.N, MODE == WGRAD && a.cin != 2 ? 27 * (a.cin >> 3) : 0);
+    return resident_grid((const void *)k_conv<MODE>, *smem, (int)a.tmem_cols, kThreads, a.units,
+                         grid);
+}
+
 // The two-channel kernels are built for the output widths 16 and 32.
 bool conv2_built(const ConvLayer &l) { return l.cin == 2 && (l.cout == 16 || l.cout == 32); }
 
-template <int N>
-cudaError_t run_conv2_fwd(const ConvArgs &a, cudaStream_t s)
+// Host plan of a slab pass; false when no tiling of it fits (rows beyond 254
+// positions, weights and two stages beyond a CTA's shared memory, TMEM columns).
+bool slab_plan(int kind, int C, int N, int64_t nb, const int *S, const int *Q, SlabArgs *out,
+               uint32_t *cols, size_t *smem)
 {
-    const size_t smem = 128 + 2 * kC2Slot + 10 * N * 16 + 32;
+    const bool s2 = kind == FWD2 || kind == WGRAD2;
+    const int halo = kind == FWD1 || kind == DGRAD1 ? 2 : 1, nc = C / 8;
+    bool found = false;
+    double best_cost = 0.0;
+    for (int R = std::min(Q[1], 256 / (Q[2] + halo)); R >= 1; --R) {
+        SlabArgs s{};
+        s.Sz = S[0], s.Sy = S[1], s.Sx = S[2];
+        s.Qz = Q[0], s.Qy = Q[1], s.Qx = Q[2];
+        s.P = s.Qx + halo;
+        s.R = R;
+        s.T = (s.R * s.P + 127) / 128;
+        s.RB = s.R + halo;
+        s.nzb = kind == DGRAD2 ? 2 : 3;
+        s.plane = s.RB * s.P * 16;
+        int sets = 1;  // accumulators of N columns
+        if (kind == WGRAD2) {
+            const int B = 3 * nc;
+            s.nk = (4 * B + 1 + 15) / 16 + 2 * ((2 * B + 15) / 16) + (B + 15) / 16;
+            s.ksteps = (s.R * s.P + 15) / 16;
+            s.gplane = s.ksteps * 256;
+            s.goff = (4 * B + 1) * s.plane;
+            s.stage = (s.goff + N / 8 * s.gplane + 127) / 128 * 128;
+            sets = s.nk;
+            s.T = 1;
+            // the last window of 16 planes runs past the ones
+            s.slack = ((4 * B + 1 + 15) / 16 * 16 - 4 * B) * s.plane;
+        } else {
+            s.nk = kind == DGRAD2 ? kRuns * C / 16 : 27 * C / 16;
+            // a tile's rows past the band, shifted, read beyond the last plane
+            s.stage = ((s2 ? 4 : 1) * s.nzb * nc * s.plane + 127) / 128 * 128;
+            s.wbytes = kind == DGRAD2 ? 27 * C * N * 2 : (27 * C + 63) / 64 * 64 * N * 2;
+            sets = kind == DGRAD2 ? 8 : 1;
+        }
+        s.accs = sets * N;
+        // a weight adjoint drains its sums once per unit: one set where two do not fit
+        s.nacc = kind == WGRAD2 && 2 * s.accs > 512 ? 1 : 2;
+        uint32_t c = 32;
+        while ((int)c < s.nacc * s.T * s.accs)
+            c <<= 1;
+        if (kind == DGRAD2 && 8 * N > 256)
+            continue;  // the widest MMA
+        const size_t fixed = 128 + (size_t)s.slack + (s.wbytes + 127) / 128 * 128 + 192;
+        // reads past the last stage land in the weights and the table behind it
+        const size_t past = kind == WGRAD2 ? 0 : (size_t)((halo * s.P + halo + s.T * 128) * 16);
+        if (c > 512 || fixed + 2 * (size_t)s.stage > (size_t)kMaxDynSmem ||
+            past > (size_t)s.RB * s.P * 16 + fixed - 192)
+            continue;
+        s.nst = (int)std::min<size_t>(4, ((size_t)kMaxDynSmem - fixed) / s.stage);
+        // staged rows per output row, and the idle MMA rows; two stages alone leave
+        // the staging's latency bare
+        const double cost =
+            ((double)(s2 ? 2 * s.R + 1 : s.RB) / s.R +
+             (kind == WGRAD2 ? (double)s.ksteps * 16 : (double)s.T * 128) / (s.R * s.P)) *
+            (s.nst > 2 ? 1.0 : 1.25);
+        s.bands = (s.Qy + s.R - 1) / s.R;
+        s.items = (int)(nb * s.Qz * s.bands);
+        if (!found || cost < best_cost) {
+            *out = s;
+            *cols = c;
+            *smem = fixed + (size_t)s.nst * s.stage;
+            best_cost = cost;
+            found = true;
+        }
+    }
+    return found;
+}
+
+template <int C, int KIND>
+cudaError_t run_slab(const ConvArgs &a, const SlabArgs &s, size_t smem, int units, cudaStream_t st)
+{
     int grid = 0;
-    const cudaError_t e = resident_grid((const void *)k_conv2_fwd<N>, smem, 2 * N, a.units, &grid);
+    const cudaError_t e = resident_grid((const void *)k_conv_slab<C, KIND>, smem,
+                                        (int)a.tmem_cols, slab_threads(KIND), units, &grid);
     if (e != cudaSuccess)
         return e;
-    ProfScope ps(s, "k_conv_fwd");
-    k_conv2_fwd<N><<<grid, kThreads, smem, s>>>(a);
+    ProfScope ps(st, KIND == WGRAD2 ? "k_conv_wgrad" : KIND == FWD1 || KIND == FWD2 ? "k_conv_fwd"
+                                                                                  : "k_conv_dgrad");
+    k_conv_slab<C, KIND><<<grid, slab_threads(KIND), smem, st>>>(a, s);
     return cudaGetLastError();
 }
 
-template <int N>
-cudaError_t run_conv2_wgrad(const ConvArgs &a, cudaStream_t s)
+template <int C>
+cudaError_t run_slab_kind(int kind, const ConvArgs &a, const SlabArgs &s, size_t smem,
+                          cudaStream_t st)
 {
-    const size_t smem = 128 + 2 * (16 + N / 8) * kC2Plane + 32;
+    switch (kind) {
+    case FWD1: return run_slab<C, FWD1>(a, s, smem, s.items, st);
+    case FWD2: return run_slab<C, FWD2>(a, s, smem, s.items, st);
+    case DGRAD1: return run_slab<C, DGRAD1>(a, s, smem, s.items, st);
+    default: return run_slab<C, DGRAD2>(a, s, smem, s.items, st);
+    }
+}
+
+// Runs a pass (a prepared) as a slab when it fits one; *ran says so. WGRAD: at
+// most *splits units, whose partial sums lie as k_wgrad_reduce reads them; the
+// number used is returned in *splits.
+cudaError_t launch_slab(int mode, const ConvLayer &l, ConvArgs a, cudaStream_t st, bool *ran,
+                        int *splits = nullptr)
+{
+    *ran = false;
+    if (mode == WGRAD && l.stride != 2)
+        return cudaSuccess;
+    const int kind = mode == WGRAD ? WGRAD2
+                     : mode == FWD ? (l.stride == 1 ? FWD1 : FWD2)
+                                   : (l.stride == 1 ? DGRAD1 : DGRAD2);
+    const int C = mode == DGRAD ? l.cout : l.cin;
+    if (C != 16 && C != 32 && (kind == WGRAD2 || (C != 48 && C != 64)))
+        return cudaSuccess;
+    const int in[3] = {l.D, l.H, l.W}, o[3] = {a.Do, a.Ho, a.Wo};
+    const int pairs[3] = {(l.D + 1) / 2, (l.H + 1) / 2, (l.W + 1) / 2};
+    const int *S = mode == DGRAD ? o : in;
+    const int *Q = mode == DGRAD ? (kind == DGRAD2 ? pairs : in) : o;
+    SlabArgs s;
+    size_t smem = 0;
+    if (!slab_plan(kind, C, a.N, l.nb, S, Q, &s, &a.tmem_cols, &smem))
+        return cudaSuccess;
+    s.src = a.act;
+    s.src_elems = a.act_elems;
+    *ran = true;
+    if (kind == WGRAD2) {
+        s.upu = (s.items + *splits - 1) / *splits;
+        a.units = *splits = (s.items + s.upu - 1) / s.upu;
+        return C == 16 ? run_slab<16, WGRAD2>(a, s, smem, a.units, st)
+                       : run_slab<32, WGRAD2>(a, s, smem, a.units, st);
+    }
+    switch (C) {
+    case 16: return run_slab_kind<16>(kind, a, s, smem, st);
+    case 32: return run_slab_kind<32>(kind, a, s, smem, st);
+    case 48: return run_slab_kind<48>(kind, a, s, smem, st);
+    default: return run_slab_kind<64>(kind, a, s, smem, st);
+    }
+}
+
+template <int N, bool PAIR>
+cudaError_t run_conv2(const ConvArgs &a, bool wgrad, cudaStream_t s)
+{
+    const size_t smem = wgrad ? 128 + 16 * kC2Plane + 32 : 128 + 10 * kC2Plane + 10 * N * 16 + 32;
+    const void *fn = wgrad ? (const void *)k_conv2_wgrad<N, PAIR> : (const void *)k_conv2_fwd<N, PAIR>;
     int grid = 0;
-    const cudaError_t e = resident_grid((const void *)k_conv2_wgrad<N>, smem, 32, a.units, &grid);
+    const cudaError_t e = resident_grid(fn, smem, 32, kThreads, a.units, &grid);
     if (e != cudaSuccess)
         return e;
-    ProfScope ps(s, "k_conv_wgrad");
-    k_conv2_wgrad<N><<<grid, kThreads, smem, s>>>(a);
+    ProfScope ps(s, wgrad ? "k_conv_wgrad" : "k_conv_fwd");
+    if (wgrad)
+        k_conv2_wgrad<N, PAIR><<<grid, kThreads, smem, s>>>(a);
+    else
+        k_conv2_fwd<N, PAIR><<<grid, kThreads, smem, s>>>(a);
     return cudaGetLastError();
+}
+
+// PAIR's 8-byte loads need stride 2, an even W and an input on 8 bytes (it is on 16).
+cudaError_t launch_conv2(const ConvArgs &a, bool wgrad, cudaStream_t s)
+{
+    const bool pair = a.stride == 2 && a.W % 2 == 0;
+    if (a.N == 16)
+        return pair ? run_conv2<16, true>(a, wgrad, s) : run_conv2<16, false>(a, wgrad, s);
+    return pair ? run_conv2<32, true>(a, wgrad, s) : run_conv2<32, false>(a, wgrad, s);
 }
 
 int blocks_for(int64_t n, int threads)
@@ -1609,6 +2435,8 @@ cudaError_t launch_adam_pack(const AdamPackArgs &a, int64_t *step, float *p, con
     return launch_step_tick(step, s);
 }
 
+static bool on32(const void *p) { return ((uintptr_t)p & 31u) == 0; }
+
 static ConvArgs base_args(const ConvLayer &l)
 {
     ConvArgs a = {};
@@ -1699,17 +2527,25 @@ cudaError_t launch_conv_forward(const ConvLayer &l, const void *in, const void *
     }
     a.relu = relu;
     a.out_f32 = out_f32;
+    a.wide = on32(out);
     a.idesc = make_idesc(a.N, false);
     a.tmem_cols = tmem_cols_for(a.N);
     if (conv2_built(l) && sp == 1)
-        return l.cout == 16 ? run_conv2_fwd<16>(a, s) : run_conv2_fwd<32>(a, s);
+        return launch_conv2(a, false, s);
+    if (sp == 1) {
+        bool ran = false;
+        const cudaError_t e = launch_slab(FWD, l, a, s, &ran);
+        if (ran)
+            return e;
+    }
     int grid = 0;
-    cudaError_t e = grid_for<FWD>(a.N, a.units, &grid);
+    size_t smem = 0;
+    cudaError_t e = conv_grid<FWD>(a, &grid, &smem);
     if (e != cudaSuccess)
         return e;
     {
         ProfScope ps(s, "k_conv_fwd");
-        k_conv<FWD><<<grid, kThreads, conv_smem_bytes(a.N), s>>>(a);
+        k_conv<FWD><<<grid, kThreads, smem, s>>>(a);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess || sp == 1)
@@ -1729,6 +2565,7 @@ cudaError_t launch_conv_dgrad(const ConvLayer &l, const void *gout, const void *
     a.act = static_cast<const __nv_bfloat16 *>(gout);
     a.wpk = static_cast<const __nv_bfloat16 *>(wpk);
     a.mask = static_cast<const __nv_bfloat16 *>(mask);
+    a.wide = on32(gin) && on32(mask);
     a.addend = static_cast<const __nv_bfloat16 *>(addend);
     a.add_stride = add_stride;
     a.add_off = add_off;
@@ -1745,12 +2582,17 @@ cudaError_t launch_conv_dgrad(const ConvLayer &l, const void *gout, const void *
     }
     a.idesc = make_idesc(a.N, false);
     a.tmem_cols = tmem_cols_for(a.N);
+    bool ran = false;
+    cudaError_t e = launch_slab(DGRAD, l, a, s, &ran);
+    if (ran)
+        return e;
     int grid = 0;
-    cudaError_t e = grid_for<DGRAD>(a.N, a.units, &grid);
+    size_t smem = 0;
+    e = conv_grid<DGRAD>(a, &grid, &smem);
     if (e != cudaSuccess)
         return e;
     ProfScope ps(s, "k_conv_dgrad");
-    k_conv<DGRAD><<<grid, kThreads, conv_smem_bytes(a.N), s>>>(a);
+    k_conv<DGRAD><<<grid, kThreads, smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -1774,15 +2616,19 @@ cudaError_t launch_conv_wgrad(const ConvLayer &l, const void *in, const void *go
     a.idesc = make_idesc(a.N, true);
     a.tmem_cols = tmem_cols_for(a.N);
     cudaError_t e;
+    bool ran = false;
     if (conv2_built(l)) {
-        e = l.cout == 16 ? run_conv2_wgrad<16>(a, s) : run_conv2_wgrad<32>(a, s);
-    } else {
+        e = launch_conv2(a, true, s);
+    } else if ((e = launch_slab(WGRAD, l, a, s, &ran, &sp)) != cudaSuccess) {
+        return e;
+    } else if (!ran) {
         int grid = 0;
-        e = grid_for<WGRAD>(a.N, a.units, &grid);
+        size_t smem = 0;
+        e = conv_grid<WGRAD>(a, &grid, &smem);
         if (e != cudaSuccess)
             return e;
         ProfScope ps(s, "k_conv_wgrad");
-        k_conv<WGRAD><<<grid, kThreads, conv_smem_bytes(a.N), s>>>(a);
+        k_conv<WGRAD><<<grid, kThreads, smem, s>>>(a);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess)
