@@ -320,98 +320,142 @@ __global__ void k_tick(int64_t *step)
 
 // out[v][z][y][x] = sum_b a_b exp(-|x - mu_b|^2 / (2 sigma_b^2)) for the
 // blob table of volume v ([blob][mu_x, mu_y, mu_z, sigma, a]). A block owns
-// an 8 x 8 x 32 box (x, y, z) and first keeps the blobs that come within 6
-// sigma of it (warp 0, in table order): a dropped term is below
-// a exp(-18) < 1.6e-8 a everywhere in the box. A Gaussian separates into
-// per-axis factors,
+// a TB x TB x 32 box (x, y, z) and takes the table in chunks of 64 blobs, of
+// which it keeps those that come within 6 sigma of the box (in table order): a
+// dropped term is below a exp(-18) < 1.6e-8 a everywhere in the box. A Gaussian
+// separates into per-axis factors,
 //   a exp(-|p - mu|^2 / (2 sigma^2)) = ex(x) ey(y) (a ez(z)),
-// so each kept blob takes 48 exponentials per box (8 + 8 + 32). A thread
-// owns 8 voxels of one (x, y) column: per blob one product ex ey, two
-// 16-byte shared-memory reads of the 8 z factors and 4 packed f32x2 FMAs.
-constexpr int kBrick = 8;                        // x and y extent of a box
-constexpr int kBrickZ = 32;                      // z extent: 4 groups of 8 slices
-constexpr int kFac = 2 * kBrick + kBrickZ;       // factors per kept blob
+// so a kept blob takes 2 TB + 32 exponentials per box. A thread owns four
+// columns (x .. x + 3, y) of 8 slices; per blob two packed products ex ey, one
+// 16-byte read of ex, one 8-byte read of ey, four 16-byte reads of the z factors
+// (y and z factors stored twice, as the packed operands want them) and 16 packed
+// f32x2 FMAs: 24 instructions for 32 voxels and a blob, the FMAs' rate (34 us for
+// 16 x 128^3 voxels, 60 blobs of sigma 3-12) being the bound. That case takes 49 us;
+// 92 with one column of 8 slices per thread and boxes of 8 x 8, whose factor loads
+// and exponentials took half the issue slots.
+constexpr int kBrickZ = 32;    // z extent: 4 groups of 8 slices
+constexpr int kBlobChunk = 64; // blobs per chunk
 
-__global__ void __launch_bounds__(256) k_render_blobs(int D, int H, int W, int nblobs,
-                                                      const float *__restrict__ table,
-                                                      float *__restrict__ out)
+template <int TB>
+__global__ void __launch_bounds__(TB * TB, TB == 16 ? 4 : 16)
+    k_render_blobs(int D, int H, int W, int nblobs, const float *__restrict__ table,
+                   float *__restrict__ out, int vec)
 {
-    extern __shared__ float4 fac4[];  // kept blob k: ex[8], ey[8], a ez[32]
+    constexpr int NT = TB * TB;               // (TB / 4) x TB x 4 threads
+    constexpr int FAC = 3 * TB + 2 * kBrickZ; // ex, (ey, ey), (a ez, a ez)
+    static_assert(NT >= kBlobChunk && FAC % 4 == 0, "a thread per blob of a chunk; 16-byte rows");
+    __shared__ float4 fac4[kBlobChunk * FAC / 4];
+    __shared__ float par[kBlobChunk][5];
+    __shared__ unsigned kept[kBlobChunk / 32];
     float *fac = reinterpret_cast<float *>(fac4);
-    __shared__ int keep[1024];        // kept blob indices, in table order (n_blobs <= 1024)
-    __shared__ int nkeep;
     const int vol = blockIdx.y;
-    const int bx = (W + kBrick - 1) / kBrick, by = (H + kBrick - 1) / kBrick;
+    const int bx = (W + TB - 1) / TB, by = (H + TB - 1) / TB;
     const int brick = blockIdx.x;
-    const int x0 = (brick % bx) * kBrick, y0 = ((brick / bx) % by) * kBrick,
+    const int x0 = (brick % bx) * TB, y0 = ((brick / bx) % by) * TB,
               z0 = (brick / (bx * by)) * kBrickZ;
     const float *tv = table + (int64_t)vol * nblobs * 5;
-    if (threadIdx.x < 32) {
-        int base = 0;
-        for (int b0 = 0; b0 < nblobs; b0 += 32) {
-            const int b = b0 + threadIdx.x;
-            bool in = false;
-            if (b < nblobs) {
-                const float *e = tv + (int64_t)b * 5;
-                const float mx = e[0], my = e[1], mz = e[2], sg = e[3];
+    const int t = threadIdx.x, lx = (t % (TB / 4)) * 4, ly = t / (TB / 4) % TB,
+              zg = t / (TB / 4 * TB);
+    float2 acc[8][2];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        acc[i][0] = acc[i][1] = make_float2(0.0f, 0.0f);
+    for (int b0 = 0; b0 < nblobs; b0 += kBlobChunk) {
+        float e[5];
+        bool in = false;
+        if (t < kBlobChunk) {
+            if (b0 + t < nblobs) {
+#pragma unroll
+                for (int k = 0; k < 5; ++k)
+                    e[k] = __ldg(tv + (int64_t)(b0 + t) * 5 + k);
                 // distance from the centre to the box
-                const float dx = fmaxf(fmaxf((float)x0 - mx, mx - (float)(x0 + kBrick - 1)), 0.0f);
-                const float dy = fmaxf(fmaxf((float)y0 - my, my - (float)(y0 + kBrick - 1)), 0.0f);
+                const float dx = fmaxf(fmaxf((float)x0 - e[0], e[0] - (float)(x0 + TB - 1)), 0.0f);
+                const float dy = fmaxf(fmaxf((float)y0 - e[1], e[1] - (float)(y0 + TB - 1)), 0.0f);
                 const float dz =
-                    fmaxf(fmaxf((float)z0 - mz, mz - (float)(z0 + kBrickZ - 1)), 0.0f);
-                in = dx * dx + dy * dy + dz * dz <= 36.0f * sg * sg;
+                    fmaxf(fmaxf((float)z0 - e[2], e[2] - (float)(z0 + kBrickZ - 1)), 0.0f);
+                in = dx * dx + dy * dy + dz * dz <= 36.0f * e[3] * e[3];
             }
             const unsigned m = __ballot_sync(0xffffffffu, in);
-            if (in)
-                keep[base + __popc(m & ((1u << threadIdx.x) - 1u))] = b;
-            base += __popc(m);
+            if (t % 32 == 0)
+                kept[t / 32] = m;
         }
-        if (threadIdx.x == 0)
-            nkeep = base;
-    }
-    __syncthreads();
-    const int n = nkeep;
-    // the per-axis factors of the kept blobs at the box's coordinates
-    for (int t = threadIdx.x; t < n * kFac; t += blockDim.x) {
-        const int k = t / kFac, r = t - k * kFac;
-        const int axis = r < kBrick ? 0 : r < 2 * kBrick ? 1 : 2;
-        const int o = r - axis * kBrick;
-        const float *e = tv + (int64_t)keep[k] * 5;
-        const float c = (float)((axis == 0 ? x0 : axis == 1 ? y0 : z0) + o) - e[axis];
-        const float v = expf(-0.5f * c * c / (e[3] * e[3]));
-        fac[t] = axis == 2 ? e[4] * v : v;
-    }
-    __syncthreads();
-    // thread: column (lx, ly), slices 8 zg .. 8 zg + 7 of the box; the 8
-    // sums as 4 pairs, each blob's 8 FMAs as 4 packed f32x2 FMAs (the same
-    // rounding per lane)
-    const int t = threadIdx.x, lx = t & 7, ly = (t >> 3) & 7, zg = t >> 6;
-    float2 acc[4];
+        __syncthreads();  // also: the previous chunk's factors are read
+        const int n0 = __popc(kept[0]), n = n0 + __popc(kept[1]);
+        if (in) {
+            const int k = (t < 32 ? 0 : n0) + __popc(kept[t / 32] & ((1u << (t % 32)) - 1u));
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-        acc[i] = make_float2(0.0f, 0.0f);
-    for (int k = 0; k < n; ++k) {
-        const float *f = fac + kFac * k;
-        const float pxy = f[lx] * f[kBrick + ly];
-        const float2 p2 = make_float2(pxy, pxy);
-        const float4 za = fac4[(kFac * k + 2 * kBrick + 8 * zg) / 4];
-        const float4 zb = fac4[(kFac * k + 2 * kBrick + 8 * zg) / 4 + 1];
-        acc[0] = __ffma2_rn(p2, make_float2(za.x, za.y), acc[0]);
-        acc[1] = __ffma2_rn(p2, make_float2(za.z, za.w), acc[1]);
-        acc[2] = __ffma2_rn(p2, make_float2(zb.x, zb.y), acc[2]);
-        acc[3] = __ffma2_rn(p2, make_float2(zb.z, zb.w), acc[3]);
+            for (int q = 0; q < 5; ++q)
+                par[k][q] = e[q];
+        }
+        __syncthreads();
+        // the per-axis factors of the kept blobs at the box's coordinates
+        constexpr int NE = 2 * TB + kBrickZ;
+        for (int i = t; i < n * NE; i += NT) {
+            const int k = i / NE, r = i - k * NE;
+            const int axis = r < TB ? 0 : r < 2 * TB ? 1 : 2;
+            const int o = r - axis * TB;
+            const float c = (float)((axis == 0 ? x0 : axis == 1 ? y0 : z0) + o) - par[k][axis];
+            const float v = expf(-0.5f * c * c / (par[k][3] * par[k][3]));
+            float *f = fac + FAC * k;
+            if (axis == 0)
+                f[o] = v;
+            else if (axis == 1)
+                reinterpret_cast<float2 *>(f + TB)[o] = make_float2(v, v);
+            else
+                reinterpret_cast<float2 *>(f + 3 * TB)[o] =
+                    make_float2(par[k][4] * v, par[k][4] * v);
+        }
+        __syncthreads();
+#pragma unroll 2
+        for (int k = 0; k < n; ++k) {
+            const float *f = fac + FAC * k;
+            const float4 ex = *reinterpret_cast<const float4 *>(f + lx);
+            const float2 ey = *reinterpret_cast<const float2 *>(f + TB + 2 * ly);
+            const float2 p0 = __fmul2_rn(make_float2(ex.x, ex.y), ey);
+            const float2 p1 = __fmul2_rn(make_float2(ex.z, ex.w), ey);
+            const float4 *zz = reinterpret_cast<const float4 *>(f + 3 * TB + 16 * zg);
+#pragma unroll
+            for (int i = 0; i < 8; i += 2) {
+                const float4 z = zz[i / 2];
+                acc[i][0] = __ffma2_rn(p0, make_float2(z.x, z.y), acc[i][0]);
+                acc[i][1] = __ffma2_rn(p1, make_float2(z.x, z.y), acc[i][1]);
+                acc[i + 1][0] = __ffma2_rn(p0, make_float2(z.z, z.w), acc[i + 1][0]);
+                acc[i + 1][1] = __ffma2_rn(p1, make_float2(z.z, z.w), acc[i + 1][1]);
+            }
+        }
     }
-    const int64_t nv = (int64_t)D * H * W;
     const int x = x0 + lx, y = y0 + ly;
-    if (x < W && y < H) {
+    if (x >= W || y >= H)
+        return;
+    float *o = out + ((int64_t)vol * D * H + y) * W + x;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int z = z0 + 8 * zg + i;
-            if (z < D)
-                out[(int64_t)vol * nv + ((int64_t)z * H + y) * W + x] =
-                    (i & 1) ? acc[i >> 1].y : acc[i >> 1].x;
+    for (int i = 0; i < 8; ++i) {
+        const int z = z0 + 8 * zg + i;
+        if (z >= D)
+            break;
+        float *oz = o + (int64_t)z * H * W;
+        const float v[4] = {acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y};
+        if (vec) {
+            *reinterpret_cast<float4 *>(oz) = make_float4(v[0], v[1], v[2], v[3]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (x + j < W)
+                    oz[j] = v[j];
         }
     }
+}
+
+template <int TB>
+cudaError_t run_render(int D, int H, int W, int count, int nblobs, const float *table, float *out,
+                       cudaStream_t s)
+{
+    const int64_t boxes = (int64_t)((W + TB - 1) / TB) * ((H + TB - 1) / TB) *
+                          ((D + kBrickZ - 1) / kBrickZ);
+    // rows of whole 16-byte pieces (out is 16-byte aligned)
+    k_render_blobs<TB><<<dim3((unsigned)boxes, count), TB * TB, 0, s>>>(D, H, W, nblobs, table, out,
+                                                                       W % 4 == 0);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -512,19 +556,13 @@ cudaError_t launch_render_blobs(int D, int H, int W, int count, int nblobs, cons
                                 float *out, cudaStream_t s)
 {
     ProfScope ps(s, "k_render_blobs");
-    const int bricks = ((W + kBrick - 1) / kBrick) * ((H + kBrick - 1) / kBrick) *
-                       ((D + kBrickZ - 1) / kBrickZ);
-    dim3 grid(bricks, count);
-    // up to 192 KB (1024 blobs), beside the 4 KB keep list
-    const size_t smem = sizeof(float) * kFac * (size_t)nblobs;
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(
-            k_render_blobs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess)
-            return e;
-    }
-    k_render_blobs<<<grid, 256, smem, s>>>(D, H, W, nblobs, table, out);
-    return cudaGetLastError();
+    const int64_t boxes16 = (int64_t)((W + 15) / 16) * ((H + 15) / 16) *
+                            ((D + kBrickZ - 1) / kBrickZ) * count;
+    // boxes of 16 x 16 need a third of the exponentials per voxel; below two per SM
+    // the smaller ones spread better (12 us either way at 48^3: launch)
+    if (boxes16 >= 2 * (int64_t)device_sms())
+        return run_render<16>(D, H, W, count, nblobs, table, out, s);
+    return run_render<8>(D, H, W, count, nblobs, table, out, s);
 }
 
 }  // namespace airgb
