@@ -31,7 +31,7 @@ struct ProbPlan {
     Grid g;
     Lattice L;
     double lambda;
-    int gt[3], ngram, nmom;
+    int gt[3], ngram, gtiles, nmom;  // Gram tiles: of every component, of one
     int gb[kMaxTiles][3], npart[kMaxTiles], nbricks[kMaxTiles], nchunks[kMaxTiles];
     size_t bpart, mpart, rpart, gR;  // workspace offsets
     double work;                     // voxels, for ordering
@@ -83,7 +83,7 @@ std::vector<BatchItem> make_items(const al_batch &b, int policy)
                 if (nb[i] < p.nbricks[t]) {
                     v.push_back({i, BATCH_BRICK, nb[i]++, 0});
                     more = true;
-                } else if (ng[i] < p.ngram) {
+                } else if (ng[i] < p.gtiles) {
                     v.push_back({i, BATCH_GRAM, ng[i]++, 0});
                     more = true;
                 }
@@ -91,7 +91,7 @@ std::vector<BatchItem> make_items(const al_batch &b, int policy)
         }
     } else if (policy == 3) {
         for (int i : order)
-            for (int t = 0; t < b.prob[i].ngram; ++t)
+            for (int t = 0; t < b.prob[i].gtiles; ++t)
                 v.push_back({i, BATCH_GRAM, t, 0});
         for (int i : order)
             for (int k = 0; k < b.prob[i].nbricks[t]; ++k)
@@ -100,7 +100,7 @@ std::vector<BatchItem> make_items(const al_batch &b, int policy)
         for (int i : order) {
             for (int k = 0; k < b.prob[i].nbricks[t]; ++k)
                 v.push_back({i, BATCH_BRICK, k, 0});
-            for (int t = 0; t < b.prob[i].ngram; ++t)
+            for (int t = 0; t < b.prob[i].gtiles; ++t)
                 v.push_back({i, BATCH_GRAM, t, 0});
         }
     }
@@ -114,7 +114,7 @@ int count_items(const al_batch &b, int t)
 {
     int n = 0;
     for (const ProbPlan &p : b.prob)
-        n += p.nbricks[t] + p.ngram + p.nchunks[t];
+        n += p.nbricks[t] + p.gtiles + p.nchunks[t];
     return n;
 }
 
@@ -132,7 +132,7 @@ al_status use_tile(al_batch &b, int t)
         q.gby = p.gb[t][1];
         q.gbz = p.gb[t][2];
         q.nbricks = p.nbricks[t];
-        q.nA = p.nbricks[t] + p.ngram;
+        q.nA = p.nbricks[t] + p.gtiles;
         q.nchunks = p.nchunks[t];
     }
     if (cudaMemcpy(b.ws + b.off_desc, b.desc.data(), sizeof(BatchProblem) * b.desc.size(),
@@ -222,7 +222,7 @@ al_status al_batch_create(const al_problem *problems, int32_t count, al_batch **
             st = check_sim(&pr.sim, p.g.ndim);
         if (st == AL_OK && !isfinite(pr.lambda))
             st = AL_ERR_INVALID_ARG;
-        if (st == AL_OK && (pr.sim.kind != AL_SIM_MSE || batch_threads(pr.bs.spacing, 0) == 0 ||
+        if (st == AL_OK && (pr.sim.kind != AL_SIM_MSE || batch_chunk(pr.bs.spacing, 0) == 0 ||
                             (i > 0 && pr.bs.spacing != problems[0].bs.spacing)))
             st = AL_ERR_UNSUPPORTED;  // MSE, one spacing in {4, 6, 8}
         if (st != AL_OK) {
@@ -234,10 +234,11 @@ al_status al_batch_create(const al_problem *problems, int32_t count, al_batch **
         for (int t = 0; t < b->ntiles; ++t) {
             batch_geometry(p.g, p.L, t, p.gb[t], p.gt, &p.npart[t], &p.nmom);
             p.nbricks[t] = p.gb[t][0] * p.gb[t][1] * p.gb[t][2];
-            const int threads = batch_threads(pr.bs.spacing, t);
-            p.nchunks[t] = (p.L.nc + threads - 1) / threads;
+            const int chunk = batch_chunk(pr.bs.spacing, t);
+            p.nchunks[t] = (p.L.nc + chunk - 1) / chunk;
         }
-        p.ngram = p.g.ndim * p.gt[0] * p.gt[1] * p.gt[2];
+        p.gtiles = p.gt[0] * p.gt[1] * p.gt[2];
+        p.ngram = p.g.ndim * p.gtiles;
         p.work = (double)p.g.nv;
         b->prob.push_back(p);
     }
@@ -275,15 +276,16 @@ int32_t al_batch_items(const al_batch *b, int32_t *per_kind)
 {
     if (!b)
         return 0;
-    if (per_kind) {
-        per_kind[0] = per_kind[1] = per_kind[2] = 0;
-        for (const ProbPlan &p : b->prob) {
-            per_kind[0] += p.nbricks[b->tile];
-            per_kind[1] += p.ngram;
-            per_kind[2] += p.nchunks[b->tile];
-        }
+    // Gram tiles counted per component (those of a tile share a queue entry)
+    int32_t n[3] = {0, 0, 0};
+    for (const ProbPlan &p : b->prob) {
+        n[0] += p.nbricks[b->tile];
+        n[1] += p.ngram;
+        n[2] += p.nchunks[b->tile];
     }
-    return b->nitems;
+    for (int k = 0; per_kind && k < 3; ++k)
+        per_kind[k] = n[k];
+    return n[0] + n[1] + n[2];
 }
 
 al_status al_batch_bind(al_batch *b, const float *const *fixed, const float *const *moving,

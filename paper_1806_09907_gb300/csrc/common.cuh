@@ -166,6 +166,22 @@ __device__ __forceinline__ bool axis_cell(int x, float u, float lo, float hi, in
     return u >= lo && u <= hi;
 }
 
+// The common half of axis_cell: true when the floor cell lies in [0, n - 2], with
+// axis_cell's cell and offset. The sample is then inside (0 <= floor(y) <= n - 2).
+// False on the last face, outside and for values that are not finite: for
+// |u| >= 2^22, infinities and NaN the bits of t give an index of magnitude above
+// 2^21, with either sign, so it never falls into the range. The cell is in range
+// either way; call axis_cell for the rest. xb = x - 0x4B400000 (wrapping).
+__device__ __forceinline__ bool axis_cell_inner(unsigned xb, float u, int n, int &cell, float &f)
+{
+    constexpr float kMagic = 12582912.0f;
+    const float t = __fadd_rd(u, kMagic);
+    const int iy = (int)(xb + (unsigned)__float_as_int(t));
+    f = u - (t - kMagic);
+    cell = __vimin_s32_relu(iy, n - 2);
+    return cell == iy;
+}
+
 // Linear interpolation value and gradient in a 3D cell: corners m[z][y][x].
 struct Interp {
     float v, gx, gy, gz;

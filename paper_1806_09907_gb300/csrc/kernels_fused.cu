@@ -40,12 +40,14 @@ __host__ __device__ constexpr int brick_bcz(int ndim) { return ndim == 3 ? 4 : 1
 
 // Brick tiles the batch kernel is built for, per spacing: control cells per
 // block in x and y, and the resident blocks per SM the kernel is compiled
-// for (its register budget). Tile 0 is the single-problem path's brick at
-// one block per SM; the others are the batch autotuner's alternatives (every
-// axis still spans >= 3 cells):
-//   spacing 4: (8, 4, 1), (8, 4, 2), (6, 4, 2)
-//   spacing 6: (4, 3, 1), (4, 3, 2), (3, 3, 2)
-//   spacing 8: (4, 3, 1), (3, 3, 1), (3, 4, 1)
+// for (its register budget). Tile 0 is the single-problem path's brick at two
+// blocks per SM, which measured best on 9 uneven problems (spacing 4: 213 us
+// against 285 with one, spacing 6: 163 against 213, though a few registers spill);
+// the others are the batch autotuner's alternatives (every axis still spans >= 3
+// cells):
+//   spacing 4: (8, 4, 2), (8, 4, 1), (6, 4, 2)
+//   spacing 6: (4, 3, 2), (4, 3, 1), (3, 3, 2)
+//   spacing 8: (4, 3, 2), (3, 3, 1), (3, 4, 2)
 constexpr int kBatchTiles = 3;
 __host__ __device__ constexpr int batch_tile_bcx(int delta, int t)
 {
@@ -55,33 +57,52 @@ __host__ __device__ constexpr int batch_tile_bcy(int delta, int t)
 {
     return delta <= 4 ? 4 : (delta == 8 && t == 2 ? 4 : 3);
 }
+// Voxel columns per thread. At spacing 8 a brick has 768 columns; one thread each
+// leaves one block per SM, and while its warps wait at the barriers of an item
+// (queue, lattice, flush, Gram phases) the SM idles: 45 % of the issue slots used.
+// Two columns per thread, one after the other, make two resident blocks of 384
+// threads whose phases overlap; with the components of a Gram tile in one item, 16
+// uneven problems go from 313 to 261 us. The smaller bricks of the other spacings
+// are two blocks per SM already.
+__host__ __device__ constexpr int batch_tile_cp(int delta, int t)
+{
+    return delta == 8 && t != 1 ? 2 : 1;
+}
 __host__ __device__ constexpr int batch_tile_minb(int delta, int t)
 {
-    return delta == 8 || t == 0 ? 1 : 2;
+    return batch_tile_cp(delta, t) == 2 ? 2 : delta == 8 || t == 1 ? 1 : 2;
 }
 
-template <int D, int DELTA, int MODE, int BCX_ = brick_bcx(DELTA), int BCY_ = brick_bcy(DELTA)>
+template <int D, int DELTA, int MODE, int BCX_ = brick_bcx(DELTA), int BCY_ = brick_bcy(DELTA),
+          int CP_ = 1>
 struct FCfg {
     static constexpr int BCX = BCX_, BCY = BCY_, BCZ = brick_bcz(D);
     static constexpr int BX = BCX * DELTA, BY = BCY * DELTA;
-    static constexpr int THREADS = BX * BY;
+    // voxel columns of the brick, and the threads that take CP columns each, one
+    // after the other (the columns COLS / CP apart)
+    static constexpr int COLS = BX * BY, CP = CP_, THREADS = COLS / CP;
+    static_assert(COLS % CP == 0 && THREADS % BX == 0, "whole rows of columns per thread group");
     static constexpr int JX = BCX + 3, JY = BCY + 3, JZ = (D == 3) ? BCZ + 3 : 1;
     static constexpr int CH = (MODE == MODE_NCC) ? 3 * D : (MODE == MODE_FWD ? 0 : D);
     static constexpr int CHS = CH > 0 ? CH : 1;  // storage size
     static constexpr int NMOM = (MODE == MODE_MSE) ? 2 : (MODE == MODE_NCC ? 6 : 0);
     static constexpr int NPART = CH * JZ * JY * JX;  // floats of one brick's partials
-    static constexpr int VC = (MODE == MODE_FWD) ? 2 : 1;  // slices whose gathers are in flight together
+    // slices whose gathers are in flight together: two hide the latency of L1 and
+    // L2 better where the registers allow (16 uneven MSE problems 349 -> 313 us);
+    // NCC's nine channels leave none
+    static constexpr int VC = (MODE == MODE_FWD || MODE == MODE_MSE) ? 2 : 1;
     // dynamic shared memory of the flush of up to NPL planes (flush_planes):
-    // region A, the column partials P[NPL][BY][BX][CHS], later their x
-    // contraction; region B, the per-cell sums S1[NPL][BY][BCX][4][CHS], later
+    // region A, the column partials P[NST][BY][BX][CHS], later the x contraction
+    // of the planes flushed; region B, the per-cell sums S1[NPL][BY][BCX][4][CHS], later
     // S2[NPL][BCY][4][JX][CHS]
     static constexpr int NPL = (D == 3) ? 4 : 1;
-    static constexpr int nP = (MODE == MODE_FWD) ? 0 : NPL * BY * BX * CHS;
+    static constexpr int NST = (D == 3 && CP > 1) ? JZ : NPL;  // planes of column partials kept
+    static constexpr int nP = (MODE == MODE_FWD) ? 0 : NST * BY * BX * CHS;
     static constexpr int nX = (MODE == MODE_FWD) ? 0 : NPL * BY * BCX * 4 * CHS;
     // the x contractions of the lattice rows of four planes, per voxel column
     // (plane_rows), after the flush buffers; GW does not expand
     static constexpr int RPL = D * JY * BX;  // floats of one plane's row contractions
-    static constexpr int nR = (MODE == MODE_GW) ? 0 : 4 * RPL;
+    static constexpr int nR = (MODE == MODE_GW) ? 0 : JZ * RPL;
     static constexpr size_t dyn_smem = (size_t)(nP + nX + nR) * sizeof(float);
 };
 
@@ -129,7 +150,8 @@ struct TCfg {
     static constexpr int oF = oRing + NSLOT * SLOTB;
     static constexpr int oU = oF + NF * FSLOTB;  // lattice rows, later the flush buffers
     static constexpr int oR = (nP1 + nX1) * 4;  // row contractions, inside the union
-    static constexpr int nU = (LSTAGE > oR + C::nR * 4) ? LSTAGE : oR + C::nR * 4;
+    static constexpr int nR = (MODE == MODE_GW) ? 0 : 4 * C::RPL;
+    static constexpr int nU = (LSTAGE > oR + nR * 4) ? LSTAGE : oR + nR * 4;
     static constexpr int oBar = oU + round128(nU);
     static constexpr int bytes = oBar + 3 * 8;
     static_assert(SLOTB % 128 == 0 && FSLOTB % 128 == 0, "TMA destinations are 128-byte aligned");
@@ -297,29 +319,32 @@ __device__ __forceinline__ void plane_cols(const float *Rw, int jz, int qy, int 
     oz = out[2];
 }
 
-// Planes 0..NPL-1 of the thread's column partials qz -> x contraction -> y
-// contraction -> the brick's partial sums of local planes lp0 .. lp0+NPL-1.
-// Every thread of the block calls it. Each axis takes two steps: the four
+// store_plane: the thread's column partials of one plane into slot `slot` of A.
+// flush_planes: planes 0..NPL-1 of A -> x contraction -> y contraction -> the
+// brick's partial sums of local planes lp0 .. lp0+NPL-1. Every thread of the
+// block calls it; after it the block may store into A again. Each axis takes two steps: the four
 // weighted sums of every cell (the DELTA voxels of the cell times the
 // compile-time weights of their phases), then for every control point the
 // sum over the (up to four) cells it supports. A holds the column partials,
 // later the x contraction; B the per-cell sums of x, later those of y.
-template <int D, int DELTA, int MODE, int NPL, int BCX_ = brick_bcx(DELTA),
-          int BCY_ = brick_bcy(DELTA)>
-__device__ __forceinline__ void flush_planes(int lp0, const float (&qz)[4][FCfg<D, DELTA, MODE>::CHS],
-                                             bool colvalid, int tx, int ty, float *A, float *B,
-                                             float *dst)
+template <int COLS, int CHS>
+__device__ __forceinline__ void store_plane(const float (&q)[CHS], bool colvalid, int slot, int col,
+                                            float *A)
 {
-    using C = FCfg<D, DELTA, MODE, BCX_, BCY_>;
+#pragma unroll
+    for (int k = 0; k < CHS; ++k)
+        A[(slot * COLS + col) * CHS + k] = colvalid ? q[k] : 0.0f;
+}
+
+template <int D, int DELTA, int MODE, int NPL, int BCX_ = brick_bcx(DELTA),
+          int BCY_ = brick_bcy(DELTA), int CP = 1>
+__device__ __forceinline__ void flush_planes(int lp0, float *A, float *B, float *dst)
+{
+    using C = FCfg<D, DELTA, MODE, BCX_, BCY_, CP>;
     constexpr int CHS = C::CHS, BX = C::BX, BY = C::BY, JX = C::JX, JY = C::JY, JZ = C::JZ;
     constexpr int BCX = C::BCX, BCY = C::BCY;
     constexpr WTab<DELTA> kW{};
     const int tid = threadIdx.x;
-#pragma unroll
-    for (int a = 0; a < NPL; ++a)
-#pragma unroll
-        for (int k = 0; k < CHS; ++k)
-            A[((a * BY + ty) * BX + tx) * CHS + k] = colvalid ? qz[a][k] : 0.0f;
     __syncthreads();
     // x, per cell: S1[(a BY + y) BCX + qx][q][k] = sum_px w[px][q] P[a][y][qx DELTA + px][k]
     for (int e = tid; e < NPL * BY * BCX * CHS; e += C::THREADS) {
@@ -398,7 +423,7 @@ __device__ __forceinline__ void flush_planes(int lp0, const float (&qz)[4][FCfg<
 // give the same bits. Returns false if a copy did not land in time (the
 // brick's partials are then not written).
 template <int D, int DELTA, int MODE, int BCX_ = brick_bcx(DELTA), int BCY_ = brick_bcy(DELTA),
-          bool TMA = false, bool PAIR = false>
+          bool TMA = false, bool PAIR = false, int CP = 1>
 __device__ __forceinline__ bool fused_brick(const Grid &g, const Lattice &L,
                                             const float *__restrict__ F,
                                             const float *__restrict__ M,
@@ -414,10 +439,10 @@ __device__ __forceinline__ bool fused_brick(const Grid &g, const Lattice &L,
     // with PAIR it writes only the bf16 pairs (W, M) of the network input,
     // W_out then pointing at them. MODE_GW reads dS/dW and those planes back
     // (no expansion, no gathers).
-    using C = FCfg<D, DELTA, MODE, BCX_, BCY_>;
+    using C = FCfg<D, DELTA, MODE, BCX_, BCY_, CP>;
     using T = TCfg<DELTA, MODE == MODE_GW ? MODE_FWD : MODE>;
     using GS = GCfg<DELTA>;
-    static_assert(!TMA || (D == 3 && BCX_ == brick_bcx(DELTA) && BCY_ == brick_bcy(DELTA)),
+    static_assert(!TMA || (D == 3 && CP == 1 && BCX_ == brick_bcx(DELTA) && BCY_ == brick_bcy(DELTA)),
                   "TMA staging: 3D single-problem bricks");
     constexpr int JX = C::JX, JY = C::JY, JZ = C::JZ, CHS = C::CHS, BX = C::BX;
     constexpr WTab<DELTA> kW{};  // weights of the compile-time z phases
@@ -436,9 +461,10 @@ __device__ __forceinline__ bool fused_brick(const Grid &g, const Lattice &L,
     const float *Fs = reinterpret_cast<const float *>(sm + T::oF);
 
     const int tid = threadIdx.x;
-    const int tx = tid % BX, ty = tid / BX;
+    const int tx = tid % BX;
+    int ty = tid / BX;
     const int cx0 = bx * C::BCX, cy0 = by * C::BCY, cz0 = bz * C::BCZ;
-    const int x = cx0 * DELTA + tx, y = cy0 * DELTA + ty, z0 = (D == 3) ? cz0 * DELTA : 0;
+    const int x = cx0 * DELTA + tx, z0 = (D == 3) ? cz0 * DELTA : 0;
     const int x0 = cx0 * DELTA, y0 = cy0 * DELTA;
 
     if (tid < DELTA * 4)
@@ -526,17 +552,41 @@ __device__ __forceinline__ bool fused_brick(const Grid &g, const Lattice &L,
     __syncthreads();
 
     const int qxl = tx / DELTA, px = tx - qxl * DELTA;
-    const int qyl = ty / DELTA, py = ty - qyl * DELTA;
-    float wx[4], wy[4];
+    float wx[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
+    for (int e = 0; e < 4; ++e)
         wx[e] = wt[px][e];
-        wy[e] = wt[py][e];
+    // xy-contracted control values of the four active planes: (x, y) packed
+    // for the f32x2 z expansion, z apart (3D)
+    if constexpr (MODE != MODE_GW) {
+        // gathered bricks: the rows of every plane, so that the layers need no
+        // barrier; staged ones have room for the active four
+#pragma unroll
+        for (int a = 0; a < (TMA ? 4 : JZ); ++a)
+            plane_rows<D, JZ, JY, JX, BX, C::THREADS>(cb, a, qxl, wx, Rw + a * C::RPL);
+        __syncthreads();
     }
-    const bool colvalid = x < g.X && y < g.Y;
-    // sample bounds of axis_cell: y = x + u inside when -x <= u <= n - 1 - x
-    const float lox = (float)(-x), hix = (float)(g.X - 1 - x);
-    const float loy = (float)(-y), hiy = (float)(g.Y - 1 - y);
+    float *const dstp = bpart + (int64_t)brick * C::NPART;
+    const int cells_z = (D == 3) ? (g.Z + DELTA - 1) / DELTA : 1;
+    const int nlayers = (D == 3) ? min(C::BCZ, cells_z - cz0) : 1;
+    constexpr int NP = D == 3 ? DELTA : 1;          // slices of a layer
+    constexpr int VC = TMA || D == 2 ? 1 : C::VC;  // slices whose loads are in flight together
+    int fail_layer = -1;
+    float qz[4][CHS];  // column partial sums of the four active planes
+    float mom[C::NMOM > 0 ? C::NMOM : 1];
+    bool colvalid = false;
+#pragma unroll 1
+    for (int h = 0; h < CP; ++h) {  // the thread's columns, body not indented further
+    const int col = tid + h * C::THREADS;
+    if (CP > 1)
+        ty = col / BX;
+    const int y = y0 + ty;
+    const int qyl = ty / DELTA, py = ty - qyl * DELTA;
+    float wy[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        wy[e] = wt[py][e];
+    colvalid = x < g.X && y < g.Y;
     // xy-contracted control values of the four active planes: (x, y) packed
     // for the f32x2 z expansion, z apart (3D)
     float2 cxy2[4];
@@ -544,32 +594,19 @@ __device__ __forceinline__ bool fused_brick(const Grid &g, const Lattice &L,
     if constexpr (MODE != MODE_GW) {
 #pragma unroll
         for (int a = 0; a < 4; ++a)
-            plane_rows<D, JZ, JY, JX, BX, C::THREADS>(cb, a, qxl, wx, Rw + a * C::RPL);
-        __syncthreads();
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
             plane_cols<D, JZ, JY, BX>(Rw + a * C::RPL, a, qyl, tx, wy, cxy2[a], cxyz[a]);
     }
-    float qz[4][CHS];  // column partial sums of the four active planes
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int k = 0; k < CHS; ++k)
             qz[a][k] = 0.0f;
-    float mom[C::NMOM > 0 ? C::NMOM : 1];
 #pragma unroll
     for (int k = 0; k < (C::NMOM > 0 ? C::NMOM : 1); ++k)
         mom[k] = 0.0f;
-
-    float *const dstp = bpart + (int64_t)brick * C::NPART;
-    const int cells_z = (D == 3) ? (g.Z + DELTA - 1) / DELTA : 1;
-    const int nlayers = (D == 3) ? min(C::BCZ, cells_z - cz0) : 1;
-    constexpr int VC = TMA ? 1 : C::VC;  // slices whose loads are in flight together
-    int fail_layer = -1;
     for (int cz = 0; cz < C::BCZ; ++cz) {
         const bool active = cz < nlayers && colvalid;
         const int zl0 = z0 + cz * DELTA;
-        const float loz0 = (float)(-zl0), hiz0 = (float)(g.Z - 1 - zl0);  // slice zl0 + pz: - pz
         // GW: the layer's loads are issued before the flush of the previous
         // plane, so they are in flight while the block contracts it
         float gv[MODE == MODE_GW ? DELTA : 1], gr[MODE == MODE_GW ? DELTA : 1][D];
@@ -590,10 +627,13 @@ __device__ __forceinline__ bool fused_brick(const Grid &g, const Lattice &L,
             }
         }
         if (cz > 0) {
-            // plane cz - 1 has all its contributions: write it out, roll
-            if (MODE != MODE_FWD)
-                flush_planes<D, DELTA, MODE, 1, BCX_, BCY_>(cz - 1, qz, colvalid, tx, ty, P, Xc,
-                                                            dstp);
+            // plane cz - 1 has all its contributions: write it out (gathered
+            // bricks: keep it for the flush at the end), roll
+            if (MODE != MODE_FWD) {
+                store_plane<C::COLS>(qz[0], colvalid, TMA ? 0 : cz - 1, col, P);
+                if constexpr (TMA)
+                    flush_planes<D, DELTA, MODE, 1, BCX_, BCY_>(cz - 1, P, Xc, dstp);
+            }
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
 #pragma unroll
@@ -607,7 +647,7 @@ __device__ __forceinline__ bool fused_brick(const Grid &g, const Lattice &L,
                 qz[3][k] = 0.0f;
             // row contractions of plane cz + 3 (into the buffer of plane
             // cz - 1, last read before the previous layer's barrier)
-            if (MODE != MODE_GW)
+            if (TMA && MODE != MODE_GW)
                 plane_rows<D, JZ, JY, JX, BX, C::THREADS>(cb, cz + 3, qxl, wx,
                                                           Rw + ((cz + 3) & 3) * C::RPL);
         }
@@ -633,12 +673,10 @@ __device__ __forceinline__ bool fused_brick(const Grid &g, const Lattice &L,
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 brick_issue<DELTA, MODE>(tm, sbase, cz + 1, x0, y0, z0);
             }
-        } else if (MODE != MODE_GW && cz > 0) {
-            __syncthreads();  // the row contractions of plane cz + 3 are written
         }
         if (MODE != MODE_GW && cz > 0)
-            plane_cols<D, JZ, JY, BX>(Rw + ((cz + 3) & 3) * C::RPL, cz + 3, qyl, tx, wy, cxy2[3],
-                                      cxyz[3]);
+            plane_cols<D, JZ, JY, BX>(Rw + (TMA ? (cz + 3) & 3 : cz + 3) * C::RPL, cz + 3, qyl, tx,
+                                      wy, cxy2[3], cxyz[3]);
         if (!active)
             continue;
         if constexpr (MODE == MODE_GW) {
@@ -677,7 +715,7 @@ __device__ __forceinline__ bool fused_brick(const Grid &g, const Lattice &L,
         } else {
         const float *Fl = Fs + (cz & 1) * (T::FSLOTB / 4) + ty * BX + tx;
 #pragma unroll
-        for (int p0 = 0; p0 < DELTA; p0 += VC) {
+        for (int p0 = 0; p0 < NP; p0 += VC) {
             // issue every load of VC slices, then use them
             // corners paired by z: mc[q] = (slice kz, slice kz + 1) at y x bits q
             float2 mc[VC][4];
@@ -686,7 +724,7 @@ __device__ __forceinline__ bool fused_brick(const Grid &g, const Lattice &L,
 #pragma unroll
             for (int j = 0; j < VC; ++j) {
                 const int pz = p0 + j;
-                if (pz >= DELTA)
+                if (pz >= NP)
                     break;
                 const int z = zl0 + pz;
                 float uu[3] = {cxy2[0].x, cxy2[0].y, 0.f};
@@ -707,10 +745,17 @@ __device__ __forceinline__ bool fused_brick(const Grid &g, const Lattice &L,
                 // cells are clamped into the volume even outside the mask, so
                 // every load is in bounds; the values outside are not used
                 int kx, ky, kz = 0;
-                bool in = axis_cell(x, uu[0], lox, hix, g.X, kx, fx[j]);
-                in &= axis_cell(y, uu[1], loy, hiy, g.Y, ky, fy[j]);
+                bool in = axis_cell_inner((unsigned)x - 0x4B400000u, uu[0], g.X, kx, fx[j]);
+                in &= axis_cell_inner((unsigned)y - 0x4B400000u, uu[1], g.Y, ky, fy[j]);
                 if (D == 3)
-                    in &= axis_cell(z, uu[2], loz0 - (float)pz, hiz0 - (float)pz, g.Z, kz, fz[j]);
+                    in &= axis_cell_inner((unsigned)z - 0x4B400000u, uu[2], g.Z, kz, fz[j]);
+                if (!in) {  // the last faces and outside
+                    in = axis_cell(x, uu[0], (float)(-x), (float)(g.X - 1 - x), g.X, kx, fx[j]);
+                    in &= axis_cell(y, uu[1], (float)(-y), (float)(g.Y - 1 - y), g.Y, ky, fy[j]);
+                    if (D == 3)
+                        in &= axis_cell(z, uu[2], (float)(-z), (float)(g.Z - 1 - z), g.Z, kz,
+                                        fz[j]);
+                }
                 inb[j] = in && (z < g.Z);
                 if (!(al_index_ok(kx, g.X - 1) & al_index_ok(ky, g.Y - 1) &
                       al_index_ok(kz, D == 3 ? g.Z - 1 : 1)))
@@ -757,7 +802,7 @@ __device__ __forceinline__ bool fused_brick(const Grid &g, const Lattice &L,
 #pragma unroll
             for (int j = 0; j < VC; ++j) {
                 const int pz = p0 + j;
-                if (pz >= DELTA)
+                if (pz >= NP)
                     break;
                 const int z = zl0 + pz;
                 if (z >= g.Z)
@@ -834,6 +879,23 @@ __device__ __forceinline__ bool fused_brick(const Grid &g, const Lattice &L,
         }
         }  // MODE != MODE_GW
     }
+    if constexpr (CP > 1) {
+        // the column's other planes, and its moments: an fp32 tree within the
+        // warp as in block_reduce_fd, the warps' sums of the columns in FP64
+#pragma unroll
+        for (int a = 0; a < (D == 3 ? 4 : 1); ++a)
+            store_plane<C::COLS>(qz[a], colvalid, (D == 3 ? C::BCZ - 1 : 0) + a, col, P);
+        constexpr int NW = (C::THREADS + 31) / 32;
+#pragma unroll
+        for (int k = 0; k < C::NMOM; ++k) {
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1)
+                mom[k] += __shfl_down_sync(0xffffffffu, mom[k], off);
+            if ((tid & 31) == 0)
+                red[k * NW + (tid >> 5)] = (h == 0 ? 0.0 : red[k * NW + (tid >> 5)]) + (double)mom[k];
+        }
+    }
+    }  // h
     if constexpr (TMA) {
         if (fail_layer >= 0) {
             // record the timeout; let the copies in flight land before the
@@ -854,25 +916,46 @@ __device__ __forceinline__ bool fused_brick(const Grid &g, const Lattice &L,
             // the last four planes one at a time (the staging leaves room for one)
 #pragma unroll
             for (int a = 0; a < 4; ++a) {
-                flush_planes<D, DELTA, MODE, 1, BCX_, BCY_>(C::BCZ - 1 + a, qz, colvalid, tx, ty,
-                                                            P, Xc, dstp);
-                if (a < 3) {
-#pragma unroll
-                    for (int b = 0; b < 3; ++b)
-#pragma unroll
-                        for (int k = 0; k < CHS; ++k)
-                            qz[b][k] = qz[b + 1][k];
-                }
+                store_plane<C::COLS>(qz[a], colvalid, 0, tid, P);
+                flush_planes<D, DELTA, MODE, 1, BCX_, BCY_>(C::BCZ - 1 + a, P, Xc, dstp);
             }
+        } else if constexpr (CP > 1 && D == 3) {
+            flush_planes<D, DELTA, MODE, C::NPL, BCX_, BCY_, CP>(0, P, Xc, dstp);
+            flush_planes<D, DELTA, MODE, C::JZ - C::NPL, BCX_, BCY_, CP>(
+                C::NPL, P + C::NPL * C::COLS * CHS, Xc, dstp);
+        } else if constexpr (CP > 1) {
+            flush_planes<D, DELTA, MODE, 1, BCX_, BCY_, CP>(0, P, Xc, dstp);
+        } else if constexpr (D == 3) {
+            // the planes kept and the first of the last four together, then
+            // the other three
+            static_assert(C::BCZ == C::NPL && C::JZ == C::NPL + 3, "seven planes in two flushes");
+            store_plane<C::COLS>(qz[0], colvalid, C::BCZ - 1, tid, P);
+            flush_planes<D, DELTA, MODE, C::NPL, BCX_, BCY_>(0, P, Xc, dstp);
+#pragma unroll
+            for (int a = 1; a < 4; ++a)
+                store_plane<C::COLS>(qz[a], colvalid, a - 1, tid, P);
+            flush_planes<D, DELTA, MODE, 3, BCX_, BCY_>(C::NPL, P, Xc, dstp);
         } else {
-            // the last four planes (a single plane in 2D), together
-            flush_planes<D, DELTA, MODE, C::NPL, BCX_, BCY_>(D == 3 ? C::BCZ - 1 : 0, qz,
-                                                             colvalid, tx, ty, P, Xc, dstp);
+            store_plane<C::COLS>(qz[0], colvalid, 0, tid, P);
+            flush_planes<D, DELTA, MODE, 1, BCX_, BCY_>(0, P, Xc, dstp);
         }
     }
     if (C::NMOM > 0) {
         double mm[C::NMOM > 0 ? C::NMOM : 1];
-        block_reduce_fd<(C::NMOM > 0 ? C::NMOM : 1)>(mom, mm, red);
+        if constexpr (CP == 1) {
+            block_reduce_fd<(C::NMOM > 0 ? C::NMOM : 1)>(mom, mm, red);
+        } else {  // the flush's barriers lie between the warps' sums and here
+            constexpr int NW = (C::THREADS + 31) / 32;
+            if (tid < 32) {
+#pragma unroll
+                for (int k = 0; k < C::NMOM; ++k) {
+                    mm[k] = tid < NW ? red[k * NW + tid] : 0.0;
+#pragma unroll
+                    for (int off = 16; off > 0; off >>= 1)
+                        mm[k] += __shfl_down_sync(0xffffffffu, mm[k], off);
+                }
+            }
+        }
         if (tid == 0) {
             for (int k = 0; k < C::NMOM; ++k)
                 mpart[(int64_t)brick * C::NMOM + k] = mm[k];
@@ -925,31 +1008,44 @@ __device__ void band_entry(const Lattice &L, int N, int n, int j, int o, float &
 
 constexpr int kGramT3 = 8, kGramT2 = 16;
 
-// One tile (tile x, y, z) of component i of dR/dc on the lattice; the
-// tile's share of R (before the 1/|X|) goes to *rpart. Every thread of the
-// block calls it (any block size up to 1024).
+// One tile (tile x, y, z) of NC components of dR/dc on the lattice, from component
+// i0; the tile's share of R (before the 1/|X|) of component i0 + k goes to
+// rpart[k * rstride]. Every thread of the block calls it (any block size up to
+// 1024). A tile is a chain of five short phases with a barrier each; with NC = D
+// the components share it and the band tables (the batch kernel, whose blocks take
+// many tiles), with NC = 1 they go to blocks of their own (one problem).
 // Shared floats a Gram tile needs (carved from the caller's dynamic memory).
-constexpr int kGram3Floats = 14 * 14 * 14 + 2 * 14 * 14 * 8 + 3 * 14 * 8 * 8 + 2 * 3 * 8 * 7;
-constexpr int kGram2Floats = 22 * 22 + 2 * 22 * 16 + 2 * 2 * 16 * 7;
+__host__ __device__ constexpr int gram3_floats(int nc)
+{
+    return nc * (14 * 14 * 14 + 2 * 14 * 14 * 8 + 3 * 14 * 8 * 8) + 2 * 3 * 8 * 7;
+}
+__host__ __device__ constexpr int gram2_floats(int nc)
+{
+    return nc * (22 * 22 + 2 * 22 * 16) + 2 * 2 * 16 * 7;
+}
 
+template <int NC>
 __device__ __forceinline__ void gram3_tile(const Grid &g, const Lattice &L,
                                            const float *__restrict__ c, float gscale,
                                            float *__restrict__ gR, int tile_x, int tile_y,
-                                           int tile_z, int i, double *rpart, float *sm)
+                                           int tile_z, int i0, double *rpart, int rstride,
+                                           float *sm)
 {
-    constexpr int T = kGramT3, H3 = T + 6;
-    static_assert(kGram3Floats == H3 * H3 * H3 + 2 * H3 * H3 * T + 3 * H3 * T * T + 2 * 3 * T * 7,
+    // rows of all components: row (k, lz) of component i0 + k at k H3 + lz
+    constexpr int T = kGramT3, H3 = T + 6, R3 = NC * H3;
+    static_assert(gram3_floats(NC) ==
+                      R3 * H3 * H3 + 2 * R3 * H3 * T + 3 * R3 * T * T + 2 * 3 * T * 7,
                   "Gram tile layout");
     auto cs = reinterpret_cast<float (*)[H3][H3]>(sm);
-    auto A = reinterpret_cast<float (*)[H3][T]>(sm + H3 * H3 * H3);
-    auto B = reinterpret_cast<float (*)[H3][T]>(sm + H3 * H3 * H3 + H3 * H3 * T);
-    float *const g0 = sm + H3 * H3 * H3 + 2 * H3 * H3 * T;
+    auto A = reinterpret_cast<float (*)[H3][T]>(sm + R3 * H3 * H3);
+    auto B = reinterpret_cast<float (*)[H3][T]>(sm + R3 * H3 * H3 + R3 * H3 * T);
+    float *const g0 = sm + R3 * H3 * H3 + 2 * R3 * H3 * T;
     auto GA = reinterpret_cast<float (*)[T][T]>(g0);
-    auto HB = reinterpret_cast<float (*)[T][T]>(g0 + H3 * T * T);
-    auto GB = reinterpret_cast<float (*)[T][T]>(g0 + 2 * H3 * T * T);
-    auto tG = reinterpret_cast<float (*)[T][7]>(g0 + 3 * H3 * T * T);
-    auto tH = reinterpret_cast<float (*)[T][7]>(g0 + 3 * H3 * T * T + 3 * T * 7);
-    __shared__ double red[32];
+    auto HB = reinterpret_cast<float (*)[T][T]>(g0 + R3 * T * T);
+    auto GB = reinterpret_cast<float (*)[T][T]>(g0 + 2 * R3 * T * T);
+    auto tG = reinterpret_cast<float (*)[T][7]>(g0 + 3 * R3 * T * T);
+    auto tH = reinterpret_cast<float (*)[T][7]>(g0 + 3 * R3 * T * T + 3 * T * 7);
+    __shared__ double red[NC * 32];
     const int nthr = blockDim.x;
     const int j0[3] = {tile_x * T, tile_y * T, tile_z * T};
     const int nn[3] = {L.nx, L.ny, L.nz};
@@ -959,19 +1055,20 @@ __device__ __forceinline__ void gram3_tile(const Grid &g, const Lattice &L,
         const int k = e / (T * 7), r = e - k * T * 7, l = r / 7, o = r - l * 7 - 3;
         band_entry(L, NN[k], nn[k], j0[k] + l, o, tG[k][l][o + 3], tH[k][l][o + 3]);
     }
-    float rsum = 0.0f;
+    float rsum[NC];
     {
         __syncthreads();
-        for (int e = tid; e < H3 * H3 * H3; e += nthr) {
+        for (int e = tid; e < R3 * H3 * H3; e += nthr) {
             const int lz = e / (H3 * H3), r = e - lz * H3 * H3, ly = r / H3, lx = r - ly * H3;
-            const int jx = j0[0] + lx - 3, jy = j0[1] + ly - 3, jz = j0[2] + lz - 3;
+            const int k = lz / H3;
+            const int jx = j0[0] + lx - 3, jy = j0[1] + ly - 3, jz = j0[2] + lz - k * H3 - 3;
             float v = 0.0f;
             if (jx >= 0 && jx < L.nx && jy >= 0 && jy < L.ny && jz >= 0 && jz < L.nz)
-                v = __ldg(c + (((int64_t)i * L.nz + jz) * L.ny + jy) * L.nx + jx);
+                v = __ldg(c + (((int64_t)(i0 + k) * L.nz + jz) * L.ny + jy) * L.nx + jx);
             (&cs[0][0][0])[e] = v;
         }
         __syncthreads();
-        for (int e = tid; e < H3 * H3 * T; e += nthr) {
+        for (int e = tid; e < R3 * H3 * T; e += nthr) {
             const int lz = e / (H3 * T), r = e - lz * H3 * T, ly = r / T, lx = r - ly * T;
             float a = 0.f, b = 0.f;
 #pragma unroll
@@ -984,7 +1081,7 @@ __device__ __forceinline__ void gram3_tile(const Grid &g, const Lattice &L,
             B[lz][ly][lx] = b;
         }
         __syncthreads();
-        for (int e = tid; e < H3 * T * T; e += nthr) {
+        for (int e = tid; e < R3 * T * T; e += nthr) {
             const int lz = e / (T * T), r = e - lz * T * T, ly = r / T, lx = r - ly * T;
             float ga = 0.f, hb = 0.f, gb = 0.f;
 #pragma unroll
@@ -999,40 +1096,50 @@ __device__ __forceinline__ void gram3_tile(const Grid &g, const Lattice &L,
             GB[lz][ly][lx] = gb;
         }
         __syncthreads();
-        for (int e = tid; e < T * T * T; e += nthr) {
-            const int lz = e / (T * T), r = e - lz * T * T, ly = r / T, lx = r - ly * T;
-            const int jx = j0[0] + lx, jy = j0[1] + ly, jz = j0[2] + lz;
-            if (jx >= L.nx || jy >= L.ny || jz >= L.nz)
-                continue;
-            float s = 0.f;
 #pragma unroll
-            for (int o = 0; o < 7; ++o) {
-                s = fmaf(tG[2][lz][o], GA[lz + o][ly][lx] + HB[lz + o][ly][lx], s);
-                s = fmaf(tH[2][lz][o], GB[lz + o][ly][lx], s);
+        for (int k = 0; k < NC; ++k) {
+            rsum[k] = 0.0f;
+            for (int e = tid; e < T * T * T; e += nthr) {
+                const int lz = e / (T * T), r = e - lz * T * T, ly = r / T, lx = r - ly * T;
+                const int jx = j0[0] + lx, jy = j0[1] + ly, jz = j0[2] + lz, rz = k * H3 + lz;
+                if (jx >= L.nx || jy >= L.ny || jz >= L.nz)
+                    continue;
+                float s = 0.f;
+#pragma unroll
+                for (int o = 0; o < 7; ++o) {
+                    s = fmaf(tG[2][lz][o], GA[rz + o][ly][lx] + HB[rz + o][ly][lx], s);
+                    s = fmaf(tH[2][lz][o], GB[rz + o][ly][lx], s);
+                }
+                rsum[k] = fmaf(cs[rz + 3][ly + 3][lx + 3], s, rsum[k]);
+                gR[(((int64_t)(i0 + k) * L.nz + jz) * L.ny + jy) * L.nx + jx] = gscale * s;
             }
-            rsum = fmaf(cs[lz + 3][ly + 3][lx + 3], s, rsum);
-            gR[(((int64_t)i * L.nz + jz) * L.ny + jy) * L.nx + jx] = gscale * s;
         }
     }
-    double acc[1] = {rsum};
-    block_reduce_d<1>(acc, red);
+    double acc[NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k)
+        acc[k] = rsum[k];
+    block_reduce_d<NC>(acc, red);
     if (tid == 0)
-        *rpart = acc[0];
+#pragma unroll
+        for (int k = 0; k < NC; ++k)
+            rpart[(int64_t)k * rstride] = acc[k];
 }
 
+template <int NC>
 __device__ __forceinline__ void gram2_tile(const Grid &g, const Lattice &L,
                                            const float *__restrict__ c, float gscale,
-                                           float *__restrict__ gR, int tile_x, int tile_y, int i,
-                                           double *rpart, float *sm)
+                                           float *__restrict__ gR, int tile_x, int tile_y, int i0,
+                                           double *rpart, int rstride, float *sm)
 {
-    constexpr int T = kGramT2, H2 = T + 6;
-    static_assert(kGram2Floats == H2 * H2 + 2 * H2 * T + 2 * 2 * T * 7, "Gram tile layout");
+    constexpr int T = kGramT2, H2 = T + 6, R2 = NC * H2;
+    static_assert(gram2_floats(NC) == R2 * H2 + 2 * R2 * T + 2 * 2 * T * 7, "Gram tile layout");
     auto cs = reinterpret_cast<float (*)[H2]>(sm);
-    auto A = reinterpret_cast<float (*)[T]>(sm + H2 * H2);
-    auto B = reinterpret_cast<float (*)[T]>(sm + H2 * H2 + H2 * T);
-    auto tG = reinterpret_cast<float (*)[T][7]>(sm + H2 * H2 + 2 * H2 * T);
-    auto tH = reinterpret_cast<float (*)[T][7]>(sm + H2 * H2 + 2 * H2 * T + 2 * T * 7);
-    __shared__ double red[32];
+    auto A = reinterpret_cast<float (*)[T]>(sm + R2 * H2);
+    auto B = reinterpret_cast<float (*)[T]>(sm + R2 * H2 + R2 * T);
+    auto tG = reinterpret_cast<float (*)[T][7]>(sm + R2 * H2 + 2 * R2 * T);
+    auto tH = reinterpret_cast<float (*)[T][7]>(sm + R2 * H2 + 2 * R2 * T + 2 * T * 7);
+    __shared__ double red[NC * 32];
     const int nthr = blockDim.x;
     const int j0[2] = {tile_x * T, tile_y * T};
     const int nn[2] = {L.nx, L.ny};
@@ -1042,19 +1149,20 @@ __device__ __forceinline__ void gram2_tile(const Grid &g, const Lattice &L,
         const int k = e / (T * 7), r = e - k * T * 7, l = r / 7, o = r - l * 7 - 3;
         band_entry(L, NN[k], nn[k], j0[k] + l, o, tG[k][l][o + 3], tH[k][l][o + 3]);
     }
-    float rsum = 0.0f;
+    float rsum[NC];
     {
         __syncthreads();
-        for (int e = tid; e < H2 * H2; e += nthr) {
+        for (int e = tid; e < R2 * H2; e += nthr) {
             const int ly = e / H2, lx = e - ly * H2;
-            const int jx = j0[0] + lx - 3, jy = j0[1] + ly - 3;
+            const int k = ly / H2;
+            const int jx = j0[0] + lx - 3, jy = j0[1] + ly - k * H2 - 3;
             float v = 0.0f;
             if (jx >= 0 && jx < L.nx && jy >= 0 && jy < L.ny)
-                v = __ldg(c + ((int64_t)i * L.ny + jy) * L.nx + jx);
+                v = __ldg(c + ((int64_t)(i0 + k) * L.ny + jy) * L.nx + jx);
             cs[ly][lx] = v;
         }
         __syncthreads();
-        for (int e = tid; e < H2 * T; e += nthr) {
+        for (int e = tid; e < R2 * T; e += nthr) {
             const int ly = e / T, lx = e - ly * T;
             float a = 0.f, b = 0.f;
 #pragma unroll
@@ -1067,25 +1175,34 @@ __device__ __forceinline__ void gram2_tile(const Grid &g, const Lattice &L,
             B[ly][lx] = b;
         }
         __syncthreads();
-        for (int e = tid; e < T * T; e += nthr) {
-            const int ly = e / T, lx = e - ly * T;
-            const int jx = j0[0] + lx, jy = j0[1] + ly;
-            if (jx >= L.nx || jy >= L.ny)
-                continue;
-            float s = 0.f;
 #pragma unroll
-            for (int o = 0; o < 7; ++o) {
-                s = fmaf(tG[1][ly][o], A[ly + o][lx], s);
-                s = fmaf(tH[1][ly][o], B[ly + o][lx], s);
+        for (int k = 0; k < NC; ++k) {
+            rsum[k] = 0.0f;
+            for (int e = tid; e < T * T; e += nthr) {
+                const int ly = e / T, lx = e - ly * T, ry = k * H2 + ly;
+                const int jx = j0[0] + lx, jy = j0[1] + ly;
+                if (jx >= L.nx || jy >= L.ny)
+                    continue;
+                float s = 0.f;
+#pragma unroll
+                for (int o = 0; o < 7; ++o) {
+                    s = fmaf(tG[1][ly][o], A[ry + o][lx], s);
+                    s = fmaf(tH[1][ly][o], B[ry + o][lx], s);
+                }
+                rsum[k] = fmaf(cs[ry + 3][lx + 3], s, rsum[k]);
+                gR[((int64_t)(i0 + k) * L.ny + jy) * L.nx + jx] = gscale * s;
             }
-            rsum = fmaf(cs[ly + 3][lx + 3], s, rsum);
-            gR[((int64_t)i * L.ny + jy) * L.nx + jx] = gscale * s;
         }
     }
-    double acc[1] = {rsum};
-    block_reduce_d<1>(acc, red);
+    double acc[NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k)
+        acc[k] = rsum[k];
+    block_reduce_d<NC>(acc, red);
     if (tid == 0)
-        *rpart = acc[0];
+#pragma unroll
+        for (int k = 0; k < NC; ++k)
+            rpart[(int64_t)k * rstride] = acc[k];
 }
 
 // ---------------------------------------------------------------------------
@@ -1500,9 +1617,9 @@ __global__ void __launch_bounds__(FCfg<D, DELTA, MODE>::THREADS,
     const int tz = r2 % gb.gtz, comp = r2 / gb.gtz;
     extern __shared__ float gtile_sm[];
     if constexpr (D == 3)
-        gram3_tile(g, L, c, gb.gscale, gb.gR, tx, ty, tz, comp, gb.rpart + w, gtile_sm);
+        gram3_tile<1>(g, L, c, gb.gscale, gb.gR, tx, ty, tz, comp, gb.rpart + w, 0, gtile_sm);
     else
-        gram2_tile(g, L, c, gb.gscale, gb.gR, tx, ty, comp, gb.rpart + w, gtile_sm);
+        gram2_tile<1>(g, L, c, gb.gscale, gb.gR, tx, ty, comp, gb.rpart + w, 0, gtile_sm);
 }
 
 // k_fused for 3D bricks staged by TMA (MSE, NCC, FWD; X a multiple of 4).
@@ -1537,14 +1654,16 @@ __global__ void __launch_bounds__(FCfg<3, DELTA, MODE>::THREADS,
     const int tx = w % gb.gtx, r = w / gb.gtx, ty = r % gb.gty, r2 = r / gb.gty;
     const int tz = r2 % gb.gtz, comp = r2 / gb.gtz;
     extern __shared__ float gtile_sm[];
-    gram3_tile(g, L, c, gb.gscale, gb.gR, tx, ty, tz, comp, gb.rpart + w, gtile_sm);
+    gram3_tile<1>(g, L, c, gb.gscale, gb.gR, tx, ty, tz, comp, gb.rpart + w, 0, gtile_sm);
 }
+
+constexpr int kStagedMseBricks = 16;
 
 // Tensor maps of the TMA brick path; false when the volume does not allow
 // them (rows not on 16-byte boundaries, a box larger than the volume) or an
 // encoding fails, and the launch then takes the gathering path.
 template <int DELTA, int MODE>
-bool brick_tmaps(const Grid &g, const Lattice &L, const float *F, const float *M, const float *c,
+bool brick_tmaps(const Grid &g, const Lattice &L, int nbricks, const float *F, const float *M, const float *c,
                  CUtensorMap *mM, CUtensorMap *mF, CUtensorMap *mC, int *lbox, int *lslot,
                  int *lplane)
 {
@@ -1552,6 +1671,13 @@ bool brick_tmaps(const Grid &g, const Lattice &L, const float *F, const float *M
     memset(mM, 0, sizeof(*mM));
     memset(mF, 0, sizeof(*mF));
     memset(mC, 0, sizeof(*mC));
+    // MSE: since gathered bricks keep their planes for one flush at the end and
+    // have two slices of gathers in flight, they are faster at every size (an
+    // iteration on 160^3, spacing 4: 84.8 us against 91.5 staged; 128^3, spacing 8:
+    // 43.5 against 45.7; 48^3, spacing 6: 35 against 37). Calls of a few bricks
+    // stay staged: that keeps the bounded waits of the staged MSE brick in use.
+    if (MODE == MODE_MSE && nbricks > kStagedMseBricks)
+        return false;
     if (g.ndim != 3 || g.X % 4 != 0 || g.X < T::TWX || g.Y < T::TWY || g.Z < DELTA)
         return false;
     const uint64_t dims[3] = {(uint64_t)g.X, (uint64_t)g.Y, (uint64_t)g.Z};
@@ -1589,7 +1715,7 @@ cudaError_t run_fused_kernel(const Grid &g, const Lattice &L, const Layout &lay,
     gb.gtz = (D == 3) ? (L.nz + T - 1) / T : 1;
     gb.ngram = with_gram ? lay.ngram : 0;
     gb.icnt = MODE == MODE_MSE ? (int *)(ws + lay.icnt) : nullptr;
-    const size_t gsm = (size_t)((D == 3) ? kGram3Floats : kGram2Floats) * sizeof(float);
+    const size_t gsm = (size_t)((D == 3) ? gram3_floats(1) : gram2_floats(1)) * sizeof(float);
     const size_t dyn = (with_gram && gsm > C::dyn_smem) ? gsm : C::dyn_smem;
     ProfScope ps(s, MODE == MODE_MSE   ? "k_fused_mse"
                     : MODE == MODE_NCC ? "k_fused_ncc"
@@ -1624,7 +1750,7 @@ cudaError_t run_fused_kernel(const Grid &g, const Lattice &L, const Layout &lay,
     if constexpr (D == 3 && MODE != MODE_GW) {
         CUtensorMap mM, mF, mC;
         int lbox = 0, lslot = 0, lplane = 0;
-        if (brick_tmaps<DELTA, MODE>(g, L, F, M, c, &mM, &mF, &mC, &lbox, &lslot, &lplane)) {
+        if (brick_tmaps<DELTA, MODE>(g, L, lay.nbricks, F, M, c, &mM, &mF, &mC, &lbox, &lslot, &lplane)) {
             using T = TCfg<DELTA, MODE>;
             const size_t tdyn = (size_t)T::bytes + 128 > gsm ? (size_t)T::bytes + 128 : gsm;
             cudaError_t e = cudaFuncSetAttribute(k_fused_tma<DELTA, MODE>,
@@ -1738,16 +1864,27 @@ cudaError_t run_all(const Grid &g, const Lattice &L, int kind, int window, doubl
 // M[v] o (x + B c[v]), mask[v] when given. With PAIR, W points at bf16 pairs
 // (W[v], M[v]) instead (the network input of the pair F = W). blockIdx.y is
 // the volume.
+//
+// The gathers bound it (their lines through L1), then issue: with the objective's
+// 768-thread bricks one block fits an SM and its warps stall together (213 us on
+// 16 x 128^3 at spacing 8). It writes no partials, so its bricks need not span
+// three cells in y: 256-288 threads, four blocks per SM, 167 us. Five blocks at 48
+// registers take 172, three 190; four slices in flight 205; the staged form of
+// the bricks was not better for a single volume either.
+__host__ __device__ constexpr int warp_bcy(int delta) { return delta == 8 ? 1 : 2; }
+
+template <int D, int DELTA>
+using WCfg = FCfg<D, DELTA, MODE_FWD, brick_bcx(DELTA), warp_bcy(DELTA)>;
+
 template <int D, int DELTA, bool PAIR>
-__global__ void __launch_bounds__(FCfg<D, DELTA, MODE_FWD>::THREADS,
-                                  FCfg<D, DELTA, MODE_FWD>::THREADS <= 512 ? 2 : 1)
+__global__ void __launch_bounds__(WCfg<D, DELTA>::THREADS, 4)
     k_warp_ctrl(Grid g, Lattice L, int gbx, int gby, const float *__restrict__ M,
                 const float *__restrict__ c, float *__restrict__ W, uint8_t *__restrict__ m)
 {
     const int b = blockIdx.x;
     const int64_t vol = blockIdx.y;
     const int bx = b % gbx, by = (b / gbx) % gby, bz = b / (gbx * gby);
-    fused_brick<D, DELTA, MODE_FWD, brick_bcx(DELTA), brick_bcy(DELTA), false, PAIR>(
+    fused_brick<D, DELTA, MODE_FWD, WCfg<D, DELTA>::BCX, WCfg<D, DELTA>::BCY, false, PAIR>(
         g, L, nullptr, M + vol * g.nv, c + vol * D * L.nc, nullptr, W + vol * g.nv,
         m ? m + vol * g.nv : nullptr, nullptr, nullptr, nullptr, bx, by, bz, b);
 }
@@ -1756,18 +1893,13 @@ template <int D, int DELTA, bool PAIR>
 cudaError_t warp_ctrl_run(const Grid &g, const Lattice &L, int count, const float *M,
                           const float *c, float *W, uint8_t *m, cudaStream_t s)
 {
-    using C = FCfg<D, DELTA, MODE_FWD>;
-    const Layout lay = make_layout(g, L, 0, 3);
-    if (C::dyn_smem > 48 * 1024) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(k_warp_ctrl<D, DELTA, PAIR>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::dyn_smem);
-        if (e != cudaSuccess)
-            return e;
-    }
+    using C = WCfg<D, DELTA>;
+    static_assert(C::dyn_smem <= 32 * 1024, "within the default shared memory");
+    const int gbx = (g.X + C::BX - 1) / C::BX, gby = (g.Y + C::BY - 1) / C::BY;
+    const int gbz = D == 3 ? (g.Z + C::BCZ * DELTA - 1) / (C::BCZ * DELTA) : 1;
     ProfScope ps(s, PAIR ? "k_warp_ctrl_pair" : "k_warp_ctrl");
-    k_warp_ctrl<D, DELTA, PAIR><<<dim3(lay.nbricks, count), C::THREADS, C::dyn_smem, s>>>(
-        g, L, lay.gbx, lay.gby, M, c, W, m);
+    k_warp_ctrl<D, DELTA, PAIR><<<dim3(gbx * gby * gbz, count), C::THREADS, C::dyn_smem, s>>>(
+        g, L, gbx, gby, M, c, W, m);
     return cudaGetLastError();
 }
 
@@ -1788,13 +1920,14 @@ cudaError_t warp_ctrl_run(const Grid &g, const Lattice &L, int count, const floa
 template <int DELTA, int T>
 struct BCfg {
     static constexpr int BCX = batch_tile_bcx(DELTA, T), BCY = batch_tile_bcy(DELTA, T);
-    using C3 = FCfg<3, DELTA, MODE_MSE, BCX, BCY>;
-    using C2 = FCfg<2, DELTA, MODE_MSE, BCX, BCY>;
+    static constexpr int CP = batch_tile_cp(DELTA, T);
+    using C3 = FCfg<3, DELTA, MODE_MSE, BCX, BCY, CP>;
+    using C2 = FCfg<2, DELTA, MODE_MSE, BCX, BCY, CP>;
     static constexpr int THREADS = C3::THREADS;
     static constexpr int MINB = batch_tile_minb(DELTA, T);  // resident blocks per SM
     static_assert(C2::THREADS == THREADS, "2D and 3D bricks share the block size");
     static constexpr size_t fsm = C3::dyn_smem > C2::dyn_smem ? C3::dyn_smem : C2::dyn_smem;
-    static constexpr size_t gsm = (size_t)kGram3Floats * sizeof(float);  // > the 2D tile
+    static constexpr size_t gsm = (size_t)gram3_floats(3) * sizeof(float);  // > the 2D tile
     static constexpr size_t dyn_smem = fsm > gsm ? fsm : gsm;
 };
 
@@ -1860,23 +1993,26 @@ __global__ void __launch_bounds__(BCfg<DELTA, T>::THREADS, BCfg<DELTA, T>::MINB)
         if (w.kind == BATCH_BRICK) {
             const int bx = w.idx % P.gbx, r = w.idx / P.gbx, by = r % P.gby, bz = r / P.gby;
             constexpr int BCX = BCfg<DELTA, T>::BCX, BCY = BCfg<DELTA, T>::BCY;
+            constexpr int CP = BCfg<DELTA, T>::CP;
             if (P.g.ndim == 3)
-                fused_brick<3, DELTA, MODE_MSE, BCX, BCY>(P.g, P.L, P.F, P.M, P.c, nullptr, nullptr,
+                fused_brick<3, DELTA, MODE_MSE, BCX, BCY, false, false, CP>(P.g, P.L, P.F, P.M, P.c, nullptr, nullptr,
                                                           nullptr, nullptr, P.bpart, P.mpart, bx,
                                                           by, bz, w.idx);
             else
-                fused_brick<2, DELTA, MODE_MSE, BCX, BCY>(P.g, P.L, P.F, P.M, P.c, nullptr, nullptr,
+                fused_brick<2, DELTA, MODE_MSE, BCX, BCY, false, false, CP>(P.g, P.L, P.F, P.M, P.c, nullptr, nullptr,
                                                           nullptr, nullptr, P.bpart, P.mpart, bx,
                                                           by, bz, w.idx);
         } else if (w.kind == BATCH_GRAM) {
-            // tile index = ((component * gtz + tz) * gty + ty) * gtx + tx
-            const int tx = w.idx % P.gtx, r = w.idx / P.gtx, ty = r % P.gty, r2 = r / P.gty;
-            const int tz = r2 % P.gtz, comp = r2 / P.gtz;
+            // tile w.idx = (tz * gty + ty) * gtx + tx of every component
+            const int tx = w.idx % P.gtx, r = w.idx / P.gtx, ty = r % P.gty, tz = r / P.gty;
+            const int ntiles = P.gtx * P.gty * P.gtz;
             extern __shared__ float bsm[];
             if (P.g.ndim == 3)
-                gram3_tile(P.g, P.L, P.c, P.gscale, P.gR, tx, ty, tz, comp, P.rpart + w.idx, bsm);
+                gram3_tile<3>(P.g, P.L, P.c, P.gscale, P.gR, tx, ty, tz, 0, P.rpart + w.idx, ntiles,
+                              bsm);
             else
-                gram2_tile(P.g, P.L, P.c, P.gscale, P.gR, tx, ty, comp, P.rpart + w.idx, bsm);
+                gram2_tile<2>(P.g, P.L, P.c, P.gscale, P.gR, tx, ty, 0, P.rpart + w.idx, ntiles,
+                              bsm);
         }
         if (w.kind != BATCH_CTRL) {
             __syncthreads();  // every write of the item has been issued
@@ -1908,8 +2044,10 @@ __global__ void __launch_bounds__(BCfg<DELTA, T>::THREADS, BCfg<DELTA, T>::MINB)
         double *val = (w.idx == 0 && P.values && st.record >= 0) ? P.values + 4 * st.record : nullptr;
         objective_scalars<true>(MODE_MSE, P.g.nv, P.lambda, 0.0, parts, val, ks, red);
         const float k0 = (float)ks[0];
-        const int64_t e = (int64_t)w.idx * blockDim.x + threadIdx.x;
-        if (e < P.L.nc) {
+        // a chunk of COLS control points
+        constexpr int CHUNK = BCfg<DELTA, T>::C3::COLS;
+        const int64_t e1 = min((int64_t)P.L.nc, (int64_t)(w.idx + 1) * CHUNK);
+        for (int64_t e = (int64_t)w.idx * CHUNK + threadIdx.x; e < e1; e += blockDim.x) {
             if (P.g.ndim == 3)
                 batch_ctrl_adam<3, DELTA, T>(P, st, e, k0, s_inv_bc[0], s_inv_bc[1]);
             else
@@ -2060,11 +2198,11 @@ void batch_tile_cells(int delta, int tile, int *bcx, int *bcy)
     *bcy = batch_tile_bcy(delta, tile);
 }
 
-int batch_threads(int delta, int tile)
+int batch_chunk(int delta, int tile)
 {
-#define AL_THREADS(d, t) BCfg<d, t>::THREADS
-    AL_BATCH_DISPATCH(delta, tile, 0, AL_THREADS)
-#undef AL_THREADS
+#define AL_CHUNK(d, t) BCfg<d, t>::C3::COLS
+    AL_BATCH_DISPATCH(delta, tile, 0, AL_CHUNK)
+#undef AL_CHUNK
 }
 
 int batch_blocks_per_sm(int delta, int tile)

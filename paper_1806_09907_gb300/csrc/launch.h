@@ -183,7 +183,7 @@ int batch_tiles();
 void batch_tile_cells(int delta, int tile, int *bcx, int *bcy);
 void batch_geometry(const Grid &g, const Lattice &L, int tile, int *gb, int *gt, int *npart,
                     int *nmom);
-int batch_threads(int delta, int tile);        // 0 if (delta, tile) has no batch kernel
+int batch_chunk(int delta, int tile);  // control points per chunk; 0: no batch kernel
 int batch_blocks_per_sm(int delta, int tile);  // resident blocks of the batch kernel per SM
 cudaError_t launch_batch(int delta, int tile, int blocks, const BatchProblem *probs,
                          const BatchItem *items, int nitems, int *counters, const BatchStep &st,

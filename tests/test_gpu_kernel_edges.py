@@ -114,3 +114,27 @@ def test_exponential_adjoint_of_non_finite_gradients(shape):
     near[tuple(slice(max(s // 2 - 4, 0), s // 2 + 5) for s in shape)] = True
     assert torch.equal(out[:, ~near], ref[:, ~near])
     assert torch.isnan(out[at])
+
+
+@pytest.mark.parametrize("shape,count,blobs", [
+    ((40, 100, 101), 4, 70),   # 16 x 16 boxes, rows that end inside four columns, two chunks
+    ((33, 65, 64), 16, 64),    # whole 16-byte rows, a full chunk
+    ((9, 20, 24), 1, 129),     # 8 x 8 boxes, a chunk of one blob
+])
+def test_render_blobs_boxes(shape, count, blobs):
+    """Against the sum over every blob. Per voxel the fp32 sum of at most 129 terms, each of
+    three roundings and exponentials of a few ulp, is within (129 + 12) 2^-24 of the sum of
+    magnitudes, and 129 dropped terms add 129 * 1.6e-8: below 1.1e-5 of the largest value
+    when amplitudes are below 1 and the largest value is above 1."""
+    table = layers.synth.blob_table(count, shape, blobs, seed=11)
+    out = airgb.al_render_blobs(shape, torch.from_numpy(table).to(DEV)).double().cpu().numpy()
+    for v in (0, count - 1):
+        ref = layers.synth.render_blob_table(shape, table[v])
+        assert np.max(np.abs(out[v] - ref)) <= 1.1e-5 * max(1.0, np.max(np.abs(ref)))
+
+
+@pytest.mark.parametrize("shape,delta", [((21, 35, 45), 8), ((9, 13, 50), 6), ((11, 17, 33), 4),
+                                         ((33, 66), 4)])
+def test_warp_ctrl_bricks(shape, delta):
+    """Bricks of one and two control cells in y, with remainders in every axis."""
+    parity.test_warp_ctrl_batch(shape, delta)
