@@ -189,19 +189,24 @@ def status_string(status: int) -> str:
 
 # The device of the tensors of the call being marshalled: set by _ptr, read
 # by _stream (the default stream is that device's current stream) and by
-# _call, which runs the C call with that device current.
-_tls = threading.local()
+# _call, which runs the C call with that device current (switching to it
+# only when it is not: the switch and back cost more than a small launch).
+class _CallState(threading.local):
+    dev = None
+
+
+_tls = _CallState()
 
 
 def _call(name, *args):
-    dev = getattr(_tls, "dev", None)
+    dev = _tls.dev
     _tls.dev = None
     fn = getattr(load(), name)
-    if dev is not None:
+    if dev is None or dev.index == torch.cuda.current_device():
+        st = fn(*args)
+    else:
         with torch.cuda.device(dev):
             st = fn(*args)
-    else:
-        st = fn(*args)
     if st != 0:
         raise AirgbError(name, st)
 
@@ -249,26 +254,28 @@ def _ptr(t):
         raise ValueError("tensors must live on a CUDA device")
     if not t.is_contiguous():
         raise ValueError("tensors must be contiguous")
-    dev = getattr(_tls, "dev", None)
+    dev, here = _tls.dev, t.device
     if dev is None:
-        _tls.dev = t.device
-    elif dev != t.device:
+        _tls.dev = here
+    elif dev != here:
         _tls.dev = None
-        raise ValueError(f"the tensors of one call must share a device ({dev} and {t.device})")
-    return ctypes.c_void_p(t.data_ptr())
+        raise ValueError(f"the tensors of one call must share a device ({dev} and {here})")
+    return t.data_ptr()  # an argument of type void *: ctypes converts the integer
 
 
 def _f32(t, shape, what):
-    if t.dtype != torch.float32 or tuple(t.shape) != tuple(shape):
+    if t.dtype != torch.float32 or (t.shape != shape and tuple(t.shape) != tuple(shape)):
         raise ValueError(f"{what}: expected float32 {tuple(shape)}, got {t.dtype} {tuple(t.shape)}")
     return _ptr(t)
 
 
 def _stream(stream=None):
     if stream is None:
-        dev = getattr(_tls, "dev", None)
-        stream = torch.cuda.current_stream(dev) if dev is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        dev = _tls.dev
+        if dev is not None:  # the current stream's handle without a Stream object
+            return torch._C._cuda_getCurrentRawStream(dev.index)
+        stream = torch.cuda.current_stream()
+    return stream.cuda_stream
 
 
 def _workspace(nbytes, device, ws=None):
