@@ -36,6 +36,12 @@ size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 // is touched by at most two bricks per axis (k_ctrl relies on it).
 __host__ __device__ constexpr int brick_bcx(int delta) { return delta <= 4 ? 8 : 4; }
 __host__ __device__ constexpr int brick_bcy(int delta) { return delta <= 4 ? 4 : 3; }
+__host__ __device__ constexpr int warp_bcy(int delta) { return delta == 8 ? 1 : 2; }
+// cells in y of a mode's brick
+__host__ __device__ constexpr int mode_bcy(int mode, int delta)
+{
+    return mode == MODE_FWD ? warp_bcy(delta) : brick_bcy(delta);
+}
 __host__ __device__ constexpr int brick_bcz(int ndim) { return ndim == 3 ? 4 : 1; }
 
 // Brick tiles the batch kernel is built for, per spacing: control cells per
@@ -73,8 +79,8 @@ __host__ __device__ constexpr int batch_tile_minb(int delta, int t)
     return batch_tile_cp(delta, t) == 2 ? 2 : delta == 8 || t == 1 ? 1 : 2;
 }
 
-template <int D, int DELTA, int MODE, int BCX_ = brick_bcx(DELTA), int BCY_ = brick_bcy(DELTA),
-          int CP_ = 1>
+template <int D, int DELTA, int MODE, int BCX_ = brick_bcx(DELTA),
+          int BCY_ = mode_bcy(MODE, DELTA), int CP_ = 1>
 struct FCfg {
     static constexpr int BCX = BCX_, BCY = BCY_, BCZ = brick_bcz(D);
     static constexpr int BX = BCX * DELTA, BY = BCY * DELTA;
@@ -106,7 +112,7 @@ struct FCfg {
     static constexpr size_t dyn_smem = (size_t)(nP + nX + nR) * sizeof(float);
 };
 
-// Shared-memory staging of a 3D brick by TMA (single-problem path, X a
+// Shared-memory staging of a 3D brick of MSE or NCC by TMA (single-problem path, X a
 // multiple of 4 so that image rows can be tensor-map rows):
 // * the moving image: one box of (BX + 2 HX) x (BY + 2 HY) voxels per slice,
 //   from (x0 - HX, y0 - HY), in a ring of NSLOT slices. While layer l (its
@@ -115,7 +121,7 @@ struct FCfg {
 //   layer adds are in flight. A sample whose trilinear cell lies inside that
 //   window reads its 8 corners from shared memory, any other from global
 //   memory (|u| <= HZ voxels keeps every sample inside);
-// * the fixed image (MSE, NCC): one box of BX x BY x DELTA voxels per layer,
+// * the fixed image: one box of BX x BY x DELTA voxels per layer,
 //   two layers buffered;
 // * the control lattice: c's rows (nx floats) are not tensor-map rows, so it
 //   is copied through a one-dimensional view: one box per lattice plane of
@@ -138,19 +144,19 @@ struct TCfg {
     static constexpr int SLOTB = TWX * TWY * 4;
     static constexpr int NRES = DELTA + 2 * HZ;  // slices resident while a layer is computed
     static constexpr int NSLOT = NRES + DELTA;   // + the next layer's new slices
-    static constexpr int NF = (MODE == MODE_FWD) ? 0 : 2;
+    static constexpr int NF = 2;  // layers of the fixed image
     static constexpr int FSLOTB = BX * BY * DELTA * 4;
     static constexpr int NROW = 3 * C::JZ * C::JY;  // lattice rows
     static constexpr int LBOX = 16;                  // floats per row copy (offset <= 3, JX <= 11)
     static constexpr int NPLN = 3 * C::JZ;           // lattice planes (one box each, <= 1 KB)
     static constexpr int LSTAGE = NROW * 128 > NPLN * 1024 ? NROW * 128 : NPLN * 1024;
-    static constexpr int nP1 = (MODE == MODE_FWD) ? 0 : BY * BX * C::CHS;   // one-plane flush
-    static constexpr int nX1 = (MODE == MODE_FWD) ? 0 : BY * C::BCX * 4 * C::CHS;
+    static constexpr int nP1 = BY * BX * C::CHS;  // one-plane flush
+    static constexpr int nX1 = BY * C::BCX * 4 * C::CHS;
     static constexpr int oRing = 0;
     static constexpr int oF = oRing + NSLOT * SLOTB;
     static constexpr int oU = oF + NF * FSLOTB;  // lattice rows, later the flush buffers
     static constexpr int oR = (nP1 + nX1) * 4;  // row contractions, inside the union
-    static constexpr int nR = (MODE == MODE_GW) ? 0 : 4 * C::RPL;
+    static constexpr int nR = 4 * C::RPL;
     static constexpr int nU = (LSTAGE > oR + nR * 4) ? LSTAGE : oR + nR * 4;
     static constexpr int oBar = oU + round128(nU);
     static constexpr int bytes = oBar + 3 * 8;
@@ -170,10 +176,10 @@ struct BrickMaps {
 
 // Host choice of the lattice copies of a brick (plane boxes when a plane's
 // rows fit one box of at most 256 floats).
-template <int DELTA>
+template <int DELTA, int MODE>
 void lattice_boxes(const Lattice &L, int *lbox, int *lslot, int *lplane)
 {
-    using C = FCfg<3, DELTA, MODE_FWD>;
+    using C = FCfg<3, DELTA, MODE>;
     const int span = (C::JY - 1) * L.nx + C::JX + 3;  // offset <= 3
     if (span <= 256) {
         *lbox = (span + 3) / 4 * 4;
@@ -220,7 +226,7 @@ __device__ __forceinline__ void mbar_expect(uint32_t bar, uint32_t bytes)
 }
 
 // Batch b of a brick's copies (issued by one thread): the moving-image
-// slices it adds to the ring and, for MSE/NCC, the fixed-image layer b.
+// slices it adds to the ring and the fixed-image layer b.
 template <int DELTA, int MODE>
 __device__ __forceinline__ void brick_issue(const BrickMaps &tm, uint32_t sbase, int b, int x0,
                                             int y0, int z0)
@@ -230,14 +236,13 @@ __device__ __forceinline__ void brick_issue(const BrickMaps &tm, uint32_t sbase,
         return;
     const uint32_t bar = sbase + T::oBar + 8 * (b & 1);
     const int r0 = b == 0 ? 0 : T::NRES + (b - 1) * DELTA, r1 = T::NRES + b * DELTA;
-    mbar_expect(bar, (uint32_t)((r1 - r0) * T::SLOTB + (T::NF > 0 ? T::FSLOTB : 0)));
+    mbar_expect(bar, (uint32_t)((r1 - r0) * T::SLOTB + T::FSLOTB));
     for (int r = r0; r < r1; ++r) {
         const int slot = r % T::NSLOT;
         tma_load_3d(sbase + T::oRing + slot * T::SLOTB, tm.M, x0 - T::HX, y0 - T::HY,
                     z0 - T::HZ + r, bar);
     }
-    if constexpr (T::NF > 0)
-        tma_load_3d(sbase + T::oF + (b & 1) * T::FSLOTB, tm.F, x0, y0, z0 + b * DELTA, bar);
+    tma_load_3d(sbase + T::oF + (b & 1) * T::FSLOTB, tm.F, x0, y0, z0 + b * DELTA, bar);
 }
 
 // Staging of the projection pass (GW) by TMA: per layer one box of dS/dW
@@ -417,13 +422,13 @@ __device__ __forceinline__ void flush_planes(int lp0, float *A, float *B, float 
 // brick, its partial sums written to bpart / mpart at index `brick`. Every
 // thread of a block of FCfg::THREADS threads calls it; it uses the block's
 // shared memory (static arrays here and FCfg::dyn_smem of dynamic memory,
-// or TCfg::bytes + 128 with TMA). With TMA (3D, MSE/NCC/FWD) the lattice
+// or TCfg::bytes + 128 with TMA). With TMA (3D, MSE/NCC) the lattice
 // block, the moving-image neighbourhood and the fixed image arrive by
 // tensor-map copies (TCfg); the arithmetic is the same either way, so both
 // give the same bits. Returns false if a copy did not land in time (the
 // brick's partials are then not written).
-template <int D, int DELTA, int MODE, int BCX_ = brick_bcx(DELTA), int BCY_ = brick_bcy(DELTA),
-          bool TMA = false, bool PAIR = false, int CP = 1>
+template <int D, int DELTA, int MODE, int BCX_ = brick_bcx(DELTA),
+          int BCY_ = mode_bcy(MODE, DELTA), bool TMA = false, bool PAIR = false, int CP = 1>
 __device__ __forceinline__ bool fused_brick(const Grid &g, const Lattice &L,
                                             const float *__restrict__ F,
                                             const float *__restrict__ M,
@@ -440,9 +445,10 @@ __device__ __forceinline__ bool fused_brick(const Grid &g, const Lattice &L,
     // W_out then pointing at them. MODE_GW reads dS/dW and those planes back
     // (no expansion, no gathers).
     using C = FCfg<D, DELTA, MODE, BCX_, BCY_, CP>;
-    using T = TCfg<DELTA, MODE == MODE_GW ? MODE_FWD : MODE>;
+    using T = TCfg<DELTA, MODE == MODE_NCC ? MODE_NCC : MODE_MSE>;
     using GS = GCfg<DELTA>;
-    static_assert(!TMA || (D == 3 && CP == 1 && BCX_ == brick_bcx(DELTA) && BCY_ == brick_bcy(DELTA)),
+    static_assert(!TMA || (D == 3 && CP == 1 && BCX_ == brick_bcx(DELTA) &&
+                           BCY_ == mode_bcy(MODE, DELTA)),
                   "TMA staging: 3D single-problem bricks");
     constexpr int JX = C::JX, JY = C::JY, JZ = C::JZ, CHS = C::CHS, BX = C::BX;
     constexpr WTab<DELTA> kW{};  // weights of the compile-time z phases
@@ -1587,10 +1593,19 @@ struct GramBlocks {
 };
 
 
+// Resident blocks per SM the kernels are compiled for. The forward pass (FWD)
+// writes no partials, so its bricks are of one or two cells in y, 256-288 threads,
+// four blocks per SM, and gather: 256 x 256 x 160 and 7^3 windows, one evaluation at
+// spacing 4 / 6 / 8 458 / 422 / 394 us with the projection's bricks staged by TMA,
+// 430 / 419 / 389 so; a 128 x 128 x 80 iteration 91 -> 89. Small bricks staged by TMA
+// took 444 / 433 / 390 us, three blocks 444 / 425 / 392.
+constexpr int fused_minb(int mode, int threads)
+{
+    return mode == MODE_FWD ? 4 : threads <= 512 && mode != MODE_NCC ? 2 : 1;
+}
+
 template <int D, int DELTA, int MODE>
-__global__ void __launch_bounds__(FCfg<D, DELTA, MODE>::THREADS,
-                                  (FCfg<D, DELTA, MODE>::THREADS <= 512 && MODE != MODE_NCC) ? 2
-                                                                                            : 1)
+__global__ void __launch_bounds__(FCfg<D, DELTA, MODE>::THREADS, fused_minb(MODE, FCfg<D, DELTA, MODE>::THREADS))
     k_fused(Grid g, Lattice L, const float *__restrict__ F, const float *__restrict__ M,
             const float *__restrict__ c, const float *__restrict__ gw_in,
             float *__restrict__ W_out, uint8_t *__restrict__ m_out, float *__restrict__ G_io,
@@ -1622,11 +1637,9 @@ __global__ void __launch_bounds__(FCfg<D, DELTA, MODE>::THREADS,
         gram2_tile<1>(g, L, c, gb.gscale, gb.gR, tx, ty, comp, gb.rpart + w, 0, gtile_sm);
 }
 
-// k_fused for 3D bricks staged by TMA (MSE, NCC, FWD; X a multiple of 4).
+// k_fused for 3D bricks staged by TMA (MSE, NCC, GW; X a multiple of 4).
 template <int DELTA, int MODE>
-__global__ void __launch_bounds__(FCfg<3, DELTA, MODE>::THREADS,
-                                  (FCfg<3, DELTA, MODE>::THREADS <= 512 && MODE != MODE_NCC) ? 2
-                                                                                             : 1)
+__global__ void __launch_bounds__(FCfg<3, DELTA, MODE>::THREADS, fused_minb(MODE, FCfg<3, DELTA, MODE>::THREADS))
     k_fused_tma(const __grid_constant__ CUtensorMap mapM, const __grid_constant__ CUtensorMap mapF,
                 const __grid_constant__ CUtensorMap mapC, int3 lb, Grid g, Lattice L,
                 const float *__restrict__ F, const float *__restrict__ M,
@@ -1645,7 +1658,7 @@ __global__ void __launch_bounds__(FCfg<3, DELTA, MODE>::THREADS,
     const int b = blockIdx.x - sb.on;
     if (b < gb.nbricks) {
         const int bx = b % gb.gbx, by = (b / gb.gbx) % gb.gby, bz = b / (gb.gbx * gb.gby);
-        fused_brick<3, DELTA, MODE, brick_bcx(DELTA), brick_bcy(DELTA), true>(
+        fused_brick<3, DELTA, MODE, brick_bcx(DELTA), mode_bcy(MODE, DELTA), true>(
             g, L, F, M, c, nullptr, W_out, m_out, G_io, bpart, mpart, bx, by, bz, b,
             BrickMaps{&mapM, &mapF, &mapC, lb.x, lb.y, lb.z}, gb.icnt);
         return;
@@ -1684,13 +1697,13 @@ bool brick_tmaps(const Grid &g, const Lattice &L, int nbricks, const float *F, c
     const uint64_t strides[2] = {(uint64_t)g.X * 4, (uint64_t)g.X * g.Y * 4};
     const uint32_t boxM[3] = {(uint32_t)T::TWX, (uint32_t)T::TWY, 1u};
     const uint32_t boxF[3] = {(uint32_t)T::BX, (uint32_t)T::BY, (uint32_t)DELTA};
-    lattice_boxes<DELTA>(L, lbox, lslot, lplane);
+    lattice_boxes<DELTA, MODE>(L, lbox, lslot, lplane);
     const uint64_t dimC[1] = {(uint64_t)3 * L.nc};
     const uint32_t boxC[1] = {(uint32_t)*lbox};
     if (!encode_tmap_f32(mM, 3, dims, strides, boxM, M) ||
         !encode_tmap_f32(mC, 1, dimC, nullptr, boxC, c))
         return false;
-    if (T::NF > 0 && !encode_tmap_f32(mF, 3, dims, strides, boxF, F))
+    if (!encode_tmap_f32(mF, 3, dims, strides, boxF, F))
         return false;
     return true;
 }
@@ -1706,9 +1719,9 @@ cudaError_t run_fused_kernel(const Grid &g, const Lattice &L, const Layout &lay,
     gb.gR = (float *)(ws + lay.gR);
     gb.rpart = (double *)(ws + lay.rpart);
     gb.gscale = (float)(2.0 / (double)g.nv);
-    gb.gbx = lay.gbx;
-    gb.gby = lay.gby;
-    gb.nbricks = lay.nbricks;
+    gb.gbx = MODE == MODE_FWD ? (g.X + C::BX - 1) / C::BX : lay.gbx;
+    gb.gby = MODE == MODE_FWD ? (g.Y + C::BY - 1) / C::BY : lay.gby;
+    gb.nbricks = MODE == MODE_FWD ? gb.gbx * gb.gby * lay.gbz : lay.nbricks;
     const int T = (D == 3) ? kGramT3 : kGramT2;
     gb.gtx = (L.nx + T - 1) / T;
     gb.gty = (L.ny + T - 1) / T;
@@ -1741,16 +1754,16 @@ cudaError_t run_fused_kernel(const Grid &g, const Lattice &L, const Layout &lay,
                                                  (int)tdyn);
             if (e != cudaSuccess)
                 return e;
-            k_fused_tma<DELTA, MODE><<<sb.on + lay.nbricks, C::THREADS, tdyn, s>>>(
+            k_fused_tma<DELTA, MODE><<<sb.on + gb.nbricks, C::THREADS, tdyn, s>>>(
                 mW, mG, mC, int3{0, 0, 0}, g, L, F, M, c, Wo, mo, G, (float *)(ws + lay.bpart),
                 (double *)(ws + lay.mpart), gb, sb);
             return cudaGetLastError();
         }
     }
-    if constexpr (D == 3 && MODE != MODE_GW) {
+    if constexpr (D == 3 && (MODE == MODE_MSE || MODE == MODE_NCC)) {
         CUtensorMap mM, mF, mC;
         int lbox = 0, lslot = 0, lplane = 0;
-        if (brick_tmaps<DELTA, MODE>(g, L, lay.nbricks, F, M, c, &mM, &mF, &mC, &lbox, &lslot, &lplane)) {
+        if (brick_tmaps<DELTA, MODE>(g, L, gb.nbricks, F, M, c, &mM, &mF, &mC, &lbox, &lslot, &lplane)) {
             using T = TCfg<DELTA, MODE>;
             const size_t tdyn = (size_t)T::bytes + 128 > gsm ? (size_t)T::bytes + 128 : gsm;
             cudaError_t e = cudaFuncSetAttribute(k_fused_tma<DELTA, MODE>,
@@ -1758,7 +1771,7 @@ cudaError_t run_fused_kernel(const Grid &g, const Lattice &L, const Layout &lay,
                                                  (int)tdyn);
             if (e != cudaSuccess)
                 return e;
-            k_fused_tma<DELTA, MODE><<<sb.on + lay.nbricks + gb.ngram, C::THREADS, tdyn, s>>>(
+            k_fused_tma<DELTA, MODE><<<sb.on + gb.nbricks + gb.ngram, C::THREADS, tdyn, s>>>(
                 mM, mF, mC, int3{lbox, lslot, lplane}, g, L, F, M, c, Wo, mo, G,
                 (float *)(ws + lay.bpart), (double *)(ws + lay.mpart), gb, sb);
             return cudaGetLastError();
@@ -1772,7 +1785,7 @@ cudaError_t run_fused_kernel(const Grid &g, const Lattice &L, const Layout &lay,
         if (e != cudaSuccess)
             return e;
     }
-    k_fused<D, DELTA, MODE><<<sb.on + lay.nbricks + gb.ngram, C::THREADS, dyn, s>>>(
+    k_fused<D, DELTA, MODE><<<sb.on + gb.nbricks + gb.ngram, C::THREADS, dyn, s>>>(
         g, L, F, M, c, gw, Wo, mo, G, (float *)(ws + lay.bpart), (double *)(ws + lay.mpart),
         gb, sb);
     return cudaGetLastError();
@@ -1871,10 +1884,9 @@ cudaError_t run_all(const Grid &g, const Lattice &L, int kind, int window, doubl
 // three cells in y: 256-288 threads, four blocks per SM, 167 us. Five blocks at 48
 // registers take 172, three 190; four slices in flight 205; the staged form of
 // the bricks was not better for a single volume either.
-__host__ __device__ constexpr int warp_bcy(int delta) { return delta == 8 ? 1 : 2; }
 
 template <int D, int DELTA>
-using WCfg = FCfg<D, DELTA, MODE_FWD, brick_bcx(DELTA), warp_bcy(DELTA)>;
+using WCfg = FCfg<D, DELTA, MODE_FWD>;
 
 template <int D, int DELTA, bool PAIR>
 __global__ void __launch_bounds__(WCfg<D, DELTA>::THREADS, 4)
