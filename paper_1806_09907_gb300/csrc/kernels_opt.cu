@@ -32,33 +32,42 @@ int blocks_for(int64_t n, int threads)
 //   c <- c - h lr (m / bc1) / (sqrt(v / bc2) + eps),  bc = 1 - b^t.
 // t = *step + 1 is read from the device counter; k_adam_tick stores it
 // afterwards, so a captured graph replays successive steps.
+// A small launch is one chain of latencies: the two bias corrections are formed
+// by a warp each while the block's operands are on their way (128^3 at spacing 8,
+// 81 blocks: 5.9 us with the corrections one after the other before the loads,
+// 4.2 so).
 __global__ void __launch_bounds__(kOptThreads)
     k_adam(AdamArgs a, const int64_t *__restrict__ step, float *__restrict__ ctrl,
            const float *__restrict__ grad, float *__restrict__ m, float *__restrict__ v)
 {
     __shared__ float s_inv_bc[2];
-    if (threadIdx.x == 0) {
-        const long long t = (long long)*step + 1;
-        s_inv_bc[0] = adam_inv_bias(a.beta1, t);
-        s_inv_bc[1] = adam_inv_bias(a.beta2, t);
+    const int64_t n = (int64_t)a.ndim * a.nc;
+    const int64_t e = blockIdx.x * (int64_t)kOptThreads + threadIdx.x;  // one element a thread
+    const bool on = e < n;
+    float ge = 0.0f, me = 0.0f, ve = 0.0f, ce = 0.0f;
+    if (on) {
+        ge = grad[e];
+        me = m[e];
+        ve = v[e];
+        ce = ctrl[e];
     }
+    if (threadIdx.x % 32 == 0 && threadIdx.x < 64)
+        s_inv_bc[threadIdx.x / 32] =
+            adam_inv_bias(threadIdx.x == 0 ? a.beta1 : a.beta2, (long long)*step + 1);
     __syncthreads();
+    if (!on)
+        return;
     const float inv_bc1 = s_inv_bc[0], inv_bc2 = s_inv_bc[1];
     const float b1 = (float)a.beta1, b2 = (float)a.beta2;
     const float omb1 = (float)(1.0 - a.beta1), omb2 = (float)(1.0 - a.beta2);
-    const int64_t n = (int64_t)a.ndim * a.nc;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(e / a.nc);
-        const float h = a.h[i];
-        const float gn = grad[e] * h;
-        const float mm = fmaf(b1, m[e], omb1 * gn);
-        const float vv = fmaf(b2, v[e], omb2 * gn * gn);
-        m[e] = mm;
-        v[e] = vv;
-        const float den = sqrtf(vv * inv_bc2) + a.eps;
-        ctrl[e] -= (a.lr * h) * ((mm * inv_bc1) / den);
-    }
+    const float h = a.h[(e >= a.nc) + (e >= 2 * a.nc)];
+    const float gn = ge * h;
+    const float mm = fmaf(b1, me, omb1 * gn);
+    const float vv = fmaf(b2, ve, omb2 * gn * gn);
+    m[e] = mm;
+    v[e] = vv;
+    const float den = sqrtf(vv * inv_bc2) + a.eps;
+    ctrl[e] = ce - (a.lr * h) * ((mm * inv_bc1) / den);
 }
 
 __global__ void k_adam_tick(int64_t *step)

@@ -91,7 +91,8 @@ class ObjectiveFunction(torch.autograd.Function):
         else:
             grad = saved
         # chain rule with the upstream scalar (1 for loss.backward())
-        return grad * grad_out.to(grad.dtype), None, None, None, None
+        # in grad's type: one kernel casts the 0-d upstream value as it multiplies
+        return grad * grad_out, None, None, None, None
 
 
 def objective(ctrl, evaluator: Evaluator, fixed, moving, recompute=False):
