@@ -350,7 +350,8 @@ void al_batch_destroy(al_batch *batch);
  * every problem's partial sums. */
 size_t al_batch_workspace_bytes(const al_batch *batch);
 /* Number of work items of one iteration; per_kind (nullable, 3 entries)
- * receives the bricks, Gram tiles and control chunks among them. */
+ * receives the bricks, Gram tiles (per component; those of one tile share a
+ * queue entry) and control chunks among them. */
 int32_t al_batch_items(const al_batch *batch, int32_t *per_kind);
 
 /* Attach the problems' device arrays (host arrays of `count` device
