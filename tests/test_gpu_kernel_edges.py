@@ -138,3 +138,28 @@ def test_render_blobs_boxes(shape, count, blobs):
 def test_warp_ctrl_bricks(shape, delta):
     """Bricks of one and two control cells in y, with remainders in every axis."""
     parity.test_warp_ctrl_batch(shape, delta)
+
+
+@pytest.mark.parametrize("shape,delta", [((9, 21, 35), 4), ((14, 20, 26), 6), ((18, 17, 33), 8),
+                                         ((40, 37), 8)])
+def test_brick_cells_at_faces_and_beyond(shape, delta):
+    """A zero displacement puts every sample on its voxel, the last faces included: the warp is
+    the image bit for bit and the mask full. Displacements far outside, at the limits of the
+    cell's integer arithmetic and not finite leave the mask empty and the warp zero."""
+    d, lat = len(shape), airgb.lattice_shape(shape, delta)
+    M = torch.rand((1,) + shape, device=DEV) + 1.0
+    mask = torch.empty((1,) + shape, dtype=torch.uint8, device=DEV)
+    c = torch.zeros((1, d) + lat, device=DEV)
+    W = airgb.al_warp_ctrl(shape, delta, M, c, mask=mask)
+    assert torch.equal(W, M) and bool(mask.all())
+    ob = airgb.Objective(shape, delta, "mse")
+    assert float(ob(M[0], M[0], c[0])[0][3]) == M[0].numel()
+    inf = float("inf")
+    for axis in range(d):
+        for v in (inf, -inf, float("nan"), 1e3, -1e3, 2.0 ** 22, -2.0 ** 22, 2.0 ** 23,
+                  -2.0 ** 24, 1e9, -3e9, 3e38, -3e38):
+            c.zero_()
+            c[0, axis] = v
+            W = airgb.al_warp_ctrl(shape, delta, M, c, mask=mask)
+            assert not bool(mask.any()) and not bool(W.any()), (axis, v)
+            assert float(ob(M[0], M[0], c[0])[0][3]) == 0.0, (axis, v)
