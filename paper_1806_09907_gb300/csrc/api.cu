@@ -45,7 +45,7 @@ al_status check_grid(const al_grid *g, Grid *out)
         out->X = (int)g->size[0];
         out->Y = (int)g->size[1];
         out->Z = (int)g->size[2];
-        out->nv = (int)nv;
+        out->nv = nv;
     }
     return AL_OK;
 }
@@ -73,7 +73,7 @@ al_status check_bspline(const al_bspline *bs, Grid *g, Lattice *L)
         L->nx = (int)n[0];
         L->ny = (int)n[1];
         L->nz = (int)n[2];
-        L->nc = (int)(n[0] * n[1] * n[2]);
+        L->nc = n[0] * n[1] * n[2];
         memset(L->w, 0, sizeof(L->w));
         for (int p = 0; p < bs->spacing; ++p)
             for (int a = 0; a < 4; ++a)

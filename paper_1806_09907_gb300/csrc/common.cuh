@@ -55,7 +55,7 @@ __device__ __forceinline__ bool al_index_ok(int64_t i, int64_t n)
 struct Grid {
     int ndim;
     int X, Y, Z;
-    int nv;
+    int64_t nv;  // below 2^31; 64 bits, so that offsets of the planes after the first are too
 };
 
 // Control lattice of the cubic B-spline transformation (Sec. III-C):
@@ -65,7 +65,7 @@ struct Grid {
 struct Lattice {
     int delta;
     int nx, ny, nz;
-    int nc;  // nx*ny*nz
+    int64_t nc;  // nx*ny*nz (above 2^31 for a thin volume at spacing 1)
     float w[kMaxDelta][4];
 };
 

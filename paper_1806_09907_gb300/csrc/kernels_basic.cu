@@ -37,10 +37,10 @@ __global__ void __launch_bounds__(kDispTX)
     const int rows = min(kDispTY, g.Y - y0);
     const int qz = z / delta, pz = z - qz * delta, py0 = y0 - jy0 * delta;
     const float z0 = L.w[pz][0], z1 = L.w[pz][1], z2 = L.w[pz][2], z3 = L.w[pz][3];
-    const int nxy = L.nx * L.ny;
+    const int64_t nxy = (int64_t)L.nx * L.ny;
     for (int col = threadIdx.x; col < D * njx; col += kDispTX) {
         const int i = D == 3 ? (col >= njx) + (col >= 2 * njx) : (col >= njx);
-        const float *src = c + (int64_t)i * L.nc + (D == 3 ? qz * nxy : 0) + jy0 * L.nx + jx0 +
+        const float *src = c + i * L.nc + (D == 3 ? qz * nxy : 0) + (int64_t)jy0 * L.nx + jx0 +
                            (col - i * njx);
         auto point = [&](int jy) {
             const float *p = src + jy * L.nx;
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(kTileX *kTileY)
     if (!c.on)
         return;
     const int sz = g.X * g.Y;
-    int v = (c.z0 * g.Y + c.y) * g.X + c.x;
+    unsigned v = (unsigned)((c.z0 * g.Y + c.y) * g.X + c.x);  // wraps after the last slice only
 #pragma unroll 2
     for (int z = c.z0; z < c.z1; ++z, v += sz) {
         Interp ip;
@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(kTileX *kTileY)
     if (!c.on)
         return;
     const int sz = g.X * g.Y;
-    int v = (c.z0 * g.Y + c.y) * g.X + c.x;
+    unsigned v = (unsigned)((c.z0 * g.Y + c.y) * g.X + c.x);  // wraps after the last slice only
     for (int z = c.z0; z < c.z1; ++z, v += sz) {
         float gx = 0.0f, gy = 0.0f, gz = 0.0f;
         const float gwv = __ldg(gw + v);
@@ -358,12 +358,12 @@ __global__ void __launch_bounds__(kTileX *kTileY)
             gu[v] += gx;
             gu[g.nv + v] += gy;
             if (D == 3)
-                gu[2 * (int64_t)g.nv + v] += gz;
+                gu[2 * g.nv + v] += gz;
         } else {
             gu[v] = gx;
             gu[g.nv + v] = gy;
             if (D == 3)
-                gu[2 * (int64_t)g.nv + v] = gz;
+                gu[2 * g.nv + v] = gz;
         }
     }
 }
@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(kTileX *kTileY, 5)
         const Column c = march_column(g, mp, tile);
         if (!c.on)
             continue;
-        int v = (c.z0 * g.Y + c.y) * g.X + c.x;
+        unsigned v = (unsigned)((c.z0 * g.Y + c.y) * g.X + c.x);
         float below[D], cur[D];
 #pragma unroll
         for (int i = 0; i < D; ++i) {
@@ -576,7 +576,7 @@ cudaError_t launch_displacement_adjoint(const Grid &g, const Lattice &L, const f
         grad_disp, D == 3 ? t2 : grad_ctrl, g.X, g.Y, t.jt, t.bj, t.nxt, t.nbands, L);
     if (D == 3) {
         // z: (D, Z, ny*nx) -> (D, nz, ny*nx)
-        const int64_t n3 = (int64_t)D * L.nc;
+        const int64_t n3 = D * L.nc;
         k_transpose_z<<<elementwise_grid(n3, kTransThreads), kTransThreads, 0, s>>>(
             t2, grad_ctrl, D, g.Z, L.nz, L.ny * L.nx, L);
     }

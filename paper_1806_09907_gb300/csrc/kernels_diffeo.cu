@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(kDiffeoThreads, 4)
     const int z1 = min((tz + 1) * zc, g.Z);
     const float *u1 = u + g.nv, *u2 = u1 + g.nv;
     float *o1 = out + g.nv, *o2 = o1 + g.nv;
-    int v = (tz * zc * g.Y + y) * g.X + x;
+    unsigned v = (unsigned)((tz * zc * g.Y + y) * g.X + x);
     for (int z = tz * zc; z < z1; ++z, v += sz) {
         const float a0 = __ldg(u + v) * sc, a1 = __ldg(u1 + v) * sc, a2 = __ldg(u2 + v) * sc;
         int cx, cy, cz;
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kDiffeoThreads, 4)
         if (SCALED && u0) {
             u0[v] = a0;
             u0[g.nv + v] = a1;
-            u0[2 * (int64_t)g.nv + v] = a2;
+            u0[2 * g.nv + v] = a2;
         }
         out[v] = a0 + r0;
         o1[v] = a1 + r1;
@@ -430,7 +430,7 @@ __global__ void __launch_bounds__(kDiffeoThreads, 3)
     const float *u1 = u + g.nv, *u2 = u1 + g.nv;
     const float *g1 = gin + g.nv, *g2 = g1 + g.nv;
     float *h1 = h + g.nv, *h2 = h1 + g.nv;
-    int v = (tz * zc * g.Y + y) * g.X + x;
+    unsigned v = (unsigned)((tz * zc * g.Y + y) * g.X + x);
     // contributions to the corners (y, x) at the far z of the last sample's cell
     Fix carry[3][4] = {};
     int cb = -1;  // their first node

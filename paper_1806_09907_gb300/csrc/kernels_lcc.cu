@@ -108,7 +108,7 @@ struct LccT {
 };
 
 // Distance in floats between the planes a', b, c of the LCC coefficients.
-__host__ __device__ inline int64_t lcc_plane(int nv) { return ((int64_t)nv * 4 + 255) / 256 * 64; }
+__host__ __device__ inline int64_t lcc_plane(int64_t nv) { return (nv * 4 + 255) / 256 * 64; }
 
 // ---- bounded waits, TMA helpers ---------------------------------------------
 constexpr int kErrTimeout = 6;  // AL_ERR_TIMEOUT

@@ -118,7 +118,7 @@ struct AdamArgs {
     double beta1, beta2;  // bias corrections are formed from these in double
     float lr, eps;
     float h[3];  // voxel units per normalised unit, (N_k - 1)/2, per component
-    int nc;      // coefficients per component plane
+    int64_t nc;  // coefficients per component plane
     int ndim;
 };
 cudaError_t launch_adam(const AdamArgs &a, int64_t *step, float *ctrl, const float *grad,
