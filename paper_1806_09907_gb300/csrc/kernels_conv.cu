@@ -262,33 +262,6 @@ __device__ __forceinline__ void tc_load16(uint32_t taddr, float (&v)[16])
         v[i] = __uint_as_float(r[i]);
 }
 
-// The same without waiting: the values are good after tc_load_wait, which takes
-// them so that no use can be moved before it.
-__device__ __forceinline__ void tc_load16_async(uint32_t taddr, uint32_t (&r)[16])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
-        "%11, %12, %13, %14, %15}, [%16];\n"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-          "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-}
-
-__device__ __forceinline__ void tc_load_wait(uint32_t (&r)[16], uint32_t (&q)[16])
-{
-    asm volatile("tcgen05.wait::ld.sync.aligned;\n"
-                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]),
-                   "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]),
-                   "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(q[0]), "+r"(q[1]),
-                   "+r"(q[2]), "+r"(q[3]), "+r"(q[4]), "+r"(q[5]), "+r"(q[6]), "+r"(q[7]),
-                   "+r"(q[8]), "+r"(q[9]), "+r"(q[10]), "+r"(q[11]), "+r"(q[12]), "+r"(q[13]),
-                   "+r"(q[14]), "+r"(q[15])
-                 :
-                 : "memory");
-}
-
 // Shared-memory matrix descriptor, no swizzle: start address, the byte
 // distance between core matrices along K (leading) and along M/N (stride),
 // descriptor version 1 (bits 46-47) of sm_100-class tensor cores.
@@ -1754,54 +1727,48 @@ __global__ void __launch_bounds__(slab_threads(KIND), 1) k_conv_slab(const ConvA
             } else {
                 int b, qz, y0;
                 decode(u, b, qz, y0);
-                // G chunks of 16 columns at a time (this warp's are PARTS apart); the ReLU
-                // factors of the next G are loaded before the sums of these are read
+                // 16 columns at a time (this warp's chunks are PARTS apart); the ReLU factors
+                // of the next chunk are loaded before the sums of this one are read
                 constexpr bool BWD = KIND == DGRAD1 || KIND == DGRAD2;
-                constexpr int G = 1;
-                const int per_tile = (s.accs - 16 * half + 16 * PARTS - 1) / (16 * PARTS);  // chunks
-                struct Group {
-                    size_t row[G];
-                    int nn[G];
-                    bool on[G];
-                    uint4 mask[G][2];
+                const int per_tile = (s.accs - 16 * half + 16 * PARTS - 1) / (16 * PARTS);
+                struct Chunk {
+                    size_t row;
+                    int nn;
+                    bool on;
+                    uint4 mask[2];
                 };
-                // group i: tile, first chunk
-                auto load = [&](int m, int j, Group &q) {
+                // chunk j of this warp in tile m
+                auto load = [&](int m, int j, Chunk &q) {
                     const int x = m ? x1 : x0, y = y0 + (m ? r1 : r0);
-                    const bool in = (m ? in1 : in0) && y < s.Qy;
-#pragma unroll
-                    for (int k = 0; k < G; ++k) {
-                        const int c0 = 16 * (half + PARTS * (j + k));
-                        bool on = in && c0 < s.accs;
-                        size_t row = 0;
-                        int nn = c0;
-                        if (KIND == DGRAD2) {
-                            const int pc = on ? chunks[c0 >> 4] : 0, cls = pc & 7;
-                            nn = pc >> 3;
-                            const int z = 2 * qz + (cls >> 2), yy = 2 * y + ((cls >> 1) & 1),
-                                      xx = 2 * x + (cls & 1);
-                            on = on && z < a.D && yy < a.H && xx < a.W;
-                            if (on)
-                                row = vox_index(b, z, yy, xx, a.D, a.H, a.W);
-                        } else if (on) {
-                            row = (((size_t)b * s.Qz + qz) * s.Qy + y) * s.Qx + x;
-                        }
-                        q.nn[k] = nn;
-                        q.row[k] = row;
-                        q.on[k] = on;
-                        if (BWD && a.mask && on) {
-                            const uint4 *p =
-                                reinterpret_cast<const uint4 *>(a.mask + row * a.N + nn);
-                            if (a.wide) {
-                                load32(p, q.mask[k]);
-                            } else {
-                                q.mask[k][0] = __ldg(p);
-                                q.mask[k][1] = __ldg(p + 1);
-                            }
+                    const int c0 = 16 * (half + PARTS * j);
+                    bool on = (m ? in1 : in0) && y < s.Qy;
+                    size_t row = 0;
+                    int nn = c0;
+                    if (KIND == DGRAD2) {
+                        const int pc = on ? chunks[c0 >> 4] : 0, cls = pc & 7;
+                        nn = pc >> 3;
+                        const int z = 2 * qz + (cls >> 2), yy = 2 * y + ((cls >> 1) & 1),
+                                  xx = 2 * x + (cls & 1);
+                        on = on && z < a.D && yy < a.H && xx < a.W;
+                        if (on)
+                            row = vox_index(b, z, yy, xx, a.D, a.H, a.W);
+                    } else if (on) {
+                        row = (((size_t)b * s.Qz + qz) * s.Qy + y) * s.Qx + x;
+                    }
+                    q.nn = nn;
+                    q.row = row;
+                    q.on = on;
+                    if (BWD && a.mask && on) {
+                        const uint4 *p = reinterpret_cast<const uint4 *>(a.mask + row * a.N + nn);
+                        if (a.wide) {
+                            load32(p, q.mask);
+                        } else {
+                            q.mask[0] = __ldg(p);
+                            q.mask[1] = __ldg(p + 1);
                         }
                     }
                 };
-                Group cur, nxt;
+                Chunk cur, nxt;
                 if (per_tile > 0)
                     load(0, 0, cur);
                 // every warp waits for the sums, also one that has no columns: the set
@@ -1811,30 +1778,17 @@ __global__ void __launch_bounds__(slab_threads(KIND), 1) k_conv_slab(const ConvA
                 int m = per_tile > 0 ? 0 : s.T, j = 0;
 #pragma unroll 1
                 while (m < s.T) {
-                    int m2 = m, j2 = j + G;
+                    int m2 = m, j2 = j + 1;
                     if (j2 >= per_tile) {
                         ++m2;
                         j2 = 0;
                     }
                     if (m2 < s.T)
                         load(m2, j2, nxt);
-                    uint32_t v[2][16];
-#pragma unroll
-                    for (int k = 0; k < G; ++k) {  // past the sums: any columns of the set
-                        const int c0 = 16 * (half + PARTS * (j + k));
-                        tc_load16_async(d0 + m * s.accs + (c0 < s.accs ? c0 : 0), v[k]);
-                    }
-                    tc_load_wait(v[0], v[G - 1]);
-#pragma unroll
-                    for (int k = 0; k < G; ++k)
-                        if (cur.on[k]) {
-                            float f[16];
-#pragma unroll
-                            for (int e = 0; e < 16; ++e)
-                                f[e] = __uint_as_float(v[k][e]);
-                            epilogue_chunk<BWD ? DGRAD : FWD>(a, cur.row[k], f, cur.nn[k], 0,
-                                                              cur.mask[k]);
-                        }
+                    float v[16];
+                    tc_load16(d0 + m * s.accs + 16 * (half + PARTS * j), v);
+                    if (cur.on)
+                        epilogue_chunk<BWD ? DGRAD : FWD>(a, cur.row, v, cur.nn, 0, cur.mask);
                     cur = nxt;
                     m = m2;
                     j = j2;
