@@ -1358,7 +1358,8 @@ struct SlabArgs {
     int stage;                 // bytes of a ring stage
     int gplane;                // WGRAD2: bytes of an output gradient plane
     int goff;                  // WGRAD2: their offset in a stage
-    int ksteps;                // WGRAD2: K steps of 16 positions of a band
+    int ksteps;                // WGRAD2: K steps of 16 positions that cover a band
+    int krow;                  // WGRAD2: K steps of a row of outputs (a multiple of 16), else 0
     int nst;                   // ring stages
     int slack;                 // bytes behind the ring that a window may read
     int nacc;                  // accumulator sets (2: double buffered)
@@ -1614,16 +1615,27 @@ __global__ void __launch_bounds__(slab_threads(KIND), 1) k_conv_slab(const ConvA
                 tc_after_sync();
                 const uint32_t base = r16 + st * stage16;
                 if (KIND == WGRAD2) {
+                    // The band's rows of outputs, row by row where a row is whole K steps.
+                    // Otherwise the steps run through the rows' spare columns and up to 15
+                    // positions beyond them, whose output gradient is zero.
+                    int ib, iz, y0;
+                    decode(item, ib, iz, y0);
+                    const int rows = min(s.R, s.Qy - y0);
+                    const int nk = s.krow ? rows * s.krow : (rows * s.P + 15) / 16;
                     // windows of 16 planes: all at shift (0, 0), blocks 1-2 one column
                     // on, 0-1 one row on, 1 both
                     constexpr int B = 3 * NC, n00 = (4 * B + 1 + 15) / 16, n2 = (2 * B + 15) / 16,
                                   n11 = (B + 15) / 16;
                     const uint32_t g0 = base + ((uint32_t)s.goff >> 4);
 #pragma unroll 1
-                    for (int j = 0; j < s.ksteps; ++j) {
+                    for (int j = 0, pos = 0, left = s.krow; j < nk; ++j, pos += 16) {
                         const uint32_t on = item != i0 || j != 0;
-                        const uint64_t b = mb + g0 + 16 * j;
-                        const uint32_t a0 = base + 16 * j;
+                        const uint64_t b = mb + g0 + pos;
+                        const uint32_t a0 = base + pos;
+                        if (--left == 0) {  // krow > 0: the next row's first position
+                            left = s.krow;
+                            pos += s.P - s.Qx;
+                        }
 #pragma unroll
                         for (int k = 0; k < n00 + 2 * n2 + n11; ++k) {
                             const int sx = (k >= n00 && k < n00 + n2) || k >= n00 + 2 * n2;
@@ -1938,6 +1950,10 @@ __global__ void k_adam_pack(AdamPackArgs a, const int64_t *__restrict__ step,
 // (G = kReduceThreads / N groups, coalesced reads of the N columns of a
 // split), in order with compensated fp32 sums; the G group sums are then added in order
 // by one thread per column, so the result does not depend on timing.
+// With recheck the partials come from slabs whose K steps run through positions without an
+// output, where a zero output gradient meets inputs that the weight does not read: an infinity
+// or a NaN among those makes a sum NaN. Sums that are not finite are formed again from
+// the voxels that they are of.
 constexpr int kReduceThreads = 512;
 
 // Compensated (Kahan) fp32 accumulation: the sum keeps about the precision of
@@ -1956,7 +1972,8 @@ struct Kahan {
 
 __global__ void __launch_bounds__(kReduceThreads)
     k_wgrad_reduce(const float *__restrict__ part, int splits, int mrows, int N, int cin,
-                   int cout, float *__restrict__ gw, float *__restrict__ gb)
+                   int cout, float *__restrict__ gw, float *__restrict__ gb,
+                   const __grid_constant__ ConvArgs a, int recheck)
 {
     __shared__ float red[kReduceThreads];
     const int m = blockIdx.x;
@@ -1980,13 +1997,37 @@ __global__ void __launch_bounds__(kReduceThreads)
         for (; sp < splits; sp += groups)
             acc.add(p[(size_t)sp * step]);
     }
-    red[threadIdx.x] = acc.s - acc.c;
-    __syncthreads();
-    if (threadIdx.x < N && co < cout) {
+    const bool mine = threadIdx.x < N && co < cout;
+    auto total = [&]() {
+        red[threadIdx.x] = acc.s - acc.c;
+        __syncthreads();
         Kahan tot;
-        for (int gi = 0; gi < groups; ++gi)
+        for (int gi = 0; mine && gi < groups; ++gi)
             tot.add(red[gi * N + co]);
-        const float v = tot.s - tot.c;
+        return tot.s - tot.c;
+    };
+    float v = total();
+    if (recheck && __syncthreads_or(mine && !isfinite(v))) {
+        const int t = m / cin, ci = m - t * cin;  // t = 27: the bias
+        acc = Kahan{};
+        for (int vox = grp; grp < groups && vox < a.rows; vox += groups) {
+            int r = vox;
+            const int x = r % a.Wo * a.stride - 1 + t % 3;
+            r /= a.Wo;
+            const int y = r % a.Ho * a.stride - 1 + t / 3 % 3;
+            r /= a.Ho;
+            const int z = r % a.Do * a.stride - 1 + t / 9;
+            float in = t == 27 ? 1.0f : 0.0f;
+            if (t < 27 && (unsigned)x < (unsigned)a.W && (unsigned)y < (unsigned)a.H &&
+                (unsigned)z < (unsigned)a.D)
+                in = __bfloat162float(
+                    a.act[vox_index(r / a.Do, z, y, x, a.D, a.H, a.W) * cin + ci]);
+            acc.add(in * __bfloat162float(a.gout[(size_t)vox * N + co]));
+        }
+        const float again = total();
+        v = isfinite(v) ? v : again;
+    }
+    if (mine) {
         if (m < 27 * cin)
             gw[(size_t)co * 27 * cin + m] = v;
         else if (gb)
@@ -2153,6 +2194,7 @@ bool slab_plan(int kind, int C, int N, int64_t nb, const int *S, const int *Q, S
             const int B = 3 * nc;
             s.nk = (4 * B + 1 + 15) / 16 + 2 * ((2 * B + 15) / 16) + (B + 15) / 16;
             s.ksteps = (s.R * s.P + 15) / 16;
+            s.krow = s.Qx % 16 == 0 ? s.Qx / 16 : 0;
             s.gplane = s.ksteps * 256;
             s.goff = (4 * B + 1) * s.plane;
             s.stage = (s.goff + N / 8 * s.gplane + 127) / 128 * 128;
@@ -2229,9 +2271,10 @@ cudaError_t run_slab_kind(int kind, const ConvArgs &a, const SlabArgs &s, size_t
 
 // Runs a pass (a prepared) as a slab when it fits one; *ran says so. WGRAD: at
 // most *splits units, whose partial sums lie as k_wgrad_reduce reads them; the
-// number used is returned in *splits.
+// number used is returned in *splits, and in *recheck whether k_wgrad_reduce has to look at
+// sums that are not finite.
 cudaError_t launch_slab(int mode, const ConvLayer &l, ConvArgs a, cudaStream_t st, bool *ran,
-                        int *splits = nullptr)
+                        int *splits = nullptr, int *recheck = nullptr)
 {
     *ran = false;
     if (mode == WGRAD && l.stride != 2)
@@ -2256,6 +2299,7 @@ cudaError_t launch_slab(int mode, const ConvLayer &l, ConvArgs a, cudaStream_t s
     if (kind == WGRAD2) {
         s.upu = (s.items + *splits - 1) / *splits;
         a.units = *splits = (s.items + s.upu - 1) / s.upu;
+        *recheck = s.krow == 0;
         return C == 16 ? run_slab<16, WGRAD2>(a, s, smem, a.units, st)
                        : run_slab<32, WGRAD2>(a, s, smem, a.units, st);
     }
@@ -2571,9 +2615,10 @@ cudaError_t launch_conv_wgrad(const ConvLayer &l, const void *in, const void *go
     a.tmem_cols = tmem_cols_for(a.N);
     cudaError_t e;
     bool ran = false;
+    int recheck = 0;
     if (conv2_built(l)) {
         e = launch_conv2(a, true, s);
-    } else if ((e = launch_slab(WGRAD, l, a, s, &ran, &sp)) != cudaSuccess) {
+    } else if ((e = launch_slab(WGRAD, l, a, s, &ran, &sp, &recheck)) != cudaSuccess) {
         return e;
     } else if (!ran) {
         int grid = 0;
@@ -2590,7 +2635,8 @@ cudaError_t launch_conv_wgrad(const ConvLayer &l, const void *in, const void *go
     ProfScope ps(s, "k_wgrad_reduce");
     // one block per M row (27 cin weights rows and the bias row)
     k_wgrad_reduce<<<27 * l.cin + 1, kReduceThreads, 0, s>>>(static_cast<const float *>(ws), sp,
-                                                             mt * 128, a.N, l.cin, l.cout, gw, gb);
+                                                             mt * 128, a.N, l.cin, l.cout, gw, gb,
+                                                             a, recheck);
     return cudaGetLastError();
 }
 
