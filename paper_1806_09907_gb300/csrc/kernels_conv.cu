@@ -1950,7 +1950,7 @@ __global__ void k_adam_pack(AdamPackArgs a, const int64_t *__restrict__ step,
 // (G = kReduceThreads / N groups, coalesced reads of the N columns of a
 // split), in order with compensated fp32 sums; the G group sums are then added in order
 // by one thread per column, so the result does not depend on timing.
-// With recheck the partials come from slabs whose K steps run through positions without an
+// With RECHECK the partials come from slabs whose K steps run through positions without an
 // output, where a zero output gradient meets inputs that the weight does not read: an infinity
 // or a NaN among those makes a sum NaN. Sums that are not finite are formed again from
 // the voxels that they are of.
@@ -1970,10 +1970,40 @@ struct Kahan {
     }
 };
 
-__global__ void __launch_bounds__(kReduceThreads)
+struct RecheckArgs {
+    const __nv_bfloat16 *act, *gout;
+    int D, H, W, Do, Ho, Wo, stride, rows;
+};
+
+// The part of column co of M row m that voxels vox0, vox0 + step, ... give.
+__device__ __forceinline__ float wgrad_voxels(const RecheckArgs &a, int m, int co, int N, int cin,
+                                           int vox0, int step)
+{
+    const int t = m / cin, ci = m - t * cin;  // t = 27: the bias
+    Kahan acc;
+    for (int vox = vox0; vox < a.rows; vox += step) {
+        int r = vox;
+        const int x = r % a.Wo * a.stride - 1 + t % 3;
+        r /= a.Wo;
+        const int y = r % a.Ho * a.stride - 1 + t / 3 % 3;
+        r /= a.Ho;
+        const int z = r % a.Do * a.stride - 1 + t / 9;
+        float in = t == 27 ? 1.0f : 0.0f;
+        if (t < 27 && (unsigned)x < (unsigned)a.W && (unsigned)y < (unsigned)a.H &&
+            (unsigned)z < (unsigned)a.D)
+            in = __bfloat162float(a.act[vox_index(r / a.Do, z, y, x, a.D, a.H, a.W) * cin + ci]);
+        acc.add(in * __bfloat162float(a.gout[(size_t)vox * N + co]));
+    }
+    return acc.s - acc.c;
+}
+
+// RECHECK: held to the registers of the plain form (four blocks per SM), so that the common
+// case, in which every sum is finite, costs the same.
+template <bool RECHECK>
+__global__ void __launch_bounds__(kReduceThreads, RECHECK ? 4 : 1)
     k_wgrad_reduce(const float *__restrict__ part, int splits, int mrows, int N, int cin,
                    int cout, float *__restrict__ gw, float *__restrict__ gb,
-                   const __grid_constant__ ConvArgs a, int recheck)
+                   const __grid_constant__ RecheckArgs a)
 {
     __shared__ float red[kReduceThreads];
     const int m = blockIdx.x;
@@ -1986,46 +2016,38 @@ __global__ void __launch_bounds__(kReduceThreads)
         int sp = grp;
         // four independent loads in flight per thread, added in split order
         for (; sp + 3 * groups < splits; sp += 4 * groups) {
-            const float a = p[(size_t)sp * step], b = p[(size_t)(sp + groups) * step],
-                        c = p[(size_t)(sp + 2 * groups) * step],
-                        d = p[(size_t)(sp + 3 * groups) * step];
-            acc.add(a);
-            acc.add(b);
-            acc.add(c);
-            acc.add(d);
+            const float a0 = p[(size_t)sp * step], a1 = p[(size_t)(sp + groups) * step],
+                        a2 = p[(size_t)(sp + 2 * groups) * step],
+                        a3 = p[(size_t)(sp + 3 * groups) * step];
+            acc.add(a0);
+            acc.add(a1);
+            acc.add(a2);
+            acc.add(a3);
         }
         for (; sp < splits; sp += groups)
             acc.add(p[(size_t)sp * step]);
     }
+    red[threadIdx.x] = acc.s - acc.c;
+    __syncthreads();
     const bool mine = threadIdx.x < N && co < cout;
-    auto total = [&]() {
-        red[threadIdx.x] = acc.s - acc.c;
-        __syncthreads();
+    float v = 0.0f;
+    if (mine) {
         Kahan tot;
-        for (int gi = 0; mine && gi < groups; ++gi)
+        for (int gi = 0; gi < groups; ++gi)
             tot.add(red[gi * N + co]);
-        return tot.s - tot.c;
-    };
-    float v = total();
-    if (recheck && __syncthreads_or(mine && !isfinite(v))) {
-        const int t = m / cin, ci = m - t * cin;  // t = 27: the bias
-        acc = Kahan{};
-        for (int vox = grp; grp < groups && vox < a.rows; vox += groups) {
-            int r = vox;
-            const int x = r % a.Wo * a.stride - 1 + t % 3;
-            r /= a.Wo;
-            const int y = r % a.Ho * a.stride - 1 + t / 3 % 3;
-            r /= a.Ho;
-            const int z = r % a.Do * a.stride - 1 + t / 9;
-            float in = t == 27 ? 1.0f : 0.0f;
-            if (t < 27 && (unsigned)x < (unsigned)a.W && (unsigned)y < (unsigned)a.H &&
-                (unsigned)z < (unsigned)a.D)
-                in = __bfloat162float(
-                    a.act[vox_index(r / a.Do, z, y, x, a.D, a.H, a.W) * cin + ci]);
-            acc.add(in * __bfloat162float(a.gout[(size_t)vox * N + co]));
+        v = tot.s - tot.c;
+    }
+    if constexpr (RECHECK) {
+        if (__syncthreads_or(mine && !isfinite(v))) {
+            red[threadIdx.x] = grp < groups ? wgrad_voxels(a, m, co, N, cin, grp, groups) : 0.0f;
+            __syncthreads();
+            if (mine && !isfinite(v)) {
+                Kahan tot;
+                for (int gi = 0; gi < groups; ++gi)
+                    tot.add(red[gi * N + co]);
+                v = tot.s - tot.c;
+            }
         }
-        const float again = total();
-        v = isfinite(v) ? v : again;
     }
     if (mine) {
         if (m < 27 * cin)
@@ -2243,6 +2265,46 @@ bool slab_plan(int kind, int C, int N, int64_t nb, const int *S, const int *Q, S
     return found;
 }
 
+// Whether a planned slab beats k_conv, by the measured times of both (k_conv / slab in us,
+// batch x size of the input). Short rows keep the staging (a warp per row) and the epilogue's
+// 16-column accesses narrow; few bands do not repay the load of large weights or the zeroing of
+// the ring:
+//   WGRAD2 16 -> 32: 8x40x40x14 (7 outputs a row, bands of 18 and 2 rows) 23.6 / 28.9, x 20 (bands of
+//          10) 29.7 / 26.8; 16x16x16x4 19.9 / 24.7, x 5 (bands of 8) 20.2 / 18.5.
+//          32 -> 48: 16x16x16x12 (128 bands) 22.8 / 26.8, x 20 (256) 29.9 / 25.0; 8x40x40x8 29.0 / 35.0
+//   DGRAD2 32 -> 16: 8x40x40x5 16.7 / 18.7, 16x16x16x5 18.7 / 13; 48 -> 32, 83 KB of weights:
+//          8x40x40x12 31.0 / 34.6, 2x16x16x24 17.4 / 18.6, 16x16x16x16 20.9 / 18.5
+//   DGRAD1 16 channels: 8x40x40x6 22.9 / 28.8, x 8 31.5 / 24; 48: 8x40x40x1 31.0 / 35.0
+//   FWD1   16 channels: 8x40x40x3 17.1 / 18.3, x 4 18.8 / 16.5
+// With two stages a band takes a latency of about 1.3 us + 0.04 us a channel, whatever its rows;
+// k_conv a chain of 1.1 us a K slice or its copies at 3.75 TB/s: FWD2 48 -> 64 8x40x40x16
+// 41.5 / 78.3, 16x16x16x14 31.1 / 21.3; FWD1 64 -> 48 8x40x40x20 262 / 319, x 16 209 / 179.
+bool slab_pays(int kind, int C, int64_t rows, const SlabArgs &s)
+{
+    switch (kind) {
+    case WGRAD2:
+        if (C == 32)
+            return s.Qx >= 5 && s.items >= 256;
+        return s.Qx >= 9 || (s.Qx >= 3 && s.R <= 8);
+    case DGRAD2:
+        if (s.wbytes > 64 * 1024)
+            return s.Qx >= 7 && s.items >= 64;
+        return s.Qx >= 7 || s.items < 160;
+    case DGRAD1:
+        if (s.items >= 320 && s.Qx < (C == 16 ? 7 : 2))
+            return false;
+        break;
+    case FWD1:
+        if (s.items >= 320 && C == 16 && s.Qx > 1 && s.Qx < 4)
+            return false;
+        break;
+    }
+    if (s.nst > 2)
+        return true;
+    const double slab = 11.0 + (s.items + 151) / 152 * (1.3 + 0.0375 * C);
+    return slab < std::max(8.0 + 1.1 * conv_slices(27 * C), 20.0 + 54e-6 / 3.75 * C * rows);
+}
+
 template <int C, int KIND>
 cudaError_t run_slab(const ConvArgs &a, const SlabArgs &s, size_t smem, int units, cudaStream_t st)
 {
@@ -2291,8 +2353,10 @@ cudaError_t launch_slab(int mode, const ConvLayer &l, ConvArgs a, cudaStream_t s
     const int *Q = mode == DGRAD ? (kind == DGRAD2 ? pairs : in) : o;
     SlabArgs s;
     size_t smem = 0;
-    if (!slab_plan(kind, C, a.N, l.nb, S, Q, &s, &a.tmem_cols, &smem))
+    uint32_t cols = 0;
+    if (!slab_plan(kind, C, a.N, l.nb, S, Q, &s, &cols, &smem) || !slab_pays(kind, C, a.rows, s))
         return cudaSuccess;
+    a.tmem_cols = cols;
     s.src = a.act;
     s.src_elems = a.act_elems;
     *ran = true;
@@ -2634,9 +2698,10 @@ cudaError_t launch_conv_wgrad(const ConvLayer &l, const void *in, const void *go
         return e;
     ProfScope ps(s, "k_wgrad_reduce");
     // one block per M row (27 cin weights rows and the bias row)
-    k_wgrad_reduce<<<27 * l.cin + 1, kReduceThreads, 0, s>>>(static_cast<const float *>(ws), sp,
-                                                             mt * 128, a.N, l.cin, l.cout, gw, gb,
-                                                             a, recheck);
+    const RecheckArgs ra{a.act, a.gout, a.D, a.H, a.W, a.Do, a.Ho, a.Wo, a.stride, a.rows};
+    auto *reduce = recheck ? k_wgrad_reduce<true> : k_wgrad_reduce<false>;
+    reduce<<<27 * l.cin + 1, kReduceThreads, 0, s>>>(static_cast<const float *>(ws), sp, mt * 128,
+                                                     a.N, l.cin, l.cout, gw, gb, ra);
     return cudaGetLastError();
 }
 

@@ -80,3 +80,19 @@ def test_staged_passes_reuse_their_ring(nb, dims, cin, cout, stride):
     layers.test_conv_dgrad_parity(nb, dims, cin, cout, stride)
     layers.test_conv_wgrad_parity(nb, dims, cin, cout, stride)
     assert airgb.al_get_device_error() == 0
+
+
+# either side of the lines at which a pass takes the gathering kernel: short rows in many bands,
+# large weights for few bands, two stages with one-row bands
+@pytest.mark.parametrize("nb,dims,cin,cout,stride", [
+    (8, (40, 40, 3), 16, 16, 1), (8, (40, 40, 4), 16, 16, 1),
+    (8, (40, 40, 6), 48, 16, 1), (8, (40, 40, 7), 48, 16, 1),
+    (8, (40, 40, 12), 16, 32, 2), (8, (40, 40, 14), 16, 32, 2), (8, (40, 40, 18), 16, 32, 2),
+    (4, (16, 16, 14), 32, 48, 2), (8, (16, 16, 14), 32, 48, 2), (8, (32, 32, 32), 32, 48, 2),
+    (8, (40, 40, 12), 48, 64, 2), (2, (12, 12, 12), 48, 64, 2),
+])
+def test_lines_between_kernels(nb, dims, cin, cout, stride):
+    check_forward(nb, dims, cin, cout, stride)
+    layers.test_conv_dgrad_parity(nb, dims, cin, cout, stride)
+    layers.test_conv_wgrad_parity(nb, dims, cin, cout, stride)
+    assert airgb.al_get_device_error() == 0
