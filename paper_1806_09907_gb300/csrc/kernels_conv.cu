@@ -1362,7 +1362,8 @@ struct SlabArgs {
     int krow;                  // WGRAD2: K steps of a row of outputs (a multiple of 16), else 0
     int nst;                   // ring stages
     int slack;                 // bytes behind the ring that a window may read
-    int nacc;                  // accumulator sets (2: double buffered)
+    int nacc;                  // accumulators in turn for tiles or units (2: double buffered)
+    int nset;                  // WGRAD2: accumulator sets that a unit's K steps take in turn
     int nk;                    // MMAs of a tile or K step
     int accs;                  // TMEM columns of one accumulator set
     int bands, items;
@@ -1491,6 +1492,13 @@ __global__ void __launch_bounds__(slab_threads(KIND), 1) k_conv_slab(const ConvA
         b = r / s.Qz;
         qz = r - b * s.Qz;
     };
+    // WGRAD2: K steps of an item. The band's rows of outputs, row by row where a row is whole
+    // steps; otherwise the steps run through the rows' spare columns and up to 15 positions
+    // beyond them, whose output gradient is zero.
+    auto ksteps_of = [&](int item) {
+        const int rows = min(s.R, s.Qy - (item % s.bands) * s.R);
+        return s.krow ? rows * s.krow : (rows * s.P + 15) / 16;
+    };
     if (warp > kSlabEpi) {
         // ---- staging: a warp per source row, lanes along its 16-byte pieces
         const int pw = warp - kSlabEpi - 1;
@@ -1608,28 +1616,25 @@ __global__ void __launch_bounds__(slab_threads(KIND), 1) k_conv_slab(const ConvA
             if (use > 0)
                 mbar_wait(bar_free + 8 * acc, (use - 1) & 1);
             const uint32_t d0 = tmem + acc * (a.tmem_cols / 2);
-            const int i0 = u * per, i1 = min((u + 1) * per, s.items);
-            for (int item = i0; item < i1; ++item, ++n) {
+            const int i1 = min((u + 1) * per, s.items);
+            int step = 0, set = 0;  // WGRAD2: K step of the unit, first column of its set
+            for (int item = u * per; item < i1; ++item, ++n) {
                 const int st = (int)(n % (uint32_t)s.nst);
                 mbar_wait(bar_full + 8 * st, (n / (uint32_t)s.nst) & 1);
                 tc_after_sync();
                 const uint32_t base = r16 + st * stage16;
                 if (KIND == WGRAD2) {
-                    // The band's rows of outputs, row by row where a row is whole K steps.
-                    // Otherwise the steps run through the rows' spare columns and up to 15
-                    // positions beyond them, whose output gradient is zero.
-                    int ib, iz, y0;
-                    decode(item, ib, iz, y0);
-                    const int rows = min(s.R, s.Qy - y0);
-                    const int nk = s.krow ? rows * s.krow : (rows * s.P + 15) / 16;
+                    const int nk = ksteps_of(item);
                     // windows of 16 planes: all at shift (0, 0), blocks 1-2 one column
                     // on, 0-1 one row on, 1 both
                     constexpr int B = 3 * NC, n00 = (4 * B + 1 + 15) / 16, n2 = (2 * B + 15) / 16,
                                   n11 = (B + 15) / 16;
                     const uint32_t g0 = base + ((uint32_t)s.goff >> 4);
 #pragma unroll 1
-                    for (int j = 0, pos = 0, left = s.krow; j < nk; ++j, pos += 16) {
-                        const uint32_t on = item != i0 || j != 0;
+                    for (int j = 0, pos = 0, left = s.krow; j < nk; ++j, pos += 16, ++step) {
+                        const uint32_t on = step >= s.nset;
+                        const uint32_t dj = d0 + set;
+                        set = set + s.accs == s.nset * s.accs ? 0 : set + s.accs;
                         const uint64_t b = mb + g0 + pos;
                         const uint32_t a0 = base + pos;
                         if (--left == 0) {  // krow > 0: the next row's first position
@@ -1644,7 +1649,7 @@ __global__ void __launch_bounds__(slab_threads(KIND), 1) k_conv_slab(const ConvA
                                            : k < n00 + n2        ? B + 16 * (k - n00)
                                            : k < n00 + 2 * n2    ? 16 * (k - n00 - n2)
                                                                  : B + 16 * (k - n00 - 2 * n2);
-                            tc_mma_if(one, d0 + k * N, ma + a0 + p0 * pl + sy * P + sx, b, a.idesc,
+                            tc_mma_if(one, dj + k * N, ma + a0 + p0 * pl + sy * P + sx, b, a.idesc,
                                       on);
                         }
                     }
@@ -1713,6 +1718,9 @@ __global__ void __launch_bounds__(slab_threads(KIND), 1) k_conv_slab(const ConvA
                 // row of window k: plane p0 + row / 8, element row % 8
                 constexpr int B = 3 * NC;
                 const int n00 = (4 * B + 1 + 15) / 16, n2 = (2 * B + 15) / 16;
+                int sets = 0;  // that hold sums
+                for (int item = u * per; item < min((u + 1) * per, s.items) && sets < s.nset; ++item)
+                    sets = min(s.nset, sets + ksteps_of(item));
                 for (int k = 0; k < s.nk; ++k) {
                     int sy = 0, sx = 0, p0 = 16 * k, b0 = 0, b1 = 4;
                     if (k >= n00 + 2 * n2)
@@ -1732,6 +1740,13 @@ __global__ void __launch_bounds__(slab_threads(KIND), 1) k_conv_slab(const ConvA
                     for (int c0 = 16 * half; c0 < a.N; c0 += 16 * PARTS) {
                         float v[16];
                         tc_load16(d0 + k * a.N + c0, v);
+                        for (int q = 1; q < sets; ++q) {
+                            float w[16];
+                            tc_load16(d0 + q * s.accs + k * a.N + c0, w);
+#pragma unroll
+                            for (int e = 0; e < 16; ++e)
+                                v[e] += w[e];
+                        }
                         if (on)
                             epilogue_chunk<WGRAD>(a, (size_t)u * a.mtiles * 128 + m, v, c0, 0);
                     }
@@ -2232,10 +2247,14 @@ bool slab_plan(int kind, int C, int N, int64_t nb, const int *S, const int *Q, S
             sets = kind == DGRAD2 ? 8 : 1;
         }
         s.accs = sets * N;
-        // a weight adjoint drains its sums once per unit: one set where two do not fit
-        s.nacc = kind == WGRAD2 && 2 * s.accs > 512 ? 1 : 2;
+        // A weight adjoint drains its sums once per unit and needs no second buffer: its K
+        // steps take what sets fit in turn, for chains of fewer roundings. (16 -> 32 channels,
+        // 16 x 64^3, error against 64 bits: k_conv 1.16e-6 of the norm, one set 1.22e-6, two
+        // 0.54e-6; the same time.)
+        s.nacc = kind == WGRAD2 ? 1 : 2;
+        s.nset = kind == WGRAD2 ? std::max(1, std::min(4, 512 / s.accs)) : 1;
         uint32_t c = 32;
-        while ((int)c < s.nacc * s.T * s.accs)
+        while ((int)c < s.nacc * s.nset * s.T * s.accs)
             c <<= 1;
         if (kind == DGRAD2 && 8 * N > 256)
             continue;  // the widest MMA
@@ -2271,7 +2290,7 @@ bool slab_plan(int kind, int C, int N, int64_t nb, const int *S, const int *Q, S
 // the ring:
 //   WGRAD2 16 -> 32: 8x40x40x14 (7 outputs a row, bands of 18 and 2 rows) 23.6 / 28.9, x 20 (bands of
 //          10) 29.7 / 26.8; 16x16x16x4 19.9 / 24.7, x 5 (bands of 8) 20.2 / 18.5.
-//          32 -> 48: 16x16x16x12 (128 bands) 22.8 / 26.8, x 20 (256) 29.9 / 25.0; 8x40x40x8 29.0 / 35.0
+//          32 -> 48: 1x32x32x32 (96 bands) 22.6 / 24.2, 16x16x16x32 33.0 / 27.5
 //   DGRAD2 32 -> 16: 8x40x40x5 16.7 / 18.7, 16x16x16x5 18.7 / 13; 48 -> 32, 83 KB of weights:
 //          8x40x40x12 31.0 / 34.6, 2x16x16x24 17.4 / 18.6, 16x16x16x16 20.9 / 18.5
 //   DGRAD1 16 channels: 8x40x40x6 22.9 / 28.8, x 8 31.5 / 24; 48: 8x40x40x1 31.0 / 35.0
@@ -2283,8 +2302,12 @@ bool slab_pays(int kind, int C, int64_t rows, const SlabArgs &s)
 {
     switch (kind) {
     case WGRAD2:
+        // A single set's chains are no longer than k_conv's only without idle positions
+        // (32 -> 48, 16 x 22 x 30 x 26: error 1.75e-7 of the norm, k_conv 1.49e-7)
+        if (s.nset == 1 && s.krow == 0)
+            return false;
         if (C == 32)
-            return s.Qx >= 5 && s.items >= 256;
+            return s.items >= 256;
         return s.Qx >= 9 || (s.Qx >= 3 && s.R <= 8);
     case DGRAD2:
         if (s.wbytes > 64 * 1024)
@@ -2303,6 +2326,22 @@ bool slab_pays(int kind, int C, int64_t rows, const SlabArgs &s)
         return true;
     const double slab = 11.0 + (s.items + 151) / 152 * (1.3 + 0.0375 * C);
     return slab < std::max(8.0 + 1.1 * conv_slices(27 * C), 20.0 + 54e-6 / 3.75 * C * rows);
+}
+
+// Slab plan of a layer's weight adjoint for at most sp units; false when the layer takes k_conv.
+bool wgrad_slab_plan(const ConvLayer &l, int sp, SlabArgs *s, int *units, uint32_t *cols,
+                     size_t *smem)
+{
+    if (l.stride != 2 || (l.cin != 16 && l.cin != 32))
+        return false;
+    const int in[3] = {l.D, l.H, l.W};
+    const int o[3] = {conv_out_size(l.D, 2), conv_out_size(l.H, 2), conv_out_size(l.W, 2)};
+    if (!slab_plan(WGRAD2, l.cin, l.cout, l.nb, in, o, s, cols, smem) ||
+        !slab_pays(WGRAD2, l.cin, 0, *s))
+        return false;
+    s->upu = (s->items + sp - 1) / sp;
+    *units = (s->items + s->upu - 1) / s->upu;
+    return true;
 }
 
 template <int C, int KIND>
@@ -2331,21 +2370,36 @@ cudaError_t run_slab_kind(int kind, const ConvArgs &a, const SlabArgs &s, size_t
     }
 }
 
-// Runs a pass (a prepared) as a slab when it fits one; *ran says so. WGRAD: at
-// most *splits units, whose partial sums lie as k_wgrad_reduce reads them; the
-// number used is returned in *splits, and in *recheck whether k_wgrad_reduce has to look at
-// sums that are not finite.
-cudaError_t launch_slab(int mode, const ConvLayer &l, ConvArgs a, cudaStream_t st, bool *ran,
-                        int *splits = nullptr, int *recheck = nullptr)
+// The weight adjoint as a slab when its plan says so (*ran), in at most *splits units. *splits
+// receives the number of partial sums, which lie as k_wgrad_reduce reads them, and *recheck
+// whether that has to look at sums that are not finite.
+cudaError_t launch_wgrad_slab(const ConvLayer &l, ConvArgs a, cudaStream_t st, bool *ran,
+                              int *splits, int *recheck)
+{
+    SlabArgs s;
+    size_t smem = 0;
+    uint32_t cols = 0;
+    int units = 0;
+    *ran = wgrad_slab_plan(l, *splits, &s, &units, &cols, &smem);
+    if (!*ran)
+        return cudaSuccess;
+    s.src = a.act;
+    s.src_elems = a.act_elems;
+    a.tmem_cols = cols;
+    a.units = *splits = units;
+    *recheck = s.krow == 0;
+    return l.cin == 16 ? run_slab<16, WGRAD2>(a, s, smem, a.units, st)
+                       : run_slab<32, WGRAD2>(a, s, smem, a.units, st);
+}
+
+// Runs a forward pass or an input adjoint (a prepared) as a slab when it fits one; *ran says so.
+cudaError_t launch_slab(int mode, const ConvLayer &l, ConvArgs a, cudaStream_t st, bool *ran)
 {
     *ran = false;
-    if (mode == WGRAD && l.stride != 2)
-        return cudaSuccess;
-    const int kind = mode == WGRAD ? WGRAD2
-                     : mode == FWD ? (l.stride == 1 ? FWD1 : FWD2)
-                                   : (l.stride == 1 ? DGRAD1 : DGRAD2);
+    const int kind = mode == FWD ? (l.stride == 1 ? FWD1 : FWD2)
+                                 : (l.stride == 1 ? DGRAD1 : DGRAD2);
     const int C = mode == DGRAD ? l.cout : l.cin;
-    if (C != 16 && C != 32 && (kind == WGRAD2 || (C != 48 && C != 64)))
+    if (C != 16 && C != 32 && C != 48 && C != 64)
         return cudaSuccess;
     const int in[3] = {l.D, l.H, l.W}, o[3] = {a.Do, a.Ho, a.Wo};
     const int pairs[3] = {(l.D + 1) / 2, (l.H + 1) / 2, (l.W + 1) / 2};
@@ -2360,13 +2414,6 @@ cudaError_t launch_slab(int mode, const ConvLayer &l, ConvArgs a, cudaStream_t s
     s.src = a.act;
     s.src_elems = a.act_elems;
     *ran = true;
-    if (kind == WGRAD2) {
-        s.upu = (s.items + *splits - 1) / *splits;
-        a.units = *splits = (s.items + s.upu - 1) / s.upu;
-        *recheck = s.krow == 0;
-        return C == 16 ? run_slab<16, WGRAD2>(a, s, smem, a.units, st)
-                       : run_slab<32, WGRAD2>(a, s, smem, a.units, st);
-    }
     switch (C) {
     case 16: return run_slab_kind<16>(kind, a, s, smem, st);
     case 32: return run_slab_kind<32>(kind, a, s, smem, st);
@@ -2682,7 +2729,7 @@ cudaError_t launch_conv_wgrad(const ConvLayer &l, const void *in, const void *go
     int recheck = 0;
     if (conv2_built(l)) {
         e = launch_conv2(a, true, s);
-    } else if ((e = launch_slab(WGRAD, l, a, s, &ran, &sp, &recheck)) != cudaSuccess) {
+    } else if ((e = launch_wgrad_slab(l, a, s, &ran, &sp, &recheck)) != cudaSuccess) {
         return e;
     } else if (!ran) {
         int grid = 0;

@@ -72,3 +72,17 @@ def test_output_gradient_that_is_not_finite(nb, dims, cin, cout):
     ref, refb = wgrad64(x, gy, 2)  # padding zeros meet the infinity here as well
     assert torch.equal(torch.isfinite(gw), torch.isfinite(ref))
     assert torch.equal(torch.isfinite(gb), torch.isfinite(refb))
+
+
+@pytest.mark.parametrize("nb,dims,cin,cout,most", [
+    (16, (64, 64, 64), 16, 32, 1.15e-6), (8, (41, 37, 29), 16, 32, 1.15e-7),
+    (12, (30, 21, 47), 16, 32, 1.16e-7), (16, (22, 30, 26), 32, 48, 1.5e-7),
+    (9, (26, 31, 20), 32, 48, 8.9e-8)])
+def test_error_against_64_bits(nb, dims, cin, cout, most):
+    """No larger than what gathered operands and chains of one split's voxels give (`most`,
+    measured for these sizes on other inputs), and a tenth for the inputs' spread."""
+    cv, x, gy = layer(nb, dims, cin, cout, seed=7)
+    gw, gb = airgb.al_conv3d_backward_weight(cv, x, gy)
+    ref, refb = wgrad64(x, gy, 2)
+    assert float((gw.double() - ref).norm() / ref.norm()) <= 1.1 * most
+    assert float((gb.double() - refb).norm() / refb.norm()) <= 1e-7
