@@ -2143,54 +2143,61 @@ int dgrad_classes(const ConvLayer &l, int *unit0, int *nst, int *slice0, int *to
     return u;
 }
 
-// Resident CTAs per SM of a kernel of `threads` threads with `smem` bytes of
-// dynamic shared memory and `cols` TMEM columns, from the kernel's own limits
-// (shared memory with the largest carveout, registers, 512 TMEM columns per
-// SM); found once per kernel, size and device.
-struct Residency {
+// What limits a kernel's resident CTAs on a device, found once per kernel and device.
+struct KernelLimits {
     const void *fn;
-    size_t smem;
-    int dev, occ;
+    int dev, regs, fixed;  // registers of a thread; static and reserved shared memory of a CTA
+    int smem_sm;
 };
 
-cudaError_t resident_grid(const void *fn, size_t smem, int cols, int threads, int units, int *grid)
+cudaError_t kernel_limits(const void *fn, KernelLimits *out)
 {
     static std::mutex mu;
-    static Residency known[64];
+    static KernelLimits known[256];  // the kernels of this file on 8 devices
     static int n = 0;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess)
         return e;
     std::lock_guard<std::mutex> lk(mu);
-    int occ = 0;
-    for (int k = 0; k < n && occ == 0; ++k)
-        if (known[k].fn == fn && known[k].smem == smem && known[k].dev == dev)
-            occ = known[k].occ;
-    if (occ == 0) {
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kMaxDynSmem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     (int)cudaSharedmemCarveoutMaxShared);
-        cudaFuncAttributes fa;
-        if (e == cudaSuccess)
-            e = cudaFuncGetAttributes(&fa, fn);
-        int smem_sm = 0, resv = 0;
-        if (e == cudaSuccess)
-            e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-        if (e == cudaSuccess)
-            e = cudaDeviceGetAttribute(&resv, cudaDevAttrReservedSharedMemoryPerBlock, dev);
-        if (e != cudaSuccess)
-            return e;
-        const int by_smem = smem_sm / (int)(smem + fa.sharedSizeBytes + resv);
-        const int by_regs = 65536 / ((fa.numRegs * 32 + 255) / 256 * 256 * (threads / 32));
-        occ = std::min(std::min(by_smem, by_regs), std::min(512 / cols, 16));
-        if (occ < 1)
-            return cudaErrorInvalidConfiguration;
-        if (n < 64)
-            known[n++] = Residency{fn, smem, dev, occ};
-    }
+    for (int k = 0; k < n; ++k)
+        if (known[k].fn == fn && known[k].dev == dev) {
+            *out = known[k];
+            return cudaSuccess;
+        }
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 (int)cudaSharedmemCarveoutMaxShared);
+    cudaFuncAttributes fa;
+    if (e == cudaSuccess)
+        e = cudaFuncGetAttributes(&fa, fn);
+    int smem_sm = 0, resv = 0;
+    if (e == cudaSuccess)
+        e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    if (e == cudaSuccess)
+        e = cudaDeviceGetAttribute(&resv, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+    if (e != cudaSuccess)
+        return e;
+    *out = KernelLimits{fn, dev, fa.numRegs, (int)fa.sharedSizeBytes + resv, smem_sm};
+    if (n < 256)
+        known[n++] = *out;
+    return cudaSuccess;
+}
+
+// Resident grid of a kernel of `threads` threads with `smem` bytes of dynamic shared memory and
+// `cols` TMEM columns: shared memory with the largest carveout, registers, 512 TMEM columns per SM.
+cudaError_t resident_grid(const void *fn, size_t smem, int cols, int threads, int units, int *grid)
+{
+    KernelLimits k;
+    const cudaError_t e = kernel_limits(fn, &k);
+    if (e != cudaSuccess)
+        return e;
+    const int by_smem = k.smem_sm / (int)(smem + k.fixed);
+    const int by_regs = 65536 / ((k.regs * 32 + 255) / 256 * 256 * (threads / 32));
+    const int occ = std::min(std::min(by_smem, by_regs), std::min(512 / cols, 16));
+    if (occ < 1)
+        return cudaErrorInvalidConfiguration;
     *grid = std::min(units, occ * device_sms());
     return cudaSuccess;
 }
