@@ -320,33 +320,39 @@ __global__ void k_tick(int64_t *step)
 
 // out[v][z][y][x] = sum_b a_b exp(-|x - mu_b|^2 / (2 sigma_b^2)) for the
 // blob table of volume v ([blob][mu_x, mu_y, mu_z, sigma, a]). A block owns
-// a TB x TB x 32 box (x, y, z) and takes the table in chunks of 64 blobs, of
-// which it keeps those that come within 6 sigma of the box (in table order): a
+// a TB x TB x 32 box (x, y, z) and takes the table in chunks of 64 or 128 blobs, of
+// which it keeps those that come within 6 sigma of the 16 x 16 x 32 box around
+// it (in table order; the same blobs whatever TB, so the same bits): a
 // dropped term is below a exp(-18) < 1.6e-8 a everywhere in the box. A Gaussian
 // separates into per-axis factors,
 //   a exp(-|p - mu|^2 / (2 sigma^2)) = ex(x) ey(y) (a ez(z)),
-// so a kept blob takes 2 TB + 32 exponentials per box. A thread owns four
+// so a kept blob takes 2 TB + 32 exponentials per box. With TB = 16 a thread owns four
 // columns (x .. x + 3, y) of 8 slices; per blob two packed products ex ey, one
 // 16-byte read of ex, one 8-byte read of ey, four 16-byte reads of the z factors
 // (y and z factors stored twice, as the packed operands want them) and 16 packed
 // f32x2 FMAs: 24 instructions for 32 voxels and a blob, the FMAs' rate (34 us for
 // 16 x 128^3 voxels, 60 blobs of sigma 3-12) being the bound. That case takes 49 us;
 // 92 with one column of 8 slices per thread and boxes of 8 x 8, whose factor loads
-// and exponentials took half the issue slots.
+// and exponentials took half the issue slots. Calls of few boxes are chains of latencies
+// instead, and take boxes of 8 x 8 with one column of 8 slices per thread: 2 volumes of
+// 64 x 64 x 20 and 500 blobs 92 us with four columns, 35 so; one of 128 x 256 x 16 and 60
+// blobs 10 us either way.
 constexpr int kBrickZ = 32;    // z extent: 4 groups of 8 slices
-constexpr int kBlobChunk = 64; // blobs per chunk
 
 template <int TB>
-__global__ void __launch_bounds__(TB * TB, TB == 16 ? 4 : 16)
+__global__ void __launch_bounds__(256, 4)
     k_render_blobs(int D, int H, int W, int nblobs, const float *__restrict__ table,
                    float *__restrict__ out, int vec)
 {
-    constexpr int NT = TB * TB;               // (TB / 4) x TB x 4 threads
-    constexpr int FAC = 3 * TB + 2 * kBrickZ; // ex, (ey, ey), (a ez, a ez)
-    static_assert(NT >= kBlobChunk && FAC % 4 == 0, "a thread per blob of a chunk; 16-byte rows");
-    __shared__ float4 fac4[kBlobChunk * FAC / 4];
-    __shared__ float par[kBlobChunk][5];
-    __shared__ unsigned kept[kBlobChunk / 32];
+    constexpr int NT = 256, CX = TB == 16 ? 4 : 1;  // threads; columns of a thread
+    // factors of a blob: TB = 16: ex, (ey, ey), (a ez, a ez); TB = 8: ex, ey, a ez
+    constexpr int OY = TB, OZ = CX == 4 ? 3 * TB : 2 * TB,
+                  FAC = OZ + (CX == 4 ? 2 : 1) * kBrickZ;
+    static_assert(NT == TB / CX * TB * 4 && FAC % 4 == 0 && OZ % 4 == 0, "16-byte rows");
+    constexpr int CH = TB == 16 ? 64 : 128;  // blobs of a chunk
+    __shared__ float4 fac4[CH * FAC / 4];
+    __shared__ float par[CH][5];
+    __shared__ unsigned kept[CH / 32];
     float *fac = reinterpret_cast<float *>(fac4);
     const int vol = blockIdx.y;
     const int bx = (W + TB - 1) / TB, by = (H + TB - 1) / TB;
@@ -354,23 +360,25 @@ __global__ void __launch_bounds__(TB * TB, TB == 16 ? 4 : 16)
     const int x0 = (brick % bx) * TB, y0 = ((brick / bx) % by) * TB,
               z0 = (brick / (bx * by)) * kBrickZ;
     const float *tv = table + (int64_t)vol * nblobs * 5;
-    const int t = threadIdx.x, lx = (t % (TB / 4)) * 4, ly = t / (TB / 4) % TB,
-              zg = t / (TB / 4 * TB);
-    float2 acc[8][2];
+    const int t = threadIdx.x, lx = (t % (TB / CX)) * CX, ly = t / (TB / CX) % TB,
+              zg = t / (TB / CX * TB);
+    // TB = 16: columns (x, x + 1), (x + 2, x + 3) of slice i; TB = 8: slices 2 i, 2 i + 1
+    float2 acc[CX == 4 ? 8 : 2][2];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < (CX == 4 ? 8 : 2); ++i)
         acc[i][0] = acc[i][1] = make_float2(0.0f, 0.0f);
-    for (int b0 = 0; b0 < nblobs; b0 += kBlobChunk) {
+    for (int b0 = 0; b0 < nblobs; b0 += CH) {
         float e[5];
         bool in = false;
-        if (t < kBlobChunk) {
+        if (t < CH) {
             if (b0 + t < nblobs) {
 #pragma unroll
                 for (int k = 0; k < 5; ++k)
                     e[k] = __ldg(tv + (int64_t)(b0 + t) * 5 + k);
-                // distance from the centre to the box
-                const float dx = fmaxf(fmaxf((float)x0 - e[0], e[0] - (float)(x0 + TB - 1)), 0.0f);
-                const float dy = fmaxf(fmaxf((float)y0 - e[1], e[1] - (float)(y0 + TB - 1)), 0.0f);
+                // distance from the centre to the 16 x 16 x 32 box
+                const int xb = x0 & ~15, yb = y0 & ~15;
+                const float dx = fmaxf(fmaxf((float)xb - e[0], e[0] - (float)(xb + 15)), 0.0f);
+                const float dy = fmaxf(fmaxf((float)yb - e[1], e[1] - (float)(yb + 15)), 0.0f);
                 const float dz =
                     fmaxf(fmaxf((float)z0 - e[2], e[2] - (float)(z0 + kBrickZ - 1)), 0.0f);
                 in = dx * dx + dy * dy + dz * dz <= 36.0f * e[3] * e[3];
@@ -380,9 +388,14 @@ __global__ void __launch_bounds__(TB * TB, TB == 16 ? 4 : 16)
                 kept[t / 32] = m;
         }
         __syncthreads();  // also: the previous chunk's factors are read
-        const int n0 = __popc(kept[0]), n = n0 + __popc(kept[1]);
+        int n = 0, before = 0;  // kept blobs, those of the warps before this one
+#pragma unroll
+        for (int w = 0; w < CH / 32; ++w) {
+            before = w == t / 32 ? n : before;
+            n += __popc(kept[w]);
+        }
         if (in) {
-            const int k = (t < 32 ? 0 : n0) + __popc(kept[t / 32] & ((1u << (t % 32)) - 1u));
+            const int k = before + __popc(kept[t / 32] & ((1u << (t % 32)) - 1u));
 #pragma unroll
             for (int q = 0; q < 5; ++q)
                 par[k][q] = e[q];
@@ -395,32 +408,45 @@ __global__ void __launch_bounds__(TB * TB, TB == 16 ? 4 : 16)
             const int axis = r < TB ? 0 : r < 2 * TB ? 1 : 2;
             const int o = r - axis * TB;
             const float c = (float)((axis == 0 ? x0 : axis == 1 ? y0 : z0) + o) - par[k][axis];
-            const float v = expf(-0.5f * c * c / (par[k][3] * par[k][3]));
+            float v = expf(-0.5f * c * c / (par[k][3] * par[k][3]));
+            if (axis == 2)
+                v = par[k][4] * v;
             float *f = fac + FAC * k;
             if (axis == 0)
                 f[o] = v;
-            else if (axis == 1)
-                reinterpret_cast<float2 *>(f + TB)[o] = make_float2(v, v);
+            else if (CX == 1)
+                f[(axis == 1 ? OY : OZ) + o] = v;
             else
-                reinterpret_cast<float2 *>(f + 3 * TB)[o] =
-                    make_float2(par[k][4] * v, par[k][4] * v);
+                reinterpret_cast<float2 *>(f + (axis == 1 ? OY : OZ))[o] = make_float2(v, v);
         }
         __syncthreads();
 #pragma unroll 2
         for (int k = 0; k < n; ++k) {
             const float *f = fac + FAC * k;
-            const float4 ex = *reinterpret_cast<const float4 *>(f + lx);
-            const float2 ey = *reinterpret_cast<const float2 *>(f + TB + 2 * ly);
-            const float2 p0 = __fmul2_rn(make_float2(ex.x, ex.y), ey);
-            const float2 p1 = __fmul2_rn(make_float2(ex.z, ex.w), ey);
-            const float4 *zz = reinterpret_cast<const float4 *>(f + 3 * TB + 16 * zg);
+            if constexpr (CX == 4) {
+                const float4 ex = *reinterpret_cast<const float4 *>(f + lx);
+                const float2 ey = *reinterpret_cast<const float2 *>(f + OY + 2 * ly);
+                const float2 p0 = __fmul2_rn(make_float2(ex.x, ex.y), ey);
+                const float2 p1 = __fmul2_rn(make_float2(ex.z, ex.w), ey);
+                const float4 *zz = reinterpret_cast<const float4 *>(f + OZ + 16 * zg);
 #pragma unroll
-            for (int i = 0; i < 8; i += 2) {
-                const float4 z = zz[i / 2];
-                acc[i][0] = __ffma2_rn(p0, make_float2(z.x, z.y), acc[i][0]);
-                acc[i][1] = __ffma2_rn(p1, make_float2(z.x, z.y), acc[i][1]);
-                acc[i + 1][0] = __ffma2_rn(p0, make_float2(z.z, z.w), acc[i + 1][0]);
-                acc[i + 1][1] = __ffma2_rn(p1, make_float2(z.z, z.w), acc[i + 1][1]);
+                for (int i = 0; i < 8; i += 2) {
+                    const float4 z = zz[i / 2];
+                    acc[i][0] = __ffma2_rn(p0, make_float2(z.x, z.y), acc[i][0]);
+                    acc[i][1] = __ffma2_rn(p1, make_float2(z.x, z.y), acc[i][1]);
+                    acc[i + 1][0] = __ffma2_rn(p0, make_float2(z.z, z.w), acc[i + 1][0]);
+                    acc[i + 1][1] = __ffma2_rn(p1, make_float2(z.z, z.w), acc[i + 1][1]);
+                }
+            } else {
+                const float pxy = f[lx] * f[OY + ly];
+                const float2 p = make_float2(pxy, pxy);
+                const float4 *zz = reinterpret_cast<const float4 *>(f + OZ + 8 * zg);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const float4 z = zz[i];
+                    acc[i][0] = __ffma2_rn(p, make_float2(z.x, z.y), acc[i][0]);
+                    acc[i][1] = __ffma2_rn(p, make_float2(z.z, z.w), acc[i][1]);
+                }
             }
         }
     }
@@ -434,14 +460,19 @@ __global__ void __launch_bounds__(TB * TB, TB == 16 ? 4 : 16)
         if (z >= D)
             break;
         float *oz = o + (int64_t)z * H * W;
-        const float v[4] = {acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y};
-        if (vec) {
-            *reinterpret_cast<float4 *>(oz) = make_float4(v[0], v[1], v[2], v[3]);
+        if constexpr (CX == 1) {
+            const float2 v = acc[i / 4][i / 2 % 2];
+            *oz = i % 2 ? v.y : v.x;
         } else {
+            const float v[4] = {acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y};
+            if (vec) {
+                *reinterpret_cast<float4 *>(oz) = make_float4(v[0], v[1], v[2], v[3]);
+            } else {
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (x + j < W)
-                    oz[j] = v[j];
+                for (int j = 0; j < 4; ++j)
+                    if (x + j < W)
+                        oz[j] = v[j];
+            }
         }
     }
 }
@@ -453,8 +484,8 @@ cudaError_t run_render(int D, int H, int W, int count, int nblobs, const float *
     const int64_t boxes = (int64_t)((W + TB - 1) / TB) * ((H + TB - 1) / TB) *
                           ((D + kBrickZ - 1) / kBrickZ);
     // rows of whole 16-byte pieces (out is 16-byte aligned)
-    k_render_blobs<TB><<<dim3((unsigned)boxes, count), TB * TB, 0, s>>>(D, H, W, nblobs, table, out,
-                                                                       W % 4 == 0);
+    k_render_blobs<TB><<<dim3((unsigned)boxes, count), 256, 0, s>>>(D, H, W, nblobs, table, out,
+                                                                   W % 4 == 0);
     return cudaGetLastError();
 }
 
