@@ -408,7 +408,10 @@ __device__ __forceinline__ void block_reduce_fd(float (&v)[K], double (&out)[K],
 // An fp32 sum kept as its value and the sum of its rounding errors (each add's
 // error is exact, Knuth's two-sum), about 2^-45 of the terms' size: what an
 // FP64 sum of fp32 terms is wanted for, on the full-rate fp32 pipe (an FP64 add
-// or conversion takes 16 cycles per warp on this part).
+// or conversion takes 16 cycles per warp on this part). It has fp32's range: terms
+// above kSum2Most are left to an FP64 sum (2^31 of the largest stay inside).
+constexpr float kSum2Most = 0x1p96f;
+
 struct Sum2 {
     float s = 0.0f, e = 0.0f;
     __device__ __forceinline__ void add(float v)
@@ -430,9 +433,8 @@ struct Sum2 {
     }
 };
 
-// Deterministic block sum of K Sum2 per thread (fixed trees): pairs within each
-// warp, then warp 0 adds the warps' sums in FP64, which has the range for any
-// number of them. Valid in thread 0. `scratch` holds at least
+// Deterministic block sum of K Sum2 of terms up to kSum2Most per thread (fixed
+// trees): pairs within each warp, then warp 0 adds the warps' sums in FP64. Valid in thread 0. `scratch` holds at least
 // K * (blockDim.x / 32) doubles.
 template <int K>
 __device__ __forceinline__ void block_reduce_s2(Sum2 (&v)[K], double (&out)[K], double *scratch)

@@ -378,10 +378,39 @@ __global__ void __launch_bounds__(kTileX *kTileY)
 // again) + 19 us (the scaling of dS/dW), 156 us so; its bytes take 51 us.
 // maxbits (nullable): the largest |grad| as the bits of a float (a NaN never
 // wins), for al_exp_field_adjoint's fixed point.
+// The thread's part of R |X| as an FP64 sum, for terms that a Sum2 does not take.
+template <int D>
+__device__ __noinline__ double regulariser_wide(const Grid &g, const March &mp,
+                                                const float *__restrict__ u)
+{
+    double total = 0.0;
+    for (int tile = blockIdx.x; tile < mp.ntiles; tile += gridDim.x) {
+        const Column c = march_column(g, mp, tile);
+        if (!c.on)
+            continue;
+        unsigned v = (unsigned)((c.z0 * g.Y + c.y) * g.X + c.x);
+        for (int z = c.z0; z < c.z1; ++z, v += g.X * g.Y) {
+            float sum = 0.0f;
+            for (int i = 0; i < D; ++i) {
+                const float *ui = u + i * g.nv + v;
+                const float m = __ldg(ui);
+                const float dx = c.x + 1 < g.X ? __ldg(ui + 1) - m : 0.0f;
+                const float dy = c.y + 1 < g.Y ? __ldg(ui + g.X) - m : 0.0f;
+                const float dz =
+                    D == 3 && z + 1 < g.Z ? __ldg(ui + (int64_t)g.X * g.Y) - m : 0.0f;
+                sum = fmaf(dz, dz, fmaf(dy, dy, fmaf(dx, dx, sum)));
+            }
+            total += (double)sum;
+        }
+    }
+    return total;
+}
+
 template <int D, int GW>
 __global__ void __launch_bounds__(kTileX *kTileY, 5)
-    k_regulariser(Grid g, March mp, const float *__restrict__ u, float gscale,
-                  float *__restrict__ gu, double *__restrict__ partials, AdjointArgs a,
+    k_regulariser(const __grid_constant__ Grid g, const __grid_constant__ March mp,
+                  const float *__restrict__ u, float gscale, float *__restrict__ gu,
+                  double *__restrict__ partials, AdjointArgs a,
                   unsigned int *__restrict__ maxbits)
 {
     __shared__ double red[kTileX * kTileY / 32];
@@ -482,7 +511,12 @@ __global__ void __launch_bounds__(kTileX *kTileY, 5)
         }
     }
     double R[1];
+    const bool wide = !(total[0].s <= kSum2Most);  // terms are not negative
     block_reduce_s2<1>(total, R, red);
+    if (__syncthreads_or(wide)) {
+        R[0] = regulariser_wide<D>(g, mp, u);
+        block_reduce_d<1>(R, red);
+    }
     if (threadIdx.x == 0)
         partials[blockIdx.x] = R[0];
     if (!maxbits)

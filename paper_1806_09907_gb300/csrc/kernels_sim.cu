@@ -80,12 +80,30 @@ __device__ __forceinline__ Sum2 sum4(const float (&v)[4])
     return t;
 }
 
-// The block's K sums as its row of partials.
+// The block's K sums of four per thread as its row of partials; by FP64 trees
+// when a thread's sum is beyond what a Sum2 takes.
 template <int K>
-__device__ __forceinline__ void store_partials(Sum2 (&v)[K], double *part, double *red)
+__device__ __forceinline__ void store_partials(const float (&v)[K][4], double *part, double *red)
 {
+    bool far = false;
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            far |= !(fabsf(v[k][i]) <= kSum2Most);
     double t[K];
-    block_reduce_s2<K>(v, t, red);
+    if (__syncthreads_or(far)) {
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            t[k] = ((double)v[k][0] + v[k][1]) + ((double)v[k][2] + v[k][3]);
+        block_reduce_d<K>(t, red);
+    } else {
+        Sum2 s[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            s[k] = sum4(v[k]);
+        block_reduce_s2<K>(s, t, red);
+    }
     if (threadIdx.x == 0)
 #pragma unroll
         for (int k = 0; k < K; ++k)
@@ -149,16 +167,15 @@ __global__ void __launch_bounds__(kRedThreads)
                    const uint8_t *__restrict__ m, double *__restrict__ part)
 {
     __shared__ double red[2 * kRedThreads / 32];
-    float s[4] = {}, c[4] = {};
+    float s[2][4] = {};
     each_voxel(nv, F, W, m, [&](int k, float f, float w, bool on) {
         if (on) {
             const float d = w - f;
-            s[k] = fmaf(d, d, s[k]);
-            c[k] += 1.0f;
+            s[0][k] = fmaf(d, d, s[0][k]);
+            s[1][k] += 1.0f;
         }
     });
-    Sum2 acc[2] = {sum4(s), sum4(c)};
-    store_partials<2>(acc, part, red);
+    store_partials<2>(s, part, red);
 }
 
 __global__ void __launch_bounds__(kRedThreads)
@@ -186,6 +203,9 @@ __global__ void __launch_bounds__(kRedThreads)
 }
 
 // ---------------------------------------------------------------- NCC ------
+constexpr float kNccScale = 0x1p-20f;
+static_assert((int64_t)kRedBlocksMax * kRedThreads * 4 <= 1 << 20, "sums of a pass");
+
 __global__ void __launch_bounds__(kRedThreads)
     k_ncc_sums(int64_t nv, const float *__restrict__ F, const float *__restrict__ W,
                const uint8_t *__restrict__ m, float2 *__restrict__ part)
@@ -199,7 +219,14 @@ __global__ void __launch_bounds__(kRedThreads)
             c[k] += 1.0f;
         }
     });
-    // sums of values, whose squares fp32 has to hold in the second pass: pairs
+    // scaled by 2^-20, at least the reciprocal of the threads' sums that are added, so that
+    // no sum of sums leaves fp32's range
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        sf[k] *= kNccScale;
+        sw[k] *= kNccScale;
+        c[k] *= kNccScale;
+    }
     Sum2 acc[3] = {sum4(sf), sum4(sw), sum4(c)};
     block_reduce_pairs<3>(acc, red);
     if (threadIdx.x == 0)
@@ -230,7 +257,8 @@ __global__ void __launch_bounds__(kRedThreads)
         }
     block_reduce_pairs<3>(t, pairs);
     if (threadIdx.x == 0) {
-        const double n = t[2].value(), sf = t[0].value(), sw = t[1].value();
+        constexpr double up = 1.0 / kNccScale;
+        const double n = t[2].value() * up, sf = t[0].value() * up, sw = t[1].value() * up;
         const double mf = n > 0.0 ? sf / n : 0.0, mw = n > 0.0 ? sw / n : 0.0;
         mu[0] = (float)mf;
         mu[1] = (float)mw;
@@ -242,17 +270,16 @@ __global__ void __launch_bounds__(kRedThreads)
     }
     __syncthreads();
     const float muf = mu[0], muw = mu[1];
-    float cov[4] = {}, vf[4] = {}, vw[4] = {};
+    float s[3][4] = {};  // cov, vf, vw
     each_voxel(nv, F, W, m, [&](int k, float f, float w, bool on) {
         if (on) {
             const float a = f - muf, b = w - muw;
-            cov[k] = fmaf(a, b, cov[k]);
-            vf[k] = fmaf(a, a, vf[k]);
-            vw[k] = fmaf(b, b, vw[k]);
+            s[0][k] = fmaf(a, b, s[0][k]);
+            s[1][k] = fmaf(a, a, s[1][k]);
+            s[2][k] = fmaf(b, b, s[2][k]);
         }
     });
-    Sum2 acc[3] = {sum4(cov), sum4(vf), sum4(vw)};
-    store_partials<3>(acc, part, red);
+    store_partials<3>(s, part, red);
 }
 
 // scal: {muF, muW, n} in; writes {.., .., .., kF, kW} with
