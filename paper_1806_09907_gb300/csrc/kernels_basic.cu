@@ -8,7 +8,7 @@ namespace airgb {
 
 namespace {
 
-constexpr int kDispTX = 128;  // x extent of a displacement tile (threads)
+constexpr int kDispTX = 128;  // x extent of a displacement tile (threads); 32 for rows up to 32
 constexpr int kDispTY = 8;    // rows per tile
 
 // Control columns a tile of n voxels can touch.
@@ -23,22 +23,22 @@ constexpr int disp_span(int n, int delta) { return (n - 1) / delta + 5; }
 // indices were divided out and buffers sized for spacing 1 (6 CTAs per SM),
 // 44.8 us so; writing u takes 18.5 us. (96 registers; held to 64, 46.6 us, to 40,
 // 61.9 us.)
-template <int D>
-__global__ void __launch_bounds__(kDispTX)
+template <int D, int TX>
+__global__ void __launch_bounds__(TX)
     k_displacement(Grid g, const __grid_constant__ Lattice L, const float *__restrict__ c,
                    float *__restrict__ u)
 {
     extern __shared__ float disp_smem[];  // [D][kDispTY][njx]
-    const int x0 = blockIdx.x * kDispTX, y0 = blockIdx.y * kDispTY, z = blockIdx.z;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * kDispTY, z = blockIdx.z;
     const int delta = L.delta;
     const int jx0 = x0 / delta, jy0 = y0 / delta;
-    const int xl = min(x0 + kDispTX, g.X) - 1;
+    const int xl = min(x0 + TX, g.X) - 1;
     const int njx = xl / delta + 4 - jx0;
     const int rows = min(kDispTY, g.Y - y0);
     const int qz = z / delta, pz = z - qz * delta, py0 = y0 - jy0 * delta;
     const float z0 = L.w[pz][0], z1 = L.w[pz][1], z2 = L.w[pz][2], z3 = L.w[pz][3];
     const int64_t nxy = (int64_t)L.nx * L.ny;
-    for (int col = threadIdx.x; col < D * njx; col += kDispTX) {
+    for (int col = threadIdx.x; col < D * njx; col += TX) {
         const int i = D == 3 ? (col >= njx) + (col >= 2 * njx) : (col >= njx);
         const float *src = c + i * L.nc + (D == 3 ? qz * nxy : 0) + (int64_t)jy0 * L.nx + jx0 +
                            (col - i * njx);
@@ -102,8 +102,9 @@ __global__ void __launch_bounds__(kDispTX)
 // cell's four weighted sums of its delta voxels, then per control point the
 // sum over the up to four cells it supports) and kept; then the kept rows are
 // contracted along y. A row's buffers belong to its warp, so only the y step
-// waits for the block, and lanes stride along x, so no index is divided. Fixed
-// order, no atomics. 256 x 256 x 160, spacing 6: 168 us for x and 31 us for y
+// waits for the block, and lanes stride along x, so no index is divided; a cell's
+// voxels lie an odd number of words from the next cell's, so that lanes read different
+// banks. Fixed order, no atomics. 256 x 256 x 160, spacing 6: 168 us for x and 31 us for y
 // with one thread per output reading 4 delta values delta apart, 70 us so;
 // reading the field takes 18.5 us.
 constexpr int kTransThreads = 256;
@@ -113,73 +114,103 @@ constexpr int kTransWidth = 320;  // voxels of a staged row at most
 struct TransPlan {
     int jt, bj;         // control columns and rows of a block
     int nxt, nbands;    // blocks per slice along x and y
+    int cells, pitch;   // staged cells of a row at most, and words from one to the next
     size_t smem;
 };
 
-// A block's columns: up to kTransWidth voxels of support (a whole row of most
-// volumes; the buffers stay within 48 KB); its rows: 16, so that 3/16 of the
-// rows are read twice, or 8 or 4 when that leaves fewer than four blocks per SM
-// of a 152-SM GB300.
+// A block's columns: as many as need up to kTransWidth voxels of support and 48 KB (a whole row of
+// most volumes); its rows: 16, so that 3/16 of the rows are read twice, or 8 or 4 when that leaves
+// fewer than four blocks per SM of a 152-SM GB300. Both evened out over the blocks.
 TransPlan trans_plan(const Grid &g, const Lattice &L)
 {
     TransPlan t;
-    t.jt = std::min(L.nx, std::max(4, std::min(kTransWidth / L.delta - 3, 96)));
+    const int ncx = (g.X - 1) / L.delta + 1;
+    t.pitch = L.delta | 1;
+    auto bytes = [&](int bj) {
+        return 4 * (kMaxDelta * 4 +
+                    (size_t)kTransWarps * (t.cells * t.pitch + (t.jt + 3) * 4) +
+                    (size_t)(bj + 3) * L.delta * t.jt);
+    };
+    const int most = std::max(1, std::min(L.nx, kTransWidth));  // columns of a first guess
+    t.nxt = (L.nx + most - 1) / most;
+    do {
+        t.jt = (L.nx + t.nxt - 1) / t.nxt;
+        t.cells = std::min(ncx, t.jt + 3);
+    } while ((std::min(t.cells * L.delta, g.X) > kTransWidth || bytes(16) > 48 * 1024) && ++t.nxt);
     t.nxt = (L.nx + t.jt - 1) / t.jt;
     for (t.bj = 16; t.bj > 4; t.bj /= 2)
         if ((int64_t)g.ndim * g.Z * t.nxt * ((L.ny + t.bj - 1) / t.bj) >= 4 * 152)
             break;
     t.nbands = (L.ny + t.bj - 1) / t.bj;
-    const int cells = t.jt + 3;
-    t.smem = 4 * (kMaxDelta * 4 + (size_t)kTransWarps * cells * (L.delta + 4) +
-                  (size_t)(t.bj + 3) * L.delta * t.jt);
+    t.bj = (L.ny + t.nbands - 1) / t.nbands;
+    t.smem = bytes(t.bj);
     return t;
 }
 
 __global__ void __launch_bounds__(kTransThreads)
-    k_transpose_xy(const float *__restrict__ in, float *__restrict__ out, int X, int Y, int jt,
-                   int bj, int nxt, int nbands, const __grid_constant__ Lattice L)
+    k_transpose_xy(const float *__restrict__ in, float *__restrict__ out, int X, int Y,
+                   const __grid_constant__ TransPlan t, const __grid_constant__ Lattice L)
 {
     extern __shared__ __align__(16) float trans_sm[];
-    const int delta = L.delta, cells = jt + 3, width = cells * delta;
+    const int delta = L.delta, jt = t.jt, cells = jt + 3, pitch = t.pitch;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float4 *w4 = reinterpret_cast<float4 *>(trans_sm);   // [delta] weights of a phase
-    float *raw = trans_sm + kMaxDelta * 4 + warp * width;                       // [width]
-    float *sums = trans_sm + kMaxDelta * 4 + kTransWarps * width + warp * cells * 4;  // [4][cells]
-    float *t1 = trans_sm + kMaxDelta * 4 + kTransWarps * (width + cells * 4);   // [rows][jt]
+    float *raw = trans_sm + kMaxDelta * 4 + warp * t.cells * pitch;  // [staged cells][pitch]
+    float *sums = trans_sm + kMaxDelta * 4 + kTransWarps * t.cells * pitch +
+                  warp * cells * 4;  // [4][cells]
+    float *t1 = trans_sm + kMaxDelta * 4 + kTransWarps * (t.cells * pitch + cells * 4);  // [rows][jt]
     if (threadIdx.x < delta)
         w4[threadIdx.x] = make_float4(L.w[threadIdx.x][0], L.w[threadIdx.x][1],
                                       L.w[threadIdx.x][2], L.w[threadIdx.x][3]);
-    const int tile = blockIdx.x, tx = tile % nxt, band = (tile / nxt) % nbands;
-    const int64_t o = tile / (nxt * nbands);
-    const int jx0 = tx * jt, jy0 = band * bj;
-    const int nj = min(jt, L.nx - jx0), nb = min(bj, L.ny - jy0);
-    // voxel (column) 0 of the tile, row 0 of the band
-    const int x0 = (jx0 - 3) * delta, y0 = (jy0 - 3) * delta;
-    const int rows = (nb + 3) * delta;
+    const int tile = blockIdx.x, tx = tile % t.nxt, band = (tile / t.nxt) % t.nbands;
+    const int64_t o = tile / (t.nxt * t.nbands);
+    const int jx0 = tx * jt, jy0 = band * t.bj;
+    const int nj = min(jt, L.nx - jx0), nb = min(t.bj, L.ny - jy0);
+    // the tile's cells inside the grid, [c0, c0 + nc), cell 0 of the tile being jx0 - 3
+    const int c0 = max(jx0 - 3, 0), nc = min(jx0 + nj, (X - 1) / delta + 1) - c0;
+    const int skip = c0 - (jx0 - 3);
+    const int x0 = c0 * delta, width = min(nc * delta, X - x0);
+    // rows of the band's support, those inside the grid
+    const int y0 = (jy0 - 3) * delta, rows = (nb + 3) * delta;
+    const int r0 = max(0, -y0), r1 = min(rows, Y - y0);
     const float *src = in + o * Y * X + x0;
     constexpr int PER = kTransWidth / 32;
+    int place[PER];  // of this lane's voxels in raw
+    const int spare = pitch - delta, inv = 65536 / delta + 1;  // i inv / 65536 = i / delta, i < 320
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const int i = lane + 32 * k;
+        place[k] = i + spare * (i * inv >> 16);
+    }
     float next[PER];
     auto fetch = [&](int r) {
-        const int y = y0 + r;
-        const bool ok = r < rows && y >= 0 && y < Y;
 #pragma unroll
-        for (int k = 0; k < PER; ++k) {
-            const int i = lane + 32 * k;
-            next[k] = ok && i < width && x0 + i >= 0 && x0 + i < X
-                          ? __ldg(src + (int64_t)y * X + i) : 0.0f;
-        }
+        for (int k = 0; k < PER; ++k)
+            next[k] = r < r1 && lane + 32 * k < width
+                          ? __ldg(src + (int64_t)(y0 + r) * X + lane + 32 * k) : 0.0f;
     };
-    fetch(warp);
+    fetch(r0 + warp);
+    // zero where no row or cell of the grid writes: cells before and beyond the grid's, the last
+    // one's voxels beyond it, and rows
+    if (skip > 0 || skip + nc < cells)
+        for (int e = lane; e < cells * 4; e += 32)
+            sums[e] = 0.0f;
+    if (lane < nc * delta - width)
+        raw[(nc - 1) * pitch + delta - 1 - lane] = 0.0f;
+    for (int e = threadIdx.x; e < r0 * jt; e += kTransThreads)
+        t1[e] = 0.0f;
+    for (int e = r1 * jt + threadIdx.x; e < rows * jt; e += kTransThreads)
+        t1[e] = 0.0f;
     __syncthreads();
-    for (int r = warp; r < rows; r += kTransWarps) {
+    for (int r = r0 + warp; r < r1; r += kTransWarps) {
 #pragma unroll
         for (int k = 0; k < PER; ++k)
             if (lane + 32 * k < width)
-                raw[lane + 32 * k] = next[k];
+                raw[place[k]] = next[k];
         __syncwarp();
         fetch(r + kTransWarps);
-        for (int e = lane; e < cells; e += 32) {
-            const float *v = raw + e * delta;
+        for (int e = lane; e < nc; e += 32) {
+            const float *v = raw + e * pitch;
             float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, s3 = 0.0f;
 #pragma unroll 4
             for (int k = 0; k < delta; ++k) {
@@ -190,10 +221,11 @@ __global__ void __launch_bounds__(kTransThreads)
                 s2 = fmaf(w.z, a, s2);
                 s3 = fmaf(w.w, a, s3);
             }
-            sums[e] = s0;
-            sums[cells + e] = s1;
-            sums[2 * cells + e] = s2;
-            sums[3 * cells + e] = s3;
+            float *d = sums + skip + e;
+            d[0] = s0;
+            d[cells] = s1;
+            d[2 * cells] = s2;
+            d[3 * cells] = s3;
         }
         __syncwarp();
         // control point j is fed by the cells j - 3 .. j (weights 3 .. 0)
@@ -220,30 +252,29 @@ __global__ void __launch_bounds__(kTransThreads)
         }
 }
 
-// A6 along z: in[o][Z][inner] -> out[o][nz][inner], one thread per output,
-// ascending z.
+// A6 along one axis: in[o][len][inner] -> out[o][n][inner], one thread per output,
+// ascending positions.
+// I: the outputs' index type, 32 bits where they allow it.
+template <typename I>
 __global__ void __launch_bounds__(kTransThreads)
-    k_transpose_z(const float *__restrict__ in, float *__restrict__ out, int outer, int Z, int nz,
-                  int inner, const __grid_constant__ Lattice L)
+    k_transpose_axis(const float *__restrict__ in, float *__restrict__ out, I total, int len,
+                     int n, I inner, const __grid_constant__ Lattice L)
 {
-    const int64_t total = (int64_t)outer * nz * inner;
     const int delta = L.delta;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int o = (int)(e / ((int64_t)nz * inner));
-        const int64_t r = e - (int64_t)o * nz * inner;
-        const int j = (int)(r / inner), k = (int)(r - (int64_t)j * inner);
-        const float *src = in + (int64_t)o * Z * inner + k;
+    for (I e = blockIdx.x * (I)blockDim.x + threadIdx.x; e < total; e += (I)gridDim.x * blockDim.x) {
+        const I oj = e / inner, k = e - oj * inner, o = oj / n;
+        const int j = (int)(oj - o * n);
+        const float *src = in + (int64_t)o * len * inner + k;
         float acc = 0.0f;
 #pragma unroll
         for (int a = 3; a >= 0; --a) {
             const int t0 = (j - a) * delta;
             if (t0 < 0)
                 continue;
-            const int n = min(delta, Z - t0);
+            const int m = min(delta, len - t0);
             const float *p = src + (int64_t)t0 * inner;
 #pragma unroll 4
-            for (int q = 0; q < n; ++q)
+            for (int q = 0; q < m; ++q)
                 acc = fmaf(L.w[q][a], __ldg(p + (int64_t)q * inner), acc);
         }
         out[e] = acc;
@@ -251,22 +282,25 @@ __global__ void __launch_bounds__(kTransThreads)
 }
 
 // ---- marching tiles ---------------------------------------------------------
-// The point-wise kernels take 32 x 8 columns a block (a warp per row) and march
+// The point-wise kernels take 32 x 8 columns a block (a warp per row; narrower rows where
+// they use more lanes, march_lx) and march
 // through zc slices, so that a column's index arithmetic is done once and its
 // z neighbours stay in registers. Tiles beyond the grid's blocks follow in
 // order (tile += gridDim).
-constexpr int kTileX = 32, kTileY = 8;
+constexpr int kTileX = 32, kTileY = 8;  // columns of a block: kTileX * kTileY
 
 struct March {
-    int ntx, nty, ntiles, zc;
+    int ntx, nty, ntiles, zc, lx;  // lx: log2 of a tile's columns in x
 };
 
 // Slices of a column: 8, fewer while that leaves less than eight blocks per SM.
 March march_plan(const Grid &g)
 {
     March m;
-    m.ntx = (g.X + kTileX - 1) / kTileX;
-    m.nty = (g.Y + kTileY - 1) / kTileY;
+    m.lx = march_lx(g.X);
+    m.ntx = (g.X + (1 << m.lx) - 1) >> m.lx;
+    const int ty = kTileX * kTileY >> m.lx;
+    m.nty = (g.Y + ty - 1) / ty;
     m.zc = 8;
     while (m.zc > 1 &&
            (int64_t)m.ntx * m.nty * ((g.Z + m.zc - 1) / m.zc) < 8 * (int64_t)device_sms())
@@ -283,8 +317,8 @@ struct Column {
 __device__ __forceinline__ Column march_column(const Grid &g, const March &m, int tile)
 {
     Column c;
-    c.x = tile % m.ntx * kTileX + (threadIdx.x & 31);
-    c.y = tile / m.ntx % m.nty * kTileY + (threadIdx.x >> 5);
+    c.x = (tile % m.ntx << m.lx) + (threadIdx.x & ((1 << m.lx) - 1));
+    c.y = tile / m.ntx % m.nty * (kTileX * kTileY >> m.lx) + (threadIdx.x >> m.lx);
     c.z0 = tile / (m.ntx * m.nty) * m.zc;
     c.z1 = min(c.z0 + m.zc, g.Z);
     c.on = c.x < g.X && c.y < g.Y;
@@ -318,10 +352,10 @@ __global__ void __launch_bounds__(kTileX *kTileY)
     const Column c = march_column(g, mp, blockIdx.x);
     if (!c.on)
         return;
-    const int sz = g.X * g.Y;
-    unsigned v = (unsigned)((c.z0 * g.Y + c.y) * g.X + c.x);  // wraps after the last slice only
+    const int sz = g.X * g.Y, v0 = (c.z0 * g.Y + c.y) * g.X + c.x;
 #pragma unroll 2
-    for (int z = c.z0; z < c.z1; ++z, v += sz) {
+    for (int z = c.z0; z < c.z1; ++z) {
+        const int v = v0 + (z - c.z0) * sz;
         Interp ip;
         const bool in = sample_at<D>(g, M, c.x, c.y, z, __ldg(u + v), __ldg(u + g.nv + v),
                                      D == 3 ? __ldg(u + 2 * (int64_t)g.nv + v) : 0.0f, ip);
@@ -576,17 +610,24 @@ int elementwise_grid(int64_t n, int threads)
 
 }  // namespace
 
+template <int TX>
+static cudaError_t run_displacement(const Grid &g, const Lattice &L, const float *ctrl,
+                                    float *disp, cudaStream_t s)
+{
+    dim3 grid((g.X + TX - 1) / TX, (g.Y + kDispTY - 1) / kDispTY, g.Z);
+    const size_t smem = (size_t)g.ndim * std::min(disp_span(TX, L.delta), L.nx) * kDispTY * 4;
+    if (g.ndim == 3)
+        k_displacement<3, TX><<<grid, TX, smem, s>>>(g, L, ctrl, disp);
+    else
+        k_displacement<2, TX><<<grid, TX, smem, s>>>(g, L, ctrl, disp);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_displacement(const Grid &g, const Lattice &L, const float *ctrl, float *disp,
                                 cudaStream_t s)
 {
-    dim3 grid((g.X + kDispTX - 1) / kDispTX, (g.Y + kDispTY - 1) / kDispTY, g.Z);
-    const size_t smem =
-        (size_t)g.ndim * std::min(disp_span(kDispTX, L.delta), L.nx) * kDispTY * 4;
-    if (g.ndim == 3)
-        k_displacement<3><<<grid, kDispTX, smem, s>>>(g, L, ctrl, disp);
-    else
-        k_displacement<2><<<grid, kDispTX, smem, s>>>(g, L, ctrl, disp);
-    return cudaGetLastError();
+    return g.X <= 32 ? run_displacement<32>(g, L, ctrl, disp, s)
+                     : run_displacement<kDispTX>(g, L, ctrl, disp, s);
 }
 
 size_t displacement_adjoint_ws(const Grid &g, const Lattice &L)
@@ -597,6 +638,19 @@ size_t displacement_adjoint_ws(const Grid &g, const Lattice &L)
     return ((t1 * 4 + 255) / 256) * 256 + ((t2 * 4 + 255) / 256) * 256;
 }
 
+static void transpose_axis(const float *in, float *out, int64_t outer, int len, int n,
+                           int64_t inner, const Lattice &L, cudaStream_t s)
+{
+    const int64_t total = outer * n * inner;
+    const int blocks = elementwise_grid(total, kTransThreads);
+    if (total < 1ll << 31)  // and a step of the grid beyond it fits 32 bits
+        k_transpose_axis<unsigned><<<blocks, kTransThreads, 0, s>>>(in, out, (unsigned)total, len,
+                                                                    n, (unsigned)inner, L);
+    else
+        k_transpose_axis<int64_t><<<blocks, kTransThreads, 0, s>>>(in, out, total, len, n, inner,
+                                                                   L);
+}
+
 cudaError_t launch_displacement_adjoint(const Grid &g, const Lattice &L, const float *grad_disp,
                                         float *grad_ctrl, void *ws, cudaStream_t s)
 {
@@ -605,15 +659,24 @@ cudaError_t launch_displacement_adjoint(const Grid &g, const Lattice &L, const f
     // second part of the workspace
     const size_t t1n = (size_t)D * g.Z * g.Y * L.nx;
     float *t2 = (float *)((char *)ws + ((t1n * 4 + 255) / 256) * 256);
+    // Few cells a row leave a row's warp most lanes idle: one thread per output and axis
+    // instead (three launches; from about 32 k rows on: 256 x 256 x 8 at spacing 16
+    // 90 us against 32, 300 x 300 x 3 at 5 87 / 25, 128 x 256 x 16 at 6 43 / 25; 128 x 200 x 24
+    // at 3 37 / 40, and 20000 x 5 at 8 20 / 31).
+    if ((int64_t)D * g.Z * g.Y >= 32768 && (g.X < 24 || g.X < 5 * L.delta)) {
+        const int64_t rows = (int64_t)D * g.Z * g.Y;
+        float *t1 = (float *)ws, *xy = D == 3 ? t2 : grad_ctrl;
+        transpose_axis(grad_disp, t1, rows, g.X, L.nx, 1, L, s);
+        transpose_axis(t1, xy, (int64_t)D * g.Z, g.Y, L.ny, L.nx, L, s);
+        if (D == 3)
+            transpose_axis(xy, grad_ctrl, D, g.Z, L.nz, (int64_t)L.ny * L.nx, L, s);
+        return cudaGetLastError();
+    }
     const TransPlan t = trans_plan(g, L);
     k_transpose_xy<<<D * g.Z * t.nxt * t.nbands, kTransThreads, t.smem, s>>>(
-        grad_disp, D == 3 ? t2 : grad_ctrl, g.X, g.Y, t.jt, t.bj, t.nxt, t.nbands, L);
-    if (D == 3) {
-        // z: (D, Z, ny*nx) -> (D, nz, ny*nx)
-        const int64_t n3 = D * L.nc;
-        k_transpose_z<<<elementwise_grid(n3, kTransThreads), kTransThreads, 0, s>>>(
-            t2, grad_ctrl, D, g.Z, L.nz, L.ny * L.nx, L);
-    }
+        grad_disp, D == 3 ? t2 : grad_ctrl, g.X, g.Y, t, L);
+    if (D == 3)  // z: (D, Z, ny*nx) -> (D, nz, ny*nx)
+        transpose_axis(t2, grad_ctrl, D, g.Z, L.nz, (int64_t)L.ny * L.nx, L, s);
     return cudaGetLastError();
 }
 

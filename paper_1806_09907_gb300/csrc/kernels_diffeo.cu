@@ -128,11 +128,12 @@ __global__ void __launch_bounds__(kDiffeoThreads)
 template <bool SCALED>
 __global__ void __launch_bounds__(kDiffeoThreads, 4)
     k_compose3(Grid g, const float *__restrict__ u, float *__restrict__ out, float scale,
-               float *__restrict__ u0, int ntx, int nty, int zc)
+               float *__restrict__ u0, int ntx, int nty, int zc, int lx)
 {
     const float sc = SCALED ? scale : 1.0f;
     const int tile = blockIdx.x, tx = tile % ntx, ty = (tile / ntx) % nty, tz = tile / (ntx * nty);
-    const int x = tx * 32 + (threadIdx.x & 31), y = ty * (kDiffeoThreads / 32) + (threadIdx.x >> 5);
+    const int x = (tx << lx) + (threadIdx.x & ((1 << lx) - 1)),
+              y = ty * (kDiffeoThreads >> lx) + (threadIdx.x >> lx);
     if (x >= g.X || y >= g.Y)
         return;
     const int sy = g.X, sz = g.X * g.Y;
@@ -416,11 +417,12 @@ __device__ __forceinline__ void add_fix(unsigned long long *a, Fix q)
 __global__ void __launch_bounds__(kDiffeoThreads, 3)
     k_compose_adjoint3(Grid g, const float *__restrict__ u, const float *__restrict__ gin,
                        float *__restrict__ h, unsigned long long *__restrict__ acc,
-                       const unsigned int *__restrict__ maxbits, int ntx, int nty, int zc)
+                       const unsigned int *__restrict__ maxbits, int ntx, int nty, int zc, int lx)
 {
     const float S = fixed_scale(*maxbits);
     const int tile = blockIdx.x, tx = tile % ntx, ty = (tile / ntx) % nty, tz = tile / (ntx * nty);
-    const int x = tx * 32 + (threadIdx.x & 31), y = ty * (kDiffeoThreads / 32) + (threadIdx.x >> 5);
+    const int x = (tx << lx) + (threadIdx.x & ((1 << lx) - 1)),
+              y = ty * (kDiffeoThreads >> lx) + (threadIdx.x >> lx);
     if (x >= g.X || y >= g.Y)
         return;
     const int sy = g.X, sz = g.X * g.Y;
@@ -522,17 +524,19 @@ __global__ void __launch_bounds__(kDiffeoThreads, 3)
     }
 }
 
-// Tiles of the marching kernels: 32 x 8 columns a block and zc slices, 8 of
+// Tiles of the marching kernels: 32 x 8 columns a block (march_lx) and zc slices, 8 of
 // them or fewer while that leaves less than eight blocks per SM.
 struct Tiles {
-    int ntx, nty, zc, blocks;
+    int ntx, nty, zc, blocks, lx;
 };
 
 Tiles tiles_of(const Grid &g)
 {
     Tiles t;
-    t.ntx = (g.X + 31) / 32;
-    t.nty = (g.Y + kDiffeoThreads / 32 - 1) / (kDiffeoThreads / 32);
+    t.lx = march_lx(g.X);
+    t.ntx = (g.X + (1 << t.lx) - 1) >> t.lx;
+    const int ty = kDiffeoThreads >> t.lx;
+    t.nty = (g.Y + ty - 1) / ty;
     t.zc = 8;
     while (t.zc > 1 &&
            (int64_t)t.ntx * t.nty * ((g.Z + t.zc - 1) / t.zc) < 8 * (int64_t)device_sms())
@@ -586,10 +590,10 @@ cudaError_t exp_run(const Grid &g, int K, const float *v, float *u, float *traj,
             const Tiles t = tiles_of(g);
             if (scaled)
                 k_compose3<true><<<t.blocks, kDiffeoThreads, 0, s>>>(g, cur, nxt, scale0, u0,
-                                                                     t.ntx, t.nty, t.zc);
+                                                                     t.ntx, t.nty, t.zc, t.lx);
             else
                 k_compose3<false><<<t.blocks, kDiffeoThreads, 0, s>>>(g, cur, nxt, 1.0f, u0,
-                                                                      t.ntx, t.nty, t.zc);
+                                                                      t.ntx, t.nty, t.zc, t.lx);
         } else {
             if (scaled)
                 k_compose2<true><<<blocks_for(g.nv), kDiffeoThreads, 0, s>>>(g, cur, nxt, scale0,
@@ -634,7 +638,7 @@ cudaError_t exp_adjoint_run(const Grid &g, int K, const float *traj, const float
         if constexpr (D == 3) {
             const Tiles t = tiles_of(g);
             k_compose_adjoint3<<<t.blocks, kDiffeoThreads, 0, s>>>(g, u, gin, out, acc, mcur,
-                                                                   t.ntx, t.nty, t.zc);
+                                                                   t.ntx, t.nty, t.zc, t.lx);
         } else {
             k_compose_adjoint2<<<blocks_for(g.nv), kDiffeoThreads, 0, s>>>(g, u, gin, out, acc,
                                                                            mcur);

@@ -66,6 +66,23 @@ cudaError_t launch_similarity_scalars(const Grid &g, int kind, int window, doubl
 // no workspace size depends on it.
 int device_sms();
 
+// log2 of the x extent of a marching tile of 256 columns: 32, or 16, 8 or 4 for rows of up to
+// 64 voxels where that uses more lanes (a line of 32 bytes a row still comes whole).
+inline int march_lx(int X)
+{
+    int best = 5;
+    double cost = 0.0;
+    for (int lx = 5; lx >= 2 && X <= 64; --lx) {
+        const double idle[4] = {1.4, 1.15, 1.05, 1.0};  // the rows' shorter accesses
+        const double c = (((X + (1 << lx) - 1) >> lx) << lx) * idle[lx - 2];
+        if (lx == 5 || c < cost) {
+            cost = c;
+            best = lx;
+        }
+    }
+    return best;
+}
+
 // LCC statistics + exact gradient, shared by the unfused similarity and the
 // fused objective: grad_unscaled = dS/dW * |X_m| (nullable; needs `coef`,
 // lcc_coef_bytes(g) of scratch), per-block {sum of rho over masked voxels, masked
