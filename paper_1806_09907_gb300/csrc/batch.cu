@@ -45,6 +45,7 @@ struct al_batch {
     size_t off_counters = 0, off_err = 0, off_desc = 0, off_items = 0, total = 0;
     int ntiles = 1;
     int tile = 0;                       // brick tile of the batch kernel in use
+    int kernel = 0;                     // tile, or kBatchSmall
     int nitems = 0;                     // items of one iteration with that tile
     int policy = 1;
     int blocks = 0;
@@ -65,6 +66,7 @@ namespace {
 //  3: every Gram tile first (largest problem first), then the bricks.
 std::vector<BatchItem> make_items(const al_batch &b, int policy)
 {
+    const bool by_component = b.kernel == kBatchSmall;
     const int n = (int)b.prob.size(), t = b.tile;
     std::vector<int> order(n);
     for (int i = 0; i < n; ++i)
@@ -73,6 +75,10 @@ std::vector<BatchItem> make_items(const al_batch &b, int policy)
         std::stable_sort(order.begin(), order.end(),
                          [&](int a, int c) { return b.prob[a].work > b.prob[c].work; });
     std::vector<BatchItem> v;
+    auto push_gram = [&](int i, int tile) {
+        for (int c = 0; c < (by_component ? b.prob[i].g.ndim : 1); ++c)
+            v.push_back({i, BATCH_GRAM, tile, c});
+    };
     if (policy == 2) {
         std::vector<int> nb(n, 0), ng(n, 0);
         bool more = true;
@@ -84,7 +90,7 @@ std::vector<BatchItem> make_items(const al_batch &b, int policy)
                     v.push_back({i, BATCH_BRICK, nb[i]++, 0});
                     more = true;
                 } else if (ng[i] < p.gtiles) {
-                    v.push_back({i, BATCH_GRAM, ng[i]++, 0});
+                    push_gram(i, ng[i]++);
                     more = true;
                 }
             }
@@ -92,7 +98,7 @@ std::vector<BatchItem> make_items(const al_batch &b, int policy)
     } else if (policy == 3) {
         for (int i : order)
             for (int t = 0; t < b.prob[i].gtiles; ++t)
-                v.push_back({i, BATCH_GRAM, t, 0});
+                push_gram(i, t);
         for (int i : order)
             for (int k = 0; k < b.prob[i].nbricks[t]; ++k)
                 v.push_back({i, BATCH_BRICK, k, 0});
@@ -101,7 +107,7 @@ std::vector<BatchItem> make_items(const al_batch &b, int policy)
             for (int k = 0; k < b.prob[i].nbricks[t]; ++k)
                 v.push_back({i, BATCH_BRICK, k, 0});
             for (int t = 0; t < b.prob[i].gtiles; ++t)
-                v.push_back({i, BATCH_GRAM, t, 0});
+                push_gram(i, t);
         }
     }
     for (int i : order)
@@ -110,19 +116,33 @@ std::vector<BatchItem> make_items(const al_batch &b, int policy)
     return v;
 }
 
-int count_items(const al_batch &b, int t)
+int count_items(const al_batch &b, int t, bool by_component)
 {
     int n = 0;
     for (const ProbPlan &p : b.prob)
-        n += p.nbricks[t] + p.gtiles + p.nchunks[t];
+        n += p.nbricks[t] + (by_component ? p.ngram : p.gtiles) + p.nchunks[t];
     return n;
+}
+
+// Kernel of brick tile t: tile 0's for few bricks up to 200 of them (160 at spacing 4), hardly more
+// than one for each of a GB300's 152 SMs. Time of the larger kernel over the smaller one's, by bricks:
+// spacing 8 130 1.25, 176 1.01, 208 1.03, 288 0.95; spacing 6 90 1.39, 192 1.08, 221 0.99; spacing 4
+// 128 1.18, 152 1.04, 190 0.86. The same coefficients, bit for bit.
+int tile_kernel(const al_batch &b, int t)
+{
+    int64_t bricks = 0;
+    for (const ProbPlan &p : b.prob)
+        bricks += p.nbricks[t];
+    return t == 0 && bricks <= (b.delta == 4 ? 160 : 200) ? kBatchSmall : t;
 }
 
 // Select brick tile t: the descriptors' brick geometry, the launch size and
 // the work items (in the current order) follow it.
 al_status use_tile(al_batch &b, int t)
 {
-    const int occ = batch_blocks_per_sm(b.delta, t);
+    const int kernel = tile_kernel(b, t);
+    const bool by_component = kernel == kBatchSmall;
+    const int occ = batch_blocks_per_sm(b.delta, kernel);
     if (occ < 1)
         return AL_ERR_CUDA;
     for (size_t i = 0; i < b.prob.size(); ++i) {
@@ -132,14 +152,15 @@ al_status use_tile(al_batch &b, int t)
         q.gby = p.gb[t][1];
         q.gbz = p.gb[t][2];
         q.nbricks = p.nbricks[t];
-        q.nA = p.nbricks[t] + p.gtiles;
+        q.nA = p.nbricks[t] + (by_component ? p.ngram : p.gtiles);
         q.nchunks = p.nchunks[t];
     }
     if (cudaMemcpy(b.ws + b.off_desc, b.desc.data(), sizeof(BatchProblem) * b.desc.size(),
                    cudaMemcpyHostToDevice) != cudaSuccess)
         return AL_ERR_CUDA;
     b.tile = t;
-    b.nitems = count_items(b, t);
+    b.kernel = kernel;
+    b.nitems = count_items(b, t, by_component);
     b.blocks = occ * device_sms();  // persistent: resident blocks of every SM
     const std::vector<BatchItem> v = make_items(b, b.policy);
     if (cudaMemcpy(b.ws + b.off_items, v.data(), v.size() * sizeof(BatchItem),
@@ -166,7 +187,7 @@ al_status launch_step(const al_batch &b, const BatchStep &st, cudaStream_t s)
     if (cudaMemsetAsync(counters, 0, sizeof(int) * (1 + b.prob.size()), s) != cudaSuccess)
         return AL_ERR_CUDA;
     const int blocks = b.blocks > 0 ? b.blocks : device_sms();
-    return launched(launch_batch(b.delta, b.tile, blocks,
+    return launched(launch_batch(b.delta, b.kernel, blocks,
                                  (const BatchProblem *)(b.ws + b.off_desc),
                                  (const BatchItem *)(b.ws + b.off_items), b.nitems, counters, st,
                                  s));
@@ -244,8 +265,7 @@ al_status al_batch_create(const al_problem *problems, int32_t count, al_batch **
     }
     b->delta = problems[0].bs.spacing;
     for (int t = 0; t < b->ntiles; ++t)
-        nitems = std::max(nitems, count_items(*b, t));
-    b->nitems = count_items(*b, 0);
+        nitems = std::max(nitems, count_items(*b, t, t == 0));
     b->off_items = off;
     off += a256(sizeof(BatchItem) * (size_t)nitems);
     for (ProbPlan &p : b->prob) {
@@ -417,7 +437,6 @@ al_status al_batch_set_tile(al_batch *b, int32_t tile)
         return AL_ERR_INVALID_ARG;
     if (!b->ws) {
         b->tile = tile;
-        b->nitems = count_items(*b, tile);
         return AL_OK;
     }
     return use_tile(*b, tile);

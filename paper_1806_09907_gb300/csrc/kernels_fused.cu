@@ -55,12 +55,20 @@ __host__ __device__ constexpr int brick_bcz(int ndim) { return ndim == 3 ? 4 : 1
 //   spacing 6: (4, 3, 2), (4, 3, 1), (3, 3, 2)
 //   spacing 8: (4, 3, 2), (3, 3, 1), (3, 4, 2)
 constexpr int kBatchTiles = 3;
+// Tile 0 of a batch of few bricks (batch.cu: use_tile): one block per SM, a thread per column
+// and a Gram tile's components apart, so that the items, which no SM has more than one or two
+// of, are short. One problem of 64 x 64 x 20 / 97 x 141 x 173 at spacing 8 and of
+// 400 x 30 x 30 at 4: 50, 67 and 47 us with tile 0's kernel, 43, 50 and 33 so.
 __host__ __device__ constexpr int batch_tile_bcx(int delta, int t)
 {
+    if (t == kBatchSmall)
+        t = 0;
     return delta <= 4 ? (t == 2 ? 6 : 8) : (t == 0 || (t == 1 && delta == 6) ? 4 : 3);
 }
 __host__ __device__ constexpr int batch_tile_bcy(int delta, int t)
 {
+    if (t == kBatchSmall)
+        t = 0;
     return delta <= 4 ? 4 : (delta == 8 && t == 2 ? 4 : 3);
 }
 // Voxel columns per thread. At spacing 8 a brick has 768 columns; one thread each
@@ -72,11 +80,11 @@ __host__ __device__ constexpr int batch_tile_bcy(int delta, int t)
 // are two blocks per SM already.
 __host__ __device__ constexpr int batch_tile_cp(int delta, int t)
 {
-    return delta == 8 && t != 1 ? 2 : 1;
+    return delta == 8 && t != 1 && t != kBatchSmall ? 2 : 1;
 }
 __host__ __device__ constexpr int batch_tile_minb(int delta, int t)
 {
-    return batch_tile_cp(delta, t) == 2 ? 2 : delta == 8 || t == 1 ? 1 : 2;
+    return batch_tile_cp(delta, t) == 2 ? 2 : delta == 8 || t == 1 || t == kBatchSmall ? 1 : 2;
 }
 
 template <int D, int DELTA, int MODE, int BCX_ = brick_bcx(DELTA),
@@ -1939,7 +1947,8 @@ struct BCfg {
     static constexpr int MINB = batch_tile_minb(DELTA, T);  // resident blocks per SM
     static_assert(C2::THREADS == THREADS, "2D and 3D bricks share the block size");
     static constexpr size_t fsm = C3::dyn_smem > C2::dyn_smem ? C3::dyn_smem : C2::dyn_smem;
-    static constexpr size_t gsm = (size_t)gram3_floats(3) * sizeof(float);  // > the 2D tile
+    static constexpr bool SMALL = T == kBatchSmall;  // Gram tiles by component
+    static constexpr size_t gsm = (size_t)gram3_floats(SMALL ? 1 : 3) * sizeof(float);  // > 2D
     static constexpr size_t dyn_smem = fsm > gsm ? fsm : gsm;
 };
 
@@ -2015,16 +2024,18 @@ __global__ void __launch_bounds__(BCfg<DELTA, T>::THREADS, BCfg<DELTA, T>::MINB)
                                                           nullptr, nullptr, P.bpart, P.mpart, bx,
                                                           by, bz, w.idx);
         } else if (w.kind == BATCH_GRAM) {
-            // tile w.idx = (tz * gty + ty) * gtx + tx of every component
+            // tile w.idx = (tz * gty + ty) * gtx + tx of every component, or of w.comp
             const int tx = w.idx % P.gtx, r = w.idx / P.gtx, ty = r % P.gty, tz = r / P.gty;
             const int ntiles = P.gtx * P.gty * P.gtz;
             extern __shared__ float bsm[];
+            constexpr bool SMALL = BCfg<DELTA, T>::SMALL;
+            double *rpart = P.rpart + (SMALL ? w.comp * ntiles : 0) + w.idx;
             if (P.g.ndim == 3)
-                gram3_tile<3>(P.g, P.L, P.c, P.gscale, P.gR, tx, ty, tz, 0, P.rpart + w.idx, ntiles,
-                              bsm);
+                gram3_tile<SMALL ? 1 : 3>(P.g, P.L, P.c, P.gscale, P.gR, tx, ty, tz,
+                                          SMALL ? w.comp : 0, rpart, ntiles, bsm);
             else
-                gram2_tile<2>(P.g, P.L, P.c, P.gscale, P.gR, tx, ty, 0, P.rpart + w.idx, ntiles,
-                              bsm);
+                gram2_tile<SMALL ? 1 : 2>(P.g, P.L, P.c, P.gscale, P.gR, tx, ty,
+                                          SMALL ? w.comp : 0, rpart, ntiles, bsm);
         }
         if (w.kind != BATCH_CTRL) {
             __syncthreads();  // every write of the item has been issued
@@ -2103,12 +2114,15 @@ int batch_occupancy()
     case 4 * 16 + 0: return CALL(4, 0);                     \
     case 4 * 16 + 1: return CALL(4, 1);                     \
     case 4 * 16 + 2: return CALL(4, 2);                     \
+    case 4 * 16 + 3: return CALL(4, kBatchSmall);           \
     case 6 * 16 + 0: return CALL(6, 0);                     \
     case 6 * 16 + 1: return CALL(6, 1);                     \
     case 6 * 16 + 2: return CALL(6, 2);                     \
+    case 6 * 16 + 3: return CALL(6, kBatchSmall);           \
     case 8 * 16 + 0: return CALL(8, 0);                     \
     case 8 * 16 + 1: return CALL(8, 1);                     \
     case 8 * 16 + 2: return CALL(8, 2);                     \
+    case 8 * 16 + 3: return CALL(8, kBatchSmall);           \
     }                                                       \
     return fail;
 

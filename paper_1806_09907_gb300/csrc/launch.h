@@ -177,7 +177,7 @@ struct BatchProblem {
 
 enum { BATCH_BRICK = 0, BATCH_GRAM = 1, BATCH_CTRL = 2 };
 struct BatchItem {
-    int prob, kind, idx, pad;
+    int prob, kind, idx, comp;  // comp: a Gram tile's component with kBatchSmall
 };
 
 // Arguments of one batched iteration.
@@ -196,6 +196,7 @@ struct BatchStep {
 // 0: the single-problem path's brick). Geometry of a problem in a batch of
 // spacing delta with a tile: brick grid, Gram tiles, floats of one brick's
 // partials and doubles of its moments.
+constexpr int kBatchSmall = 3;  // kernel of tile 0 for few bricks; not one of the tiles
 int batch_tiles();
 void batch_tile_cells(int delta, int tile, int *bcx, int *bcy);
 void batch_geometry(const Grid &g, const Lattice &L, int tile, int *gb, int *gt, int *npart,
