@@ -1604,9 +1604,9 @@ struct GramBlocks {
 // Resident blocks per SM the kernels are compiled for. The forward pass (FWD)
 // writes no partials, so its bricks are of one or two cells in y, 256-288 threads,
 // four blocks per SM, and gather: 256 x 256 x 160 and 7^3 windows, one evaluation at
-// spacing 4 / 6 / 8 458 / 422 / 394 us with the larger bricks staged by TMA,
-// 430 / 419 / 389 so; a 128 x 128 x 80 iteration 91 -> 89. Small bricks staged by TMA
-// took 444 / 433 / 390 us, three blocks 444 / 425 / 392.
+// spacing 4 / 6 / 8 458 / 420 / 394 us with the larger bricks staged by TMA,
+// 430 / 420 / 389 so (no gain at 6); a 128 x 128 x 80 iteration 92 -> 90. Small bricks staged by
+// TMA took 444 / 433 / 390 us, three blocks 444 / 425 / 392.
 constexpr int fused_minb(int mode, int threads)
 {
     return mode == MODE_FWD ? 4 : threads <= 512 && mode != MODE_NCC ? 2 : 1;
@@ -1651,8 +1651,7 @@ __global__ void __launch_bounds__(FCfg<3, DELTA, MODE>::THREADS, fused_minb(MODE
     k_fused_tma(const __grid_constant__ CUtensorMap mapM, const __grid_constant__ CUtensorMap mapF,
                 const __grid_constant__ CUtensorMap mapC, int3 lb, Grid g, Lattice L,
                 const float *__restrict__ F, const float *__restrict__ M,
-                const float *__restrict__ c, float *__restrict__ W_out,
-                uint8_t *__restrict__ m_out, float *__restrict__ G_io, float *__restrict__ bpart,
+                const float *__restrict__ c, float *__restrict__ bpart,
                 double *__restrict__ mpart, GramBlocks gb, ScalBlock sb)
 {
     if (sb.on && blockIdx.x == 0) {
@@ -1667,7 +1666,7 @@ __global__ void __launch_bounds__(FCfg<3, DELTA, MODE>::THREADS, fused_minb(MODE
     if (b < gb.nbricks) {
         const int bx = b % gb.gbx, by = (b / gb.gbx) % gb.gby, bz = b / (gb.gbx * gb.gby);
         fused_brick<3, DELTA, MODE, brick_bcx(DELTA), mode_bcy(MODE, DELTA), true>(
-            g, L, F, M, c, nullptr, W_out, m_out, G_io, bpart, mpart, bx, by, bz, b,
+            g, L, F, M, c, nullptr, nullptr, nullptr, nullptr, bpart, mpart, bx, by, bz, b,
             BrickMaps{&mapM, &mapF, &mapC, lb.x, lb.y, lb.z}, gb.icnt);
         return;
     }
@@ -1763,7 +1762,7 @@ cudaError_t run_fused_kernel(const Grid &g, const Lattice &L, const Layout &lay,
             if (e != cudaSuccess)
                 return e;
             k_fused_tma<DELTA, MODE><<<sb.on + gb.nbricks, C::THREADS, tdyn, s>>>(
-                mW, mG, mC, int3{0, 0, 0}, g, L, F, M, c, Wo, mo, G, (float *)(ws + lay.bpart),
+                mW, mG, mC, int3{0, 0, 0}, g, L, F, M, c, (float *)(ws + lay.bpart),
                 (double *)(ws + lay.mpart), gb, sb);
             return cudaGetLastError();
         }
@@ -1780,7 +1779,7 @@ cudaError_t run_fused_kernel(const Grid &g, const Lattice &L, const Layout &lay,
             if (e != cudaSuccess)
                 return e;
             k_fused_tma<DELTA, MODE><<<sb.on + gb.nbricks + gb.ngram, C::THREADS, tdyn, s>>>(
-                mM, mF, mC, int3{lbox, lslot, lplane}, g, L, F, M, c, Wo, mo, G,
+                mM, mF, mC, int3{lbox, lslot, lplane}, g, L, F, M, c,
                 (float *)(ws + lay.bpart), (double *)(ws + lay.mpart), gb, sb);
             return cudaGetLastError();
         }

@@ -4,9 +4,9 @@
 // levels (multi-resolution strategy of Sec. IV-A).
 //
 // All three are light: Adam streams 7 floats per coefficient (0.19 M
-// coefficients at 256x256x160, spacing 6), the pyramid reads an image once per
-// axis pass, the refinement gathers at most 27 coarse coefficients per fine
-// one. They are plain elementwise / gather kernels sized to the data; what
+// coefficients at 256x256x160, spacing 6), the pyramid reads an image once,
+// the refinement gathers at most 27 coarse coefficients per fine
+// one. They are elementwise, filter and gather kernels sized to the data; what
 // matters is that the whole loop stays on the device (no host round trip per
 // iteration) so that a level's iterations can be captured in a CUDA graph.
 #include "launch.h"
