@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(kTileX *kTileY)
 // wins), for al_exp_field_adjoint's fixed point.
 // The thread's part of R |X| as an FP64 sum, for terms that a Sum2 does not take.
 template <int D>
-__device__ __noinline__ double regulariser_wide(const Grid &g, const March &mp,
+__device__ __forceinline__ double regulariser_wide(const Grid &g, const March &mp,
                                                 const float *__restrict__ u)
 {
     double total = 0.0;
