@@ -1311,7 +1311,8 @@ __device__ __forceinline__ int class_ntaps(int cls);
 // Warps: the first 8 (16 for the input adjoints, whose epilogues read and write
 // the most) take the epilogue, the warps of a TMEM quarter sharing its columns;
 // one issues the MMAs; the others stage the slabs (16-byte asynchronous copies
-// along rows) into a ring, two in flight. D is double buffered in TMEM, so
+// along rows) into a ring, two in flight. D is double buffered in TMEM (the weight
+// adjoint drains once per unit; its K steps take the sets in turn), so
 // staging, MMAs and epilogues of successive bands overlap. What it took, measured
 // on 16 x 64^3 -> 32^3, 16 -> 32 channels, stride 2 (forward / input adjoint /
 // weight adjoint):
